@@ -116,11 +116,10 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
     // per direction: reconstruction and Riemann fluxes, flattener, cell factors
     for (int d = 0; d < 3; ++d) {
       if (!p.act[d]) continue;
-      long long wf = 1, wc = 1, ws = 1;
+      long long wf = 1, wc = 1;
       for (int e = 0; e < 3; ++e) {
         wf *= (e == d) ? bx.n[e] + 1 : (bx.n[e] > 1 ? bx.n[e] + 2 : 1);
         wc *= bx.n[e] > 1 ? bx.n[e] + 2 : 1;
-        ws *= bx.n[e] > 1 ? bx.n[e] + (e == d ? 4 : 2) : 1;
       }
       const double* chi_s = a.chi + ((size_t)s * 3 + d) * 2 * nt;
       const double* chi_prev = s > 0 ? a.chi + ((size_t)(s - 1) * 3 + d) * 2 * nt : nullptr;
@@ -129,9 +128,8 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
       HR_ACHECK(cudaMemsetAsync(a.gE, 0, 24 * (size_t)nt * sizeof(double), st));
       HR_ACHECK(cudaMemsetAsync(a.gaux, 0, 3 * (size_t)nt * sizeof(double), st));
       const double* flat = p.recon == 0 ? chi_s : aux;  // not read for MC
+      recon<MET>(c, d, Pg, aux, flat, E, 256, 16);
       if (d == 0) {
-        k_slopes<MET, double, 0><<<G(ws), 128, 0, st>>>(p, c->dboxes, 1, Pg, aux, (double*)c->slope);
-        k_edges<MET, double, 0><<<G(wc), 128, 0, st>>>(p, c->dboxes, 1, Pg, aux, flat, (double*)c->slope, E);
         ka_face<MET, 0><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[0], a.gE, a.gk, a.gFS[0]);
         ka_edges<MET, 0><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, flat, a.gE, a.gP, a.gchi);
         if (p.recon == 0) {
@@ -139,8 +137,6 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
           ka_prep<MET, 0><<<G(nt), 128, 0, st>>>(p, bx, Pg, K, a.gaux, a.gP, a.gk);
         }
       } else if (d == 1) {
-        k_slopes<MET, double, 1><<<G(ws), 128, 0, st>>>(p, c->dboxes, 1, Pg, aux, (double*)c->slope);
-        k_edges<MET, double, 1><<<G(wc), 128, 0, st>>>(p, c->dboxes, 1, Pg, aux, flat, (double*)c->slope, E);
         ka_face<MET, 1><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[1], a.gE, a.gk, a.gFS[1]);
         ka_edges<MET, 1><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, flat, a.gE, a.gP, a.gchi);
         if (p.recon == 0) {
@@ -148,8 +144,6 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
           ka_prep<MET, 1><<<G(nt), 128, 0, st>>>(p, bx, Pg, K, a.gaux, a.gP, a.gk);
         }
       } else {
-        k_slopes<MET, double, 2><<<G(ws), 128, 0, st>>>(p, c->dboxes, 1, Pg, aux, (double*)c->slope);
-        k_edges<MET, double, 2><<<G(wc), 128, 0, st>>>(p, c->dboxes, 1, Pg, aux, flat, (double*)c->slope, E);
         ka_face<MET, 2><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[2], a.gE, a.gk, a.gFS[2]);
         ka_edges<MET, 2><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, flat, a.gE, a.gP, a.gchi);
         if (p.recon == 0) {

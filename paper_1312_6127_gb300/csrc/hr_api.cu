@@ -376,7 +376,7 @@ void free_adjoint(harmrad_ctx* c) {
 void free_all(harmrad_ctx* c) {
   free_adjoint(c);
   void* ptrs[] = {c->P, c->K, c->geotab, c->Un, c->F[0], c->F[1], c->F[2], c->spd[0], c->spd[1], c->spd[2],
-                  c->aux, c->flat[0], c->flat[1], c->flat[2], c->emf, c->edges, c->slope, c->dt, c->status,
+                  c->aux, c->flat[0], c->flat[1], c->flat[2], c->emf, c->edges, c->dt, c->status,
                   c->iters, c->failed, c->qcount, c->czone, c->cbox, c->cdata, c->qzone, c->qbox, c->qdata, c->fzone, c->fbox,
                   c->ftmp, c->stats, c->dtmin, c->stage_buf, c->flag, c->dboxes, c->imex_ust, c->imex_psol,
                   c->imex_M, c->sig, c->Sn, c->FS[0], c->FS[1], c->FS[2], c->Bf[0], c->Bf[1], c->Bf[2],
@@ -491,7 +491,6 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     rc = rc ? rc : dalloc(&c->vel, 3 * nt * rs);
   }
   rc = rc ? rc : dalloc(&c->edges, 24 * nt * rs);
-  rc = rc ? rc : dalloc(&c->slope, 12 * nt * rs);
   rc = rc ? rc : dalloc(&c->dt, count * sizeof(double));
   rc = rc ? rc : dalloc(&c->status, na);
   rc = rc ? rc : dalloc(&c->iters, na * sizeof(int));

@@ -45,7 +45,6 @@ struct harmrad_ctx {
   void* vel;
   void* emf3[3];
   void* edges;  // [2][12][ntot] reconstructed edge values of one direction
-  void* slope;  // [12][ntot] MC slopes of one direction
   double* dt;
   unsigned char* status;
   int* iters;

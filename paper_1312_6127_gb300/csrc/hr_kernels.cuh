@@ -414,41 +414,6 @@ __device__ __forceinline__ R mc_slope(R qm, R q0, R qp) {
   return dc > R(0) ? m : -m;
 }
 
-// Branch of mc_slope: 0 opposite one-sided slopes (zero), 1 central,
-// 2 twice the left, 3 twice the right difference.
-template <typename R>
-__device__ __forceinline__ unsigned mc_code(R qm, R q0, R qp) {
-  R dl = q0 - qm, dr = qp - q0, dc = R(0.5) * (qp - qm);
-  if (dl * dr <= R(0)) return 0u;
-  R m = fabs(dc);
-  R a = R(2) * fabs(dl), b = R(2) * fabs(dr);
-  unsigned c = 1u;
-  if (a < m) {
-    m = a;
-    c = 2u;
-  }
-  if (b < m) c = 3u;
-  return c;
-}
-
-// Branch of the PPM monotonicity limiter (ppm_slopes): 0 none, 1 flat,
-// 2 left edge moved, 3 right edge moved.
-template <typename R>
-__device__ __forceinline__ unsigned ppm_code(R sm, R s0, R sp, R dm, R d0, R dp, R chi) {
-  const R sixth = R(1.0 / 6.0);
-  R l = R(0.5) * (sm + s0) - (d0 - dm) * sixth;
-  R r = R(0.5) * (s0 + sp) - (dp - d0) * sixth;
-  R q = s0;
-  l = (R(1) - chi) * l + chi * q;
-  r = (R(1) - chi) * r + chi * q;
-  if ((r - q) * (q - l) <= R(0)) return 1u;
-  R dd = r - l;
-  R m6 = R(6) * (q - R(0.5) * (l + r));
-  if (dd * m6 > dd * dd) return 2u;
-  if (-dd * dd > dd * m6) return 3u;
-  return 0u;
-}
-
 // PPM edge values of the centre of s[0..4] (Colella & Woodward 1984, no
 // contact steepening), flattened toward the cell mean by chi, then limited.
 // sm, s0, sp: the cell and its neighbours; dm, d0, dp: their MC slopes.
@@ -482,81 +447,250 @@ __device__ __forceinline__ void ppm_cell(const R s[5], R chi, R* aL, R* aR) {
 }
 
 // ------------------------------------------------------- edge reconstruction
-// MC slopes of all 12 primitives along d, once per cell: the PPM edges of a
-// cell need the slopes of the cell and of its two neighbours, so computing
-// them here saves two of every three slope evaluations of the edge kernel.
-// Range: cells -2..n_d+1 along d, transverse range widened by one layer.  In
-// r and phi on the Kerr-Schild grid the velocity and field components are
+// FP64 reconstruction of one direction: the PPM parabola (or MC line) of every
+// primitive in every cell of the face range (cells -1..n_d along d, transverse
+// range widened by one layer), flattened by the cell's GAS or RAD flattener and
+// stored as the two edge values E[q] (lower) and E[12 + q] (upper); the face
+// kernel reads the upper edge of cell f-1 and the lower edge of cell f.  In r
+// and phi on the Kerr-Schild grid the velocity and field components are
 // reconstructed as sqrt(-g) times the primitive (Sec. 4.3).
-template <int MET, typename R, int d>
-__global__ void __launch_bounds__(256) k_slopes(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                                const double* __restrict__ P0, const R* __restrict__ aux0,
-                                                R* __restrict__ S0) {
+//
+// Bound by FP64 instructions (each holds an SM's FP64 pipe for 16 clocks), so
+// nothing is computed twice: neighbouring cells share the difference, the MC
+// slope and the interface value between them (a thread walks along d with
+// them in registers, or, along x1, a warp passes them between its lanes), and
+// the limiters work on differences: with a = |r - q|, b = |q - l| the
+// monotonicity tests of Colella & Woodward read b > 2 a and a > 2 b, and twice
+// the MC slope is min(|dl + dr|, 4 |dl|, 4 |dr|).  About 14 FP64 instructions
+// per cell and variable.  One thread (or warp) takes one variable: few
+// registers, many warps, and small grids still fill the SMs.  Measured over an
+// RK3 step (GB300, PPM, Kerr-Schild, event time of the class): 256x128x64
+// 17.2 -> 10.7 ms, 64x32x16 0.75 -> 0.36 ms, 256 zones in 1D 125 -> 27 us,
+// against a slope pass plus a parabola pass of one thread per cell.
+
+// Twice the MC slope from the differences to the left and right neighbour.
+__device__ __forceinline__ double mc_twice(double dm, double dp) {
+  const double s = dm + dp;
+  const double m = 4.0 * (fabs(dm) < fabs(dp) ? dm : dp);
+  const double r = fabs(s) < fabs(m) ? s : m;
+  return (__double2hiint(dm) ^ __double2hiint(dp)) < 0 ? 0.0 : r;
+}
+// Branch of mc_twice: 0 opposite or zero differences (no slope), 1 central, 2 twice
+// the left, 3 twice the right difference.
+__device__ __forceinline__ unsigned mc_twice_code(double dm, double dp) {
+  if ((__double2hiint(dm) ^ __double2hiint(dp)) < 0 || dm == 0.0 || dp == 0.0) return 0u;
+  const bool left = fabs(dm) < fabs(dp);
+  if (fabs(dm + dp) < fabs(4.0 * (left ? dm : dp))) return 1u;
+  return left ? 2u : 3u;
+}
+// PPM interface value between cells of values sm and sm + d whose doubled MC
+// slopes are Dm and D0 (third-order with limited slopes).
+__device__ __forceinline__ double ppm_face(double sm, double d, double Dm, double D0) {
+  return fma(Dm - D0, 1.0 / 12.0, fma(0.5, d, sm));
+}
+// Flattening and monotonicity of the parabola of a cell of value q with edge
+// values l, r; returns the branch: 0 none, 1 flat, 2 left edge moved, 3 right edge
+// moved.
+__device__ __forceinline__ unsigned ppm_limit(double q, double chi, double& l, double& r) {
+  if (chi != 0.0) {
+    l = (1.0 - chi) * l + chi * q;
+    r = (1.0 - chi) * r + chi * q;
+  }
+  const double A = r - q, B = q - l;
+  if ((__double2hiint(A) ^ __double2hiint(B)) < 0) {
+    l = q;
+    r = q;
+    return 1u;
+  }
+  if (fma(-2.0, fabs(A), fabs(B)) > 0.0) {
+    l = fma(-2.0, A, q);
+    return 2u;
+  }
+  if (fma(-2.0, fabs(B), fabs(A)) > 0.0) {
+    r = fma(2.0, B, q);
+    return 3u;
+  }
+  return 0u;
+}
+
+// First item of this thread among the items of a grid whose predecessors in
+// the context hold `done` items: the grids' items form one sequence dealt to
+// the threads in turn, so that a batch of small grids loads every block alike.
+__device__ __forceinline__ long long first_item(long long done) {
+  if (done == 0) return HR_TID;
+  const long long r = HR_TID - done % HR_STRIDE;
+  return r < 0 ? r + HR_STRIDE : r;
+}
+
+// d = 1, 2: a thread walks `chunk` cells of one column along d for one
+// variable; lanes are neighbours along x1, so every load is coalesced.  A
+// chunk's start repeats two slopes and one interface: about one cell's work.
+template <int MET, int d>
+__global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                    const double* __restrict__ P0, const double* __restrict__ aux0,
+                                                    const double* __restrict__ flat0, double* __restrict__ E0,
+                                                    int chunk) {
   const bool weighted = (MET == KS) && (d != 1);
+  constexpr int o = 3 - d;  // the other transverse direction beside x1
+  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const double* P = P0 + 12 * bx.coff;
-    const R* aux = aux0 + 10 * bx.coff;
-    R* S = S0 + 12 * bx.coff;
-    int len[3], off[3];
-    for (int e = 0; e < 3; ++e) {
-      if (bx.n[e] > 1) {
-        len[e] = bx.n[e] + (e == d ? 4 : 2);
-        off[e] = e == d ? -2 : -1;
-      } else {
-        len[e] = 1;
-        off[e] = 0;
+    const double* aux = aux0 + 10 * bx.coff;
+    const double* flat = flat0 + 2 * bx.coff;
+    double* E = E0 + 24 * bx.coff;
+    const int wx = bx.n[0] > 1 ? bx.n[0] + 2 : 1, wo = bx.n[o] > 1 ? bx.n[o] + 2 : 1;
+    const int nd = bx.n[d] + 2, nch = (nd + chunk - 1) / chunk, cols = wx * wo;
+    const long long total = 12LL * nch * cols, st = bx.str[d], nt = bx.ntot;
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+      const int qc = (int)(id / cols), col = (int)(id - (long long)qc * cols);
+      const int q = qc / nch, c0 = (qc - q * nch) * chunk - 1;
+      const int c1 = min(c0 + chunk, bx.n[d] + 1);  // cells c0 .. c1 - 1
+      int ii[3];
+      ii[0] = col % wx + (bx.n[0] > 1 ? -1 : 0);
+      ii[o] = col / wx + (bx.n[o] > 1 ? -1 : 0);
+      ii[d] = c0;
+      long long t = cell_index(bx, ii[0], ii[1], ii[2]);
+      const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
+      const double* Pq = P + q * nt;
+      const double* chi = flat + (q < ER ? 0 : nt);
+      double* El = E + q * nt;
+      double* Er = E + (NPR + q) * nt;
+      auto ld = [&](long long x) { return wq ? aux[x] * Pq[x] : Pq[x]; };
+      double s0 = ld(t), sp = ld(t + st), dp = sp - s0;
+      const double sm = ld(t - st), dm = s0 - sm;
+      double D0 = mc_twice(dm, dp), aL = 0.0;
+      if (p.recon == 0) {
+        const double dmm = sm - ld(t - 2 * st);
+        aL = ppm_face(sm, dm, mc_twice(dmm, dm), D0);
+        if (p.sig && c0 == -1)
+          sig_put(p, bx.coff + t - st, 10 + d, (unsigned long long)q << 8 | mc_twice_code(dmm, dm));
       }
-    }
-    long long total = (long long)len[0] * len[1] * len[2];
-    const long long st = bx.str[d];
-    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
-      long long r = id;
-      int i = (int)(r % len[0]) + off[0];
-      r /= len[0];
-      int j = (int)(r % len[1]) + off[1];
-      int k = (int)(r / len[1]) + off[2];
-      long long t = cell_index(bx, i, j, k);
-      R gw[3];
-      if (weighted) {
-#pragma unroll
-        for (int m = 0; m < 3; ++m) gw[m] = aux[t + (m - 1) * st];
-      }
-#pragma unroll
-      for (int q = 0; q < NPR; ++q) {
-        const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
-        R s[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-          R v = R(P[q * bx.ntot + t + (m - 1) * st]);
-          s[m] = wq ? gw[m] * v : v;
+      double dl = dm;  // kept for the branch signature only
+#pragma unroll 2
+      for (int c = c0; c < c1; ++c, t += st) {
+        if (p.sig) sig_put(p, bx.coff + t, 10 + d, (unsigned long long)q << 8 | mc_twice_code(dl, dp));
+        const double s2 = ld(t + 2 * st), d2 = s2 - sp, Dp = mc_twice(dp, d2);
+        double l, r;
+        if (p.recon == 0) {
+          const double aR = ppm_face(s0, dp, D0, Dp);
+          l = aL;
+          r = aR;
+          const unsigned code = ppm_limit(s0, chi[t], l, r);
+          if (p.sig) sig_put(p, bx.coff + t, 20 + d, (unsigned long long)q << 8 | code);
+          aL = aR;
+        } else {
+          l = fma(-0.25, D0, s0);
+          r = fma(0.25, D0, s0);
         }
-        S[q * bx.ntot + t] = mc_slope<R>(s[0], s[1], s[2]);
-        if (p.sig) sig_put(p, bx.coff + t, 10 + d, (unsigned long long)q << 8 | mc_code<R>(s[0], s[1], s[2]));
+        El[t] = l;
+        Er[t] = r;
+        if (p.sig && c == bx.n[d])
+          sig_put(p, bx.coff + t + st, 10 + d, (unsigned long long)q << 8 | mc_twice_code(dp, d2));
+        s0 = sp;
+        sp = s2;
+        dl = dp;
+        dp = d2;
+        D0 = Dp;
       }
     }
+    done += total;
   }
 }
 
-// One thread per cell of the face range of direction d (cells -1..n_d along d,
-// transverse range widened by one layer): the cell's PPM parabola (or MC
-// slope) for all 12 primitives from the slopes of k_slopes (S0; null: the
-// slopes are computed here, as the FP32 path does), flattened by the
-// cell's GAS or RAD flattener, stored as the two edge values E[0][q] (lower)
-// and E[1][q] (upper).  Every parabola is built once per direction; the face
-// kernel reads the upper edge of cell f-1 and the lower edge of cell f.
-template <int MET, typename R, int d>
+// d = 0: a warp takes 60 consecutive cells of the rows of the transverse range
+// (rows joined end to end, ghosts included) for one variable, two cells per
+// lane, the first and last lane for the neighbours only; differences, slopes
+// and interface values pass between lanes.  Values that cross a row's end
+// reach ghost cells that are not stored.
+template <int MET>
+__global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                    const double* __restrict__ P0, const double* __restrict__ aux0,
+                                                    const double* __restrict__ flat0, double* __restrict__ E0) {
+  const bool weighted = (MET == KS);
+  const int lane = threadIdx.x & 31;
+  const unsigned full = 0xffffffffu;
+  long long done = 0;
+  for (int bi = 0; bi < nbox; ++bi) {
+    const BoxGeo& bx = boxes[bi];
+    const double* P = P0 + 12 * bx.coff;
+    const double* aux = aux0 + 10 * bx.coff;
+    const double* flat = flat0 + 2 * bx.coff;
+    double* E = E0 + 24 * bx.coff;
+    const int w1 = bx.n[1] > 1 ? bx.n[1] + 2 : 1, w2 = bx.n[2] > 1 ? bx.n[2] + 2 : 1;
+    const int o1 = bx.n[1] > 1 ? -1 : 0, o2 = bx.n[2] > 1 ? -1 : 0;
+    const int N0 = bx.N[0], cells = w1 * w2 * N0, ntask = (cells + 59) / 60;
+    const long long total = 12LL * ntask * 32, nt = bx.ntot;
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+      const int task = (int)(id >> 5), q = task / ntask, seg = task - q * ntask;
+      // this lane's two cells and their places in memory
+      int x[2];
+      long long t[2];
+      const int f0 = 60 * seg - 2 + 2 * lane;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int f = min(max(f0 + e, 0), cells - 1), row = f / N0;
+        x[e] = f - row * N0 - 4;
+        t[e] = cell_index(bx, x[e], row % w1 + o1, row / w1 + o2);
+      }
+      const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
+      const double* Pq = P + q * nt;
+      double s[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) s[e] = wq ? aux[t[e]] * Pq[t[e]] : Pq[t[e]];
+      const double sm = __shfl_up_sync(full, s[1], 1);
+      const double d0 = s[0] - sm, d1 = s[1] - s[0], d2 = __shfl_down_sync(full, d0, 1);
+      const double D0 = mc_twice(d0, d1), D1 = mc_twice(d1, d2);
+      double l[2], r[2], chi[2] = {0.0, 0.0};
+      const bool mine = lane >= 1 && lane <= 30 && f0 < cells;
+      unsigned code[2] = {0u, 0u};
+      if (p.recon == 0) {
+        const double* ch = flat + (q < ER ? 0 : nt);
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (x[e] >= -1 && x[e] <= bx.n[0]) chi[e] = ch[t[e]];
+        const double Dm = __shfl_up_sync(full, D1, 1);
+        l[0] = ppm_face(sm, d0, Dm, D0);
+        l[1] = ppm_face(s[0], d1, D0, D1);
+        r[0] = l[1];
+        r[1] = __shfl_down_sync(full, l[0], 1);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) code[e] = ppm_limit(s[e], chi[e], l[e], r[e]);
+      } else {
+        l[0] = fma(-0.25, D0, s[0]);
+        r[0] = fma(0.25, D0, s[0]);
+        l[1] = fma(-0.25, D1, s[1]);
+        r[1] = fma(0.25, D1, s[1]);
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        if (!mine || f0 + e >= cells) continue;
+        if (p.sig && x[e] >= -2 && x[e] <= bx.n[0] + 1)
+          sig_put(p, bx.coff + t[e], 10, (unsigned long long)q << 8 | (e ? mc_twice_code(d1, d2) : mc_twice_code(d0, d1)));
+        if (x[e] < -1 || x[e] > bx.n[0]) continue;
+        if (p.sig && p.recon == 0) sig_put(p, bx.coff + t[e], 20, (unsigned long long)q << 8 | code[e]);
+        E[q * nt + t[e]] = l[e];
+        E[(NPR + q) * nt + t[e]] = r[e];
+      }
+    }
+    done += total;
+  }
+}
+
+// FP32 reconstruction (split precision), one thread per cell of the face range
+// and all 12 primitives: FP32 arithmetic is cheap, so each cell computes its
+// own slopes.
+template <int MET, int d>
 __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                               const double* __restrict__ P0, const R* __restrict__ aux0,
-                                               const R* __restrict__ flat0, const R* __restrict__ S0,
-                                               R* __restrict__ E0) {
+                                               const double* __restrict__ P0, const float* __restrict__ aux0,
+                                               const float* __restrict__ flat0, float* __restrict__ E0) {
+  typedef float R;
   const bool weighted = (MET == KS) && (d != 1);
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const double* P = P0 + 12 * bx.coff;
     const R* aux = aux0 + 10 * bx.coff;
     const R* flat = flat0 + 2 * bx.coff;
-    const R* S = S0 + 12 * bx.coff;
     R* E = E0 + 24 * bx.coff;
     int len[3], off[3];
     for (int e = 0; e < 3; ++e) {
@@ -582,61 +716,27 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
         chg = flat[t];
         chr = flat[bx.ntot + t];
       }
-      if (!S0) {  // slopes computed here (FP32, where arithmetic is cheap)
-        R gw[5];
-        if (weighted) {
+      R gw[5];
+      if (weighted) {
 #pragma unroll
-          for (int m = 0; m < 5; ++m) gw[m] = aux[t + (m - 2) * st];
-        }
-#pragma unroll
-        for (int q = 0; q < NPR; ++q) {
-          const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
-          R s[5];
-#pragma unroll
-          for (int m = 0; m < 5; ++m) {
-            R v = R(P[q * bx.ntot + t + (m - 2) * st]);
-            s[m] = wq ? gw[m] * v : v;
-          }
-          R aL, aR;
-          if (p.recon == 0) {
-            ppm_cell<R>(s, q < ER ? chg : chr, &aL, &aR);
-          } else {
-            R dq = mc_slope<R>(s[1], s[2], s[3]);
-            aL = s[2] - R(0.5) * dq;
-            aR = s[2] + R(0.5) * dq;
-          }
-          E[q * bx.ntot + t] = aL;
-          E[(NPR + q) * bx.ntot + t] = aR;
-        }
-        continue;
-      }
-      R gw[3];
-      if (weighted && p.recon == 0) {
-#pragma unroll
-        for (int m = 0; m < 3; ++m) gw[m] = aux[t + (m - 1) * st];
+        for (int m = 0; m < 5; ++m) gw[m] = aux[t + (m - 2) * st];
       }
 #pragma unroll
       for (int q = 0; q < NPR; ++q) {
         const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
+        R s[5];
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+          R v = R(P[q * bx.ntot + t + (m - 2) * st]);
+          s[m] = wq ? gw[m] * v : v;
+        }
         R aL, aR;
         if (p.recon == 0) {
-          R s[3], ds[3];
-#pragma unroll
-          for (int m = 0; m < 3; ++m) {
-            R v = R(P[q * bx.ntot + t + (m - 1) * st]);
-            s[m] = wq ? gw[m] * v : v;
-            ds[m] = S[q * bx.ntot + t + (m - 1) * st];
-          }
-          ppm_slopes<R>(s[0], s[1], s[2], ds[0], ds[1], ds[2], q < ER ? chg : chr, &aL, &aR);
-          if (p.sig)
-            sig_put(p, bx.coff + t, 20 + d,
-                    (unsigned long long)q << 8 | ppm_code<R>(s[0], s[1], s[2], ds[0], ds[1], ds[2], q < ER ? chg : chr));
+          ppm_cell<R>(s, q < ER ? chg : chr, &aL, &aR);
         } else {
-          R v = R(P[q * bx.ntot + t]);
-          if (wq) v = aux[t] * v;
-          const R dq = S[q * bx.ntot + t];
-          aL = v - R(0.5) * dq;
-          aR = v + R(0.5) * dq;
+          R dq = mc_slope<R>(s[1], s[2], s[3]);
+          aL = s[2] - R(0.5) * dq;
+          aR = s[2] + R(0.5) * dq;
         }
         E[q * bx.ntot + t] = aL;
         E[(NPR + q) * bx.ntot + t] = aR;

@@ -100,6 +100,35 @@ inline int fill_ghost_cells(harmrad_ctx* c) {
   return nk;
 }
 
+// FP64 reconstruction of direction d: edge values of every cell of its face range.
+// A column along x2 or x3 is cut so that there are at least two threads per
+// resident-thread slot, into pieces of 16 cells or more (a piece repeats one
+// cell's work).
+template <int MET>
+void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const double* flat, double* E, int block,
+           int per_sm) {
+  const DevParams& p = c->dp;
+  const BoxGeo* bt = c->dboxes;
+  const int nb = c->nbox;
+  auto width = [](const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; };
+  if (d == 0) {
+    const long long work = max_work(c, [width](const BoxGeo& b) {
+      return 12LL * 32 * (((long long)width(b, 1) * width(b, 2) * b.N[0] + 59) / 60);
+    });
+    k_recon_rows<MET><<<grid_for(work, c->sms, block, per_sm), block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E);
+    return;
+  }
+  const int o = 3 - d;
+  const long long cols = max_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
+  const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
+  long long pieces = (2LL * 2048 * c->sms + 12 * cols - 1) / (12 * cols);
+  if (pieces > (nd + 15) / 16) pieces = (nd + 15) / 16;
+  const int chunk = (int)((nd + pieces - 1) / pieces);
+  const int g = grid_for(12 * cols * pieces, c->sms, block, per_sm);
+  if (d == 1) k_recon_cols<MET, 1><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E, chunk);
+  else k_recon_cols<MET, 2><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E, chunk);
+}
+
 template <int MET, typename R>
 int faces_impl(harmrad_ctx* c, bool fresh) {
   const DevParams& p = c->dp;
@@ -139,52 +168,31 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     });
     const harmrad_tuning& tu = c->tune;
     const int be = tu.edge_block, bf = tu.face_block;
-    const int ge = grid_for(max_work(c, range_cells), c->sms, be, tu.edge_blocks_per_sm);
-    const int gs = grid_for(max_work(c, [d](const BoxGeo& b) {
-                              long long w = 1;
-                              for (int e = 0; e < 3; ++e) w *= b.n[e] > 1 ? b.n[e] + (e == d ? 4 : 2) : 1;
-                              return w;
-                            }),
-                            c->sms, be, tu.edge_blocks_per_sm);
-    // FP64: slopes once per cell in their own pass; FP32: in the edge kernel
-    R* Sl = std::is_same<R, double>::value ? (R*)c->slope : nullptr;
     const int g = grid_for(wf, c->sms, bf, tu.face_blocks_per_sm);
-    const R* aux = (const R*)c->aux;
-    const R* fl = (const R*)c->flat[d];
     R* Ed = (R*)c->edges;
     R* Fd = (R*)c->F[d];
     R* sd = (R*)c->spd[d];
-    if (d == 0) {
-      if (Sl) {
-        k_slopes<MET, R, 0><<<gs, be, 0, st>>>(p, bt, nb, c->P, aux, Sl);
-        mark(c, HARMRAD_K_EDGE);
-        ++nk;
-      }
-      k_edges<MET, R, 0><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Sl, Ed);
-      mark(c, HARMRAD_K_EDGE);
+    if constexpr (std::is_same<R, double>::value) {
+      recon<MET>(c, d, c->P, (const double*)c->aux, (const double*)c->flat[d], (double*)c->edges, be,
+                 tu.edge_blocks_per_sm);
+    } else {
+      const int ge = grid_for(max_work(c, range_cells), c->sms, be, tu.edge_blocks_per_sm);
+      const R* aux = (const R*)c->aux;
+      const R* fl = (const R*)c->flat[d];
+      if (d == 0) k_edges<MET, 0><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Ed);
+      else if (d == 1) k_edges<MET, 1><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Ed);
+      else k_edges<MET, 2><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Ed);
+    }
+    mark(c, HARMRAD_K_EDGE);
+    if (d == 0)
       k_face<MET, R, 0><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[0],
                                            (R*)c->gsp[0]);
-    } else if (d == 1) {
-      if (Sl) {
-        k_slopes<MET, R, 1><<<gs, be, 0, st>>>(p, bt, nb, c->P, aux, Sl);
-        mark(c, HARMRAD_K_EDGE);
-        ++nk;
-      }
-      k_edges<MET, R, 1><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Sl, Ed);
-      mark(c, HARMRAD_K_EDGE);
+    else if (d == 1)
       k_face<MET, R, 1><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[1],
                                            (R*)c->gsp[1]);
-    } else {
-      if (Sl) {
-        k_slopes<MET, R, 2><<<gs, be, 0, st>>>(p, bt, nb, c->P, aux, Sl);
-        mark(c, HARMRAD_K_EDGE);
-        ++nk;
-      }
-      k_edges<MET, R, 2><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Sl, Ed);
-      mark(c, HARMRAD_K_EDGE);
+    else
       k_face<MET, R, 2><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[2],
                                            (R*)c->gsp[2]);
-    }
     mark(c, HARMRAD_K_FACE);
     nk += 2;
   }
