@@ -81,10 +81,14 @@ __device__ __forceinline__ double kfield(const DevParams& p, const double* K, lo
 // The FP64 kernels then read 16 doubles (L2-resident: a few MB per grid)
 // instead of evaluating exp, sin, cos and four divisions per zone and face,
 // which matters because the step is bound by FP64 arithmetic.
-// Layout of a grid's table (offset BoxGeo::goff, in doubles): [16][N2][N1]
-// centres, [16][N2][N1] centre derivatives, [16][N2][n1+1] x1 faces,
-// [16][n2+1][N1] x2 faces; fields in the order of Geo (g00 g01 g03 g11 g13
+// Layout of a grid's table (offset BoxGeo::goff, in doubles): [GEO_C][N2][N1]
+// centres, [16][N2][N1] centre derivatives, [GEO_F][N2][n1+1] x1 faces,
+// [GEO_F][n2+1][N1] x2 faces; fields in the order of Geo (g00 g01 g03 g11 g13
 // g22 g33 G00 G01 G11 G13 G22 G33 gdet alpha ialpha) and of MetricDeriv.
+// Centres add 1/sqrt(-g) (plane 16) and sqrt(g_dd) of the three directions
+// (17..19), faces 1/sqrt(-g) (16) and sqrt(g_dd) of their direction (17):
+// each saves a division or a square root per zone or face.
+constexpr int GEO_C = 20, GEO_F = 18;
 struct GeoTab {
   const double* C;
   const double* M;
@@ -95,7 +99,7 @@ struct GeoTab {
 
 __host__ __device__ __forceinline__ long long geotab_size(const BoxGeo& b) {
   const long long sC = (long long)b.N[0] * b.N[1];
-  return 16 * (2 * sC + (long long)(b.n[0] + 1) * b.N[1] + (long long)b.N[0] * (b.n[1] + 1));
+  return (GEO_C + 16) * sC + GEO_F * ((long long)(b.n[0] + 1) * b.N[1] + (long long)b.N[0] * (b.n[1] + 1));
 }
 
 __device__ __forceinline__ GeoTab geotab(const double* base, const BoxGeo& b) {
@@ -104,9 +108,9 @@ __device__ __forceinline__ GeoTab geotab(const double* base, const BoxGeo& b) {
   t.sF0 = (long long)(b.n[0] + 1) * b.N[1];
   t.sF1 = (long long)b.N[0] * (b.n[1] + 1);
   t.C = base + b.goff;
-  t.M = t.C + 16 * t.sC;
+  t.M = t.C + GEO_C * t.sC;
   t.F0 = t.M + 16 * t.sC;
-  t.F1 = t.F0 + 16 * t.sF0;
+  t.F1 = t.F0 + GEO_F * t.sF0;
   return t;
 }
 
@@ -875,22 +879,22 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
         continue;
       }
       Geo<MET, R> g;
-      bool tab = false;
+      R igf = R(1), dl = dxd;  // FP64: 1/sqrt(-g) and the cell's proper length along d
       if constexpr (MET == KS && std::is_same<R, double>::value) {
-        if (geo0 && bx.goff >= 0) {
-          const GeoTab T = geotab(geo0, bx);
-          if (d == 0) g = geo_load<MET>(T.F0, T.sF0, gidx_f0(bx, ii[0], ii[1]));
-          else if (d == 1) g = geo_load<MET>(T.F1, T.sF1, gidx_f1(bx, ii[0], ii[1]));
-          else g = geo_load<MET>(T.C, T.sC, gidx_c(bx, ii[0], ii[1]));
-          tab = true;
-        }
-      }
-      if (!tab) {
+        const GeoTab T = geotab(geo0, bx);
+        const double* tab = d == 0 ? T.F0 : (d == 1 ? T.F1 : T.C);
+        const long long sz = d == 0 ? T.sF0 : (d == 1 ? T.sF1 : T.sC);
+        const long long x = d == 0 ? gidx_f0(bx, ii[0], ii[1])
+                                   : (d == 1 ? gidx_f1(bx, ii[0], ii[1]) : gidx_c(bx, ii[0], ii[1]));
+        g = geo_load<MET>(tab, sz, x);
+        if (weighted) igf = __ldg(tab + 16 * sz + x);
+        dl = dxd * __ldg(tab + (d == 2 ? 19 : 17) * sz + x);
+      } else {
         R xf[3];
         for (int e = 0; e < 3; ++e) xf[e] = R(bx.x0[e] + (ii[e] + (e == d ? 0.0 : 0.5)) * bx.dx[e]);
         g = make_geo<MET, R>(p, xf[0], xf[1]);
+        igf = weighted ? R(1) / g.gdet : R(1);
       }
-      const R igf = weighted ? R(1) / g.gdet : R(1);
       R PL[NPR], PR[NPR];
 #pragma unroll
       for (int q = 0; q < NPR; ++q) {
@@ -904,8 +908,12 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
       R out[NPR], smax;
       unsigned fcode = 0;
       R fsv, gs[2];
-      face_flux<MET, R, d>(p, g, dxd, kL, kR, R(p.kscale), PL, PR, out, &smax, p.sig ? &fcode : nullptr,
-                           FS ? &fsv : nullptr, gs);
+      if constexpr (std::is_same<R, double>::value)
+        face_flux64<MET, d + 1>(p, g, dl, kL, kR, PL, PR, out, &smax, p.sig ? &fcode : nullptr, FS ? &fsv : nullptr,
+                                gsp ? gs : nullptr);
+      else
+        face_flux<MET, R, d>(p, g, dxd, kL, kR, R(p.kscale), PL, PR, out, &smax, p.sig ? &fcode : nullptr,
+                             FS ? &fsv : nullptr, gs);
       if (p.sig) sig_put(p, bx.coff + t, 40 + d, fcode);
       if (FS) FS[t] = fsv;
       if (gsp) {
@@ -1361,7 +1369,12 @@ static __global__ void k_geo_init(DevParams p, const BoxGeo* __restrict__ boxes,
       if (id < T.sC) {  // centres and their derivatives
         const int i = (int)(id % bx.N[0]) - bx.ng[0], j = (int)(id / bx.N[0]) - bx.ng[1];
         const double x1 = xcen(bx, 0, i), x2 = xcen(bx, 1, j);
-        geo_store<KS>(C, T.sC, id, make_geo<KS, double>(p, x1, x2));
+        const Geo<KS, double> g = make_geo<KS, double>(p, x1, x2);
+        geo_store<KS>(C, T.sC, id, g);
+        C[16 * T.sC + id] = 1.0 / g.gdet;
+        C[17 * T.sC + id] = sqrt(g.g11);
+        C[18 * T.sC + id] = sqrt(g.g22);
+        C[19 * T.sC + id] = sqrt(g.g33);
         const MetricDeriv md = ks_derivs(p, x1, x2);
         const double* v = reinterpret_cast<const double*>(&md);
         for (int f = 0; f < 16; ++f) M[f * T.sC + id] = v[f];
@@ -1369,12 +1382,18 @@ static __global__ void k_geo_init(DevParams p, const BoxGeo* __restrict__ boxes,
         const long long e = id - T.sC;
         const int i = (int)(e % (bx.n[0] + 1)), j = (int)(e / (bx.n[0] + 1)) - bx.ng[1];
         const double x1 = bx.x0[0] + (i + 0.0) * bx.dx[0], x2 = bx.x0[1] + (j + 0.5) * bx.dx[1];
-        geo_store<KS>(F0, T.sF0, e, make_geo<KS, double>(p, x1, x2));
+        const Geo<KS, double> g = make_geo<KS, double>(p, x1, x2);
+        geo_store<KS>(F0, T.sF0, e, g);
+        F0[16 * T.sF0 + e] = 1.0 / g.gdet;
+        F0[17 * T.sF0 + e] = sqrt(g.g11);
       } else if (id < T.sC + T.sF0 + T.sF1) {  // x2 faces
         const long long e = id - T.sC - T.sF0;
         const int i = (int)(e % bx.N[0]) - bx.ng[0], j = (int)(e / bx.N[0]);
         const double x1 = bx.x0[0] + (i + 0.5) * bx.dx[0], x2 = bx.x0[1] + (j + 0.0) * bx.dx[1];
-        geo_store<KS>(F1, T.sF1, e, make_geo<KS, double>(p, x1, x2));
+        const Geo<KS, double> g = make_geo<KS, double>(p, x1, x2);
+        geo_store<KS>(F1, T.sF1, e, g);
+        F1[16 * T.sF1 + e] = 1.0 / g.gdet;
+        F1[17 * T.sF1 + e] = sqrt(g.g22);
       }
     }
   }

@@ -12,6 +12,7 @@
 #include <type_traits>
 
 #include "hr_dual.cuh"
+#include "hr_math.cuh"
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -509,6 +510,257 @@ __device__ __forceinline__ void face_accum(const DevParams& p, const Geo<MET, R>
   for (int n = 0; n < 4; ++n)
     out[8 + n] += gd * (aFr * (e43 * urc[d] * urv[n] + (n == d ? e13 : R(0))) +
                         aUr * (e43 * urc[0] * urv[n] + (n == 0 ? e13 : R(0))));
+}
+
+// ------------------------------------------------- FP64 face (hot path)
+// The Riemann flux of one face in FP64, arranged for few FP64 instructions
+// (face_speeds and face_accum above state the same physics term by term and
+// serve FP32 and the adjoint's dual numbers).  With l_i = g_ij u~^j = u_i (the
+// ZAMO's n_i vanish): gamma^2 = 1 + u~^i l_i and u_t = -alpha gamma + beta^i l_i,
+// beta^i = alpha^2 g^{ti}; likewise B_mu from m_i = g_ij B^j.  With
+// b_mu = (B_mu + b^t u_mu) / u^t a state's share aF F^d + aU U of every gas row
+// is Z u_mu + Y B_mu + p_tot (aF delta^d_mu + aU delta^t_mu) for two scalars
+// Z and Y per state, and of every radiation row one product.  The dispersion
+// relation (Sec. 4.4) is solved from its discriminant in factored form,
+// c^2 (H + c^2 (C0 - H)), which keeps its digits for small c^2, and
+// c_ms^2 = (Gamma p + b^2) / (w + b^2).  Both states live in registers (210 of
+// them, 2 blocks of 128 threads per SM as with the 184 before), so nothing is
+// formed twice.  Measured over an RK3 step (GB300, event time of the class):
+// 256x128x64 Kerr-Schild torus 28.0 -> 17.6 ms, 64x32x16 0.67 -> 0.45 ms,
+// 93x71x45 Minkowski box with HLL 3.31 -> 2.29 ms.
+
+// Metric factors of a face of direction d (1..3) beside the Geo components.
+template <int MET, int d>
+struct FaceGeo {
+  double a01;  // alpha g^{t1}
+  double b1;   // beta^1 = alpha^2 g^{t1}
+  double C0;   // (g^{td})^2 - g^{dd} g^{tt}
+  __device__ __forceinline__ explicit FaceGeo(const Geo<MET, double>& g) {
+    if constexpr (MET == MINK) {
+      a01 = b1 = 0.0;
+      C0 = 1.0;
+    } else {
+      a01 = g.alpha * g.G01;
+      b1 = g.alpha * a01;
+      C0 = d == 1 ? fma(g.G01, g.G01, -g.G11 * g.G00) : -g.Gdd(d) * g.G00;
+    }
+  }
+};
+
+// g_ij v^j
+template <int MET>
+__device__ __forceinline__ void lower3(const Geo<MET, double>& g, double v1, double v2, double v3, double l[3]) {
+  if constexpr (MET == MINK) {
+    l[0] = v1;
+    l[1] = v2;
+    l[2] = v3;
+  } else {
+    l[0] = fma(g.g13, v3, g.g11 * v1);
+    l[1] = g.g22 * v2;
+    l[2] = fma(g.g33, v3, g.g13 * v1);
+  }
+}
+
+// Absorption plus scattering opacity (opacity_ks) at temperature T(): the
+// temperature is formed only where the opacity depends on it.
+template <class Temp>
+__device__ __forceinline__ double opacity_sum(const DevParams& p, double rho, Temp T, double kf) {
+  double kabs;
+  if (p.opacity == 2) {
+    kabs = p.kscale * kf;
+  } else if (p.opacity == 1) {
+    const double Tg = T(), Tc = Tg > p.Tmin ? Tg : p.Tmin, T2 = Tc * Tc;
+    kabs = p.kscale * p.kabs0 * rho * rho * rsqrt64(T2 * T2 * T2 * Tc);
+  } else {
+    kabs = p.kscale * p.kabs0 * rho;
+  }
+  return fma(p.kscale * p.kes0, rho, kabs);
+}
+
+// One reconstructed state of a face: 4-velocities (contravariant time and d
+// components, covariant components), field, enthalpy and signal speeds
+// (Bq +- sd) iq of the gas [0] and the radiation [1].
+template <int MET, int d>
+struct FaceSide {
+  double u0, u1, l0, l[3], bt, m0, m[3], iut, wb, pt;
+  double r0, rd, k0, k[3];
+  double Bq[2], sd[2], iq[2];
+
+  __device__ __forceinline__ void speeds(const Geo<MET, double>& g, const FaceGeo<MET, d>& f, int w, double ut,
+                                         double ud, double c2) {
+    const double u02 = ut * ut, mix = ut * ud;
+    double H, AB = 0.0;
+    if constexpr (MET == MINK) {
+      H = fma(-ud, ud, u02);
+    } else {
+      H = fma(ud * ud, g.G00, u02 * g.Gdd(d));
+      if (d == 1) {
+        AB = g.G01;
+        H = fma(-2.0 * AB, mix, H);
+      }
+    }
+    const double K = c2 * fma(c2, f.C0 - H, H);
+    Bq[w] = d == 1 && MET == KS ? fma(-c2, AB + mix, mix) : fma(-c2, mix, mix);
+    iq[w] = rcp(fma(-c2, g.Gtt() + u02, u02));
+    sd[w] = K > 0.0 ? sqrt64(K) : 0.0;
+  }
+
+  // dl: proper length of the cell along d; kf: its per-zone opacity; code:
+  // branches (1, 2: c_ms^2 clamped, 4: optically thick radiation speed)
+  __device__ __forceinline__ void build(const DevParams& p, const Geo<MET, double>& g, const FaceGeo<MET, d>& f,
+                                        double dl, double kf, const double P[NPR], unsigned* code) {
+    const double rho = P[RHO], pg = (p.gam - 1.0) * P[UU], w = rho + P[UU] + pg;
+    lower3<MET>(g, P[U1], P[U2], P[U3], l);
+    double igm;
+    const double gm = sqrt_rsqrt(fma(P[U1], l[0], fma(P[U2], l[1], fma(P[U3], l[2], 1.0))), &igm);
+    lower3<MET>(g, P[B1], P[B2], P[B3], m);
+    bt = fma(P[B1], l[0], fma(P[B2], l[1], P[B3] * l[2]));
+    const double BB = fma(P[B1], m[0], fma(P[B2], m[1], P[B3] * m[2]));
+    double k2;
+    lower3<MET>(g, P[UR1], P[UR2], P[UR3], k);
+    k2 = sqrt64(fma(P[UR1], k[0], fma(P[UR2], k[1], fma(P[UR3], k[2], 1.0))));
+    if constexpr (MET == MINK) {
+      u0 = gm;
+      u1 = P[U1];
+      l0 = -gm;
+      m0 = 0.0;
+      iut = igm;
+      r0 = k2;
+      k0 = -k2;
+      rd = P[UR1 + d - 1];
+    } else {
+      u0 = gm * g.ialpha;
+      u1 = fma(-gm, f.a01, P[U1]);
+      l0 = fma(f.b1, l[0], -g.alpha * gm);
+      m0 = f.b1 * m[0];
+      iut = g.alpha * igm;
+      r0 = k2 * g.ialpha;
+      k0 = fma(f.b1, k[0], -g.alpha * k2);
+      rd = d == 1 ? fma(-k2, f.a01, P[UR1]) : P[UR1 + d - 1];
+    }
+    const double bsq = fma(bt, bt, BB) * (iut * iut);
+    wb = w + bsq;
+    pt = fma(0.5, bsq, pg);
+    double c2 = fma(p.gam, pg, bsq) * rcp(wb);
+    unsigned cd = 0;
+    if ((unsigned)__double2hiint(c2) >= 0x3ff00000u) {  // at least 1, negative or NaN
+      cd = (c2 > 1.0 ? 1u : 0u) | (c2 < 0.0 ? 2u : 0u);
+      c2 = c2 > 1.0 ? 1.0 : (c2 < 0.0 ? 0.0 : c2);
+    }
+    speeds(g, f, 0, u0, d == 1 ? u1 : P[U1 + d - 1], c2);
+    const double tau = opacity_sum(p, rho, [&] { return pg * rcp(rho); }, kf) * dl;
+    double cr2 = 1.0 / 3.0;
+    if (__double2hiint(tau) >= 0x40020000) {  // tau >= 2.25: (4 / (3 tau))^2 may lie below 1/3
+      const double lim = (4.0 / 3.0) * rcp(tau), l2 = lim * lim;
+      if (l2 < cr2) {
+        cr2 = l2;
+        cd |= 4u;
+      }
+    }
+    speeds(g, f, 1, r0, rd, cr2);
+    if (code) *code = cd;
+  }
+  __device__ __forceinline__ double vmax(int w) const { return (Bq[w] + sd[w]) * iq[w]; }
+  __device__ __forceinline__ double vmin(int w) const { return (Bq[w] - sd[w]) * iq[w]; }
+  __device__ __forceinline__ double vabs(int w) const { return (fabs(Bq[w]) + sd[w]) * iq[w]; }
+
+  // out += aF F + aU U over sqrt(-g), gas rows with (aFg, aUg), radiation with
+  // (aFr, aUr); ONE: aF = 1.  Returns the share of the mass row.
+  template <bool ONE>
+  __device__ __forceinline__ double add(const Geo<MET, double>& g, const double P[NPR], double aFg, double aUg,
+                                        double aFr, double aUr, double out[NPR]) const {
+    (void)g;
+    const double ud = d == 1 ? u1 : P[U1 + d - 1], Bd = P[B1 + d - 1];
+    const double V = ONE ? fma(aUg, u0, ud) : fma(aUg, u0, aFg * ud);
+    const double M = P[RHO] * V, bu = bt * u0, bd = fma(bt, ud, Bd);
+    const double Y = -(iut * iut) * (ONE ? fma(aUg, bu, bd) : fma(aUg, bu, aFg * bd));
+    const double Z = fma(bt, Y, wb * V);
+    out[0] += M;
+    out[1] = fma(Z, l0, fma(Y, m0, fma(aUg, pt, out[1] + M)));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[2 + i] = fma(Z, l[i], fma(Y, m[i], out[2 + i]));
+    out[1 + d] += ONE ? pt : aFg * pt;
+    const double vi = V * iut, Bi = ONE ? Bd * iut : aFg * (Bd * iut);
+#pragma unroll
+    for (int i = 1; i <= 3; ++i)
+      if (i != d) out[4 + i] = fma(vi, P[B1 + i - 1], fma(-Bi, i == 1 ? u1 : P[U1 + i - 1], out[4 + i]));
+    const double E = P[ER], e13 = E * (1.0 / 3.0);
+    const double R = ((4.0 / 3.0) * E) * (ONE ? fma(aUr, r0, rd) : fma(aUr, r0, aFr * rd));
+    out[8] = fma(R, k0, fma(aUr, e13, out[8]));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[9 + i] = fma(R, k[i], out[9 + i]);
+    out[8 + d] += ONE ? e13 : aFr * e13;
+    return M;
+  }
+};
+
+// HLL or LAXF flux of one face (face_flux in FP64): out the 12 rows with
+// F[B_d] = 0, smax the largest speed, fs (optional) the entropy flux, gas
+// (optional) the gas speeds v_max, v_min, code (optional) the branches.
+template <int MET, int d>
+__device__ __forceinline__ void face_flux64(const DevParams& p, const Geo<MET, double>& g, double dl, double kL,
+                                            double kR, const double PL[NPR], const double PR[NPR], double out[NPR],
+                                            double* smax, unsigned* code, double* fs, double* gas) {
+  const FaceGeo<MET, d> f(g);
+  FaceSide<MET, d> L, R;
+  unsigned cL = 0, cR = 0;
+  L.build(p, g, f, dl, kL, PL, code ? &cL : nullptr);
+  R.build(p, g, f, dl, kR, PR, code ? &cR : nullptr);
+  double cp[2], cm[2], c[2];  // v_max, v_min, largest of the gas and the radiation
+  if (p.flux != 0 || gas || code) {
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      cp[w] = fmax(0.0, fmax(L.vmax(w), R.vmax(w)));
+      cm[w] = -fmin(0.0, fmin(L.vmin(w), R.vmin(w)));
+      c[w] = fmax(cp[w], cm[w]);
+    }
+    if (code) {  // which signal speed each maximum took, and the speed caps
+      unsigned k = cL | (cR << 3);
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const double l1 = L.vmax(w), r1 = R.vmax(w), l0 = L.vmin(w), r0 = R.vmin(w);
+        k |= (l1 >= r1 ? 0u : 1u) << (6 + 4 * w) | (0.0 > fmax(l1, r1) ? 1u : 0u) << (7 + 4 * w);
+        k |= (l0 <= r0 ? 0u : 1u) << (8 + 4 * w) | (0.0 < fmin(l0, r0) ? 1u : 0u) << (9 + 4 * w);
+        k |= (cp[w] > cm[w] ? 1u : 0u) << (14 + w);
+      }
+      *code = k;
+    }
+    if (gas) {
+      gas[0] = cp[0];
+      gas[1] = cm[0];
+    }
+  } else {
+#pragma unroll
+    for (int w = 0; w < 2; ++w) c[w] = fmax(L.vabs(w), R.vabs(w));
+  }
+  *smax = fmax(c[0], c[1]);
+#pragma unroll
+  for (int q = 0; q < NPR; ++q) out[q] = 0.0;
+  double mL, mR, sc[2];
+  if (p.flux == 0) {  // LAXF: 1/2 (F_L + F_R - c (U_R - U_L))
+    mL = L.template add<true>(g, PL, 1.0, c[0], 1.0, c[1], out);
+    mR = R.template add<true>(g, PR, 1.0, -c[0], 1.0, -c[1], out);
+    sc[0] = sc[1] = 0.5 * g.gdet;
+  } else {  // HLL: (c- F_R + c+ F_L - c- c+ (U_R - U_L)) / (c- + c+)
+    double aL[2], aR[2], aU[2];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      const double sum = cp[w] + cm[w];
+      const bool ok = sum > 0.0;
+      aL[w] = ok ? cp[w] : 1.0;
+      aR[w] = ok ? cm[w] : 1.0;
+      aU[w] = ok ? cm[w] * cp[w] : 0.0;
+      sc[w] = g.gdet * (ok ? rcp(sum) : 0.5);
+    }
+    mL = L.template add<false>(g, PL, aL[0], aU[0], aL[1], aU[1], out);
+    mR = R.template add<false>(g, PR, aR[0], -aU[0], aR[1], -aU[1], out);
+  }
+  if (fs)  // entropy flux: s_gas times the mass flux of each state (Sec. 2, Eq. S)
+    *fs = sc[0] * fma(entropy_per_baryon<double>(p, PL[RHO], PL[UU]), mL,
+                      entropy_per_baryon<double>(p, PR[RHO], PR[UU]) * mR);
+#pragma unroll
+  for (int q = 0; q < NPR; ++q) out[q] *= sc[q < ER ? 0 : 1];
+  out[B1 + d - 1] = 0.0;
 }
 
 // ------------------------------------------------------ M1 inversion (FP64)
