@@ -337,18 +337,21 @@ void prim_to_cons(const orc_params& p, const Geom& G, const double Gam[4][4][4],
 // Lab-frame characteristic speeds along direction d for a fluid with
 // 4-velocity u and rest-frame signal speed^2 c2 (Sec. 4.4): the covector
 // k_mu = delta^d_mu - v delta^t_mu must satisfy (k.u)^2 = c2 (k.k + (k.u)^2).
+// In extended precision: for small c2 (cold gas, optically thick radiation) the
+// discriminant is c2 times a number of order one, left over from terms of
+// order one, and loses -log10(c2) digits.
 void char_speeds(const Geom& G, const double ucon[4], double c2, int d, double* vmin,
                  double* vmax) {
-  double Au = ucon[d], Bu = ucon[0];
-  double AA = G.gcon[d][d], BB = G.gcon[0][0], AB = G.gcon[0][d];
-  double qa = Bu * Bu - c2 * (BB + Bu * Bu);
-  double qb = -2.0 * (Au * Bu - c2 * (AB + Au * Bu));
-  double qc = Au * Au - c2 * (AA + Au * Au);
-  double disc = qb * qb - 4.0 * qa * qc;
-  if (disc < 0.0) disc = 0.0;
-  double sd = std::sqrt(disc);
-  double v1 = (-qb + sd) / (2.0 * qa);
-  double v2 = (-qb - sd) / (2.0 * qa);
+  const long double Au = ucon[d], Bu = ucon[0];
+  const long double AA = G.gcon[d][d], BB = G.gcon[0][0], AB = G.gcon[0][d];
+  const long double qa = Bu * Bu - c2 * (BB + Bu * Bu);
+  const long double qb = -2.0L * (Au * Bu - c2 * (AB + Au * Bu));
+  const long double qc = Au * Au - c2 * (AA + Au * Au);
+  long double disc = qb * qb - 4.0L * qa * qc;
+  if (disc < 0.0L) disc = 0.0L;
+  const long double sd = std::sqrt(disc);
+  const double v1 = (double)((-qb + sd) / (2.0L * qa));
+  const double v2 = (double)((-qb - sd) / (2.0L * qa));
   *vmax = std::max(v1, v2);
   *vmin = std::min(v1, v2);
 }

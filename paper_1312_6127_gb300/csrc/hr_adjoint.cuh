@@ -159,12 +159,13 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
     const double Sz = ent ? a.Sst[(long long)s * bx.nact + z] : 0.0;
     const Geo<MET, D4> g4 = geo_cast<D4>(g);
     {  // floors: gq <- (d floors / d P)^T gq at the solution
-      const double rr = log_r<MET>(p, x1);
+      double fl[2];
+      floor_values<MET>(p, x1, &fl[0], &fl[1]);
       double gs[NPR];
       for (int ch = 0; ch < 3; ++ch) {
         D4 PD[NPR];
         for (int q = 0; q < NPR; ++q) PD[q] = D4::seed(Ps[q], q - 4 * ch);
-        apply_floors<MET, D4>(p, g4, rr, PD);
+        apply_floors<MET, D4>(p, g4, fl[0], fl[1], PD);
         for (int c = 0; c < 4; ++c) {
           double v = 0.0;
           for (int q = 0; q < NPR; ++q) v += gq[q] * PD[q].d[c];

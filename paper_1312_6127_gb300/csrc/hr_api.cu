@@ -158,6 +158,12 @@ int fill_physics(const harmrad_params* p, DevParams& d) {
   d.integrator = p->integrator;
   if (p->emf != 0 && p->emf != 1) return HARMRAD_E_ARG;
   d.emf = p->emf;
+  d.gm1 = d.gam - 1.0;
+  d.igam = 1.0 / d.gam;
+  d.gfac = d.gm1 / d.gam;
+  d.ibsq_rho = 1.0 / d.bsq_rho_max;
+  d.ibsq_u = 1.0 / d.bsq_u_max;
+  d.iu_rho = 1.0 / d.u_rho_max;
   d.gm1f = (float)(d.gam - 1.0);
   d.ymaxf = (float)d.ymax_rad;
   d.Tminf = (float)d.Tmin;

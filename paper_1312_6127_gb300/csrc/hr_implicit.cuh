@@ -26,10 +26,28 @@
 
 namespace hr {
 
+// Factors of a zone that every FP64 evaluation of the error function reads
+// (pmhd_res64): the ZAMO's metric factors, the covariant field B_mu = (m0, m),
+// B^2, and the constant parts of the error norms.
+template <typename T>
+struct ImpPre {};
+template <>
+struct ImpPre<double> {
+  double a2, b1, c11;      // alpha^2, beta^1 = alpha^2 g^{t1}, gamma^{11} = g^{11} + alpha^2 (g^{t1})^2
+  double m0, m[3], BB;     // B_t, B_i, B^i B_i
+  double sT, sR;           // sum_k sqrt(gamma^{kk}) |T*^t_k|, the same of R*^t_k
+};
+
 // The implicit system of one zone.  T is double in the step; the adjoint
-// evaluates the same functions on dual numbers.
-template <int MET, typename T = double>
+// evaluates the same functions on dual numbers.  FAST: FP64 with pmhd_res64
+// and hr_math.cuh; otherwise the term-by-term functions with the language's
+// divisions (dual numbers, and split precision, whose FP32 stages round the
+// primitives so that a last-bit change here moves a rounding there: its
+// results are kept to the bit).
+template <int MET, typename T = double, bool FAST = std::is_same<T, double>::value>
 struct ImpSysT {
+  static constexpr bool fast = FAST;
+  ImpPre<T> pre;
   Geo<MET, T> g;
   T Dlab;   // rho0 u^t
   T iDlab;  // 1 / (rho0 u^t)
@@ -44,8 +62,8 @@ struct ImpSysT {
   T Sstar;       // explicit S u^t (the conserved entropy over sqrt(-g))
   bool cold;     // cold MHD (Sec. 4.11): u_g held, the momentum rows only
 };
-template <int MET>
-using ImpSys = ImpSysT<MET, double>;
+template <int MET, bool FAST = true>
+using ImpSys = ImpSysT<MET, double, FAST>;
 
 template <typename T = double>
 struct ImpResT {
@@ -89,8 +107,8 @@ __device__ __forceinline__ void four_force_rad(const DevParams& p, T rho, T Tg, 
   for (int n = 0; n < 4; ++n) G[n] = A * urv[n] + C * ucov[n];
 }
 
-template <int MET, typename T = double>
-__device__ __forceinline__ void normalise(const ImpSysT<MET, T>& s, const T Tc[4], const T Rc[4],
+template <int MET, typename T = double, bool FAST>
+__device__ __forceinline__ void normalise(const ImpSysT<MET, T, FAST>& s, const T Tc[4], const T Rc[4],
                                           const T G[4], bool iter_gas, ImpResT<T>& r, T eS = T(-1.0),
                                           T eSr = T(-1.0)) {
   T dg0 = fabs(Tc[0]) + fabs(s.Ts[0]) + s.h * fabs(G[0]);
@@ -152,10 +170,173 @@ struct nondeduced {
   using type = X;
 };
 
-template <int MET, typename T = double>
-__device__ __forceinline__ void pmhd_res(const DevParams& p, const ImpSysT<MET, T>& s, const T x[4],
+// The error function in FP64, arranged for few FP64 instructions (pmhd_res
+// below states the same term by term).  With l_i = g_ij u~^j = u_i and
+// q_i = alpha R_i the gas and radiation frames follow from covariant
+// components: u_t = beta^1 l_1 - alpha gamma, T^t_mu = Z u_mu - (b^t / u^t) B_mu
+// + p_tot delta with Z = (w + b^2) u^t - (b^t)^2 / u^t; E_rad = beta^1 R_1 - R_0,
+// U~^2 = alpha^2 gamma^{ij} R_i R_j; with s = sqrt(4 - 3y) and
+// rr = 1/sqrt((s + 2)(s - 1)) the radiation frame has u_r_i = 1.5 rr q_i / E_rad
+// and gamma_r = (s + 2) rr / 2; u_r.u = u_r_i u~^i - gamma_r gamma.  Signs are
+// read from the bit patterns.  About 215 FP64 instructions with the error
+// norms, 335 before.
+__device__ __forceinline__ bool positive64(double x) { return __double_as_longlong(x) > 0; }  // not for NaN
+__device__ __forceinline__ bool finite64(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+
+template <int MET>
+__device__ __forceinline__ void pmhd_res64(const DevParams& p, const ImpSys<MET>& s, const double x[4], ImpRes& r,
+                                           ImpState* st, bool norm) {
+  const auto& g = s.g;
+  const auto& c = s.pre;
+  double l[3], igm;
+  lower3<MET>(g, x[1], x[2], x[3], l);
+  const double gm = sqrt_rsqrt(fma(x[1], l[0], fma(x[2], l[1], fma(x[3], l[2], 1.0))), &igm);
+  const double u0 = MET == MINK ? gm : gm * g.ialpha, iut = MET == MINK ? igm : g.alpha * igm;
+  const double l0 = MET == MINK ? -gm : fma(c.b1, l[0], -g.alpha * gm);
+  const double rho = s.Dlab * iut;
+  const double bt = fma(s.B[0], l[0], fma(s.B[1], l[1], s.B[2] * l[2])), bu = bt * iut;
+  const double bsq = fma(bt, bt, c.BB) * (iut * iut);
+  const double pg = p.gm1 * x[0], pt = fma(0.5, bsq, pg);
+  const double Z = fma(-bt, bu, (rho + fma(p.gam, x[0], bsq)) * u0);
+  double Tc[4], dT[4], Rt[4];
+  Tc[0] = fma(rho, u0, fma(Z, l0, MET == MINK ? pt : fma(-bu, c.m0, pt)));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) Tc[1 + k] = fma(Z, l[k], -bu * c.m[k]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    dT[k] = Tc[k] - s.Ts[k];
+    Rt[k] = s.Rs[k] - dT[k];
+  }
+  // M1 inversion with the TYPE2 limiter (rad_invert)
+  double E = MET == MINK ? -Rt[0] : fma(c.b1, Rt[1], -Rt[0]), t[3];
+  if constexpr (MET == MINK) {
+    t[0] = Rt[1];
+    t[1] = Rt[2];
+    t[2] = Rt[3];
+  } else {
+    t[0] = fma(g.G13, Rt[3], c.c11 * Rt[1]);
+    t[1] = g.G22 * Rt[2];
+    t[2] = fma(g.G33, Rt[3], g.G13 * Rt[1]);
+  }
+  double U2 = fma(Rt[1], t[0], fma(Rt[2], t[1], Rt[3] * t[2]));
+  if constexpr (MET != MINK) U2 *= c.a2;
+  r.negE = !positive64(E);
+  double ie = 0.0, y = HUGE_VAL;
+  if (!r.negE) {
+    ie = rcp(E);
+    y = positive64(U2) ? (U2 * ie) * ie : 0.0;
+  }
+  if (y > p.ymax_rad) {
+    E = 1e-150 + sqrt(U2 / p.ymax_rad);
+    ie = 1.0 / E;
+    y = (U2 * ie) * ie;
+  }
+  const double sq = sqrt64(fma(-3.0, y, 4.0)), sm1 = sq - 1.0, sp2 = sq + 2.0;
+  const double rr = rsqrt64(sp2 * sm1);
+  E *= sm1;
+  const double fa = MET == MINK ? (1.5 * ie) * rr : (1.5 * ie) * rr * g.alpha;
+  const double gr = 0.5 * sp2 * rr;
+  double v0, v[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = fa * Rt[1 + k];
+  v0 = MET == MINK ? -gr : fma(c.b1, v[0], -g.alpha * gr);
+  // four-force (four_force_rad), times h
+  const double Tg = pg * u0 * s.iDlab;  // p_g / rho0
+  double kabs;
+  if (p.opacity == 2) {
+    kabs = s.ks * s.kf;
+  } else if (p.opacity == 1) {
+    const double Tl = Tg > p.Tmin ? Tg : p.Tmin, T2 = Tl * Tl;
+    kabs = s.ks * p.kabs0 * rho * rho * rsqrt64(T2 * T2 * T2 * Tl);
+  } else {
+    kabs = s.ks * p.kabs0 * rho;
+  }
+  const double ksca = s.ks * p.kes0 * rho, kt = kabs + ksca;
+  const double uru = fma(v[0], x[1], fma(v[1], x[2], fma(v[2], x[3], -gr * gm)));
+  const double e43 = (4.0 / 3.0) * E, c2 = E * (1.0 / 3.0), c1 = e43 * uru;
+  const double T2 = Tg * Tg, lam = kabs * p.a_rad * T2 * T2;
+  const double hA = -s.h * (kt * c1), hC = -s.h * (fma(kt, c2, lam) + ksca * fma(c1, uru, -c2));
+  double hG[4];
+  hG[0] = fma(hA, v0, hC * l0);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) hG[1 + k] = fma(hA, v[k], hC * l[k]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) r.Eg[k] = dT[k] - hG[k];
+  double eS = -1.0;
+  if (s.entropy) {  // the entropy row (pmhd_res); h G_mu u^mu = hA u_r.u - hC
+    const double hGu = fma(hA, uru, -hC);
+    const double Su = s.Dlab * entropy_per_baryon<double>(p, rho, x[0]);
+    r.Eg[0] = fma(Tg, Su - s.Sstar, hGu);
+    if (norm) {
+      const double d0 = Tg * (fabs(Su) + fabs(s.Sstar)) + fabs(hGu) + (fabs(Tc[0]) + fabs(s.Ts[0]) + fabs(hG[0]));
+      eS = d0 > 0.0 ? fabs(r.Eg[0]) / d0 : 0.0;
+    }
+  }
+  r.ok = true;
+  if (norm) {  // normalise
+    const double ku = MET == MINK ? e43 * gr : e43 * (gr * g.ialpha);
+    double Rc[4];
+    Rc[0] = fma(ku, v0, c2);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) Rc[1 + k] = ku * v[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r.Er[k] = (Rc[k] - s.Rs[k]) + hG[k];
+    const double dg0 = (fabs(Tc[0]) + fabs(s.Ts[0])) + fabs(hG[0]);
+    const double dr0 = (fabs(Rc[0]) + fabs(s.Rs[0])) + fabs(hG[0]);
+    double dgs = dg0 + c.sT, drs = dr0 + c.sR;
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+      dgs = fma(s.sgk[k - 1], fabs(Tc[k]) + fabs(hG[k]), dgs);
+      drs = fma(s.sgk[k - 1], fabs(Rc[k]) + fabs(hG[k]), drs);
+    }
+    double eg0 = positive64(dg0) ? fabs(r.Eg[0]) * rcp(dg0) : 0.0;
+    double er0 = positive64(dr0) ? fabs(r.Er[0]) * rcp(dr0) : 0.0;
+    const double ig = positive64(dgs) ? rcp(dgs) : 0.0, ir = positive64(drs) ? rcp(drs) : 0.0;
+    if (r.negE) eg0 = er0 = 0.0;
+    if (eS >= 0.0) {  // entropy row in place of the gas energy row
+      eg0 = r.negE ? 0.0 : eS;
+      er0 = 0.0;
+    }
+    r.eg0 = eg0;
+    r.er0 = er0;
+    double sT = 0.0, sI = 0.0;
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+      const double eg = fabs(r.Eg[k]) * ig;
+      sT = fma(s.sgk[k - 1], fmax(eg, fabs(r.Er[k]) * ir), sT);
+      sI = fma(s.sgk[k - 1], eg, sI);
+    }
+    if (s.cold) {  // the mean of the momentum rows
+      r.eT = sT / 3.0;
+      r.eI = sI / 3.0;
+    } else {
+      r.eT = 0.25 * (fmax(eg0, er0) + sT);
+      r.eI = 0.25 * (eg0 + sI);
+    }
+    r.ok = finite64(r.eT);
+  }
+  if (st) {
+    st->negE = r.negE;
+    st->rho = rho;
+    st->ug = x[0];
+    st->Pr[0] = E;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) st->Pr[1 + k] = fa * t[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) st->Rt_pre[k] = Rt[k];
+  }
+}
+
+template <int MET, typename T = double, bool FAST>
+__device__ __forceinline__ void pmhd_res(const DevParams& p, const ImpSysT<MET, T, FAST>& s, const T x[4],
                                          ImpResT<T>& r, typename nondeduced<ImpStateT<T>>::type* st,
                                          bool norm) {
+  if constexpr (FAST) {
+    pmhd_res64<MET>(p, s, x, r, st, norm);
+    return;
+  }
   const auto& g = s.g;
   T ucon[4], ucov[4], gm, bcon[4], bcov[4], bsq;
   fourvel<MET, T>(g, x[1], x[2], x[3], ucon, ucov, &gm);
@@ -205,7 +386,7 @@ __device__ __forceinline__ void pmhd_res(const DevParams& p, const ImpSysT<MET, 
     for (int k = 1; k < 4; ++k) Rc[k] = e43 * urc[0] * urv[k];
 #pragma unroll
     for (int k = 0; k < 4; ++k) r.Er[k] = Rc[k] - s.Rs[k] + s.h * G[k];
-    normalise<MET, T>(s, Tc, Rc, G, true, r, eS);
+    normalise<MET, T, FAST>(s, Tc, Rc, G, true, r, eS);
     r.ok = isfinite(r.eT);
   } else {
     r.ok = true;
@@ -222,6 +403,7 @@ __device__ __forceinline__ void pmhd_res(const DevParams& p, const ImpSysT<MET, 
   }
 }
 
+template <bool FAST = true>
 __device__ __forceinline__ bool solve4(double A[4][4], double b[4], double z[4]) {
   double ipv[4];  // reciprocals of the pivots, reused by the back-substitution
 #pragma unroll
@@ -234,7 +416,7 @@ __device__ __forceinline__ bool solve4(double A[4][4], double b[4], double z[4])
         best = fabs(A[r][c]);
         piv = r;
       }
-    if (best == 0.0 || !isfinite(best)) return false;
+    if (best == 0.0 || !finite64(best)) return false;
     if (piv != c) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -246,7 +428,7 @@ __device__ __forceinline__ bool solve4(double A[4][4], double b[4], double z[4])
       b[c] = b[piv];
       b[piv] = t;
     }
-    const double ip = 1.0 / A[c][c];
+    const double ip = FAST ? rcp(A[c][c]) : 1.0 / A[c][c];
     ipv[c] = ip;
 #pragma unroll
     for (int r = c + 1; r < 4; ++r) {
@@ -265,7 +447,7 @@ __device__ __forceinline__ bool solve4(double A[4][4], double b[4], double z[4])
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i)
-    if (!isfinite(z[i])) return false;
+    if (!finite64(z[i])) return false;
   return true;
 }
 
@@ -330,8 +512,8 @@ __device__ __forceinline__ void newton_pmhd_init(const double x0[4], NewtonState
 // Finite-difference PMHD Jacobian (one-sided, the paper's numerical
 // Jacobian): column j from the error at x + dj e_j, dj = eps |u_g| for j = 0
 // and eps max(1, |u~|)/sqrt(g_jj) for the velocities.
-template <int MET>
-__device__ __forceinline__ void pmhd_jacobian_fd(const DevParams& p, const ImpSys<MET>& s, const double x[4],
+template <int MET, bool FAST>
+__device__ __forceinline__ void pmhd_jacobian_fd(const DevParams& p, const ImpSys<MET, FAST>& s, const double x[4],
                                                  const ImpRes& r, double eps, double J[4][4]) {
   double umag = fmax(1.0, sqrt(s.g.sq3(x[1], x[2], x[3])));
 #pragma unroll 1
@@ -355,14 +537,14 @@ __device__ __forceinline__ void pmhd_jacobian_fd(const DevParams& p, const ImpSy
 // Newton step dx = J^-1 E at x: the FP32 tangent Jacobian while *jac32, else
 // (or when it is not finite or singular, which clears *jac32) the
 // finite-difference one.  Returns false if no Jacobian could be solved.
-template <int MET>
-__device__ __forceinline__ bool pmhd_newton_dx(const DevParams& p, const ImpSys<MET>& s, const double x[4],
+template <int MET, bool FAST>
+__device__ __forceinline__ bool pmhd_newton_dx(const DevParams& p, const ImpSys<MET, FAST>& s, const double x[4],
                                                const ImpRes& r, const double Rt[4], double eps, int* jac32,
                                                double dx[4], TanStage& ts) {
   if (*jac32) {
     double J[4][4];
     double E[4] = {r.Eg[0], r.Eg[1], r.Eg[2], r.Eg[3]};
-    if (pmhd_jacobian_fp32<MET>(p, s, ts, x, Rt, J) && solve4(J, E, dx)) return true;
+    if (pmhd_jacobian_fp32<MET>(p, s, ts, x, Rt, J) && solve4<FAST>(J, E, dx)) return true;
     *jac32 = 0;
   }
   double J[4][4];
@@ -376,7 +558,7 @@ __device__ __forceinline__ bool pmhd_newton_dx(const DevParams& p, const ImpSys<
     }
     E[0] = 0.0;
   }
-  return solve4(J, E, dx);
+  return solve4<FAST>(J, E, dx);
 }
 
 // PMHD Newton iterations from the state st until a stopping rule ends the
@@ -384,8 +566,8 @@ __device__ __forceinline__ bool pmhd_newton_dx(const DevParams& p, const ImpSys<
 // (returns false; st holds what the remaining iterations need).  best_x /
 // best_eT hold the lowest-error iterate (best_eT = inf if no residual was
 // finite).
-template <int MET>
-__device__ __forceinline__ bool newton_pmhd_run(const DevParams& p, const ImpSys<MET>& s, NewtonState& st, int kstop) {
+template <int MET, bool FAST>
+__device__ __forceinline__ bool newton_pmhd_run(const DevParams& p, const ImpSys<MET, FAST>& s, NewtonState& st, int kstop) {
   TanStage ts;
   for (;; ++st.k) {
     if (st.k >= kstop) return false;
@@ -436,8 +618,8 @@ __device__ __forceinline__ bool newton_pmhd_run(const DevParams& p, const ImpSys
 // without a pause, in local variables).  Returns the number of Newton steps;
 // best_x / best_eT hold the lowest-error iterate (best_eT = inf if no
 // residual was finite).
-template <int MET>
-__device__ int newton_pmhd(const DevParams& p, const ImpSys<MET>& s, const double x0[4],
+template <int MET, bool FAST>
+__device__ int newton_pmhd(const DevParams& p, const ImpSys<MET, FAST>& s, const double x0[4],
                            double best_x[4], double* best_eT, ImpState* best_st = nullptr) {
   double x[4] = {x0[0], x0[1], x0[2], x0[3]};
   Hist hs = {HUGE_VAL, HUGE_VAL, HUGE_VAL, HUGE_VAL, HUGE_VAL, HUGE_VAL, HUGE_VAL, HUGE_VAL, 0};
@@ -1016,32 +1198,59 @@ __device__ __forceinline__ int newton_urad(const DevParams& p, const ImpSys<MET>
   return newton_rad<MET, false>(p, s, x0, Pg, best_x, best_Pg, best_eT);
 }
 
-template <int MET, typename T = double>
-__device__ __forceinline__ void build_sys(const DevParams& p, const Geo<MET, T>& g, const T Us[12], double h,
-                                          T kf, ImpSysT<MET, T>& s) {
+// The zone's implicit system from U*: igd = 1/sqrt(-g), sgk = sqrt(gamma^{kk}).
+template <int MET, typename T, bool FAST>
+__device__ __forceinline__ void build_sys_with(const DevParams& p, const Geo<MET, T>& g, T igd, const T sgk[3],
+                                               const T Us[12], double h, T kf, ImpSysT<MET, T, FAST>& s) {
   s.g = g;
   s.kf = kf;
   s.ks = T(p.kscale);
-  T igd = 1.0 / g.gdet;
   s.Dlab = Us[0] * igd;
-  s.iDlab = 1.0 / s.Dlab;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     s.Ts[k] = Us[1 + k] * igd;
     s.Rs[k] = Us[8 + k] * igd;
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) s.B[i] = Us[5 + i] * igd;
+  for (int i = 0; i < 3; ++i) {
+    s.B[i] = Us[5 + i] * igd;
+    s.sgk[i] = sgk[i];
+  }
   s.h = T(h);
-  // orthonormal (ZAMO) size of covariant spatial components:
-  // sqrt(gamma^{kk}), gamma^{kk} = g^{kk} - (g^{tk})^2 / g^{tt} > 0 everywhere
-  // on the slice, inside the horizon too
-#pragma unroll
-  for (int k = 1; k < 4; ++k) s.sgk[k - 1] = sqrt(g.Gdd(k) - g.Gt(k) * g.Gt(k) / g.Gtt());
   s.entropy = false;
   s.cold = false;
   s.Sstar = T(0.0);
-  (void)p;
+  if constexpr (FAST) {
+    s.iDlab = rcp(s.Dlab);
+    ImpPre<double>& c = s.pre;
+    lower3<MET>(g, s.B[0], s.B[1], s.B[2], c.m);
+    c.BB = fma(s.B[0], c.m[0], fma(s.B[1], c.m[1], s.B[2] * c.m[2]));
+    c.sT = fma(sgk[0], fabs(s.Ts[1]), fma(sgk[1], fabs(s.Ts[2]), sgk[2] * fabs(s.Ts[3])));
+    c.sR = fma(sgk[0], fabs(s.Rs[1]), fma(sgk[1], fabs(s.Rs[2]), sgk[2] * fabs(s.Rs[3])));
+    if constexpr (MET == MINK) {
+      c.a2 = c.c11 = 1.0;
+      c.b1 = c.m0 = 0.0;
+    } else {
+      c.a2 = g.alpha * g.alpha;
+      c.b1 = c.a2 * g.G01;
+      c.c11 = fma(c.b1, g.G01, g.G11);
+      c.m0 = c.b1 * c.m[0];
+    }
+  } else {
+    s.iDlab = 1.0 / s.Dlab;
+  }
+}
+
+template <int MET, typename T = double>
+__device__ __forceinline__ void build_sys(const DevParams& p, const Geo<MET, T>& g, const T Us[12], double h,
+                                          T kf, ImpSysT<MET, T>& s) {
+  // orthonormal (ZAMO) size of covariant spatial components:
+  // sqrt(gamma^{kk}), gamma^{kk} = g^{kk} - (g^{tk})^2 / g^{tt} > 0 everywhere
+  // on the slice, inside the horizon too
+  T sgk[3];
+#pragma unroll
+  for (int k = 1; k < 4; ++k) sgk[k - 1] = sqrt(g.Gdd(k) - g.Gt(k) * g.Gt(k) / g.Gtt());
+  build_sys_with<MET, T>(p, g, 1.0 / g.gdet, sgk, Us, h, kf, s);
 }
 
 }  // namespace hr

@@ -85,10 +85,15 @@ __device__ __forceinline__ double kfield(const DevParams& p, const double* K, lo
 // centres, [16][N2][N1] centre derivatives, [GEO_F][N2][n1+1] x1 faces,
 // [GEO_F][n2+1][N1] x2 faces; fields in the order of Geo (g00 g01 g03 g11 g13
 // g22 g33 G00 G01 G11 G13 G22 G33 gdet alpha ialpha) and of MetricDeriv.
-// Centres add 1/sqrt(-g) (plane 16) and sqrt(g_dd) of the three directions
-// (17..19), faces 1/sqrt(-g) (16) and sqrt(g_dd) of their direction (17):
-// each saves a division or a square root per zone or face.
-constexpr int GEO_C = 20, GEO_F = 18;
+// Centres add 1/sqrt(-g) (plane 16), sqrt(g_dd) of the three directions
+// (17..19), sqrt(gamma^{kk}) of the ZAMO slice (20..22), the density and
+// internal-energy floors (23, 24) and the longest active proper edge of the
+// cell (25); faces add 1/sqrt(-g) (16) and sqrt(g_dd) of their direction (17).
+// Each saves divisions, square roots or exponentials per zone or face.  The
+// derivatives are stored as the geometric source contracts them (split
+// precision: plain): 1/2 sqrt(-g) d_nu g_{mu kappa}, off-diagonals doubled, and
+// d_nu sqrt(-g).
+constexpr int GEO_C = 26, GEO_F = 18;
 struct GeoTab {
   const double* C;
   const double* M;
@@ -993,56 +998,68 @@ __global__ void k_ct(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, co
 // ----------------------------------------------------------------- floors
 // Lorentz-factor caps, density and internal-energy floors f0 r^pow,
 // magnetisation caps b^2/rho, b^2/u_g, u_g/rho, and Ebar > 0.
-// ln r of the cell centre at x1 (0 on the Minkowski grid, where the floors
-// take r = 1): x1 itself when r = e^x1 (R0 = 0).
+
+// The floors f0 r^pow at x1 as f0 exp(pow ln r), with ln r = x1 itself when
+// r = e^x1 (R0 = 0); on the Minkowski grid r = 1.
 template <int MET>
-__device__ __forceinline__ double log_r(const DevParams& p, double x1) {
-  if constexpr (MET == KS) return p.R0 == 0.0 ? x1 : log(p.R0 + exp(x1));
-  else return 0.0;
+__device__ __forceinline__ void floor_values(const DevParams& p, double x1, double* rfl, double* ufl) {
+  double lr = 0.0;
+  if constexpr (MET == KS) lr = p.R0 == 0.0 ? x1 : log(p.R0 + exp(x1));
+  *rfl = p.rf0 * (p.rfp == 0.0 ? 1.0 : exp(p.rfp * lr));
+  *ufl = p.uf0 * (p.ufp == 0.0 ? 1.0 : exp(p.ufp * lr));
+}
+
+// b^2 of u~^i and B^i by b^2 = (B^i B_i + (B^i u_i)^2) / (u^t)^2, and
+// gamma^2 of u~^i; both in FP64 or on dual numbers.
+template <int MET, typename T>
+__device__ __forceinline__ T floor_bsq(const Geo<MET, T>& g, const T P[NPR], T* g2) {
+  if constexpr (std::is_same<T, double>::value) {
+    double l[3], m[3];
+    lower3<MET>(g, P[U1], P[U2], P[U3], l);
+    lower3<MET>(g, P[B1], P[B2], P[B3], m);
+    *g2 = fma(P[U1], l[0], fma(P[U2], l[1], fma(P[U3], l[2], 1.0)));
+    const double bt = fma(P[B1], l[0], fma(P[B2], l[1], P[B3] * l[2]));
+    const double BB = fma(P[B1], m[0], fma(P[B2], m[1], P[B3] * m[2]));
+    return fma(bt, bt, BB) * (MET == MINK ? rcp(*g2) : (g.alpha * g.alpha) * rcp(*g2));
+  } else {
+    T ucon[4], ucov[4], bcon[4], bcov[4], bsq, gm;
+    fourvel<MET, T>(g, P[U1], P[U2], P[U3], ucon, ucov, &gm);
+    bvec<MET, T>(g, ucon, ucov, P[B1], P[B2], P[B3], bcon, bcov, &bsq);
+    *g2 = gm * gm;
+    return bsq;
+  }
 }
 
 template <int MET, typename T = double>
-__device__ __forceinline__ void apply_floors(const DevParams& p, const Geo<MET, T>& g, double lr, T P[NPR],
-                                             unsigned* code = nullptr) {
-  T gm = sqrt(1.0 + g.sq3(P[U1], P[U2], P[U3]));
-  if (code) {  // which floors act (the branch signature)
-    *code = 0;
-    const T gr0 = sqrt(1.0 + g.sq3(P[UR1], P[UR2], P[UR3]));
-    if (gm > p.ggas_max) *code |= 1u;
-    if (gr0 > p.grad_max) *code |= 2u;
-  }
-  if (gm > p.ggas_max) {
-    T f = sqrt((p.ggas_max * p.ggas_max - 1.0) / (gm * gm - 1.0));
+__device__ __forceinline__ void apply_floors(const DevParams& p, const Geo<MET, T>& g, double rf0, double uf0,
+                                             T P[NPR], unsigned* code = nullptr) {
+  T g2, bsq = floor_bsq<MET, T>(g, P, &g2);
+  const T r2 = 1.0 + g.sq3(P[UR1], P[UR2], P[UR3]);
+  const double gc = p.ggas_max * p.ggas_max, rc = p.grad_max * p.grad_max;
+  if (code) *code = (g2 > gc ? 1u : 0u) | (r2 > rc ? 2u : 0u);  // which floors act (the branch signature)
+  if (g2 > gc) {
+    T f = sqrt((gc - 1.0) / (g2 - 1.0));
     P[U1] *= f;
     P[U2] *= f;
     P[U3] *= f;
+    bsq = floor_bsq<MET, T>(g, P, &g2);
   }
-  T gr = sqrt(1.0 + g.sq3(P[UR1], P[UR2], P[UR3]));
-  if (gr > p.grad_max) {
-    T f = sqrt((p.grad_max * p.grad_max - 1.0) / (gr * gr - 1.0));
+  if (r2 > rc) {
+    T f = sqrt((rc - 1.0) / (r2 - 1.0));
     P[UR1] *= f;
     P[UR2] *= f;
     P[UR3] *= f;
   }
-  T ucon[4], ucov[4], bcon[4], bcov[4], bsq;
-  fourvel<MET, T>(g, P[U1], P[U2], P[U3], ucon, ucov, &gm);
-  bvec<MET, T>(g, ucon, ucov, P[B1], P[B2], P[B3], bcon, bcov, &bsq);
-  // f0 r^pow as exp(pow ln r): the floor needs ln r only (x1 itself on the
-  // Kerr-Schild grid with R0 = 0, where r = e^x1)
-  T rfl = T(p.rf0 * (p.rfp == 0.0 ? 1.0 : exp(p.rfp * lr)));
-  T ufl = T(p.uf0 * (p.ufp == 0.0 ? 1.0 : exp(p.ufp * lr)));
+  const T rb = bsq * p.ibsq_rho, ub = bsq * p.ibsq_u;
+  const T rfl = fmax(T(rf0), rb), ufl = fmax(T(uf0), ub);
   if (code) {
-    const T rb = bsq / p.bsq_rho_max, ub = bsq / p.bsq_u_max;
-    const T rf = fmax(rfl, rb), uf = fmax(ufl, ub);
-    const T u1 = fmax(P[UU], uf);
-    *code |= (rb > rfl ? 4u : 0u) | (ub > ufl ? 8u : 0u) | (rf > P[RHO] ? 16u : 0u) | (uf > P[UU] ? 32u : 0u) |
-             (u1 / p.u_rho_max > fmax(P[RHO], rf) ? 64u : 0u) | (!(P[ER] > 0.0) ? 128u : 0u);
+    const T u1 = fmax(P[UU], ufl);
+    *code |= (rb > rf0 ? 4u : 0u) | (ub > uf0 ? 8u : 0u) | (rfl > P[RHO] ? 16u : 0u) | (ufl > P[UU] ? 32u : 0u) |
+             (u1 * p.iu_rho > fmax(P[RHO], rfl) ? 64u : 0u) | (!(P[ER] > 0.0) ? 128u : 0u);
   }
-  rfl = fmax(rfl, bsq / p.bsq_rho_max);
-  ufl = fmax(ufl, bsq / p.bsq_u_max);
   P[RHO] = fmax(P[RHO], rfl);
   P[UU] = fmax(P[UU], ufl);
-  P[RHO] = fmax(P[RHO], P[UU] / p.u_rho_max);
+  P[RHO] = fmax(P[RHO], P[UU] * p.iu_rho);
   if (!(P[ER] > 0.0)) P[ER] = T(1e-150);
 }
 
@@ -1051,8 +1068,8 @@ __device__ __forceinline__ void apply_floors(const DevParams& p, const Geo<MET, 
 // Final primitives from the error function's state at x (pmhd_res), without
 // evaluating it again: gas from x, B fixed, radiation re-inverted with BASIC
 // if the TYPE2 branch saw a negative energy (Sec. 4.10).
-template <int MET>
-__device__ __forceinline__ void pmhd_final_state(const DevParams& p, const ImpSys<MET>& s, const double x[4],
+template <int MET, bool FAST>
+__device__ __forceinline__ void pmhd_final_state(const DevParams& p, const ImpSys<MET, FAST>& s, const double x[4],
                                                  const ImpState& st, double P[NPR]) {
   P[RHO] = st.rho;
   P[UU] = x[0];
@@ -1070,8 +1087,8 @@ __device__ __forceinline__ void pmhd_final_state(const DevParams& p, const ImpSy
   P[UR3] = Pr[3];
 }
 
-template <int MET, typename T = double>
-__device__ __forceinline__ void pmhd_final(const DevParams& p, const ImpSysT<MET, T>& s, const T x[4], T P[NPR],
+template <int MET, typename T = double, bool FAST>
+__device__ __forceinline__ void pmhd_final(const DevParams& p, const ImpSysT<MET, T, FAST>& s, const T x[4], T P[NPR],
                                            T* Eg = nullptr, unsigned* code = nullptr) {
   ImpResT<T> r;
   ImpStateT<T> stt;
@@ -1375,9 +1392,20 @@ static __global__ void k_geo_init(DevParams p, const BoxGeo* __restrict__ boxes,
         C[17 * T.sC + id] = sqrt(g.g11);
         C[18 * T.sC + id] = sqrt(g.g22);
         C[19 * T.sC + id] = sqrt(g.g33);
+        double dl = 0.0;
+        for (int k = 1; k < 4; ++k) {
+          C[(19 + k) * T.sC + id] = sqrt(g.Gdd(k) - g.Gt(k) * g.Gt(k) / g.Gtt());
+          if (p.act[k - 1]) dl = fmax(dl, sqrt(g.gdd(k)) * bx.dx[k - 1]);
+        }
+        floor_values<KS>(p, x1, &C[23 * T.sC + id], &C[24 * T.sC + id]);
+        C[25 * T.sC + id] = dl;
         const MetricDeriv md = ks_derivs(p, x1, x2);
         const double* v = reinterpret_cast<const double*>(&md);
-        for (int f = 0; f < 16; ++f) M[f * T.sC + id] = v[f];
+        for (int f = 0; f < 16; ++f) {
+          const int c = f / 2;  // g00 g01 g03 g11 g13 g22 g33 sg, two derivatives each
+          const double w = c == 7 || p.precision ? 1.0 : (c == 1 || c == 2 || c == 4 ? g.gdet : 0.5 * g.gdet);
+          M[f * T.sC + id] = w * v[f];
+        }
       } else if (id < T.sC + T.sF0) {  // x1 faces
         const long long e = id - T.sC;
         const int i = (int)(e % (bx.n[0] + 1)), j = (int)(e / (bx.n[0] + 1)) - bx.ng[1];
@@ -1440,6 +1468,70 @@ __device__ __forceinline__ void cons_source(const DevParams& p, const Geo<MET, T
   (void)x2;
 }
 
+// The same in FP64 with the metric derivatives of the table (md: 1/2 sqrt(-g)
+// d_nu g_{mu kappa}, off-diagonals doubled): the source contracts T^{mu kappa}
+// once per nu, and the rows of U take the two-scalar form of pmhd_res64.
+template <int MET>
+__device__ __forceinline__ void cons_source64(const DevParams& p, const Geo<MET, double>& g, const double Ps[NPR],
+                                              double Us[NPR], double X[NPR], const MetricDeriv& md) {
+  double l[3], m[3], k[3], igm;
+  lower3<MET>(g, Ps[U1], Ps[U2], Ps[U3], l);
+  lower3<MET>(g, Ps[B1], Ps[B2], Ps[B3], m);
+  lower3<MET>(g, Ps[UR1], Ps[UR2], Ps[UR3], k);
+  const double gm = sqrt_rsqrt(fma(Ps[U1], l[0], fma(Ps[U2], l[1], fma(Ps[U3], l[2], 1.0))), &igm);
+  const double gr = sqrt64(fma(Ps[UR1], k[0], fma(Ps[UR2], k[1], fma(Ps[UR3], k[2], 1.0))));
+  const double bt = fma(Ps[B1], l[0], fma(Ps[B2], l[1], Ps[B3] * l[2]));
+  const double BB = fma(Ps[B1], m[0], fma(Ps[B2], m[1], Ps[B3] * m[2]));
+  double u0 = gm, l0 = -gm, iut = igm, r0 = gr, k0 = -gr, m0 = 0.0, a01 = 0.0;
+  if constexpr (MET == KS) {
+    a01 = g.alpha * g.G01;
+    const double b1 = g.alpha * a01;
+    u0 = gm * g.ialpha;
+    l0 = fma(b1, l[0], -g.alpha * gm);
+    iut = g.alpha * igm;
+    r0 = gr * g.ialpha;
+    k0 = fma(b1, k[0], -g.alpha * gr);
+    m0 = b1 * m[0];
+  }
+  const double bu = bt * iut, bsq = fma(bt, bt, BB) * (iut * iut);
+  const double pg = p.gm1 * Ps[UU], wb = Ps[RHO] + fma(p.gam, Ps[UU], bsq), pt = fma(0.5, bsq, pg);
+  const double wu = wb * u0, Z = fma(-bt, bu, wu), mt = Ps[RHO] * u0;
+  const double E = Ps[ER], e43 = (4.0 / 3.0) * E, e13 = E * (1.0 / 3.0), er = e43 * r0, gd = g.gdet;
+  Us[0] = gd * mt;
+  Us[1] = gd * fma(Z, l0, fma(-bu, m0, pt + mt));
+#pragma unroll
+  for (int n = 0; n < 3; ++n) {
+    Us[2 + n] = gd * fma(Z, l[n], -bu * m[n]);
+    Us[5 + n] = gd * Ps[B1 + n];
+    Us[9 + n] = gd * (er * k[n]);
+  }
+  Us[8] = gd * fma(er, k0, e13);
+#pragma unroll
+  for (int q = 0; q < NPR; ++q) X[q] = 0.0;
+  if constexpr (MET == KS) {
+    const double u1 = fma(-gm, a01, Ps[U1]), u2 = Ps[U2], u3 = Ps[U3];
+    const double b1 = fma(bt, u1, Ps[B1]) * iut, b2 = fma(bt, u2, Ps[B2]) * iut, b3 = fma(bt, u3, Ps[B3]) * iut;
+    const double w1 = wb * u1;
+    const double T[7] = {fma(wu, u0, -bt * bt), fma(wu, u1, -bt * b1),      fma(wu, u3, -bt * b3),
+                         fma(w1, u1, -b1 * b1), fma(w1, u3, -b1 * b3),      fma(wb * u2, u2, -b2 * b2),
+                         fma(wb * u3, u3, -b3 * b3)};
+    const double r1 = fma(-gr, a01, Ps[UR1]), r2 = Ps[UR2], r3 = Ps[UR3], e1 = e43 * r1;
+    const double R[7] = {er * r0, er * r1, er * r3, e1 * r1, e1 * r3, e43 * r2 * r2, e43 * r3 * r3};
+    const double* d = reinterpret_cast<const double*>(&md);
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+      double xg = pt * md.sg[n], xr = e13 * md.sg[n];
+#pragma unroll
+      for (int c = 0; c < 7; ++c) {
+        xg = fma(T[c], d[2 * c + n], xg);
+        xr = fma(R[c], d[2 * c + n], xr);
+      }
+      X[2 + n] = xg;
+      X[9 + n] = xr;
+    }
+  }
+}
+
 constexpr int CSTRIDE = NPR + 23;  // continuation queue record: U*, Newton state, S*
 
 __device__ __forceinline__ void newton_state_store(const NewtonState& st, double* d) {
@@ -1486,9 +1578,9 @@ __device__ __forceinline__ void newton_state_load(const double* d, NewtonState& 
 
 // End of a zone's PMHD solve: accept (e_T < 1e-9: final primitives, floors,
 // write) or queue the zone for URAD.  Returns whether it was accepted.
-template <int MET>
+template <int MET, bool FAST>
 __device__ __forceinline__ bool pmhd_finish(const DevParams& p, const BoxGeo& bx, int bi, long long z, long long t,
-                                            double x1, const Geo<MET, double>& g, const ImpSys<MET>& s,
+                                            const double fl[2], const Geo<MET, double>& g, const ImpSys<MET, FAST>& s,
                                             const double Ust[NPR], double h, const double best_x[4],
                                             double beT, int steps, double* P, const Bufs& b, double Sst,
                                             double acc_tol = 1e-9, const ImpState* bst = nullptr) {
@@ -1505,7 +1597,7 @@ __device__ __forceinline__ bool pmhd_finish(const DevParams& p, const BoxGeo& bx
     if (b.psol_rec)
       for (int q = 0; q < NPR; ++q) b.psol_rec[12 * bx.aoff + q * bx.nact + z] = Pn[q];
     unsigned fcode = 0;
-    apply_floors<MET>(p, g, log_r<MET>(p, x1), Pn, p.sig ? &fcode : nullptr);
+    apply_floors<MET>(p, g, fl[0], fl[1], Pn, p.sig ? &fcode : nullptr);
     if (p.sig) sig_put(p, bx.coff + t, 60, (fcode << 2 | lcode) << 4 | ST_PMHD);
 #pragma unroll
     for (int q = 0; q < NPR; ++q) P[q * bx.ntot + t] = Pn[q];
@@ -1710,24 +1802,37 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
       int j = (int)(r % bx.n[1]);
       int k = (int)(r / bx.n[1]);
       long long t = cell_index(bx, i, j, k);
-      double x1 = xcen(bx, 0, i), x2 = xcen(bx, 1, j);
-      const bool tab = MET == KS && b.geo && bx.goff >= 0;
+      // the zone's metric, 1/sqrt(-g), sqrt(gamma^{kk}), floors and longest edge
       Geo<MET, double> g;
-      MetricDeriv mdt;
-      if (tab) {
+      MetricDeriv mdt{};
+      double igd, sgk[3], fl[2], dl;
+      if constexpr (MET == KS) {
         const GeoTab T = geotab(b.geo, bx);
         const long long gi = gidx_c(bx, i, j);
         g = geo_load<MET>(T.C, T.sC, gi);
         mdt = md_load(T.M, T.sC, gi);
+        igd = __ldg(T.C + 16 * T.sC + gi);
+        for (int e = 0; e < 3; ++e) sgk[e] = __ldg(T.C + (20 + e) * T.sC + gi);
+        fl[0] = __ldg(T.C + 23 * T.sC + gi);
+        fl[1] = __ldg(T.C + 24 * T.sC + gi);
+        dl = __ldg(T.C + 25 * T.sC + gi);
       } else {
-        g = make_geo<MET, double>(p, x1, x2);
+        g = make_geo<MET, double>(p, 0.0, 0.0);
+        igd = sgk[0] = sgk[1] = sgk[2] = 1.0;
+        fl[0] = p.rf0;
+        fl[1] = p.uf0;
+        dl = 0.0;
+        for (int e = 0; e < 3; ++e)
+          if (p.act[e]) dl = fmax(dl, bx.dx[e]);
       }
       double Ps[NPR];
 #pragma unroll
       for (int q = 0; q < NPR; ++q) Ps[q] = P[q * bx.ntot + t];
       const double kz = kfield(p, K, t);
       double Us[NPR], X[NPR];
-      cons_source<MET, double>(p, g, x1, x2, Ps, Us, X, tab ? &mdt : nullptr);
+      constexpr bool FAST = std::is_same<R, double>::value;
+      if constexpr (FAST) cons_source64<MET>(p, g, Ps, Us, X, mdt);
+      else cons_source<MET, double>(p, g, 0.0, 0.0, Ps, Us, X, &mdt);
       // flux divergence (an IMEX stage without flux term reads no fluxes)
       const bool rhs = !IMEX || im.d != 0.0;
 #pragma unroll
@@ -1736,6 +1841,7 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
         const long long s = bx.str[d];
 #pragma unroll
         for (int q = 0; q < NPR; ++q) {
+          if (q == B1 + d) continue;  // F_d[B_d] = 0
           R df = Fd[d][q * bx.ntot + t + s] - Fd[d][q * bx.ntot + t];
           X[q] -= double(df) * idx[d];
         }
@@ -1810,25 +1916,26 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
       // extremely sub-dominant radiation: no PMHD attempt; the zone goes to
       // the retry queue for URAD with a negative PMHD error as the mark
       const bool subdom = radiation_subdominant<MET>(g, Ust, Ps);
-      ImpSys<MET> s;
-      build_sys<MET>(p, g, Ust, h, kz, s);
-      double x0[4] = {Ps[UU], Ps[U1], Ps[U2], Ps[U3]};
-      {
+      ImpSys<MET, FAST> s;
+      build_sys_with<MET, double>(p, g, igd, sgk, Ust, h, kz, s);
+      double x0[4] = {Ps[UU], Ps[U1], Ps[U2], Ps[U3]}, kt;
+      if constexpr (FAST) {
+        kt = opacity_sum(p, Ps[RHO], [&] { return p.gm1 * Ps[UU] * rcp(Ps[RHO]); }, kz);
+      } else {
         double kabs, ksca;
         opacity<double>(p, Ps[RHO], Ps[UU], kz, &kabs, &ksca);
-        double dl = 0.0;
-#pragma unroll
-        for (int d = 1; d <= 3; ++d)
-          if (p.act[d - 1]) dl = fmax(dl, sqrt(g.gdd(d)) * bx.dx[d - 1]);
-        if ((kabs + ksca) * dl < 2.0 / 3.0) {
-          double go[5];
-          double T3[3] = {s.Ts[1], s.Ts[2], s.Ts[3]};
-          if (gas_invert<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, Ps, 1e-9, go) == 0) {
-            x0[0] = go[1];
-            x0[1] = go[2];
-            x0[2] = go[3];
-            x0[3] = go[4];
-          }
+        kt = kabs + ksca;
+      }
+      if (kt * dl < 2.0 / 3.0) {
+        double go[5];
+        double T3[3] = {s.Ts[1], s.Ts[2], s.Ts[3]};
+        const int rc = FAST ? gas_invert<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, Ps, 1e-9, go)
+                            : gas_invert_ieee<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, Ps, 1e-9, go);
+        if (rc == 0) {
+          x0[0] = go[1];
+          x0[1] = go[2];
+          x0[2] = go[3];
+          x0[3] = go[4];
         }
       }
       bool accept = false;
@@ -1838,19 +1945,19 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
         // e_T >= 1e-9 goes to the retry queue for the entropy URAD and PRAD
         // (the methods' sequence, Sec. 4.10-4.11)
         s.entropy = true;
-        s.Sstar = Sst / g.gdet;
+        s.Sstar = Sst * igd;
         double bxn[4] = {0.0, 0.0, 0.0, 0.0}, beT = HUGE_VAL;
         double xe[4] = {x0[0], x0[1], x0[2], x0[3]};
         entropy_ug_guess(p, Sst, s.Dlab * g.gdet, Ps[RHO], xe);
         const int steps = newton_pmhd<MET>(p, s, xe, bxn, &beT);
-        accept = pmhd_finish<MET>(p, bx, bi, z, t, x1, g, s, Ust, h, bxn, beT, steps, P, b, Sst, 1e-9);
+        accept = pmhd_finish<MET>(p, bx, bi, z, t, fl, g, s, Ust, h, bxn, beT, steps, P, b, Sst, 1e-9);
         done_steps = (unsigned)steps;
         warp_add(&b.stats[ST_ENTROPY], accept ? 1u : 0u);
       } else if constexpr (!CONT) {
         double bxn[4] = {0.0, 0.0, 0.0, 0.0}, beT = -1.0;
         ImpState bst;
         const int steps = subdom ? 0 : newton_pmhd<MET>(p, s, x0, bxn, &beT, &bst);
-        accept = pmhd_finish<MET>(p, bx, bi, z, t, x1, g, s, Ust, h, bxn, beT, steps, P, b, Sst, 1e-9,
+        accept = pmhd_finish<MET>(p, bx, bi, z, t, fl, g, s, Ust, h, bxn, beT, steps, P, b, Sst, 1e-9,
                                   subdom ? nullptr : &bst);
         done_steps = (unsigned)steps;
       } else {
@@ -1861,7 +1968,7 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
         newton_pmhd_init(x0, ns);
         if (subdom) ns.best_eT = -1.0;
         if (subdom || newton_pmhd_run<MET>(p, s, ns, split)) {
-          accept = pmhd_finish<MET>(p, bx, bi, z, t, x1, g, s, Ust, h, ns.best_x, ns.best_eT, ns.steps, P, b, Sst);
+          accept = pmhd_finish<MET>(p, bx, bi, z, t, fl, g, s, Ust, h, ns.best_x, ns.best_eT, ns.steps, P, b, Sst);
           done_steps = (unsigned)ns.steps;
         } else {
           const int slot = atomicAdd(&b.qcount[2], 1);
@@ -1899,8 +2006,9 @@ __global__ void __launch_bounds__(128) k_newton_cont(DevParams p, const BoxGeo* 
     const int j = (int)(r % bx.n[1]);
     const int k = (int)(r / bx.n[1]);
     const long long t = cell_index(bx, i, j, k);
-    const double x1 = xcen(bx, 0, i);
     const Geo<MET, double> g = geo_centre<MET, double>(p, bx, b.geo, i, j);
+    double fl[2];
+    floor_values<MET>(p, xcen(bx, 0, i), &fl[0], &fl[1]);
     const double* cd = b.cdata + (long long)e * CSTRIDE;
     double Ust[NPR];
     for (int q = 0; q < NPR; ++q) Ust[q] = cd[q];
@@ -1910,7 +2018,7 @@ __global__ void __launch_bounds__(128) k_newton_cont(DevParams p, const BoxGeo* 
     ImpSys<MET> s;
     build_sys<MET>(p, g, Ust, h, kfield(p, b.K + bx.coff, t), s);
     newton_pmhd_run<MET>(p, s, ns, 1 << 30);
-    const bool accept = pmhd_finish<MET>(p, bx, bi, z, t, x1, g, s, Ust, h, ns.best_x, ns.best_eT, ns.steps,
+    const bool accept = pmhd_finish<MET>(p, bx, bi, z, t, fl, g, s, Ust, h, ns.best_x, ns.best_eT, ns.steps,
                                          b.P + 12 * bx.coff, b, cd[NPR + 22]);
     if (accept) atomicAdd(&b.stats[ST_PMHD], 1ULL);
     atomicAdd(&b.stats[ST_ITERS], (unsigned long long)ns.steps);
@@ -1955,7 +2063,7 @@ __global__ void k_imex_store(DevParams p, const BoxGeo* __restrict__ boxes, int 
       double Pz[NPR], Uz[NPR], Xz[NPR];
 #pragma unroll
       for (int q = 0; q < NPR; ++q) Pz[q] = Ps[q * bx.nact + z];
-      cons_source<MET, double>(p, g, x1, x2, Pz, Uz, Xz, nullptr);
+      cons_source<MET, double>(p, g, x1, x2, Pz, Uz, Xz);
 #pragma unroll
       for (int q = 0; q < 4; ++q) M[(4 * j + q) * bx.nact + z] = (Uz[UU + q] - Us[(UU + q) * bx.nact + z]) / h;
     }
@@ -2025,7 +2133,9 @@ __global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __rest
     if (b.psol_rec)
       for (int q = 0; q < NPR; ++q) b.psol_rec[12 * bx.aoff + q * bx.nact + z] = Pn[q];
     unsigned fcode = 0;
-    apply_floors<MET>(p, g, log_r<MET>(p, x1), Pn, p.sig ? &fcode : nullptr);
+    double fl[2];
+    floor_values<MET>(p, x1, &fl[0], &fl[1]);
+    apply_floors<MET>(p, g, fl[0], fl[1], Pn, p.sig ? &fcode : nullptr);
     if (p.sig) sig_put(p, bx.coff + t, 60, fcode << 4 | (unsigned)method);
     for (int q = 0; q < NPR; ++q) P[q * bx.ntot + t] = Pn[q];
     unsigned char m = (unsigned char)method;
@@ -2122,7 +2232,9 @@ __global__ void k_backup_apply(DevParams p, const BoxGeo* __restrict__ boxes, Bu
     double Pn[NPR];
     for (int q = 0; q < NPR; ++q) Pn[q] = b.ftmp[(long long)e * NPR + q];
     unsigned fcode = 0;
-    apply_floors<MET>(p, g, log_r<MET>(p, x1), Pn, p.sig ? &fcode : nullptr);
+    double fl[2];
+    floor_values<MET>(p, x1, &fl[0], &fl[1]);
+    apply_floors<MET>(p, g, fl[0], fl[1], Pn, p.sig ? &fcode : nullptr);
     if (p.sig) sig_put(p, bx.coff + t, 62, fcode);
     for (int q = 0; q < NPR; ++q) P[q * bx.ntot + t] = Pn[q];
   }

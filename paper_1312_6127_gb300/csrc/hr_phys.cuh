@@ -44,6 +44,9 @@ struct DevParams {
   // FP32 copies of the parameters the FP32 tangent pass reads (converted once
   // on the host, not per use on the device)
   float gm1f, ymaxf, Tminf, kabs0f, kes0f, aradf;
+  // constants the FP64 kernels would otherwise divide for: Gamma - 1, 1/Gamma,
+  // (Gamma - 1)/Gamma, 1/bsq_rho_max, 1/bsq_u_max, 1/u_rho_max
+  double gm1, igam, gfac, ibsq_rho, ibsq_u, iu_rho;
   // branch signature (a test instrument; null unless enabled): per cell a
   // 64-bit word into which every branch decision of the step is folded
   unsigned long long* sig;
@@ -609,7 +612,7 @@ struct FaceSide {
   // branches (1, 2: c_ms^2 clamped, 4: optically thick radiation speed)
   __device__ __forceinline__ void build(const DevParams& p, const Geo<MET, double>& g, const FaceGeo<MET, d>& f,
                                         double dl, double kf, const double P[NPR], unsigned* code) {
-    const double rho = P[RHO], pg = (p.gam - 1.0) * P[UU], w = rho + P[UU] + pg;
+    const double rho = P[RHO], pg = p.gm1 * P[UU], w = rho + P[UU] + pg;
     lower3<MET>(g, P[U1], P[U2], P[U3], l);
     double igm;
     const double gm = sqrt_rsqrt(fma(P[U1], l[0], fma(P[U2], l[1], fma(P[U3], l[2], 1.0))), &igm);
@@ -830,8 +833,127 @@ __device__ __forceinline__ int rad_invert(const DevParams& p, const Geo<MET, T>&
 // conserved form: Dlab = rho0 u^t, taue = T^t_t + rho0 u^t, Tt[3] = T^t_i,
 // B[3] lab field; guess primitives give the starting W'.  Writes rho0, u_g,
 // u~^i into out[0..4].  Returns 0 on success.
+//
+// With T_i = T^t_i the momentum is Q~_i = alpha T_i, so Q~^2 = alpha^2
+// gamma^{ij} T_i T_j and E = beta^1 T_1 - T_t.  The residual takes two
+// reciprocals and one reciprocal square root; an unmagnetised zone skips the
+// field's terms; a step within the tolerance goes straight to the final state.
 template <int MET>
 __device__ __forceinline__ int gas_invert(const DevParams& p, const Geo<MET, double>& g, double Dlab,
+                                          double taue, const double Tt[3], const double B[3],
+                                          const double* Pg, double tol, double out[5]) {
+  const double a = g.alpha, gam = p.gam;
+  const double D = a * Dlab;
+  double Ep, Qt[3], l[3];  // Q~^i / alpha
+  if constexpr (MET == MINK) {
+    Ep = -taue;
+    Qt[0] = Tt[0];
+    Qt[1] = Tt[1];
+    Qt[2] = Tt[2];
+  } else {
+    const double a01 = a * g.G01;
+    Ep = fma(a * a01, Tt[0], fma(1.0 - a, Dlab, -taue));
+    Qt[0] = fma(g.G13, Tt[2], fma(a01, a01, g.G11) * Tt[0]);
+    Qt[1] = g.G22 * Tt[1];
+    Qt[2] = fma(g.G33, Tt[2], g.G13 * Tt[0]);
+  }
+  const double E = Ep + D, a2 = a * a;
+  const double Qtsq = a2 * fma(Tt[0], Qt[0], fma(Tt[1], Qt[1], Tt[2] * Qt[2]));
+  lower3<MET>(g, B[0], B[1], B[2], l);
+  const double Bsq = a2 * fma(B[0], l[0], fma(B[1], l[1], B[2] * l[2]));
+  const double QdB = a2 * fma(Tt[0], B[0], fma(Tt[1], B[1], Tt[2] * B[2]));
+  const double S2 = QdB * QdB;
+  const bool nomag = Bsq == 0.0;
+  if (!(D > 0.0) || !isfinite(E)) return 1;
+  lower3<MET>(g, Pg[U1], Pg[U2], Pg[U3], l);
+  const double q0 = fma(Pg[U1], l[0], fma(Pg[U2], l[1], Pg[U3] * l[2])), ug0 = Pg[UU] > 0.0 ? Pg[UU] : 0.0;
+  double Wp = fma(D * q0, rcp(1.0 + sqrt64(1.0 + q0)), gam * ug0 * (1.0 + q0));
+  if (!(Wp > 0.0)) Wp = fmax(fabs(Ep), 1e-300);
+  const double gfac = p.gfac;
+  // 1/W, 1/(B^2 + W) and 1 - v~^2 at W' (false where v~^2 >= 1)
+  auto speed = [&](double Wpv, double& W, double& iW, double& iWB, double& vsq, double& omv) -> bool {
+    W = Wpv + D;
+    iW = rcp(W);
+    if (nomag) {
+      iWB = iW;
+      vsq = Qtsq * (iW * iW);
+    } else {
+      iWB = rcp(Bsq + W);
+      vsq = fma(Qtsq * W, W, S2 * fma(2.0, W, Bsq)) * ((iWB * iWB) * (iW * iW));
+    }
+    omv = 1.0 - vsq;
+    return vsq < 1.0 && W > 0.0;
+  };
+  auto resid = [&](double Wpv, double* fo, double* dfo) -> bool {
+    double W, iW, iWB, vsq, omv;
+    if (!speed(Wpv, W, iW, iWB, vsq, omv)) return false;
+    const double gg = rsqrt64(omv);
+    const double chi = fma(-D * ((gg * gg) * vsq), rcp(gg + 1.0), Wpv) * omv;
+    double f = fma(-gfac, chi, Wpv - Ep), df, dvsq;
+    if (nomag) {
+      dvsq = -2.0 * vsq * iW;
+      df = 1.0;
+    } else {
+      const double iW2 = iW * iW, iW3 = iW2 * iW, WB = Bsq + W;
+      f = fma(0.5 * Bsq, 1.0 + vsq, fma(-0.5 * S2, iW2, f));
+      dvsq = -2.0 * iW3 * (iWB * iWB * iWB) * fma(S2, fma(3.0 * W, WB, Bsq * Bsq), Qtsq * W * W * W);
+      df = fma(0.5 * Bsq, dvsq, fma(S2, iW3, 1.0));
+    }
+    *fo = f;
+    *dfo = fma(-gfac, fma(-dvsq, fma(-0.5 * D, gg, W), omv), df);
+    return true;
+  };
+  // primitives at W' (-1 where v~^2 >= 1)
+  auto finish = [&](double Wpv) -> int {
+    double W, iW, iWB, vsq, omv;
+    if (!speed(Wpv, W, iW, iWB, vsq, omv)) return -1;
+    const double gg = rsqrt64(omv);
+    const double chi = fma(-D * ((gg * gg) * vsq), rcp(gg + 1.0), Wpv) * omv;
+    const double rho = D * (omv * gg), ug = chi * p.igam;
+    if (!(rho > 0.0) || !(ug > 0.0) || !isfinite(ug)) return 6;
+    out[0] = rho;
+    out[1] = ug;
+    const double iv = a * gg * iWB, sb = QdB * iW;
+    out[2] = iv * fma(sb, B[0], Qt[0]);
+    out[3] = iv * fma(sb, B[1], Qt[1]);
+    out[4] = iv * fma(sb, B[2], Qt[2]);
+    return 0;
+  };
+  double f = 0.0, df = 0.0;
+  int guard = 0;
+  while (!resid(Wp, &f, &df) && guard < 200) {
+    Wp = 2.0 * Wp + 1e-300;
+    ++guard;
+  }
+  if (guard >= 200) return 2;
+  for (int it = 0; it < 50; ++it) {
+    if (!(df != 0.0) || !isfinite(f) || !isfinite(df)) return 3;
+    double dW = -f * rcp(df);
+    double Wn = Wp + dW, fn = 0.0, dfn = 0.0;
+    if (Wn > 0.0 && fabs(dW) <= tol * Wn) {
+      const int rc = finish(Wn);
+      if (rc >= 0) return rc;
+    }
+    int back = 0;
+    while ((!(Wn > 0.0) || !resid(Wn, &fn, &dfn)) && back < 60) {
+      dW *= 0.5;
+      Wn = Wp + dW;
+      ++back;
+    }
+    if (back >= 60) return 4;
+    Wp = Wn;
+    f = fn;
+    df = dfn;
+    if (fabs(dW) <= tol * fabs(Wp)) return finish(Wp);
+  }
+  return 5;
+}
+
+// The same inversion in the language's divisions and square roots, for split
+// precision: its FP32 stages round the primitives, so a last-bit change here
+// moves a rounding there, and its results are kept to the bit.
+template <int MET>
+__device__ __forceinline__ int gas_invert_ieee(const DevParams& p, const Geo<MET, double>& g, double Dlab,
                                           double taue, const double Tt[3], const double B[3],
                                           const double* Pg, double tol, double out[5]) {
   const double a = g.alpha, gam = p.gam;
@@ -885,6 +1007,14 @@ __device__ __forceinline__ int gas_invert(const DevParams& p, const Geo<MET, dou
     if (!(df != 0.0) || !isfinite(f) || !isfinite(df)) return 3;
     double dW = -f / df;
     double Wn = Wp + dW, fn = 0.0, dfn = 0.0;
+    if (Wn > 0.0 && fabs(dW) <= tol * Wn) {  // converged, unless v~^2 >= 1 there
+      const double W = Wn + D, iW = 1.0 / W, iWB = 1.0 / (Bsq + W);
+      if ((Qtsq * W * W + S2 * (Bsq + 2.0 * W)) * (iWB * iWB) * (iW * iW) < 1.0) {
+        Wp = Wn;
+        conv = true;
+        break;
+      }
+    }
     int back = 0;
     while ((!(Wn > 0.0) || !resid(Wn, &fn, &dfn)) && back < 60) {
       dW *= 0.5;
