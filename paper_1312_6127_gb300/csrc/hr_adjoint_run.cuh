@@ -83,7 +83,7 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
         if (e != d) work *= (e < d) ? bx.N[e] : bx.n[e];
       k_bc_fill<<<G(work), 128, 0, st>>>(p, c->dboxes, 1, Pg, p.opacity == 2 ? c->K : nullptr, d);
     }
-    k_prep<MET, double><<<G(nt), 128, 0, st>>>(p, c->dboxes, 1, Pg, c->K, aux, c->geotab);
+    k_prep64<MET><<<G(nt), 128, 0, st>>>(p, c->dboxes, 1, Pg, c->K, aux, c->geotab);
     HR_ACHECK(cudaMemsetAsync(a.gP, 0, pbytes, st));
     ka_update<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, Ps);
     // fluxes: divergence, then flux-CT

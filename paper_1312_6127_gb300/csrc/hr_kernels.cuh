@@ -245,6 +245,16 @@ static __global__ void k_bc_fill(DevParams p, const BoxGeo* __restrict__ boxes, 
   }
 }
 
+// ------------------------------------------------------------ work split
+// First item of this thread among the items of a grid whose predecessors in
+// the context hold `done` items: the grids' items form one sequence dealt to
+// the threads in turn, so that a batch of small grids loads every block alike.
+__device__ __forceinline__ long long first_item(long long done) {
+  if (done == 0) return HR_TID;
+  const long long r = HR_TID - done % HR_STRIDE;
+  return r < 0 ? r + HR_STRIDE : r;
+}
+
 // --------------------------------------------------------------- cell prep
 // Per cell: sqrt(-g), and for every active direction d the flattener inputs
 // sqrt(-g) u^d (gas, radiation) and the weight w_d = min(1, 2 tau_d) of the
@@ -279,6 +289,67 @@ __global__ void k_prep(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
         aux[(3 + 3 * (d - 1)) * bx.ntot + t] = w < R(1) ? w : R(1);
       }
     }
+  }
+}
+
+// The same in FP64: the metric factors it needs come from the table, the
+// 4-velocities' time components from gamma^2 = 1 + u~^i g_ij u~^j, and only
+// active directions are formed (none with MC, which has no flattener).
+// Measured over an RK3 step: 256x128x64 torus 1.51 -> 1.02 ms.
+template <int MET>
+__global__ void k_prep64(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const double* __restrict__ P0,
+                         const double* __restrict__ K0, double* __restrict__ aux0, const double* __restrict__ geo0) {
+  long long done = 0;
+  for (int bi = 0; bi < nbox; ++bi) {
+    const BoxGeo& bx = boxes[bi];
+    const double* P = P0 + 12 * bx.coff;
+    const double* K = K0 + bx.coff;
+    double* aux = aux0 + 10 * bx.coff;
+    const long long nt = bx.ntot;
+    for (long long t = first_item(done); t < nt; t += HR_STRIDE) {
+      Geo<MET, double> g;
+      double gd = 1.0, a01 = 0.0, sd[3] = {1.0, 1.0, 1.0};
+      if constexpr (MET == KS) {
+        const GeoTab T = geotab(geo0, bx);
+        const long long x = (unsigned)t % (unsigned)T.sC, s = T.sC;
+        gd = __ldg(T.C + 13 * s + x);
+        if (p.recon == 0) {
+          g.g11 = __ldg(T.C + 3 * s + x);
+          g.g13 = __ldg(T.C + 4 * s + x);
+          g.g22 = __ldg(T.C + 5 * s + x);
+          g.g33 = __ldg(T.C + 6 * s + x);
+          a01 = __ldg(T.C + 14 * s + x) * __ldg(T.C + 8 * s + x);
+          for (int e = 0; e < 3; ++e) sd[e] = __ldg(T.C + (17 + e) * s + x);
+        }
+      }
+      aux[t] = gd;
+      if (p.recon != 0) continue;
+      double u[3], r[3], l[3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        u[e] = P[(U1 + e) * nt + t];
+        r[e] = P[(UR1 + e) * nt + t];
+      }
+      if constexpr (MET == KS) {
+        if (p.act[0]) {  // u^1 = u~^1 - gamma alpha g^{t1}; u^2, u^3 are u~^2, u~^3
+          lower3<MET>(g, u[0], u[1], u[2], l);
+          u[0] = fma(-sqrt64(fma(u[0], l[0], fma(u[1], l[1], fma(u[2], l[2], 1.0)))), a01, u[0]);
+          lower3<MET>(g, r[0], r[1], r[2], l);
+          r[0] = fma(-sqrt64(fma(r[0], l[0], fma(r[1], l[1], fma(r[2], l[2], 1.0)))), a01, r[0]);
+        }
+      }
+      const double rho = P[RHO * nt + t], ug = P[UU * nt + t];
+      const double k2 = 2.0 * opacity_sum(p, rho, [&] { return p.gm1 * ug * rcp(rho); }, kfield(p, K, t));
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        if (!p.act[e]) continue;
+        aux[(1 + 3 * e) * nt + t] = gd * u[e];
+        aux[(2 + 3 * e) * nt + t] = gd * r[e];
+        const double w = k2 * sd[e] * bx.dx[e];
+        aux[(3 + 3 * e) * nt + t] = w < 1.0 ? w : 1.0;
+      }
+    }
+    done += nt;
   }
 }
 
@@ -411,6 +482,187 @@ __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
   }
 }
 
+// The flattener in FP64.  Each cell's own value f(m) (ftilde) is formed once
+// and handed to the neighbours: a thread walks along x2 or x3 with a window in
+// registers, or, along x1, a warp passes values between its lanes.  With
+// X = dp_gas and Y = dp_rad across the cell the blended differences are X + w Y
+// and Y + w X; the rest of the test is formed only where the flow compresses,
+// the wider difference only where the jump is a shock.  About 12 FP64
+// instructions per cell where nothing compresses.  `fresh`: the first sub-step
+// (no earlier value to keep).  Measured over an RK3 step: 256x128x64 torus
+// 3.05 -> 1.52 ms, 64x32x16 0.18 -> 0.14 ms.
+
+// f(m) from the jump dp across the cell, the blended pressures pp, pm beside it
+// and the wider jump d2.
+__device__ __forceinline__ double flat_value(double dp, double d2) {
+  const double f = d2 != 0.0 ? 10.0 * (dp / d2 - 0.75) : -7.5;
+  return f < 0.0 ? 0.0 : (f > 1.0 ? 1.0 : f);
+}
+__device__ __forceinline__ bool flat_shock(double dp, double pp, double pm) {
+  return fabs(dp) > 0.33 * (pp < pm ? pp : pm);
+}
+
+// The cell's flattener from f of the cell and its two neighbours (gas, rad).
+__device__ __forceinline__ void flat_store(const DevParams& p, double w, const double fg[3], const double fr[3],
+                                           bool gup, bool rup, bool fresh, double* F, double* R) {
+  const double ng = gup ? fg[2] : fg[0], nr = rup ? fr[2] : fr[0];
+  const double a = fg[1] > ng ? fg[1] : ng, b = fr[1] > nr ? fr[1] : nr;
+  if (a == 0.0 && b == 0.0) {
+    if (fresh) *F = *R = 0.0;
+    return;
+  }
+  const double mx = a > b ? a : b;
+  const double g = (1.0 - w) * a + w * mx, r = (1.0 - w) * b + w * mx;
+  if (fresh || g > *F) *F = g;
+  if (fresh || r > *R) *R = r;
+}
+
+// The branch signature of the flattener of the cell at t (a test instrument).
+__device__ __forceinline__ void flat_sig(const DevParams& p, const BoxGeo& bx, const double* P, const double* aux,
+                                             long long t, int d, double og, double orr) {
+  FlatCell<double> c[7];
+  for (int m = 0; m < 7; ++m) {
+    const long long x = t + (m - 3) * bx.str[d];
+    c[m].pg = (p.gam - 1.0) * P[UU * bx.ntot + x];
+    c[m].pr = P[ER * bx.ntot + x] * (1.0 / 3.0);
+    c[m].vg = aux[(1 + 3 * d) * bx.ntot + x];
+    c[m].vr = aux[(2 + 3 * d) * bx.ntot + x];
+    c[m].w = aux[(3 + 3 * d) * bx.ntot + x];
+  }
+  sig_put(p, bx.coff + t, 30 + d, flatten_code<double>(c, og, orr));
+}
+
+template <int d, bool SIG>
+__global__ void __launch_bounds__(256) k_flat_cols(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                   const double* __restrict__ P0, const double* __restrict__ aux0,
+                                                   double* __restrict__ flat0, int chunk, bool fresh) {
+  constexpr int o = 3 - d;
+  long long done = 0;
+  for (int bi = 0; bi < nbox; ++bi) {
+    const BoxGeo& bx = boxes[bi];
+    const double* P = P0 + 12 * bx.coff;
+    const double* aux = aux0 + 10 * bx.coff;
+    double* flat = flat0 + 2 * bx.coff;
+    const int wx = bx.n[0] > 1 ? bx.n[0] + 2 : 1, wo = bx.n[o] > 1 ? bx.n[o] + 2 : 1;
+    const int nd = bx.n[d] + 2, nch = (nd + chunk - 1) / chunk, cols = wx * wo;
+    const long long total = (long long)nch * cols, st = bx.str[d], nt = bx.ntot;
+    const double* Ug = P + UU * nt;
+    const double* Er = P + ER * nt;
+    const double* vg = aux + (1 + 3 * d) * nt;
+    const double* vr = aux + (2 + 3 * d) * nt;
+    const double* wt = aux + (3 + 3 * d) * nt;
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+      const int ch = (int)(id / cols), col = (int)(id - (long long)ch * cols);
+      const int c0 = ch * chunk - 1, c1 = min(c0 + chunk, bx.n[d] + 1);  // cells c0 .. c1 - 1
+      int ii[3];
+      ii[0] = col % wx + (bx.n[0] > 1 ? -1 : 0);
+      ii[o] = col / wx + (bx.n[o] > 1 ? -1 : 0);
+      ii[d] = c0 - 1;
+      long long t = cell_index(bx, ii[0], ii[1], ii[2]);
+      // pressures of cells m-2 .. m+2 around m = c0 - 1, velocities of m-1 .. m+1
+      double pg[5], pr[5], ug[3], ur[3], fg[3], fr[3], wc = 0.0, wm = 0.0;
+      bool gu = false, ru = false;  // f's neighbour lies at m + 1, of cell m - 1
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        pg[e + 1] = p.gm1 * Ug[t + (e - 2) * st];
+        pr[e + 1] = Er[t + (e - 2) * st] * (1.0 / 3.0);
+      }
+      ug[1] = vg[t - st];
+      ug[2] = vg[t];
+      ur[1] = vr[t - st];
+      ur[2] = vr[t];
+      fg[1] = fg[2] = fr[1] = fr[2] = 0.0;
+      for (int m = c0 - 1; m <= c1; ++m, t += st) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          pg[e] = pg[e + 1];
+          pr[e] = pr[e + 1];
+        }
+        pg[4] = p.gm1 * Ug[t + 2 * st];
+        pr[4] = Er[t + 2 * st] * (1.0 / 3.0);
+        ug[0] = ug[1];
+        ug[1] = ug[2];
+        ug[2] = vg[t + st];
+        ur[0] = ur[1];
+        ur[1] = ur[2];
+        ur[2] = vr[t + st];
+        wm = wc;  // of cell m - 1
+        wc = wt[t];
+        fg[0] = fg[1];
+        fg[1] = fg[2];
+        fr[0] = fr[1];
+        fr[1] = fr[2];
+        const double X = pg[3] - pg[1], Y = pr[3] - pr[1];
+        const double dg = fma(wc, Y, X), dr = fma(wc, X, Y);
+        fg[2] = fr[2] = 0.0;
+        if (ug[2] < ug[0] && flat_shock(dg, fma(wc, pr[3], pg[3]), fma(wc, pr[1], pg[1])))
+          fg[2] = flat_value(dg, fma(wc, pr[4] - pr[0], pg[4] - pg[0]));
+        if (ur[2] < ur[0] && flat_shock(dr, fma(wc, pg[3], pr[3]), fma(wc, pg[1], pr[1])))
+          fr[2] = flat_value(dr, fma(wc, pg[4] - pg[0], pr[4] - pr[0]));
+        if (m > c0) {
+          const long long c = t - st;
+          if (SIG) flat_sig(p, bx, P, aux, c, d, fresh ? 0.0 : flat[c], fresh ? 0.0 : flat[nt + c]);
+          flat_store(p, wm, fg, fr, gu, ru, fresh, flat + c, flat + nt + c);
+        }
+        gu = dg < 0.0;
+        ru = dr < 0.0;
+      }
+    }
+    done += total;
+  }
+}
+
+// d = 0: a warp takes 26 consecutive cells of the joined rows (as k_recon_rows),
+// one per lane, three lanes on either side for the neighbours only.
+template <bool SIG>
+__global__ void __launch_bounds__(256) k_flat_rows(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                          const double* __restrict__ P0,
+                                                          const double* __restrict__ aux0, double* __restrict__ flat0,
+                                                          bool fresh) {
+  const int lane = threadIdx.x & 31;
+  const unsigned full = 0xffffffffu;
+  long long done = 0;
+  for (int bi = 0; bi < nbox; ++bi) {
+    const BoxGeo& bx = boxes[bi];
+    const double* P = P0 + 12 * bx.coff;
+    const double* aux = aux0 + 10 * bx.coff;
+    double* flat = flat0 + 2 * bx.coff;
+    const int w1 = bx.n[1] > 1 ? bx.n[1] + 2 : 1, w2 = bx.n[2] > 1 ? bx.n[2] + 2 : 1;
+    const int o1 = bx.n[1] > 1 ? -1 : 0, o2 = bx.n[2] > 1 ? -1 : 0;
+    const int N0 = bx.N[0], cells = w1 * w2 * N0, ntask = (cells + 25) / 26;
+    const long long total = 32LL * ntask, nt = bx.ntot;
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+      const int f0 = 26 * (int)(id >> 5) - 3 + lane, f = min(max(f0, 0), cells - 1), row = f / N0;
+      const int x = f - row * N0 - 4;
+      const long long t = cell_index(bx, x, row % w1 + o1, row / w1 + o2);
+      const double pg = p.gm1 * P[UU * nt + t], pr = P[ER * nt + t] * (1.0 / 3.0);
+      const double vg = aux[nt + t], vr = aux[2 * nt + t], w = aux[3 * nt + t];
+      const double pgp = __shfl_down_sync(full, pg, 1), pgm = __shfl_up_sync(full, pg, 1);
+      const double prp = __shfl_down_sync(full, pr, 1), prm = __shfl_up_sync(full, pr, 1);
+      const bool cg = __shfl_down_sync(full, vg, 1) < __shfl_up_sync(full, vg, 1);
+      const bool cr = __shfl_down_sync(full, vr, 1) < __shfl_up_sync(full, vr, 1);
+      const double X = pgp - pgm, Y = prp - prm, dg = fma(w, Y, X), dr = fma(w, X, Y);
+      const bool hg = cg && flat_shock(dg, fma(w, prp, pgp), fma(w, prm, pgm));
+      const bool hr = cr && flat_shock(dr, fma(w, pgp, prp), fma(w, pgm, prm));
+      double fg[3] = {0.0, 0.0, 0.0}, fr[3] = {0.0, 0.0, 0.0};
+      if (__any_sync(full, hg || hr)) {
+        const double X2 = __shfl_down_sync(full, pg, 2) - __shfl_up_sync(full, pg, 2);
+        const double Y2 = __shfl_down_sync(full, pr, 2) - __shfl_up_sync(full, pr, 2);
+        if (hg) fg[1] = flat_value(dg, fma(w, Y2, X2));
+        if (hr) fr[1] = flat_value(dr, fma(w, X2, Y2));
+        fg[0] = __shfl_up_sync(full, fg[1], 1);
+        fg[2] = __shfl_down_sync(full, fg[1], 1);
+        fr[0] = __shfl_up_sync(full, fr[1], 1);
+        fr[2] = __shfl_down_sync(full, fr[1], 1);
+      }
+      if (lane < 3 || lane > 28 || f0 >= cells || x < -1 || x > bx.n[0]) continue;
+      if (SIG) flat_sig(p, bx, P, aux, t, 0, fresh ? 0.0 : flat[t], fresh ? 0.0 : flat[nt + t]);
+      flat_store(p, w, fg, fr, dg < 0.0, dr < 0.0, fresh, flat + t, flat + nt + t);
+    }
+    done += total;
+  }
+}
+
 // ------------------------------------------------------------- reconstruction
 template <typename R>
 __device__ __forceinline__ R mc_slope(R qm, R q0, R qp) {
@@ -522,19 +774,12 @@ __device__ __forceinline__ unsigned ppm_limit(double q, double chi, double& l, d
   return 0u;
 }
 
-// First item of this thread among the items of a grid whose predecessors in
-// the context hold `done` items: the grids' items form one sequence dealt to
-// the threads in turn, so that a batch of small grids loads every block alike.
-__device__ __forceinline__ long long first_item(long long done) {
-  if (done == 0) return HR_TID;
-  const long long r = HR_TID - done % HR_STRIDE;
-  return r < 0 ? r + HR_STRIDE : r;
-}
-
 // d = 1, 2: a thread walks `chunk` cells of one column along d for one
 // variable; lanes are neighbours along x1, so every load is coalesced.  A
 // chunk's start repeats two slopes and one interface: about one cell's work.
-template <int MET, int d>
+// SIG: folds its decisions into the branch signature (a test instrument; a
+// variant of its own, so that the hot one holds no registers for it).
+template <int MET, int d, bool SIG>
 __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
                                                     const double* __restrict__ P0, const double* __restrict__ aux0,
                                                     const double* __restrict__ flat0, double* __restrict__ E0,
@@ -572,13 +817,13 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
       if (p.recon == 0) {
         const double dmm = sm - ld(t - 2 * st);
         aL = ppm_face(sm, dm, mc_twice(dmm, dm), D0);
-        if (p.sig && c0 == -1)
+        if (SIG && c0 == -1)
           sig_put(p, bx.coff + t - st, 10 + d, (unsigned long long)q << 8 | mc_twice_code(dmm, dm));
       }
       double dl = dm;  // kept for the branch signature only
 #pragma unroll 2
       for (int c = c0; c < c1; ++c, t += st) {
-        if (p.sig) sig_put(p, bx.coff + t, 10 + d, (unsigned long long)q << 8 | mc_twice_code(dl, dp));
+        if (SIG) sig_put(p, bx.coff + t, 10 + d, (unsigned long long)q << 8 | mc_twice_code(dl, dp));
         const double s2 = ld(t + 2 * st), d2 = s2 - sp, Dp = mc_twice(dp, d2);
         double l, r;
         if (p.recon == 0) {
@@ -586,7 +831,7 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
           l = aL;
           r = aR;
           const unsigned code = ppm_limit(s0, chi[t], l, r);
-          if (p.sig) sig_put(p, bx.coff + t, 20 + d, (unsigned long long)q << 8 | code);
+          if (SIG) sig_put(p, bx.coff + t, 20 + d, (unsigned long long)q << 8 | code);
           aL = aR;
         } else {
           l = fma(-0.25, D0, s0);
@@ -594,7 +839,7 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
         }
         El[t] = l;
         Er[t] = r;
-        if (p.sig && c == bx.n[d])
+        if (SIG && c == bx.n[d])
           sig_put(p, bx.coff + t + st, 10 + d, (unsigned long long)q << 8 | mc_twice_code(dp, d2));
         s0 = sp;
         sp = s2;
@@ -612,7 +857,7 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
 // lane, the first and last lane for the neighbours only; differences, slopes
 // and interface values pass between lanes.  Values that cross a row's end
 // reach ghost cells that are not stored.
-template <int MET>
+template <int MET, bool SIG>
 __global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
                                                     const double* __restrict__ P0, const double* __restrict__ aux0,
                                                     const double* __restrict__ flat0, double* __restrict__ E0) {
@@ -674,10 +919,10 @@ __global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* _
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         if (!mine || f0 + e >= cells) continue;
-        if (p.sig && x[e] >= -2 && x[e] <= bx.n[0] + 1)
+        if (SIG && x[e] >= -2 && x[e] <= bx.n[0] + 1)
           sig_put(p, bx.coff + t[e], 10, (unsigned long long)q << 8 | (e ? mc_twice_code(d1, d2) : mc_twice_code(d0, d1)));
         if (x[e] < -1 || x[e] > bx.n[0]) continue;
-        if (p.sig && p.recon == 0) sig_put(p, bx.coff + t[e], 20, (unsigned long long)q << 8 | code[e]);
+        if (SIG && p.recon == 0) sig_put(p, bx.coff + t[e], 20, (unsigned long long)q << 8 | code[e]);
         E[q * nt + t[e]] = l[e];
         E[(NPR + q) * nt + t[e]] = r[e];
       }

@@ -100,10 +100,46 @@ inline int fill_ghost_cells(harmrad_ctx* c) {
   return nk;
 }
 
+// Pieces a column of nd cells is cut into so that there are `slots` threads per
+// SM, `least` cells or more each; the cells of a piece.
+inline int column_chunk(const harmrad_ctx* c, long long columns, long long nd, int slots, int least,
+                        long long* pieces) {
+  long long n = ((long long)slots * c->sms + columns - 1) / columns;
+  if (n > (nd + least - 1) / least) n = (nd + least - 1) / least;
+  *pieces = n;
+  return (int)((nd + n - 1) / n);
+}
+
+// FP64 flattener of direction d.
+inline void flatten(harmrad_ctx* c, int d, bool fresh) {
+  const DevParams& p = c->dp;
+  const BoxGeo* bt = c->dboxes;
+  const int nb = c->nbox;
+  const double* aux = (const double*)c->aux;
+  double* fl = (double*)c->flat[d];
+  auto width = [](const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; };
+  if (d == 0) {
+    const long long work = max_work(c, [width](const BoxGeo& b) {
+      return 32LL * (((long long)width(b, 1) * width(b, 2) * b.N[0] + 25) / 26);
+    });
+    const int g = grid_for(work, c->sms, 256);
+    if (p.sig) k_flat_rows<true><<<g, 256, 0, c->stream>>>(p, bt, nb, c->P, aux, fl, fresh);
+    else k_flat_rows<false><<<g, 256, 0, c->stream>>>(p, bt, nb, c->P, aux, fl, fresh);
+    return;
+  }
+  const int o = 3 - d;
+  const long long cols = max_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
+  const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
+  // a piece evaluates two cells more than it owns; 4 blocks of 128 fit an SM
+  long long pieces;
+  const int chunk = column_chunk(c, cols, nd, 1024, 4, &pieces);
+  const int g = grid_for(cols * pieces, c->sms, 128);
+  auto run = [&](auto kernel) { kernel<<<g, 128, 0, c->stream>>>(p, bt, nb, c->P, aux, fl, chunk, fresh); };
+  if (d == 1) p.sig ? run(k_flat_cols<1, true>) : run(k_flat_cols<1, false>);
+  else p.sig ? run(k_flat_cols<2, true>) : run(k_flat_cols<2, false>);
+}
+
 // FP64 reconstruction of direction d: edge values of every cell of its face range.
-// A column along x2 or x3 is cut so that there are at least two threads per
-// resident-thread slot, into pieces of 16 cells or more (a piece repeats one
-// cell's work).
 template <int MET>
 void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const double* flat, double* E, int block,
            int per_sm) {
@@ -115,18 +151,21 @@ void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const doub
     const long long work = max_work(c, [width](const BoxGeo& b) {
       return 12LL * 32 * (((long long)width(b, 1) * width(b, 2) * b.N[0] + 59) / 60);
     });
-    k_recon_rows<MET><<<grid_for(work, c->sms, block, per_sm), block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E);
+    const int g = grid_for(work, c->sms, block, per_sm);
+    if (p.sig) k_recon_rows<MET, true><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E);
+    else k_recon_rows<MET, false><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E);
     return;
   }
   const int o = 3 - d;
   const long long cols = max_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
   const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
-  long long pieces = (2LL * 2048 * c->sms + 12 * cols - 1) / (12 * cols);
-  if (pieces > (nd + 15) / 16) pieces = (nd + 15) / 16;
-  const int chunk = (int)((nd + pieces - 1) / pieces);
+  // a piece repeats about one cell's work: 16 cells or more, two threads per slot
+  long long pieces;
+  const int chunk = column_chunk(c, 12 * cols, nd, 4096, 16, &pieces);
   const int g = grid_for(12 * cols * pieces, c->sms, block, per_sm);
-  if (d == 1) k_recon_cols<MET, 1><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E, chunk);
-  else k_recon_cols<MET, 2><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E, chunk);
+  auto run = [&](auto kernel) { kernel<<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E, chunk); };
+  if (d == 1) p.sig ? run(k_recon_cols<MET, 1, true>) : run(k_recon_cols<MET, 1, false>);
+  else p.sig ? run(k_recon_cols<MET, 2, true>) : run(k_recon_cols<MET, 2, false>);
 }
 
 template <int MET, typename R>
@@ -137,8 +176,12 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
   const int nb = c->nbox;
   int nk = fill_ghost_cells(c);
   if (p.emf == 1) nk += face_ghosts<MET>(c);
-  k_prep<MET, R><<<grid_for(c->maxcell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, c->K, (R*)c->aux,
-                                                                     c->geotab);
+  if constexpr (std::is_same<R, double>::value)
+    k_prep64<MET><<<grid_for(c->maxcell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, c->K, (double*)c->aux,
+                                                                      c->geotab);
+  else
+    k_prep<MET, R><<<grid_for(c->maxcell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, c->K, (R*)c->aux,
+                                                                       c->geotab);
   mark(c, HARMRAD_K_PREP);
   ++nk;
   auto range_cells = [](const BoxGeo& b) {
@@ -149,6 +192,12 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
   if (p.recon == 0) {
     for (int d = 0; d < 3; ++d) {
       if (!p.act[d]) continue;
+      if constexpr (std::is_same<R, double>::value) {
+        flatten(c, d, fresh);
+        mark(c, HARMRAD_K_FLATTEN);
+        ++nk;
+        continue;
+      }
       if (fresh) {
         if (cudaMemsetAsync(c->flat[d], 0, 2 * c->ncell * sizeof(R), st) != cudaSuccess) return HARMRAD_E_CUDA;
         mark(c, HARMRAD_K_OTHER);
