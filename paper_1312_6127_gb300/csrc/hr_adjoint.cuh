@@ -444,7 +444,7 @@ __global__ void ka_ct_T(BoxGeo bx, const double* __restrict__ gemf, double* __re
 // Per face: cotangents of the two reconstructed states from the flux's
 // cotangent (25 inputs: P_L, P_R, kappa_scale; five dual passes).
 template <int MET, int d>
-__global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, const double* __restrict__ E,
+__global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, EdgeSet E,
                                                const double* __restrict__ K, const double* __restrict__ gF,
                                                double* __restrict__ gE, double* gk_out,
                                                const double* __restrict__ gFS) {
@@ -492,8 +492,8 @@ __global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, const dou
     double PL[NPR], PR[NPR], wL[NPR];
     for (int q = 0; q < NPR; ++q) {
       const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
-      const double aR = E[(NPR + q) * bx.ntot + t - st];
-      const double bL = E[q * bx.ntot + t];
+      const double aR = E.plane(1, q, bx.ntot)[t - st];
+      const double bL = E.plane(0, q, bx.ntot)[t];
       PL[q] = wq ? aR * igf : aR;
       PR[q] = wq ? bL * igf : bL;
       wL[q] = wq ? igf : 1.0;

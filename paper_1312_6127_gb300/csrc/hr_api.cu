@@ -385,7 +385,7 @@ void free_all(harmrad_ctx* c) {
                   c->aux, c->flat[0], c->flat[1], c->flat[2], c->emf, c->edges, c->dt, c->status,
                   c->iters, c->failed, c->qcount, c->czone, c->cbox, c->cdata, c->qzone, c->qbox, c->qdata, c->fzone, c->fbox,
                   c->ftmp, c->stats, c->dtmin, c->stage_buf, c->flag, c->dboxes, c->imex_ust, c->imex_psol,
-                  c->imex_M, c->sig, c->Sn, c->FS[0], c->FS[1], c->FS[2], c->Bf[0], c->Bf[1], c->Bf[2],
+                  c->imex_M, c->sig, c->Sn, c->FS[0], c->FS[1], c->FS[2], c->ES[0], c->ES[1], c->ES[2], c->Bf[0], c->Bf[1], c->Bf[2],
                   c->Bfn[0], c->Bfn[1], c->Bfn[2], c->gsp[0], c->gsp[1], c->gsp[2], c->vel, c->emf3[0],
                   c->emf3[1], c->emf3[2]};
   for (void* q : ptrs)
@@ -477,11 +477,13 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
   rc = rc ? rc : dalloc(&c->K, nk * sizeof(double));
   if (goff > 0) rc = rc ? rc : dalloc(&c->geotab, goff * sizeof(double));
   rc = rc ? rc : dalloc(&c->Un, 12 * na * sizeof(double));
-  if (dp.integrator == 0) rc = rc ? rc : dalloc(&c->Sn, na * sizeof(double));
+  const bool f64 = rs == sizeof(double);
+  if (dp.integrator == 0) rc = rc ? rc : dalloc(&c->Sn, (f64 ? 2 : 1) * na * sizeof(double));
   for (int d = 0; d < 3; ++d) {
     size_t fn = dp.act[d] ? nt : 0;
     rc = rc ? rc : dalloc(&c->F[d], 12 * fn * rs);
     if (dp.integrator == 0 && fn) rc = rc ? rc : dalloc(&c->FS[d], fn * rs);
+    if (f64 && fn) rc = rc ? rc : dalloc(&c->ES[d], 4 * fn * rs);
     rc = rc ? rc : dalloc(&c->spd[d], fn * rs);
     rc = rc ? rc : dalloc(&c->flat[d], 2 * fn * rs);
   }
@@ -496,7 +498,7 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     }
     rc = rc ? rc : dalloc(&c->vel, 3 * nt * rs);
   }
-  rc = rc ? rc : dalloc(&c->edges, 24 * nt * rs);
+  rc = rc ? rc : dalloc(&c->edges, (f64 ? 20 : 24) * nt * rs);
   rc = rc ? rc : dalloc(&c->dt, count * sizeof(double));
   rc = rc ? rc : dalloc(&c->status, na);
   rc = rc ? rc : dalloc(&c->iters, na * sizeof(int));

@@ -28,8 +28,9 @@ struct harmrad_ctx {
   double* K;
   double* geotab;  // metric tables of Kerr-Schild grids (null for Minkowski)
   double* Un;
-  double* Sn;   // [nact] conserved entropy sqrt(-g) S u^t at the start of the step (RK3)
-  void* FS[3];  // [ntot] entropy face fluxes of each active direction (RK3; null otherwise)
+  double* Sn;   // RK3: FP64 [2][nact] rho0, u_g at the start of the step; split [nact] sqrt(-g) S u^t
+  void* FS[3];  // RK3, [ntot] per active direction: FP64 left mass flux, split entropy face flux (null otherwise)
+  double* ES[3];  // FP64: [4][ntot] edges of rho0 and u_g of each active direction
   void* F[3];
   void* spd[3];
   void* aux;
@@ -44,7 +45,7 @@ struct harmrad_ctx {
   void* gsp[3];
   void* vel;
   void* emf3[3];
-  void* edges;  // [2][12][ntot] reconstructed edge values of one direction
+  void* edges;  // reconstructed edge values of one direction: FP64 [2][10][ntot] (without rho0, u_g), split [2][12][ntot]
   double* dt;
   unsigned char* status;
   int* iters;

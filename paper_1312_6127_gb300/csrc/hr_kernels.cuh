@@ -22,14 +22,17 @@ struct Bufs {
   double* P;       // [12][ntot] primitives, ghosts included (per grid)
   double* K;       // [ntot] per-zone absorption opacity (opacity field mode), ghosts included
   double* Un;      // [12][nact] conserved state at the start of the step
-  double* Sn;      // [nact] conserved entropy at the start of the step (RK3; null otherwise)
+  double* Sn;      // RK3, null otherwise.  FP64: [2][nact] rho0 and u_g at the start of the
+                   // step; split: [nact] the conserved entropy there
   void* F[3];      // [12][ntot] face fluxes (real type of the precision mode)
-  void* FS[3];     // [ntot] entropy face fluxes (RK3; null otherwise)
+  void* FS[3];     // RK3, null otherwise: [ntot] FP64: left state's share of the mass flux;
+                   // split: the entropy face flux
+  double* ES[3];   // FP64: [4][ntot] edges of rho0 and u_g of each direction (EdgeSet)
   void* spd[3];    // [ntot] per-face max signal speed
   void* aux;       // [10][ntot] per-cell gdet, sqrt(-g) u^d gas/rad, tau weights
   void* flat[3];   // [2][ntot] flattener, max over the sub-steps of the step
   void* emf;       // [ntot] edge EMF scratch
-  void* edges;     // [24][ntot] reconstructed edges of one direction
+  void* edges;     // reconstructed edges of one direction: FP64 [20][ntot] (EdgeSet), split [24][ntot]
   double* dt;      // [nbox] time step of each grid
   unsigned char* status;  // [nact] worst outcome over the sub-steps
   int* iters;             // [nact] Newton steps summed over the sub-steps
@@ -57,6 +60,20 @@ struct Bufs {
   double* Bf[3];              // staggered field: sqrt(-g) B^d on the d-faces [ntot] (null: flux-CT)
 };
 
+
+// FP64 edge values of one direction: [lower, upper][q - 2][ntot] of the primitives
+// q >= 2 in E, which every direction reuses, and [lower, upper][q][ntot] of rho0
+// and u_g in S, which each direction keeps: the entropy fluxes are formed from
+// them where a zone needs them (entropy_flux).
+struct EdgeSet {
+  double* E;
+  double* S;
+  __device__ __forceinline__ EdgeSet box(const BoxGeo& b) const { return {E + 20 * b.coff, S + 4 * b.coff}; }
+  // plane of primitive q's lower (up = 0) or upper (1) edges
+  __device__ __forceinline__ double* plane(int up, int q, long long nt) const {
+    return q < U1 ? S + (2 * up + q) * nt : E + (10 * up + q - U1) * nt;
+  }
+};
 
 // Counter update aggregated over the converged lanes of a warp.
 __device__ __forceinline__ void warp_add(unsigned long long* dst, unsigned v) {
@@ -711,8 +728,7 @@ __device__ __forceinline__ void ppm_cell(const R s[5], R chi, R* aL, R* aR) {
 // FP64 reconstruction of one direction: the PPM parabola (or MC line) of every
 // primitive in every cell of the face range (cells -1..n_d along d, transverse
 // range widened by one layer), flattened by the cell's GAS or RAD flattener and
-// stored as the two edge values E[q] (lower) and E[12 + q] (upper); the face
-// kernel reads the upper edge of cell f-1 and the lower edge of cell f.  In r
+// stored as its two edge values (EdgeSet); the face kernel reads the upper edge of cell f-1 and the lower edge of cell f.  In r
 // and phi on the Kerr-Schild grid the velocity and field components are
 // reconstructed as sqrt(-g) times the primitive (Sec. 4.3).
 //
@@ -782,8 +798,7 @@ __device__ __forceinline__ unsigned ppm_limit(double q, double chi, double& l, d
 template <int MET, int d, bool SIG>
 __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
                                                     const double* __restrict__ P0, const double* __restrict__ aux0,
-                                                    const double* __restrict__ flat0, double* __restrict__ E0,
-                                                    int chunk) {
+                                                    const double* __restrict__ flat0, EdgeSet E0, int chunk) {
   const bool weighted = (MET == KS) && (d != 1);
   constexpr int o = 3 - d;  // the other transverse direction beside x1
   long long done = 0;
@@ -792,7 +807,7 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
     const double* P = P0 + 12 * bx.coff;
     const double* aux = aux0 + 10 * bx.coff;
     const double* flat = flat0 + 2 * bx.coff;
-    double* E = E0 + 24 * bx.coff;
+    const EdgeSet E = E0.box(bx);
     const int wx = bx.n[0] > 1 ? bx.n[0] + 2 : 1, wo = bx.n[o] > 1 ? bx.n[o] + 2 : 1;
     const int nd = bx.n[d] + 2, nch = (nd + chunk - 1) / chunk, cols = wx * wo;
     const long long total = 12LL * nch * cols, st = bx.str[d], nt = bx.ntot;
@@ -808,8 +823,8 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
       const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
       const double* Pq = P + q * nt;
       const double* chi = flat + (q < ER ? 0 : nt);
-      double* El = E + q * nt;
-      double* Er = E + (NPR + q) * nt;
+      double* __restrict__ El = E.plane(0, q, nt);
+      double* __restrict__ Er = E.plane(1, q, nt);
       auto ld = [&](long long x) { return wq ? aux[x] * Pq[x] : Pq[x]; };
       double s0 = ld(t), sp = ld(t + st), dp = sp - s0;
       const double sm = ld(t - st), dm = s0 - sm;
@@ -860,7 +875,7 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
 template <int MET, bool SIG>
 __global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
                                                     const double* __restrict__ P0, const double* __restrict__ aux0,
-                                                    const double* __restrict__ flat0, double* __restrict__ E0) {
+                                                    const double* __restrict__ flat0, EdgeSet E0) {
   const bool weighted = (MET == KS);
   const int lane = threadIdx.x & 31;
   const unsigned full = 0xffffffffu;
@@ -870,7 +885,7 @@ __global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* _
     const double* P = P0 + 12 * bx.coff;
     const double* aux = aux0 + 10 * bx.coff;
     const double* flat = flat0 + 2 * bx.coff;
-    double* E = E0 + 24 * bx.coff;
+    const EdgeSet E = E0.box(bx);
     const int w1 = bx.n[1] > 1 ? bx.n[1] + 2 : 1, w2 = bx.n[2] > 1 ? bx.n[2] + 2 : 1;
     const int o1 = bx.n[1] > 1 ? -1 : 0, o2 = bx.n[2] > 1 ? -1 : 0;
     const int N0 = bx.N[0], cells = w1 * w2 * N0, ntask = (cells + 59) / 60;
@@ -923,8 +938,8 @@ __global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* _
           sig_put(p, bx.coff + t[e], 10, (unsigned long long)q << 8 | (e ? mc_twice_code(d1, d2) : mc_twice_code(d0, d1)));
         if (x[e] < -1 || x[e] > bx.n[0]) continue;
         if (SIG && p.recon == 0) sig_put(p, bx.coff + t[e], 20, (unsigned long long)q << 8 | code[e]);
-        E[q * nt + t[e]] = l[e];
-        E[(NPR + q) * nt + t[e]] = r[e];
+        E.plane(0, q, nt)[t[e]] = l[e];
+        E.plane(1, q, nt)[t[e]] = r[e];
       }
     }
     done += total;
@@ -1085,11 +1100,13 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
                                               const R* __restrict__ E0, const double* __restrict__ K0,
                                               R* __restrict__ F0, R* __restrict__ spd0,
                                               const double* __restrict__ geo0, R* __restrict__ FS0,
-                                              R* __restrict__ gsp0 = nullptr) {
+                                              R* __restrict__ gsp0, const double* __restrict__ S0) {
   const bool weighted = (MET == KS) && (d != 1);
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
-    const R* E = E0 + 24 * bx.coff;
+    constexpr bool F64 = std::is_same<R, double>::value;
+    const R* E = E0 + (F64 ? 20 : 24) * bx.coff;
+    const double* S = F64 ? S0 + 4 * bx.coff : nullptr;  // edges of rho0 and u_g
     const double* K = K0 + bx.coff;
     R* F = F0 + 12 * bx.coff;
     R* spd = spd0 + bx.coff;
@@ -1149,8 +1166,14 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
 #pragma unroll
       for (int q = 0; q < NPR; ++q) {
         const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
-        R aR = E[(NPR + q) * bx.ntot + t - st];  // upper edge of cell f-1
-        R bL = E[q * bx.ntot + t];               // lower edge of cell f
+        R aR, bL;  // upper edge of cell f-1, lower edge of cell f
+        if constexpr (F64) {
+          aR = q < U1 ? S[(2 + q) * bx.ntot + t - st] : E[(10 + q - U1) * bx.ntot + t - st];
+          bL = q < U1 ? S[q * bx.ntot + t] : E[(q - U1) * bx.ntot + t];
+        } else {
+          aR = E[(NPR + q) * bx.ntot + t - st];
+          bL = E[q * bx.ntot + t];
+        }
         PL[q] = wq ? aR * igf : aR;
         PR[q] = wq ? bL * igf : bL;
       }
@@ -2018,6 +2041,44 @@ __device__ int backup_equations(const DevParams& p, const Geo<MET, double>& g, c
   return 0;
 }
 
+// The explicit entropy S* = a_s S^n + b_s (S(P_s) + dt X_S) of a zone (FP64,
+// RK3), formed where it is read: by the zones that reach the entropy equation
+// (Sec. 4.7, 4.11), few in any run, or by all zones in the entropy-everywhere
+// mode.  Two logarithms per face were a quarter of the face kernel when every
+// face formed its flux (256x128x64 torus, per RK3 step: faces 17.4 -> 13.8 ms,
+// update 21.7 -> 20.5 ms without); the face kernel now keeps the left state's mass flux
+// mL, and the flux is s_L mL + s_R (F_rho - mL) with the entropy per baryon s
+// of the kept edges (Sec. 2, Eq. S).
+static __device__ __forceinline__ double entropy_flux(const DevParams& p, const BoxGeo& bx, const Bufs& b, int d,
+                                                      long long t) {
+  const double* S = b.ES[d] + 4 * bx.coff;
+  const long long nt = bx.ntot, tm = t - bx.str[d];
+  const double mL = ((const double*)b.FS[d])[bx.coff + t], m = ((const double*)b.F[d])[12 * bx.coff + t];
+  return entropy_per_baryon<double>(p, S[2 * nt + tm], S[3 * nt + tm]) * mL +
+         entropy_per_baryon<double>(p, S[t], S[nt + t]) * (m - mL);
+}
+// Us0 = sqrt(-g) rho0 u^t of the sub-step's input, rho, ug its density and
+// internal energy; z, t the zone's active and cell index.
+__device__ __forceinline__ double entropy_star(const DevParams& p, const BoxGeo& bx, const Bufs& b, long long z,
+                                               long long t, int stage, double dt, double Us0, double rho,
+                                               double ug) {
+  const double A = stage == 0 ? 0.0 : (stage == 1 ? 0.75 : 1.0 / 3.0);
+  const double Bc = stage == 0 ? 1.0 : (stage == 1 ? 0.25 : 2.0 / 3.0);
+  const double Su = Us0 * entropy_per_baryon<double>(p, rho, ug);
+  const double* Sn = b.Sn + 2 * bx.aoff;
+  const double sn =
+      stage == 0 ? Su : b.Un[12 * bx.aoff + z] * entropy_per_baryon<double>(p, Sn[z], Sn[bx.nact + z]);
+  double div = 0.0;
+#pragma unroll 1
+  for (int f = 0; f < 6; ++f) {  // the upper and the lower face of each direction
+    const int d = f >> 1;
+    if (!p.act[d]) continue;
+    const double v = entropy_flux(p, bx, b, d, t + (f & 1 ? 0 : bx.str[d])) / bx.dx[d];
+    div += f & 1 ? -v : v;
+  }
+  return A * sn + Bc * (Su - dt * div);
+}
+
 // ------------------------------------------------------- update + implicit
 // One thread per active zone: U(P_s), the geometric source
 // SM_nu = 1/2 sqrt(-g) T^{mu kappa} d_nu g_{mu kappa}  (equal to
@@ -2132,29 +2193,37 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
 #pragma unroll
         for (int q = 0; q < NPR; ++q) b.ust_rec[12 * bx.aoff + q * bx.nact + z] = Ust[q];
       }
-      // RK3: the explicit entropy S* = a_s S^n + b_s (S(P_s) + dt X_S), the
-      // conserved entropy sqrt(-g) S u^t = U_rho s_gas (Sec. 2, Eq. S), for the
-      // entropy equation of the implicit solve (Sec. 4.7, 4.11); NaN: none
+      // RK3: what the explicit entropy needs of the step's start (FP64,
+      // entropy_star; where every zone takes the entropy equation it is formed
+      // here), or, in split precision, the explicit entropy
+      // S* = a_s S^n + b_s (S(P_s) + dt X_S) itself; NaN: none
       double Sst = NAN;
       if (!IMEX && b.Sn) {
-        const double Su = Us[RHO] * entropy_per_baryon<double>(p, Ps[RHO], Ps[UU]);
-        double* Sn = b.Sn + bx.aoff;
-        double sn;
-        if (stage == 0) {
-          Sn[z] = Su;
-          sn = Su;
+        if constexpr (std::is_same<R, double>::value) {
+          if (stage == 0) {
+            b.Sn[2 * bx.aoff + z] = Ps[RHO];
+            b.Sn[2 * bx.aoff + bx.nact + z] = Ps[UU];
+          }
+          if (p.implicit_eq == 1) Sst = entropy_star(p, bx, b, z, t, stage, dt, Us[RHO], Ps[RHO], Ps[UU]);
         } else {
-          sn = Sn[z];
-        }
-        double divS = 0.0;
+          const double Su = Us[RHO] * entropy_per_baryon<double>(p, Ps[RHO], Ps[UU]);
+          double* Sn = b.Sn + bx.aoff;
+          double sn;
+          if (stage == 0) {
+            Sn[z] = Su;
+            sn = Su;
+          } else {
+            sn = Sn[z];
+          }
+          double divS = 0.0;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          if (!p.act[d]) continue;
-          const R* FSd = (const R*)b.FS[d] + bx.coff;
-          divS += double(FSd[t + bx.str[d]] - FSd[t]) * idx[d];
+          for (int d = 0; d < 3; ++d) {
+            if (!p.act[d]) continue;
+            const R* FSd = (const R*)b.FS[d] + bx.coff;
+            divS += double(FSd[t + bx.str[d]] - FSd[t]) * idx[d];
+          }
+          Sst = A * sn + Bc * (Su - dt * divS);
         }
-        Sst = A * sn + Bc * (Su - dt * divS);
-        if (b.sst_rec) b.sst_rec[bx.aoff + z] = Sst;
       }
       // implicit solve
       const double h = IMEX ? im.g * dt : Bc * dt;
@@ -2321,7 +2390,7 @@ __global__ void k_imex_store(DevParams p, const BoxGeo* __restrict__ boxes, int 
 // then PRAD (retry_sequence); e_T > 1e-7 sends the zone to the
 // neighbour-average back-up.
 template <int MET>
-__global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __restrict__ boxes, Bufs b) {
+__global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __restrict__ boxes, Bufs b, int stage) {
   const int nq = b.qcount[0];
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nq; e += gridDim.x * blockDim.x) {
     const long long z = b.qzone[e];
@@ -2355,7 +2424,15 @@ __global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __rest
     int steps;
     const double tau = zone_tau<MET>(p, g, bx.dx, Ps, kfield(p, K, t));
     int method;
-    const double Sst = qd[18];
+    double Sst = qd[18];
+    // FP64: the explicit entropy, where the sequence reads it
+    auto entropy = [&] {
+      if (p.precision != 0 || !b.Sn) return;
+      double u[4], v[4], gm;
+      fourvel<MET, double>(g, Ps[U1], Ps[U2], Ps[U3], u, v, &gm);
+      Sst = entropy_star(p, bx, b, z, t, stage, b.dt[bi], g.gdet * Ps[RHO] * u[0], Ps[RHO], Ps[UU]);
+      if (b.sst_rec) b.sst_rec[zg] = Sst;
+    };
     if (p.implicit_eq == 1) {  // the entropy PMHD of the update kernel left e_T >= 1e-9
       for (int q = 0; q < NPR; ++q) Pn[q] = Ps[q];
       for (int c = 0; c < 3; ++c) Pn[B1 + c] = s.B[c];
@@ -2363,11 +2440,13 @@ __global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __rest
       steps = 0;
       method = ST_BACKUP;
     } else {
+      if (subdom) entropy();
       method = retry_sequence<MET>(p, g, s, Ps, px, peT, tau, Pn, &eT, &steps, subdom, Sst);
     }
     // no energy-based solution: the entropy, then the cold-MHD equations
     int by = 0;
     if (method == ST_BACKUP) {
+      if (p.implicit_eq != 1 && !subdom) entropy();
       by = p.implicit_eq == 1 ? backup_equations<MET>(p, g, s, Ust, Ps, Sst, 2, tau, Pn, &eT, &steps, px, peT)
                               : backup_equations<MET>(p, g, s, Ust, Ps, Sst, 1, tau, Pn, &eT, &steps);
       // a retry method's solution, except that in the entropy-everywhere

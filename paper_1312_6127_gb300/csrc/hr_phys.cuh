@@ -698,12 +698,13 @@ struct FaceSide {
 };
 
 // HLL or LAXF flux of one face (face_flux in FP64): out the 12 rows with
-// F[B_d] = 0, smax the largest speed, fs (optional) the entropy flux, gas
-// (optional) the gas speeds v_max, v_min, code (optional) the branches.
+// F[B_d] = 0, smax the largest speed, mass (optional) the left state's share of
+// the mass flux (for the entropy flux, see entropy_flux), gas (optional) the gas
+// speeds v_max, v_min, code (optional) the branches.
 template <int MET, int d>
 __device__ __forceinline__ void face_flux64(const DevParams& p, const Geo<MET, double>& g, double dl, double kL,
                                             double kR, const double PL[NPR], const double PR[NPR], double out[NPR],
-                                            double* smax, unsigned* code, double* fs, double* gas) {
+                                            double* smax, unsigned* code, double* mass, double* gas) {
   const FaceGeo<MET, d> f(g);
   FaceSide<MET, d> L, R;
   unsigned cL = 0, cR = 0;
@@ -739,10 +740,10 @@ __device__ __forceinline__ void face_flux64(const DevParams& p, const Geo<MET, d
   *smax = fmax(c[0], c[1]);
 #pragma unroll
   for (int q = 0; q < NPR; ++q) out[q] = 0.0;
-  double mL, mR, sc[2];
+  double mL, sc[2];
   if (p.flux == 0) {  // LAXF: 1/2 (F_L + F_R - c (U_R - U_L))
     mL = L.template add<true>(g, PL, 1.0, c[0], 1.0, c[1], out);
-    mR = R.template add<true>(g, PR, 1.0, -c[0], 1.0, -c[1], out);
+    R.template add<true>(g, PR, 1.0, -c[0], 1.0, -c[1], out);
     sc[0] = sc[1] = 0.5 * g.gdet;
   } else {  // HLL: (c- F_R + c+ F_L - c- c+ (U_R - U_L)) / (c- + c+)
     double aL[2], aR[2], aU[2];
@@ -756,11 +757,9 @@ __device__ __forceinline__ void face_flux64(const DevParams& p, const Geo<MET, d
       sc[w] = g.gdet * (ok ? rcp(sum) : 0.5);
     }
     mL = L.template add<false>(g, PL, aL[0], aU[0], aL[1], aU[1], out);
-    mR = R.template add<false>(g, PR, aR[0], -aU[0], aR[1], -aU[1], out);
+    R.template add<false>(g, PR, aR[0], -aU[0], aR[1], -aU[1], out);
   }
-  if (fs)  // entropy flux: s_gas times the mass flux of each state (Sec. 2, Eq. S)
-    *fs = sc[0] * fma(entropy_per_baryon<double>(p, PL[RHO], PL[UU]), mL,
-                      entropy_per_baryon<double>(p, PR[RHO], PR[UU]) * mR);
+  if (mass) *mass = sc[0] * mL;
 #pragma unroll
   for (int q = 0; q < NPR; ++q) out[q] *= sc[q < ER ? 0 : 1];
   out[B1 + d - 1] = 0.0;

@@ -15,6 +15,7 @@ inline Bufs make_bufs(harmrad_ctx* c) {
   for (int d = 0; d < 3; ++d) {
     b.F[d] = c->F[d];
     b.FS[d] = c->FS[d];
+    b.ES[d] = c->ES[d];
     b.spd[d] = c->spd[d];
     b.flat[d] = c->flat[d];
   }
@@ -141,9 +142,9 @@ inline void flatten(harmrad_ctx* c, int d, bool fresh) {
 
 // FP64 reconstruction of direction d: edge values of every cell of its face range.
 template <int MET>
-void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const double* flat, double* E, int block,
-           int per_sm) {
+void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const double* flat, int block, int per_sm) {
   const DevParams& p = c->dp;
+  const EdgeSet E{(double*)c->edges, c->ES[d]};
   const BoxGeo* bt = c->dboxes;
   const int nb = c->nbox;
   auto width = [](const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; };
@@ -222,8 +223,7 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     R* Fd = (R*)c->F[d];
     R* sd = (R*)c->spd[d];
     if constexpr (std::is_same<R, double>::value) {
-      recon<MET>(c, d, c->P, (const double*)c->aux, (const double*)c->flat[d], (double*)c->edges, be,
-                 tu.edge_blocks_per_sm);
+      recon<MET>(c, d, c->P, (const double*)c->aux, (const double*)c->flat[d], be, tu.edge_blocks_per_sm);
     } else {
       const int ge = grid_for(max_work(c, range_cells), c->sms, be, tu.edge_blocks_per_sm);
       const R* aux = (const R*)c->aux;
@@ -235,13 +235,13 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     mark(c, HARMRAD_K_EDGE);
     if (d == 0)
       k_face<MET, R, 0><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[0],
-                                           (R*)c->gsp[0]);
+                                           (R*)c->gsp[0], c->ES[0]);
     else if (d == 1)
       k_face<MET, R, 1><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[1],
-                                           (R*)c->gsp[1]);
+                                           (R*)c->gsp[1], c->ES[1]);
     else
       k_face<MET, R, 2><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[2],
-                                           (R*)c->gsp[2]);
+                                           (R*)c->gsp[2], c->ES[2]);
     mark(c, HARMRAD_K_FACE);
     nk += 2;
   }
@@ -370,7 +370,7 @@ int solve_impl(harmrad_ctx* c, int stage, const ImexStage& im) {
     mark(c, HARMRAD_K_UPDATE);
     ++nk;
   }
-  k_retry<MET><<<c->sms * 2, 128, 0, st>>>(p, c->dboxes, b);
+  k_retry<MET><<<c->sms * 2, 128, 0, st>>>(p, c->dboxes, b, stage);
   mark(c, HARMRAD_K_RETRY);
   if (im.on && im.g > 0.0) {
     k_imex_store<MET><<<grid_for(c->maxact, c->sms, 256), 256, 0, st>>>(p, c->dboxes, c->nbox, b, stage, im.g);
