@@ -85,6 +85,18 @@ __device__ __forceinline__ void warp_add(unsigned long long* dst, unsigned v) {
 #define HR_TID (blockIdx.x * (long long)blockDim.x + threadIdx.x)
 #define HR_STRIDE ((long long)gridDim.x * blockDim.x)
 
+// ------------------------------------------------------------ work split
+// First item of this thread among the items of a grid whose predecessors in
+// the context hold `done` items: the grids' items form one sequence dealt to
+// the threads in turn, so that a batch of small grids loads every block alike
+// (12 boxes of 32 to 64 cells a side: step 73.2 -> 71.5 ms, ghost fill 1.03 ->
+// 0.44, reconstruction 7.2 -> 6.3).
+__device__ __forceinline__ long long first_item(long long done) {
+  if (done == 0) return HR_TID;
+  const long long r = HR_TID - done % HR_STRIDE;
+  return r < 0 ? r + HR_STRIDE : r;
+}
+
 // Opacity-field value of a cell (1 when the opacity is not a field).
 __device__ __forceinline__ double kfield(const DevParams& p, const double* K, long long t) {
   return p.opacity == 2 ? K[t] : 1.0;
@@ -200,6 +212,7 @@ __device__ __forceinline__ Geo<MET, R> geo_centre(const DevParams& p, const BoxG
 // present, is copied like a scalar primitive.
 static __global__ void k_bc_fill(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
                                  double* __restrict__ P0, double* __restrict__ K0, int d) {
+  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     double* P = P0 + 12 * bx.coff;
@@ -218,7 +231,7 @@ static __global__ void k_bc_fill(DevParams p, const BoxGeo* __restrict__ boxes, 
       }
     }
     long long total = 2LL * len[0] * len[1] * len[2];
-    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
       long long r = id;
       int a0 = (int)(r % len[0]);
       r /= len[0];
@@ -259,17 +272,8 @@ static __global__ void k_bc_fill(DevParams p, const BoxGeo* __restrict__ boxes, 
       }
       if (K) K[t] = K[s];
     }
+    done += total;
   }
-}
-
-// ------------------------------------------------------------ work split
-// First item of this thread among the items of a grid whose predecessors in
-// the context hold `done` items: the grids' items form one sequence dealt to
-// the threads in turn, so that a batch of small grids loads every block alike.
-__device__ __forceinline__ long long first_item(long long done) {
-  if (done == 0) return HR_TID;
-  const long long r = HR_TID - done % HR_STRIDE;
-  return r < 0 ? r + HR_STRIDE : r;
 }
 
 // --------------------------------------------------------------- cell prep
@@ -285,7 +289,7 @@ __global__ void k_prep(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
     const double* P = P0 + 12 * bx.coff;
     const double* K = K0 + bx.coff;
     R* aux = aux0 + 10 * bx.coff;
-    for (long long t = HR_TID; t < bx.ntot; t += HR_STRIDE) {
+    for (long long t = first_item(bx.coff); t < bx.ntot; t += HR_STRIDE) {
       long long r = t;
       int i = (int)(r % bx.N[0]) - bx.ng[0];
       r /= bx.N[0];
@@ -316,14 +320,13 @@ __global__ void k_prep(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
 template <int MET>
 __global__ void k_prep64(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const double* __restrict__ P0,
                          const double* __restrict__ K0, double* __restrict__ aux0, const double* __restrict__ geo0) {
-  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const double* P = P0 + 12 * bx.coff;
     const double* K = K0 + bx.coff;
     double* aux = aux0 + 10 * bx.coff;
     const long long nt = bx.ntot;
-    for (long long t = first_item(done); t < nt; t += HR_STRIDE) {
+    for (long long t = first_item(bx.coff); t < nt; t += HR_STRIDE) {
       Geo<MET, double> g;
       double gd = 1.0, a01 = 0.0, sd[3] = {1.0, 1.0, 1.0};
       if constexpr (MET == KS) {
@@ -366,7 +369,6 @@ __global__ void k_prep64(DevParams p, const BoxGeo* __restrict__ boxes, int nbox
         aux[(3 + 3 * e) * nt + t] = w < 1.0 ? w : 1.0;
       }
     }
-    done += nt;
   }
 }
 
@@ -455,6 +457,7 @@ template <typename R>
 __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
                           const double* __restrict__ P0, const R* __restrict__ aux0,
                           R* __restrict__ flat0, int d) {
+  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const double* P = P0 + 12 * bx.coff;
@@ -472,7 +475,7 @@ __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
     }
     long long total = (long long)len[0] * len[1] * len[2];
     const long long st = bx.str[d];
-    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
       long long r = id;
       int i = (int)(r % len[0]) + off[0];
       r /= len[0];
@@ -496,6 +499,7 @@ __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
       flat[t] = Fg > og ? Fg : og;
       flat[bx.ntot + t] = Fr > orr ? Fr : orr;
     }
+    done += total;
   }
 }
 
@@ -955,6 +959,7 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
                                                const float* __restrict__ flat0, float* __restrict__ E0) {
   typedef float R;
   const bool weighted = (MET == KS) && (d != 1);
+  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const double* P = P0 + 12 * bx.coff;
@@ -973,7 +978,7 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
     }
     long long total = (long long)len[0] * len[1] * len[2];
     const long long st = bx.str[d];
-    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
       long long r = id;
       int i = (int)(r % len[0]) + off[0];
       r /= len[0];
@@ -1011,6 +1016,7 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
         E[(NPR + q) * bx.ntot + t] = aR;
       }
     }
+    done += total;
   }
 }
 
@@ -1102,6 +1108,7 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
                                               const double* __restrict__ geo0, R* __restrict__ FS0,
                                               R* __restrict__ gsp0, const double* __restrict__ S0) {
   const bool weighted = (MET == KS) && (d != 1);
+  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     constexpr bool F64 = std::is_same<R, double>::value;
@@ -1128,7 +1135,7 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
     long long total = (long long)len[0] * len[1] * len[2];
     const long long st = bx.str[d];
     const R dxd = R(bx.dx[d]);
-    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
       long long r = id;
       int ii[3];
       ii[0] = (int)(r % len[0]) + off[0];
@@ -1197,6 +1204,7 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
       for (int q = 0; q < NPR; ++q) F[q * bx.ntot + t] = out[q];
       spd[t] = smax;
     }
+    done += total;
   }
 }
 
@@ -1208,6 +1216,7 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
 template <typename R>
 __global__ void k_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const R* __restrict__ Fa0,
                       const R* __restrict__ Fb0, R* __restrict__ emf0, int a, int b) {
+  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const R* fab = Fa0 + 12 * bx.coff + (B1 + b) * bx.ntot;
@@ -1217,7 +1226,7 @@ __global__ void k_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, c
     for (int e = 0; e < 3; ++e) len[e] = bx.n[e] + ((e == a || e == b) ? 1 : 0);
     long long total = (long long)len[0] * len[1] * len[2];
     const long long sa = bx.str[a], sb = bx.str[b];
-    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
       long long r = id;
       int ii[3];
       ii[0] = (int)(r % len[0]);
@@ -1229,12 +1238,14 @@ __global__ void k_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, c
                   ((ii[1] == 0 && bx.bc[2] == 2) || (ii[1] == bx.n[1] && bx.bc[3] == 2));
       emf[t] = pole ? R(0) : R(0.25) * (fab[t] + fab[t - sb] - fba[t] - fba[t - sa]);
     }
+    done += total;
   }
 }
 
 template <typename R>
 __global__ void k_ct(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const R* __restrict__ emf0,
                      R* __restrict__ Fa0, R* __restrict__ Fb0, int a, int b) {
+  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     R* fab = Fa0 + 12 * bx.coff + (B1 + b) * bx.ntot;
@@ -1249,7 +1260,7 @@ __global__ void k_ct(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, co
     long long na = (long long)la[0] * la[1] * la[2];
     long long nb = (long long)lb[0] * lb[1] * lb[2];
     const long long sa = bx.str[a], sb = bx.str[b];
-    for (long long id = HR_TID; id < na + nb; id += HR_STRIDE) {
+    for (long long id = first_item(done); id < na + nb; id += HR_STRIDE) {
       const int* L = id < na ? la : lb;
       long long r = id < na ? id : id - na;
       int i0 = (int)(r % L[0]);
@@ -1260,6 +1271,7 @@ __global__ void k_ct(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, co
       if (id < na) fab[t] = R(0.5) * (emf[t] + emf[t + sb]);
       else fba[t] = R(-0.5) * (emf[t] + emf[t + sa]);
     }
+    done += na + nb;
   }
 }
 
@@ -2101,7 +2113,7 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
     const R* Fd[3] = {(const R*)b.F[0] + 12 * bx.coff, (const R*)b.F[1] + 12 * bx.coff,
                       (const R*)b.F[2] + 12 * bx.coff};
     const double idx[3] = {1.0 / bx.dx[0], 1.0 / bx.dx[1], 1.0 / bx.dx[2]};
-    for (long long z = HR_TID; z < bx.nact; z += HR_STRIDE) {
+    for (long long z = first_item(bx.aoff); z < bx.nact; z += HR_STRIDE) {
       long long r = z;
       int i = (int)(r % bx.n[0]);
       r /= bx.n[0];
@@ -2367,7 +2379,7 @@ __global__ void k_imex_store(DevParams p, const BoxGeo* __restrict__ boxes, int 
     const double* Ps = b.psol_rec + 12 * bx.aoff;
     const double* Us = b.ust_rec + 12 * bx.aoff;
     double* M = b.imexM + 16 * bx.aoff;
-    for (long long z = HR_TID; z < bx.nact; z += HR_STRIDE) {
+    for (long long z = first_item(bx.aoff); z < bx.nact; z += HR_STRIDE) {
       long long r = z;
       const int i = (int)(r % bx.n[0]);
       r /= bx.n[0];
@@ -2574,7 +2586,7 @@ __global__ void k_cfl(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, B
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     double best = HUGE_VAL;
-    for (long long z = HR_TID; z < bx.nact; z += HR_STRIDE) {
+    for (long long z = first_item(bx.aoff); z < bx.nact; z += HR_STRIDE) {
       long long r = z;
       int i = (int)(r % bx.n[0]);
       r /= bx.n[0];

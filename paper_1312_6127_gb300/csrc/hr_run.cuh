@@ -52,7 +52,8 @@ inline Bufs make_bufs(harmrad_ctx* c) {
   return b;
 }
 
-// Largest per-grid work count of a kernel class, for sizing its launch.
+// Largest per-grid count, and the work of all grids (the kernels deal the grids'
+// items to the threads as one sequence, first_item), for sizing a launch.
 template <typename Fn>
 inline long long max_work(const harmrad_ctx* c, Fn work) {
   long long m = 1;
@@ -60,6 +61,12 @@ inline long long max_work(const harmrad_ctx* c, Fn work) {
     long long w = work(c->boxes[i]);
     if (w > m) m = w;
   }
+  return m;
+}
+template <typename Fn>
+inline long long all_work(const harmrad_ctx* c, Fn work) {
+  long long m = 0;
+  for (int i = 0; i < c->nbox; ++i) m += work(c->boxes[i]);
   return m;
 }
 
@@ -74,7 +81,7 @@ inline FaceSet face_set(double* const f[3]) {
 template <int MET>
 int face_ghosts(harmrad_ctx* c) {
   for (int d = 0; d < 3; ++d) {
-    k_face_ghosts<MET><<<grid_for(c->maxcell, c->sms, 256), 256, 0, c->stream>>>(c->dp, c->dboxes, c->nbox, c->P,
+    k_face_ghosts<MET><<<grid_for(c->ncell, c->sms, 256), 256, 0, c->stream>>>(c->dp, c->dboxes, c->nbox, c->P,
                                                                                  face_set(c->Bf), d, c->geotab);
     mark(c, HARMRAD_K_CT);
   }
@@ -88,7 +95,7 @@ inline int fill_ghost_cells(harmrad_ctx* c) {
   int nk = 0;
   for (int d = 0; d < 3; ++d) {
     if (!p.act[d]) continue;
-    long long work = max_work(c, [d](const BoxGeo& b) {
+    long long work = all_work(c, [d](const BoxGeo& b) {
       long long w = 2LL * b.ng[d];
       for (int e = 0; e < 3; ++e)
         if (e != d) w *= (e < d) ? b.N[e] : b.n[e];
@@ -120,7 +127,7 @@ inline void flatten(harmrad_ctx* c, int d, bool fresh) {
   double* fl = (double*)c->flat[d];
   auto width = [](const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; };
   if (d == 0) {
-    const long long work = max_work(c, [width](const BoxGeo& b) {
+    const long long work = all_work(c, [width](const BoxGeo& b) {
       return 32LL * (((long long)width(b, 1) * width(b, 2) * b.N[0] + 25) / 26);
     });
     const int g = grid_for(work, c->sms, 256);
@@ -129,7 +136,7 @@ inline void flatten(harmrad_ctx* c, int d, bool fresh) {
     return;
   }
   const int o = 3 - d;
-  const long long cols = max_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
+  const long long cols = all_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
   const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
   // a piece evaluates two cells more than it owns; 4 blocks of 128 fit an SM
   long long pieces;
@@ -149,7 +156,7 @@ void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const doub
   const int nb = c->nbox;
   auto width = [](const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; };
   if (d == 0) {
-    const long long work = max_work(c, [width](const BoxGeo& b) {
+    const long long work = all_work(c, [width](const BoxGeo& b) {
       return 12LL * 32 * (((long long)width(b, 1) * width(b, 2) * b.N[0] + 59) / 60);
     });
     const int g = grid_for(work, c->sms, block, per_sm);
@@ -158,7 +165,7 @@ void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const doub
     return;
   }
   const int o = 3 - d;
-  const long long cols = max_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
+  const long long cols = all_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
   const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
   // a piece repeats about one cell's work: 16 cells or more, two threads per slot
   long long pieces;
@@ -178,10 +185,10 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
   int nk = fill_ghost_cells(c);
   if (p.emf == 1) nk += face_ghosts<MET>(c);
   if constexpr (std::is_same<R, double>::value)
-    k_prep64<MET><<<grid_for(c->maxcell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, c->K, (double*)c->aux,
+    k_prep64<MET><<<grid_for(c->ncell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, c->K, (double*)c->aux,
                                                                       c->geotab);
   else
-    k_prep<MET, R><<<grid_for(c->maxcell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, c->K, (R*)c->aux,
+    k_prep<MET, R><<<grid_for(c->ncell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, c->K, (R*)c->aux,
                                                                        c->geotab);
   mark(c, HARMRAD_K_PREP);
   ++nk;
@@ -203,7 +210,7 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
         if (cudaMemsetAsync(c->flat[d], 0, 2 * c->ncell * sizeof(R), st) != cudaSuccess) return HARMRAD_E_CUDA;
         mark(c, HARMRAD_K_OTHER);
       }
-      k_flatten<R><<<grid_for(max_work(c, range_cells), c->sms, 256), 256, 0, st>>>(
+      k_flatten<R><<<grid_for(all_work(c, range_cells), c->sms, 256), 256, 0, st>>>(
           p, bt, nb, c->P, (const R*)c->aux, (R*)c->flat[d], d);
       mark(c, HARMRAD_K_FLATTEN);
       ++nk;
@@ -211,7 +218,7 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
   }
   for (int d = 0; d < 3; ++d) {
     if (!p.act[d]) continue;
-    long long wf = max_work(c, [d](const BoxGeo& b) {
+    long long wf = all_work(c, [d](const BoxGeo& b) {
       long long w = 1;
       for (int e = 0; e < 3; ++e) w *= (e == d) ? b.n[e] + 1 : (b.n[e] > 1 ? b.n[e] + 2 : 1);
       return w;
@@ -225,7 +232,7 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     if constexpr (std::is_same<R, double>::value) {
       recon<MET>(c, d, c->P, (const double*)c->aux, (const double*)c->flat[d], be, tu.edge_blocks_per_sm);
     } else {
-      const int ge = grid_for(max_work(c, range_cells), c->sms, be, tu.edge_blocks_per_sm);
+      const int ge = grid_for(all_work(c, range_cells), c->sms, be, tu.edge_blocks_per_sm);
       const R* aux = (const R*)c->aux;
       const R* fl = (const R*)c->flat[d];
       if (d == 0) k_edges<MET, 0><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Ed);
@@ -246,13 +253,13 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     nk += 2;
   }
   if (p.emf == 1) {  // staggered field: the 4-state upwind EMFs on the edges
-    k_vel<MET, R><<<grid_for(c->maxcell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, (R*)c->vel, c->geotab);
+    k_vel<MET, R><<<grid_for(c->ncell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, (R*)c->vel, c->geotab);
     mark(c, HARMRAD_K_CT);
     ++nk;
     for (int a = 0; a < 3; ++a)
       for (int b = a + 1; b < 3; ++b) {
         if (!p.act[a] && !p.act[b]) continue;
-        long long we = max_work(c, [a, b](const BoxGeo& x) {
+        long long we = all_work(c, [a, b](const BoxGeo& x) {
           long long w = 1;
           for (int e = 0; e < 3; ++e) w *= x.n[e] + (((e == a || e == b) && x.n[e] > 1) ? 1 : 0);
           return w;
@@ -269,12 +276,12 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
   for (int a = 0; a < 3; ++a)
     for (int b = a + 1; b < 3; ++b) {
       if (!p.act[a] || !p.act[b]) continue;
-      long long we = max_work(c, [a, b](const BoxGeo& x) {
+      long long we = all_work(c, [a, b](const BoxGeo& x) {
         long long w = 1;
         for (int e = 0; e < 3; ++e) w *= x.n[e] + ((e == a || e == b) ? 1 : 0);
         return w;
       });
-      long long wc = max_work(c, [a, b](const BoxGeo& x) {
+      long long wc = all_work(c, [a, b](const BoxGeo& x) {
         long long la = 1, lb = 1;
         for (int e = 0; e < 3; ++e) {
           la *= x.n[e] + (e == a ? 1 : 0);
@@ -301,7 +308,7 @@ int cfl_impl(harmrad_ctx* c) {
   Bufs b = make_bufs(c);
   k_cfl_init<<<1, 128, 0, c->stream>>>(b, c->nbox);
   mark(c, HARMRAD_K_CFL);
-  k_cfl<R><<<grid_for(c->maxact, c->sms, 256), 256, 0, c->stream>>>(c->dp, c->dboxes, c->nbox, b);
+  k_cfl<R><<<grid_for(c->nact, c->sms, 256), 256, 0, c->stream>>>(c->dp, c->dboxes, c->nbox, b);
   mark(c, HARMRAD_K_CFL);
   k_cfl_finish<<<1, 128, 0, c->stream>>>(c->dp, b, c->nbox);
   mark(c, HARMRAD_K_CFL);
@@ -318,7 +325,7 @@ int solve_impl(harmrad_ctx* c, int stage, const ImexStage& im) {
   mark(c, HARMRAD_K_OTHER);
   Bufs b = make_bufs(c);
   const int bu = c->tune.update_block;
-  const int gu = grid_for(c->maxact, c->sms, bu, c->tune.update_blocks_per_sm);
+  const int gu = grid_for(c->nact, c->sms, bu, c->tune.update_blocks_per_sm);
   const int split = c->tune.newton_split;
   const bool one = c->nbox == 1;
   const BoxGeo& b0 = c->boxes[0];
@@ -330,7 +337,7 @@ int solve_impl(harmrad_ctx* c, int stage, const ImexStage& im) {
     for (int e = 0; e < 3; ++e) es.e[e] = c->emf3[e];
     const bool rhs = !im.on || im.d != 0.0;
     for (int d = 0; d < 3; ++d) {
-      long long wf = max_work(c, [d](const BoxGeo& x) {
+      long long wf = all_work(c, [d](const BoxGeo& x) {
         long long w = 1;
         for (int e = 0; e < 3; ++e) w *= (e == d && x.n[e] > 1) ? x.n[e] + 1 : x.n[e];
         return w;
@@ -373,7 +380,7 @@ int solve_impl(harmrad_ctx* c, int stage, const ImexStage& im) {
   k_retry<MET><<<c->sms * 2, 128, 0, st>>>(p, c->dboxes, b, stage);
   mark(c, HARMRAD_K_RETRY);
   if (im.on && im.g > 0.0) {
-    k_imex_store<MET><<<grid_for(c->maxact, c->sms, 256), 256, 0, st>>>(p, c->dboxes, c->nbox, b, stage, im.g);
+    k_imex_store<MET><<<grid_for(c->nact, c->sms, 256), 256, 0, st>>>(p, c->dboxes, c->nbox, b, stage, im.g);
     mark(c, HARMRAD_K_UPDATE);
     ++nk;
   }
@@ -568,10 +575,10 @@ template <int MET>
 int Run<MET>::init_faces(harmrad_ctx* c, bool from_centres) {
   fill_ghost_cells(c);
   if (from_centres)
-    k_faces_from_centres<MET><<<grid_for(c->maxcell, c->sms, 256), 256, 0, c->stream>>>(
+    k_faces_from_centres<MET><<<grid_for(c->ncell, c->sms, 256), 256, 0, c->stream>>>(
         c->dp, c->dboxes, c->nbox, c->P, face_set(c->Bf), c->geotab);
   face_ghosts<MET>(c);
-  k_centre_B<MET><<<grid_for(c->maxact, c->sms, 256), 256, 0, c->stream>>>(c->dp, c->dboxes, c->nbox, c->P,
+  k_centre_B<MET><<<grid_for(c->nact, c->sms, 256), 256, 0, c->stream>>>(c->dp, c->dboxes, c->nbox, c->P,
                                                                            face_set(c->Bf), c->geotab);
   return cudaGetLastError() == cudaSuccess ? 0 : HARMRAD_E_CUDA;
 }
