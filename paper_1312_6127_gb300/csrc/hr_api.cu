@@ -28,61 +28,48 @@ namespace {
 
 // Active layout of a context: the grids' [nv][n3][n2][n1] blocks one after the
 // other.  These kernels move nv planes between it and the ghost-inclusive
-// cell layout (nv = 12 for the primitives, 1 for the opacity field).
-__global__ void k_unpack(const BoxGeo* __restrict__ boxes, int nbox, int nv,
-                         const double* __restrict__ src, double* __restrict__ dst0) {
+// cell layout (nv = 12 for the primitives, 1 for the opacity field).  A thread
+// takes one cell and all its planes, so that the cell's place costs two
+// divisions, not the six 64-bit ones per value that bounded these kernels, and
+// the check of the input reads what the copy reads (it was a pass of its own).
+
+// flag = 1 if any value is not finite or rho0, u_g, Ebar is not positive
+// (nv = 12), or if any opacity-field value is negative or not finite (nv = 1)
+template <int nv>
+__global__ void k_unpack(const BoxGeo* __restrict__ boxes, int nbox, const double* __restrict__ src,
+                         double* __restrict__ dst0, int* flag) {
+  bool bad = false;
   for (int b = 0; b < nbox; ++b) {
-    const BoxGeo bx = boxes[b];
+    const BoxGeo& bx = boxes[b];
     const double* s = src + nv * bx.aoff;
     double* dst = dst0 + nv * bx.coff;
-    long long total = (long long)nv * bx.nact;
-    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < total;
-         id += (long long)gridDim.x * blockDim.x) {
-      long long q = id / bx.nact, z = id % bx.nact, r = z;
-      int i = (int)(r % bx.n[0]);
-      r /= bx.n[0];
-      int j = (int)(r % bx.n[1]);
-      int k = (int)(r / bx.n[1]);
-      dst[q * bx.ntot + hr::cell_index(bx, i, j, k)] = s[id];
+    for (long long z = hr::first_item(bx.aoff); z < bx.nact; z += HR_STRIDE) {
+      const int r = (int)(z / bx.n[0]), i = (int)(z - (long long)r * bx.n[0]);
+      const long long t = hr::cell_index(bx, i, r % bx.n[1], r / bx.n[1]);
+#pragma unroll
+      for (int q = 0; q < nv; ++q) {
+        const double v = s[q * bx.nact + z];
+        dst[q * bx.ntot + t] = v;
+        bad = bad || !isfinite(v);
+        if (nv == 12) bad = bad || ((q == hr::RHO || q == hr::UU || q == hr::ER) && !(v > 0.0));
+        else bad = bad || v < 0.0;
+      }
     }
   }
+  if (bad) atomicOr(flag, 1);
 }
 
 __global__ void k_pack(const BoxGeo* __restrict__ boxes, int nbox, const double* __restrict__ P0,
                        double* __restrict__ dst0) {
   for (int b = 0; b < nbox; ++b) {
-    const BoxGeo bx = boxes[b];
+    const BoxGeo& bx = boxes[b];
     const double* P = P0 + 12 * bx.coff;
     double* d = dst0 + 12 * bx.aoff;
-    long long total = (long long)hr::NPR * bx.nact;
-    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < total;
-         id += (long long)gridDim.x * blockDim.x) {
-      long long q = id / bx.nact, z = id % bx.nact, r = z;
-      int i = (int)(r % bx.n[0]);
-      r /= bx.n[0];
-      int j = (int)(r % bx.n[1]);
-      int k = (int)(r / bx.n[1]);
-      d[id] = P[q * bx.ntot + hr::cell_index(bx, i, j, k)];
-    }
-  }
-}
-
-// flag = 1 if any value is not finite or rho0, u_g, Ebar is not positive
-// (nv = 12), or if any opacity-field value is negative or not finite (nv = 1)
-__global__ void k_validate(const BoxGeo* __restrict__ boxes, int nbox, int nv,
-                           const double* __restrict__ src, int* flag) {
-  for (int b = 0; b < nbox; ++b) {
-    const BoxGeo bx = boxes[b];
-    const double* s = src + nv * bx.aoff;
-    long long total = (long long)nv * bx.nact;
-    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < total;
-         id += (long long)gridDim.x * blockDim.x) {
-      double v = s[id];
-      long long q = id / bx.nact;
-      bool bad = !isfinite(v);
-      if (nv == 12) bad = bad || ((q == hr::RHO || q == hr::UU || q == hr::ER) && !(v > 0.0));
-      else bad = bad || v < 0.0;
-      if (bad) atomicOr(flag, 1);
+    for (long long z = hr::first_item(bx.aoff); z < bx.nact; z += HR_STRIDE) {
+      const int r = (int)(z / bx.n[0]), i = (int)(z - (long long)r * bx.n[0]);
+      const long long t = hr::cell_index(bx, i, r % bx.n[1], r / bx.n[1]);
+#pragma unroll
+      for (int q = 0; q < hr::NPR; ++q) d[q * bx.nact + z] = P[q * bx.ntot + t];
     }
   }
 }
@@ -416,7 +403,7 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
   int rc = fill_physics(&p[0], dp);
   if (rc) return rc;
   std::vector<BoxGeo> boxes(count);
-  long long coff = 0, aoff = 0, maxc = 0, maxa = 0, goff = 0;
+  long long coff = 0, aoff = 0, goff = 0;
   for (int b = 0; b < count; ++b) {
     if (b > 0 && !same_physics(p[0], p[b])) return HARMRAD_E_ARG;
     rc = fill_geometry(&p[b], boxes[b]);
@@ -429,8 +416,6 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     }
     coff += boxes[b].ntot;
     aoff += boxes[b].nact;
-    maxc = boxes[b].ntot > maxc ? boxes[b].ntot : maxc;
-    maxa = boxes[b].nact > maxa ? boxes[b].nact : maxa;
   }
   harmrad_ctx* c = (harmrad_ctx*)calloc(1, sizeof(harmrad_ctx));
   if (!c) return HARMRAD_E_OOM;
@@ -445,8 +430,6 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
   memcpy(c->boxes, boxes.data(), sizeof(BoxGeo) * count);
   c->ncell = coff;
   c->nact = aoff;
-  c->maxcell = maxc;
-  c->maxact = maxa;
   c->real_size = p[0].precision == HARMRAD_PREC_SPLIT ? 4 : 8;
   c->use_graph = getenv("HARMRAD_NO_GRAPH") == nullptr;
   c->tune = default_tuning();
@@ -568,9 +551,9 @@ int upload_planes(harmrad_ctx* c, int nv, const double* src_in, int on_device, d
     src = c->stage_buf;
   }
   HR_CHECK(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
-  int g = hr::grid_for(nv * c->maxact, c->sms, 256);
-  k_validate<<<g, 256, 0, c->stream>>>(c->dboxes, c->nbox, nv, src, c->flag);
-  k_unpack<<<g, 256, 0, c->stream>>>(c->dboxes, c->nbox, nv, src, dst);
+  const int g = hr::grid_for(c->nact, c->sms, 256);
+  if (nv == 12) k_unpack<12><<<g, 256, 0, c->stream>>>(c->dboxes, c->nbox, src, dst, c->flag);
+  else k_unpack<1><<<g, 256, 0, c->stream>>>(c->dboxes, c->nbox, src, dst, c->flag);
   HR_CHECK(cudaGetLastError());
   int flag = 0;
   HR_CHECK(cudaMemcpyAsync(&flag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -691,7 +674,7 @@ int harmrad_set_opacity_field(harmrad_ctx* c, const double* kabs, int on_device)
 int harmrad_get_prims(harmrad_ctx* c, double* P, int on_device) {
   if (!c || !P) return HARMRAD_E_ARG;
   size_t bytes = 12 * (size_t)c->nact * sizeof(double);
-  int g = hr::grid_for(12 * c->maxact, c->sms, 256);
+  int g = hr::grid_for(c->nact, c->sms, 256);
   double* dst = on_device ? P : c->stage_buf;
   k_pack<<<g, 256, 0, c->stream>>>(c->dboxes, c->nbox, c->P, dst);
   HR_CHECK(cudaGetLastError());

@@ -17,7 +17,6 @@ struct harmrad_ctx {
   hr::BoxGeo* boxes;         // host copy of the grid table
   hr::BoxGeo* dboxes;        // device copy
   long long ncell, nact;     // totals over the grids
-  long long maxcell, maxact; // largest grid
   cudaStream_t stream;
   bool own_stream;
   int device;
