@@ -441,14 +441,199 @@ __global__ void ka_ct_T(BoxGeo bx, const double* __restrict__ gemf, double* __re
 }
 
 // ------------------------------------------------------ Riemann fluxes (T)
-// Per face: cotangents of the two reconstructed states from the flux's
-// cotangent (25 inputs: P_L, P_R, kappa_scale; five dual passes).
+// Reverse sweep of face_flux64: the cotangents of the two states and of
+// kappa_scale from those of the 12 fluxes and of the entropy flux, each
+// operation of FaceSide transposed by hand.  About 1,500 FP64 instructions per
+// face; 25 forward derivatives on dual numbers took fifteen times as many.
+
+// Cotangents of one side's intermediates (names as in FaceSide).
+struct SideCot {
+  double u0, ud, u1, l0, l[3], bt, m0, m[3], iut, wb, pt, r0, rd, k0, k[3];
+  double aF[2], aU[2];  // of the weights, gas and radiation
+};
+
+// FaceSide::add transposed: o the cotangents of out, oM that of the returned
+// mass share.  Adds to gP what does not pass through the intermediates.
 template <int MET, int d>
-__global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, EdgeSet E,
-                                               const double* __restrict__ K, const double* __restrict__ gF,
-                                               double* __restrict__ gE, double* gk_out,
-                                               const double* __restrict__ gFS) {
-  typedef Dn<5> D5;
+__device__ __forceinline__ void side_add_T(const FaceSide<MET, d>& s, const double P[NPR], const double aF[2],
+                                           const double aU[2], const double o[NPR], double oM, double gP[NPR],
+                                           SideCot& c) {
+  const double ud = d == 1 ? s.u1 : P[U1 + d - 1], Bd = P[B1 + d - 1], iut = s.iut;
+  const double V = fma(aU[0], s.u0, aF[0] * ud), bu = s.bt * s.u0, bd = fma(s.bt, ud, Bd);
+  const double S = fma(aU[0], bu, aF[0] * bd), Y = -(iut * iut) * S, Z = fma(s.bt, Y, s.wb * V);
+  double gZ = o[1] * s.l0, gY = o[1] * s.m0;
+  c.l0 = o[1] * Z;
+  c.m0 = o[1] * Y;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    gZ = fma(o[2 + i], s.l[i], gZ);
+    gY = fma(o[2 + i], s.m[i], gY);
+    c.l[i] = o[2 + i] * Z;
+    c.m[i] = o[2 + i] * Y;
+  }
+  c.pt = fma(o[1], aU[0], o[1 + d] * aF[0]);
+  double gaU = o[1] * s.pt, gaF = o[1 + d] * s.pt;
+  const double gM = o[0] + o[1] + oM;
+  // induction rows
+  const double vi = V * iut, Bi = aF[0] * Bd * iut;
+  double gvi = 0.0, gBi = 0.0;
+  c.u1 = 0.0;
+#pragma unroll
+  for (int i = 1; i <= 3; ++i) {
+    if (i == d) continue;
+    const double oi = o[4 + i];
+    gvi = fma(oi, P[B1 + i - 1], gvi);
+    gBi = fma(-oi, i == 1 ? s.u1 : P[U1 + i - 1], gBi);
+    gP[B1 + i - 1] = fma(oi, vi, gP[B1 + i - 1]);
+    if (i == 1) c.u1 = -oi * Bi;
+    else gP[U1 + i - 1] = fma(-oi, Bi, gP[U1 + i - 1]);
+  }
+  double gV = gvi * iut, gBd = gBi * aF[0] * iut;
+  c.iut = fma(gvi, V, gBi * aF[0] * Bd);
+  gaF = fma(gBi, Bd * iut, gaF);
+  // Z, M, Y
+  c.bt = gZ * Y;
+  gY = fma(gZ, s.bt, gY);
+  c.wb = gZ * V;
+  gV = fma(gZ, s.wb, fma(gM, P[RHO], gV));
+  gP[RHO] = fma(gM, V, gP[RHO]);
+  c.iut = fma(-2.0 * gY * iut, S, c.iut);
+  const double gS = -(iut * iut) * gY, gbu = gS * aU[0], gbd = gS * aF[0];
+  gaU = fma(gS, bu, gaU);
+  gaF = fma(gS, bd, gaF);
+  c.bt = fma(gbd, ud, fma(gbu, s.u0, c.bt));
+  gBd += gbd;
+  gP[B1 + d - 1] += gBd;
+  c.u0 = fma(gbu, s.bt, gV * aU[0]);
+  c.ud = fma(gbd, s.bt, gV * aF[0]);
+  c.aU[0] = fma(gV, s.u0, gaU);
+  c.aF[0] = fma(gV, ud, gaF);
+  // radiation
+  const double E = P[ER], e13 = E * (1.0 / 3.0), W = fma(aU[1], s.r0, aF[1] * s.rd), e43 = (4.0 / 3.0) * E, R = e43 * W;
+  double gR = o[8] * s.k0;
+  c.k0 = o[8] * R;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    gR = fma(o[9 + i], s.k[i], gR);
+    c.k[i] = o[9 + i] * R;
+  }
+  const double ge13 = fma(o[8], aU[1], o[8 + d] * aF[1]), gW = gR * e43;
+  gP[ER] += fma(gR * (4.0 / 3.0), W, ge13 * (1.0 / 3.0));
+  c.aU[1] = fma(gW, s.r0, o[8] * e13);
+  c.aF[1] = fma(gW, s.rd, o[8 + d] * e13);
+  c.r0 = gW * aU[1];
+  c.rd = gW * aF[1];
+}
+
+// FaceSide::build transposed: gvp, gvm the cotangents of v_max and v_min (gas,
+// radiation), c those of the other intermediates; adds to gP and *gks.
+template <int MET, int d>
+__device__ __forceinline__ void side_build_T(const DevParams& p, const Geo<MET, double>& g,
+                                             const FaceGeo<MET, d>& f, const FaceSide<MET, d>& s, double dl,
+                                             double kf, const double P[NPR], const double gvp[2],
+                                             const double gvm[2], SideCot& c, double gP[NPR], double* gks) {
+  double gc2[2];
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {  // speeds
+    const double ut = w ? s.r0 : s.u0, ud = w ? s.rd : (d == 1 ? s.u1 : P[U1 + d - 1]), c2 = s.c2[w], H = s.H[w];
+    const double sum = gvp[w] + gvm[w], dif = gvp[w] - gvm[w], iq = s.iq[w];
+    const double gBq = sum * iq, gqa = -(fma(sum, s.Bq[w], dif * s.sd[w])) * (iq * iq);
+    const double gK = s.sd[w] > 0.0 ? 0.5 * dif * iq * rcp(s.sd[w]) : 0.0;
+    const double AB = d == 1 ? g.Gt(1) : 0.0, u02 = ut * ut, mix = ut * ud;
+    double gx = fma(gK, fma(c2, f.C0 - H, H) + c2 * (f.C0 - H), fma(-gBq, AB + mix, -gqa * (g.Gtt() + u02)));
+    const double gH = gK * c2 * (1.0 - c2);
+    const double gmix = fma(gBq, 1.0 - c2, -2.0 * AB * gH);
+    const double gu02 = fma(gqa, 1.0 - c2, gH * g.Gdd(d));
+    const double gu = fma(gmix, ud, 2.0 * ut * gu02), gd = fma(gmix, ut, 2.0 * ud * g.Gtt() * gH);
+    if (w) {
+      c.r0 += gu;
+      c.rd += gd;
+    } else {
+      c.u0 += gu;
+      c.ud += gd;
+    }
+    gc2[w] = gx;
+  }
+  const double rho = P[RHO], iwb = rcp(s.wb), ia = MET == MINK ? 1.0 : g.ialpha, al = MET == MINK ? 1.0 : g.alpha;
+  double gpg = c.pt, gbsq = 0.5 * c.pt, gwb = c.wb;
+  if (!(s.cd & 3u)) {  // c_ms^2 = (Gamma p + b^2) / (w + b^2), unclamped
+    gpg = fma(gc2[0] * p.gam, iwb, gpg);
+    gbsq = fma(gc2[0], iwb, gbsq);
+    gwb = fma(-gc2[0] * s.c2[0], iwb, gwb);
+  }
+  if (s.cd & 4u) {  // (4 / (3 tau))^2: d/dtau = -2 c^2 / tau
+    const double Tg = p.gm1 * P[UU] / rho;
+    double ka, dr = 0.0, du = 0.0;  // absorption over kappa_scale and its derivatives
+    if (p.opacity == 2) {
+      ka = kf;
+    } else if (p.opacity == 1) {
+      const double Tc = Tg > p.Tmin ? Tg : p.Tmin, T2 = Tc * Tc;
+      ka = p.kabs0 * rho * rho * rsqrt64(T2 * T2 * T2 * Tc);
+      dr = (Tg > p.Tmin ? 5.5 : 2.0) * ka / rho;
+      du = Tg > p.Tmin ? -3.5 * ka / P[UU] : 0.0;
+    } else {
+      ka = p.kabs0 * rho;
+      dr = p.kabs0;
+    }
+    const double kt = fma(p.kes0, rho, ka);
+    const double gk = -2.0 * s.c2[1] / (p.kscale * kt) * gc2[1];  // of kappa_scale kt
+    *gks = fma(gk, kt, *gks);
+    gP[RHO] = fma(gk * p.kscale, dr + p.kes0, gP[RHO]);
+    gP[UU] = fma(gk * p.kscale, du, gP[UU]);
+  }
+  (void)dl;
+  // w + b^2, p_tot, b^2
+  gbsq += gwb;
+  gP[RHO] += gwb;
+  gP[UU] += fma(p.gm1, gpg, p.gam * gwb);
+  const double i2 = s.iut * s.iut, gBB = gbsq * i2;
+  c.bt = fma(2.0 * gBB, s.bt, c.bt);
+  c.iut = fma(2.0 * gbsq, s.bsq * rcp(s.iut), c.iut);
+  // gas frame
+  double ggm = fma(-c.iut * s.iut, s.igm, c.u0 * ia) - al * c.l0;
+  if (d == 1) c.u1 += c.ud;
+  else gP[U1 + d - 1] += c.ud;
+  gP[U1] += c.u1;
+  ggm = fma(-c.u1, f.a01, ggm);
+  c.l[0] = fma(f.b1, c.l0, c.l[0]);
+  c.m[0] = fma(f.b1, c.m0, c.m[0]);
+  const double gg = 0.5 * ggm * s.igm;
+  double gl[3], gmm[3], t[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    gP[B1 + i] = fma(c.bt, s.l[i], fma(gBB, s.m[i], gP[B1 + i]));
+    gl[i] = fma(c.bt, P[B1 + i], fma(gg, P[U1 + i], c.l[i]));
+    gmm[i] = fma(gBB, P[B1 + i], c.m[i]);
+    gP[U1 + i] = fma(gg, s.l[i], gP[U1 + i]);
+  }
+  lower3<MET>(g, gl[0], gl[1], gl[2], t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) gP[U1 + i] += t[i];
+  lower3<MET>(g, gmm[0], gmm[1], gmm[2], t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) gP[B1 + i] += t[i];
+  // radiation frame
+  double ggr = fma(c.r0, ia, -al * c.k0);
+  gP[UR1 + d - 1] += c.rd;
+  if (d == 1) ggr = fma(-c.rd, f.a01, ggr);
+  c.k[0] = fma(f.b1, c.k0, c.k[0]);
+  const double gq = 0.5 * ggr * rcp(s.gr);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    gP[UR1 + i] = fma(gq, s.k[i], gP[UR1 + i]);
+    gl[i] = fma(gq, P[UR1 + i], c.k[i]);
+  }
+  lower3<MET>(g, gl[0], gl[1], gl[2], t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) gP[UR1 + i] += t[i];
+}
+
+template <int MET, int d>
+__global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, EdgeSet E, const double* __restrict__ K,
+                                               const double* __restrict__ gF, double* __restrict__ gE,
+                                               double* gk_out, const double* __restrict__ gFS,
+                                               const double* __restrict__ geo) {
+  constexpr int dd = d + 1;
   const bool weighted = (MET == KS) && (d != 1);
   int len[3], off[3];
   for (int e = 0; e < 3; ++e) {
@@ -463,7 +648,7 @@ __global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, EdgeSet E
       off[e] = 0;
     }
   }
-  const long long total = (long long)len[0] * len[1] * len[2];
+  const long long total = (long long)len[0] * len[1] * len[2], nt = bx.ntot;
   const long long st = bx.str[d];
   double gk = 0.0;
   for (long long id = HR_TID; id < total; id += HR_STRIDE) {
@@ -474,54 +659,133 @@ __global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, EdgeSet E
     ii[1] = (int)(r % len[1]) + off[1];
     ii[2] = (int)(r / len[1]) + off[2];
     const long long t = cell_index(bx, ii[0], ii[1], ii[2]);
-    const int f = ii[d];
-    if (MET == KS && d == 1 && ((f == 0 && bx.bc[2] == 2) || (f == bx.n[1] && bx.bc[3] == 2))) continue;
-    double gq[NPR];
+    const int fi = ii[d];
+    if (MET == KS && d == 1 && ((fi == 0 && bx.bc[2] == 2) || (fi == bx.n[1] && bx.bc[3] == 2))) continue;
+    double o[NPR];
     bool any = false;
+#pragma unroll
     for (int q = 0; q < NPR; ++q) {
-      gq[q] = gF[q * bx.ntot + t];
-      any = any || gq[q] != 0.0;
+      o[q] = q == B1 + d ? 0.0 : gF[q * nt + t];
+      any = any || o[q] != 0.0;
     }
     const double gfs = gFS ? gFS[t] : 0.0;
     any = any || gfs != 0.0;
     if (!any) continue;
-    double xf[3];
-    for (int e = 0; e < 3; ++e) xf[e] = bx.x0[e] + (ii[e] + (e == d ? 0.0 : 0.5)) * bx.dx[e];
-    const Geo<MET, double> g = make_geo<MET, double>(p, xf[0], xf[1]);
-    const double igf = weighted ? 1.0 / g.gdet : 1.0;
-    double PL[NPR], PR[NPR], wL[NPR];
+    Geo<MET, double> g;
+    double igf = 1.0, dl = bx.dx[d];
+    if constexpr (MET == KS) {
+      const GeoTab T = geotab(geo, bx);
+      const double* tab = d == 0 ? T.F0 : (d == 1 ? T.F1 : T.C);
+      const long long sz = d == 0 ? T.sF0 : (d == 1 ? T.sF1 : T.sC);
+      const long long x = d == 0 ? gidx_f0(bx, ii[0], ii[1])
+                                 : (d == 1 ? gidx_f1(bx, ii[0], ii[1]) : gidx_c(bx, ii[0], ii[1]));
+      g = geo_load<MET>(tab, sz, x);
+      if (weighted) igf = __ldg(tab + 16 * sz + x);
+      dl *= __ldg(tab + (d == 2 ? 19 : 17) * sz + x);
+    } else {
+      g = make_geo<MET, double>(p, 0.0, 0.0);
+    }
+    double PL[NPR], PR[NPR];
+#pragma unroll
     for (int q = 0; q < NPR; ++q) {
       const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
-      const double aR = E.plane(1, q, bx.ntot)[t - st];
-      const double bL = E.plane(0, q, bx.ntot)[t];
-      PL[q] = wq ? aR * igf : aR;
-      PR[q] = wq ? bL * igf : bL;
-      wL[q] = wq ? igf : 1.0;
+      const double w = wq ? igf : 1.0;
+      PL[q] = E.plane(1, q, nt)[t - st] * w;
+      PR[q] = E.plane(0, q, nt)[t] * w;
     }
     const double kL = kfield(p, K, t - st), kR = kfield(p, K, t);
-    const Geo<MET, D5> g5 = geo_cast<D5>(g);
-    double gin[25];
-    for (int ch = 0; ch < 5; ++ch) {
-      D5 PLd[NPR], PRd[NPR], out[NPR], smax;
-      for (int q = 0; q < NPR; ++q) {
-        PLd[q] = D5::seed(PL[q], q - 5 * ch);
-        PRd[q] = D5::seed(PR[q], NPR + q - 5 * ch);
-      }
-      const D5 ks = D5::seed(p.kscale, 24 - 5 * ch);
-      D5 fs;
-      face_flux<MET, D5, d>(p, g5, D5(bx.dx[d]), D5(kL), D5(kR), ks, PLd, PRd, out, &smax, nullptr,
-                            gfs != 0.0 ? &fs : nullptr);
-      for (int c = 0; c < 5; ++c) {
-        double v = gfs != 0.0 ? gfs * fs.d[c] : 0.0;
-        for (int q = 0; q < NPR; ++q) v += gq[q] * out[q].d[c];
-        gin[5 * ch + c] = v;
+    const FaceGeo<MET, dd> f(g);
+    FaceSide<MET, dd> L, R;
+    L.build(p, g, f, dl, kL, PL, nullptr);
+    R.build(p, g, f, dl, kR, PR, nullptr);
+    double cp[2], cm[2], aFL[2], aFR[2], aUL[2], aUR[2], sc[2];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      cp[w] = fmax(0.0, fmax(L.vmax(w), R.vmax(w)));
+      cm[w] = -fmin(0.0, fmin(L.vmin(w), R.vmin(w)));
+      if (p.flux == 0) {
+        aFL[w] = aFR[w] = 1.0;
+        aUL[w] = cp[w] > cm[w] ? cp[w] : cm[w];
+        aUR[w] = -aUL[w];
+        sc[w] = 0.5 * g.gdet;
+      } else {
+        const double sum = cp[w] + cm[w];
+        const bool ok = sum > 0.0;
+        aFL[w] = ok ? cp[w] : 1.0;
+        aFR[w] = ok ? cm[w] : 1.0;
+        aUL[w] = ok ? cm[w] * cp[w] : 0.0;
+        aUR[w] = -aUL[w];
+        sc[w] = g.gdet * (ok ? 1.0 / sum : 0.5);
       }
     }
+    // the entropy flux s_L M_L + s_R M_R (over the scale of the gas rows)
+    double sL = 0.0, sR = 0.0;
+    if (gfs != 0.0) {
+      sL = entropy_per_baryon<double>(p, PL[RHO], PL[UU]);
+      sR = entropy_per_baryon<double>(p, PR[RHO], PR[UU]);
+    }
+    double gsc[2] = {0.0, 0.0};  // cotangents of the scales (HLL)
+    if (p.flux != 0) {
+      double raw[NPR];
+#pragma unroll
+      for (int q = 0; q < NPR; ++q) raw[q] = 0.0;
+      const double mL = L.template add<false>(g, PL, aFL[0], aUL[0], aFL[1], aUL[1], raw);
+      const double mR = R.template add<false>(g, PR, aFR[0], aUR[0], aFR[1], aUR[1], raw);
+#pragma unroll
+      for (int q = 0; q < NPR; ++q)
+        if (q != B1 + d) gsc[q < ER ? 0 : 1] = fma(o[q], raw[q], gsc[q < ER ? 0 : 1]);
+      gsc[0] += gfs * (sL * mL + sR * mR);
+    }
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) o[q] *= sc[q < ER ? 0 : 1];
+    double gL[NPR], gR[NPR];
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) gL[q] = gR[q] = 0.0;
+    SideCot cL, cR;
+    side_add_T<MET, dd>(L, PL, aFL, aUL, o, gfs * sc[0] * sL, gL, cL);
+    side_add_T<MET, dd>(R, PR, aFR, aUR, o, gfs * sc[0] * sR, gR, cR);
+    if (gfs != 0.0) {  // d s = n d ug / ug - (n + 1) d rho / rho
+      const double n = 1.0 / (p.gam - 1.0), ud1 = dd == 1 ? L.u1 : PL[U1 + d], ud2 = dd == 1 ? R.u1 : PR[U1 + d];
+      const double gl = gfs * sc[0] * PL[RHO] * fma(aUL[0], L.u0, aFL[0] * ud1);
+      const double gr = gfs * sc[0] * PR[RHO] * fma(aUR[0], R.u0, aFR[0] * ud2);
+      gL[UU] += gl * n / PL[UU];
+      gL[RHO] -= gl * (n + 1.0) / PL[RHO];
+      gR[UU] += gr * n / PR[UU];
+      gR[RHO] -= gr * (n + 1.0) / PR[RHO];
+    }
+    // weights -> v_max, v_min of the sides, by the branches the maxima took
+    double vpL[2], vpR[2], vmL[2], vmR[2];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      double gp, gm;
+      const double gU = cL.aU[w] - cR.aU[w];
+      if (p.flux == 0) {
+        gp = cp[w] > cm[w] ? gU : 0.0;
+        gm = cp[w] > cm[w] ? 0.0 : gU;
+      } else if (cp[w] + cm[w] > 0.0) {
+        const double gs = -gsc[w] * sc[w] / (cp[w] + cm[w]);
+        gp = cL.aF[w] + gU * cm[w] + gs;
+        gm = cR.aF[w] + gU * cp[w] + gs;
+      } else {
+        gp = gm = 0.0;
+      }
+      const double a = L.vmax(w), b = R.vmax(w), e = L.vmin(w), h = R.vmin(w);
+      if (!(cp[w] > 0.0)) gp = 0.0;
+      if (!(cm[w] > 0.0)) gm = 0.0;
+      vpL[w] = a >= b ? gp : 0.0;
+      vpR[w] = a >= b ? 0.0 : gp;
+      vmL[w] = e <= h ? -gm : 0.0;
+      vmR[w] = e <= h ? 0.0 : -gm;
+    }
+    side_build_T<MET, dd>(p, g, f, L, dl, kL, PL, vpL, vmL, cL, gL, &gk);
+    side_build_T<MET, dd>(p, g, f, R, dl, kR, PR, vpR, vmR, cR, gR, &gk);
+#pragma unroll
     for (int q = 0; q < NPR; ++q) {
-      gE[(NPR + q) * bx.ntot + t - st] = gin[q] * wL[q];  // upper edge of cell f-1
-      gE[q * bx.ntot + t] = gin[NPR + q] * wL[q];         // lower edge of cell f
+      const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
+      const double w = wq ? igf : 1.0;
+      gE[(NPR + q) * nt + t - st] = gL[q] * w;  // upper edge of cell f-1
+      gE[q * nt + t] = gR[q] * w;               // lower edge of cell f
     }
-    gk += gin[24];
   }
   warp_atomic_add(gk_out, gk);
 }

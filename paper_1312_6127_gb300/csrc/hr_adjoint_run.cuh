@@ -130,21 +130,21 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
       const double* flat = p.recon == 0 ? chi_s : aux;  // not read for MC
       recon<MET>(c, d, Pg, aux, flat, 256, 16);
       if (d == 0) {
-        ka_face<MET, 0><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[0], a.gE, a.gk, a.gFS[0]);
+        ka_face<MET, 0><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[0], a.gE, a.gk, a.gFS[0], c->geotab);
         ka_edges<MET, 0><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, flat, a.gE, a.gP, a.gchi);
         if (p.recon == 0) {
           ka_flatten<0><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, chi_prev, a.gchi, carry, a.gP, a.gaux);
           ka_prep<MET, 0><<<G(nt), 128, 0, st>>>(p, bx, Pg, K, a.gaux, a.gP, a.gk);
         }
       } else if (d == 1) {
-        ka_face<MET, 1><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[1], a.gE, a.gk, a.gFS[1]);
+        ka_face<MET, 1><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[1], a.gE, a.gk, a.gFS[1], c->geotab);
         ka_edges<MET, 1><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, flat, a.gE, a.gP, a.gchi);
         if (p.recon == 0) {
           ka_flatten<1><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, chi_prev, a.gchi, carry, a.gP, a.gaux);
           ka_prep<MET, 1><<<G(nt), 128, 0, st>>>(p, bx, Pg, K, a.gaux, a.gP, a.gk);
         }
       } else {
-        ka_face<MET, 2><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[2], a.gE, a.gk, a.gFS[2]);
+        ka_face<MET, 2><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[2], a.gE, a.gk, a.gFS[2], c->geotab);
         ka_edges<MET, 2><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, flat, a.gE, a.gP, a.gchi);
         if (p.recon == 0) {
           ka_flatten<2><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, chi_prev, a.gchi, carry, a.gP, a.gaux);

@@ -588,21 +588,26 @@ struct FaceSide {
   double u0, u1, l0, l[3], bt, m0, m[3], iut, wb, pt;
   double r0, rd, k0, k[3];
   double Bq[2], sd[2], iq[2];
+  // for the adjoint (unused, and dropped by the compiler, in the forward kernel)
+  double gm, igm, gr, bsq, c2[2], H[2];
+  unsigned cd;
 
   __device__ __forceinline__ void speeds(const Geo<MET, double>& g, const FaceGeo<MET, d>& f, int w, double ut,
                                          double ud, double c2) {
     const double u02 = ut * ut, mix = ut * ud;
-    double H, AB = 0.0;
+    double h, AB = 0.0;
     if constexpr (MET == MINK) {
-      H = fma(-ud, ud, u02);
+      h = fma(-ud, ud, u02);
     } else {
-      H = fma(ud * ud, g.G00, u02 * g.Gdd(d));
+      h = fma(ud * ud, g.G00, u02 * g.Gdd(d));
       if (d == 1) {
         AB = g.G01;
-        H = fma(-2.0 * AB, mix, H);
+        h = fma(-2.0 * AB, mix, h);
       }
     }
-    const double K = c2 * fma(c2, f.C0 - H, H);
+    H[w] = h;
+    this->c2[w] = c2;
+    const double K = c2 * fma(c2, f.C0 - h, h);
     Bq[w] = d == 1 && MET == KS ? fma(-c2, AB + mix, mix) : fma(-c2, mix, mix);
     iq[w] = rcp(fma(-c2, g.Gtt() + u02, u02));
     sd[w] = K > 0.0 ? sqrt64(K) : 0.0;
@@ -614,14 +619,12 @@ struct FaceSide {
                                         double dl, double kf, const double P[NPR], unsigned* code) {
     const double rho = P[RHO], pg = p.gm1 * P[UU], w = rho + P[UU] + pg;
     lower3<MET>(g, P[U1], P[U2], P[U3], l);
-    double igm;
-    const double gm = sqrt_rsqrt(fma(P[U1], l[0], fma(P[U2], l[1], fma(P[U3], l[2], 1.0))), &igm);
+    gm = sqrt_rsqrt(fma(P[U1], l[0], fma(P[U2], l[1], fma(P[U3], l[2], 1.0))), &igm);
     lower3<MET>(g, P[B1], P[B2], P[B3], m);
     bt = fma(P[B1], l[0], fma(P[B2], l[1], P[B3] * l[2]));
     const double BB = fma(P[B1], m[0], fma(P[B2], m[1], P[B3] * m[2]));
-    double k2;
     lower3<MET>(g, P[UR1], P[UR2], P[UR3], k);
-    k2 = sqrt64(fma(P[UR1], k[0], fma(P[UR2], k[1], fma(P[UR3], k[2], 1.0))));
+    const double k2 = gr = sqrt64(fma(P[UR1], k[0], fma(P[UR2], k[1], fma(P[UR3], k[2], 1.0))));
     if constexpr (MET == MINK) {
       u0 = gm;
       u1 = P[U1];
@@ -641,11 +644,11 @@ struct FaceSide {
       k0 = fma(f.b1, k[0], -g.alpha * k2);
       rd = d == 1 ? fma(-k2, f.a01, P[UR1]) : P[UR1 + d - 1];
     }
-    const double bsq = fma(bt, bt, BB) * (iut * iut);
+    bsq = fma(bt, bt, BB) * (iut * iut);
     wb = w + bsq;
     pt = fma(0.5, bsq, pg);
     double c2 = fma(p.gam, pg, bsq) * rcp(wb);
-    unsigned cd = 0;
+    cd = 0;
     if ((unsigned)__double2hiint(c2) >= 0x3ff00000u) {  // at least 1, negative or NaN
       cd = (c2 > 1.0 ? 1u : 0u) | (c2 < 0.0 ? 2u : 0u);
       c2 = c2 > 1.0 ? 1.0 : (c2 < 0.0 ? 0.0 : c2);
