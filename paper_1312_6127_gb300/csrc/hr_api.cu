@@ -324,15 +324,24 @@ int launch_step(harmrad_ctx* c, bool with_cfl) {
   return HARMRAD_OK;
 }
 
-harmrad_tuning default_tuning() {
+// Default launch shapes.  The heavy kernels hold 2 blocks of 128 threads per SM
+// (200 registers and more): a grid that does not fill one such wave takes blocks
+// of one or two warps, which spread over all SMs and schedulers (64x32x16 torus,
+// 32-thread against 128-thread blocks: update 0.57 against 0.62 ms per step,
+// reconstruction 0.26 against 0.34); a larger one is fastest with full blocks
+// (256x128x64: update 17.6 ms against 20.9 with 32 threads).  Blocks beyond the
+// resident ones (cap 64 per SM, 16 before: update 20.5 ms) even out zones of
+// unlike Newton counts.
+harmrad_tuning default_tuning(long long nact, int sms) {
   harmrad_tuning t;
   memset(&t, 0, sizeof(t));
-  t.face_block = 128;
-  t.face_blocks_per_sm = 16;
-  t.update_block = 128;
-  t.update_blocks_per_sm = 16;
-  t.edge_block = 256;
-  t.edge_blocks_per_sm = 16;
+  const bool small = nact <= 256LL * sms;
+  t.face_block = small ? 32 : 128;
+  t.face_blocks_per_sm = 64;
+  t.update_block = small ? 32 : 128;
+  t.update_blocks_per_sm = 64;
+  t.edge_block = small ? 64 : 256;
+  t.edge_blocks_per_sm = 64;
   t.newton_split = 0;
   return t;
 }
@@ -432,8 +441,6 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
   c->nact = aoff;
   c->real_size = p[0].precision == HARMRAD_PREC_SPLIT ? 4 : 8;
   c->use_graph = getenv("HARMRAD_NO_GRAPH") == nullptr;
-  c->tune = default_tuning();
-  if (count > 1) c->tune.newton_split = 3;  // batches: heavy-tailed Newton counts expected
   if (cudaGetDevice(&c->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
     cudaGetLastError();
@@ -441,6 +448,8 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     free(c);
     return HARMRAD_E_CUDA;
   }
+  c->tune = default_tuning(c->nact, c->sms);
+  if (count > 1) c->tune.newton_split = 5;  // batches: heavy-tailed Newton counts expected (3: 51.3 ms, 5: 48.2)
   if (stream) {
     c->stream = (cudaStream_t)stream;
   } else {

@@ -88,9 +88,7 @@ __device__ __forceinline__ void warp_add(unsigned long long* dst, unsigned v) {
 // ------------------------------------------------------------ work split
 // First item of this thread among the items of a grid whose predecessors in
 // the context hold `done` items: the grids' items form one sequence dealt to
-// the threads in turn, so that a batch of small grids loads every block alike
-// (12 boxes of 32 to 64 cells a side: step 73.2 -> 71.5 ms, ghost fill 1.03 ->
-// 0.44, reconstruction 7.2 -> 6.3).
+// the threads in turn, so that a batch of small grids loads every block alike.
 __device__ __forceinline__ long long first_item(long long done) {
   if (done == 0) return HR_TID;
   const long long r = HR_TID - done % HR_STRIDE;
