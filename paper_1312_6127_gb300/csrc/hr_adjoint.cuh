@@ -792,12 +792,22 @@ __global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, EdgeSet E
 
 // ----------------------------------------------------- reconstruction (T)
 // Per cell of the edge range: cotangents of the five stencil primitives of
-// every variable (atomic, the stencils overlap) and of the cell's flattener.
+// every variable (atomic, the stencils overlap) and of the cell's flattener,
+// from the edge formulas of the reconstruction transposed by hand (twice the
+// MC slope D, the interface values, flattening, monotonicity) along the
+// branches they take.
+
+// D = mc_twice(dm, dp) transposed.
+__device__ __forceinline__ void mc_twice_T(double dm, double dp, double gD, double& gm, double& gp) {
+  const unsigned c = mc_twice_code(dm, dp);
+  gm = c == 1 ? gD : (c == 2 ? 4.0 * gD : 0.0);
+  gp = c == 1 ? gD : (c == 3 ? 4.0 * gD : 0.0);
+}
+
 template <int MET, int d>
 __global__ void ka_edges(DevParams p, BoxGeo bx, const double* __restrict__ P, const double* __restrict__ aux,
                          const double* __restrict__ flat, const double* __restrict__ gE, double* gP,
                          double* __restrict__ gchi) {
-  typedef Dn<6> D6;
   const bool weighted = (MET == KS) && (d != 1);
   int len[3], off[3];
   for (int e = 0; e < 3; ++e) {
@@ -810,7 +820,7 @@ __global__ void ka_edges(DevParams p, BoxGeo bx, const double* __restrict__ P, c
     }
   }
   const long long total = (long long)len[0] * len[1] * len[2];
-  const long long st = bx.str[d];
+  const long long st = bx.str[d], nt = bx.ntot;
   for (long long id = HR_TID; id < total; id += HR_STRIDE) {
     long long r = id;
     int i = (int)(r % len[0]) + off[0];
@@ -819,37 +829,72 @@ __global__ void ka_edges(DevParams p, BoxGeo bx, const double* __restrict__ P, c
     int k = (int)(r / len[1]) + off[2];
     const long long t = cell_index(bx, i, j, k);
     double gcg = 0.0, gcr = 0.0;
-    const double chg = p.recon == 0 ? flat[t] : 0.0, chr = p.recon == 0 ? flat[bx.ntot + t] : 0.0;
+    const double chg = p.recon == 0 ? flat[t] : 0.0, chr = p.recon == 0 ? flat[nt + t] : 0.0;
     double gw[5];
+#pragma unroll
     for (int m = 0; m < 5; ++m) gw[m] = weighted ? aux[t + (m - 2) * st] : 1.0;
+#pragma unroll 2
     for (int q = 0; q < NPR; ++q) {
-      const double gl = gE[q * bx.ntot + t], gr = gE[(NPR + q) * bx.ntot + t];
+      double gl = gE[q * nt + t], gr = gE[(NPR + q) * nt + t];
       if (gl == 0.0 && gr == 0.0) continue;
       const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
-      D6 sD[5];
+      double s[5], dd[4], gs[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, gd[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
       for (int m = 0; m < 5; ++m) {
-        const double v = P[q * bx.ntot + t + (m - 2) * st];
-        sD[m] = D6::seed(wq ? gw[m] * v : v, m);
+        const double v = P[q * nt + t + (m - 2) * st];
+        s[m] = wq ? gw[m] * v : v;
       }
-      D6 aL, aR;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) dd[m] = s[m + 1] - s[m];
       if (p.recon == 0) {
-        D6 chi = D6::seed(q < ER ? chg : chr, 5);
-        ppm_cell<D6>(sD, chi, &aL, &aR);
-      } else {
-        D6 dq = mc_slope<D6>(sD[1], sD[2], sD[3]);
-        aL = sD[2] - 0.5 * dq;
-        aR = sD[2] + 0.5 * dq;
+        const double chi = q < ER ? chg : chr, qc = s[2];
+        const double D1 = mc_twice(dd[0], dd[1]), D2 = mc_twice(dd[1], dd[2]), D3 = mc_twice(dd[2], dd[3]);
+        const double l0 = ppm_face(s[1], dd[1], D1, D2), r0 = ppm_face(s[2], dd[2], D2, D3);
+        double l = l0, rr = r0;
+        const unsigned code = ppm_limit(qc, chi, l, rr);
+        if (code == 1) {
+          gs[2] = gl + gr;
+          gl = gr = 0.0;
+        } else if (code == 2) {  // l = 3 q - 2 r
+          gs[2] = 3.0 * gl;
+          gr -= 2.0 * gl;
+          gl = 0.0;
+        } else if (code == 3) {  // r = 3 q - 2 l
+          gs[2] = 3.0 * gr;
+          gl -= 2.0 * gr;
+          gr = 0.0;
+        }
+        const double gc = gl * (qc - l0) + gr * (qc - r0);
+        if (q < ER) gcg += gc;
+        else gcr += gc;
+        gs[2] += chi * (gl + gr);
+        gl *= 1.0 - chi;
+        gr *= 1.0 - chi;
+        // l0 = s1 + d1 / 2 + (D1 - D2) / 12, r0 = s2 + d2 / 2 + (D2 - D3) / 12
+        gs[1] = gl;
+        gs[2] += gr;
+        double a, b;
+        mc_twice_T(dd[0], dd[1], gl * (1.0 / 12.0), a, b);
+        gd[0] = a;
+        gd[1] = b + 0.5 * gl;
+        mc_twice_T(dd[1], dd[2], (gr - gl) * (1.0 / 12.0), a, b);
+        gd[1] += a;
+        gd[2] = b + 0.5 * gr;
+        mc_twice_T(dd[2], dd[3], gr * (-1.0 / 12.0), a, b);
+        gd[2] += a;
+        gd[3] = b;
+      } else {  // s -+ D / 4
+        gs[2] = gl + gr;
+        mc_twice_T(dd[1], dd[2], 0.25 * (gr - gl), gd[1], gd[2]);
       }
+#pragma unroll
       for (int m = 0; m < 5; ++m) {
-        const double v = gl * aL.d[m] + gr * aR.d[m];
-        if (v != 0.0) atomicAdd(&gP[q * bx.ntot + t + (m - 2) * st], wq ? v * gw[m] : v);
+        const double v = gs[m] + (m > 0 ? gd[m - 1] : 0.0) - (m < 4 ? gd[m] : 0.0);
+        if (v != 0.0) atomicAdd(&gP[q * nt + t + (m - 2) * st], wq ? v * gw[m] : v);
       }
-      const double vc = gl * aL.d[5] + gr * aR.d[5];
-      if (q < ER) gcg += vc;
-      else gcr += vc;
     }
     gchi[t] = gcg;
-    gchi[bx.ntot + t] = gcr;
+    gchi[nt + t] = gcr;
   }
 }
 
