@@ -112,6 +112,193 @@ static __global__ void ka_backup_T(BoxGeo bx, const unsigned char* __restrict__ 
   }
 }
 
+// ------------------------------------------------------------- frames (T)
+// 4-velocities, field and b^2 of a state transposed (FaceSide, Frame): from the
+// cotangents of u^t, u^1, u_t, u_i, B_t, B_i, b^t, 1/u^t, b^2 and the radiation's
+// u^t, u^1, u_t, u_i to those of u~^i, B^i and u~_rad^i (added to gP).
+template <int MET, class S>
+__device__ __forceinline__ void gas_frame_T(const Geo<MET, double>& g, double a01, double b1, const S& s,
+                                            const double P[NPR], double gu0, double gu1, double gl0,
+                                            const double gl[3], double gm0, const double gmv[3], double gbt,
+                                            double giut, double gbsq, double gP[NPR]) {
+  const double ia = MET == MINK ? 1.0 : g.ialpha, al = MET == MINK ? 1.0 : g.alpha;
+  const double gBB = gbsq * (s.iut * s.iut);
+  gbt = fma(2.0 * gBB, s.bt, gbt);
+  giut = fma(2.0 * gbsq, s.bsq * rcp(s.iut), giut);
+  // gamma: u^t = gamma / alpha, u^1 = u~^1 - gamma a01, u_t = b1 l_1 - alpha gamma, 1/u^t = alpha / gamma
+  double ggm = fma(-giut * s.iut, s.igm, gu0 * ia) - al * gl0;
+  ggm = fma(-gu1, a01, ggm);
+  gP[U1] += gu1;
+  const double gg = 0.5 * ggm * s.igm;
+  double a[3], b[3], t[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    gP[B1 + i] = fma(gbt, s.l[i], fma(gBB, s.m[i], gP[B1 + i]));
+    a[i] = fma(gbt, P[B1 + i], fma(gg, P[U1 + i], gl[i]));
+    b[i] = fma(gBB, P[B1 + i], gmv[i]);
+    gP[U1 + i] = fma(gg, s.l[i], gP[U1 + i]);
+  }
+  a[0] = fma(b1, gl0, a[0]);
+  b[0] = fma(b1, gm0, b[0]);
+  lower3<MET>(g, a[0], a[1], a[2], t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) gP[U1 + i] += t[i];
+  lower3<MET>(g, b[0], b[1], b[2], t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) gP[B1 + i] += t[i];
+}
+template <int MET, class S>
+__device__ __forceinline__ void frame_T(const Geo<MET, double>& g, double a01, double b1, const S& s,
+                                        const double P[NPR], double gu0, double gu1, double gl0, const double gl[3],
+                                        double gm0, const double gmv[3], double gbt, double giut, double gbsq,
+                                        double gr0, double gr1, double gk0, const double gk[3], double gP[NPR]) {
+  gas_frame_T<MET>(g, a01, b1, s, P, gu0, gu1, gl0, gl, gm0, gmv, gbt, giut, gbsq, gP);
+  const double ia = MET == MINK ? 1.0 : g.ialpha, al = MET == MINK ? 1.0 : g.alpha;
+  double a[3], t[3];
+  gP[UR1] += gr1;
+  const double ggr = fma(-gr1, a01, fma(gr0, ia, -al * gk0));
+  const double gq = 0.5 * ggr * rcp(s.gr);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    gP[UR1 + i] = fma(gq, s.k[i], gP[UR1 + i]);
+    a[i] = fma(gq, P[UR1 + i], gk[i]);
+  }
+  a[0] = fma(b1, gk0, a[0]);
+  lower3<MET>(g, a[0], a[1], a[2], t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) gP[UR1 + i] += t[i];
+}
+
+// The frames of a zone's state, as FaceSide forms them.
+template <int MET>
+struct Frame {
+  double gm, igm, gr, u0, u1, l0, l[3], bt, m0, m[3], iut, bsq, r0, r1, k0, k[3];
+  __device__ __forceinline__ Frame(const Geo<MET, double>& g, double a01, double b1, const double P[NPR]) {
+    const double ia = MET == MINK ? 1.0 : g.ialpha, al = MET == MINK ? 1.0 : g.alpha;
+    lower3<MET>(g, P[U1], P[U2], P[U3], l);
+    lower3<MET>(g, P[B1], P[B2], P[B3], m);
+    lower3<MET>(g, P[UR1], P[UR2], P[UR3], k);
+    gm = sqrt_rsqrt(fma(P[U1], l[0], fma(P[U2], l[1], fma(P[U3], l[2], 1.0))), &igm);
+    gr = sqrt64(fma(P[UR1], k[0], fma(P[UR2], k[1], fma(P[UR3], k[2], 1.0))));
+    bt = fma(P[B1], l[0], fma(P[B2], l[1], P[B3] * l[2]));
+    u0 = gm * ia;
+    u1 = fma(-gm, a01, P[U1]);
+    l0 = fma(b1, l[0], -al * gm);
+    iut = al * igm;
+    m0 = b1 * m[0];
+    r0 = gr * ia;
+    r1 = fma(-gr, a01, P[UR1]);
+    k0 = fma(b1, k[0], -al * gr);
+    bsq = fma(bt, bt, fma(P[B1], m[0], fma(P[B2], m[1], P[B3] * m[2]))) * (iut * iut);
+  }
+};
+
+// U(P) and the geometric source of cons_source64 transposed: gU the cotangents
+// of U, gX those of the source rows (2, 3 gas, 9, 10 radiation), gs that of the
+// conserved entropy U_rho s; md the scaled metric derivatives.  Adds to gP.
+template <int MET>
+__device__ __forceinline__ void cons_T(const DevParams& p, const Geo<MET, double>& g, const MetricDeriv& md,
+                                       const double P[NPR], const double gU[NPR], const double gX[NPR], double gs,
+                                       double gP[NPR]) {
+  const double a01 = MET == MINK ? 0.0 : g.alpha * g.G01, b1 = MET == MINK ? 0.0 : g.alpha * a01;
+  const Frame<MET> s(g, a01, b1, P);
+  const double wb = P[RHO] + fma(p.gam, P[UU], s.bsq), bu = s.bt * s.iut, wu = wb * s.u0, Z = fma(-s.bt, bu, wu);
+  const double E = P[ER], e43 = (4.0 / 3.0) * E, er = e43 * s.r0;
+  double o[NPR];
+#pragma unroll
+  for (int q = 0; q < NPR; ++q) o[q] = g.gdet * gU[q];
+  double gmt = o[0] + o[1], gpt = o[1], gZ = o[1] * s.l0, gbu = -o[1] * s.m0, gl0 = o[1] * Z, gm0 = -o[1] * bu;
+  double ger = o[8] * s.k0, gk0 = o[8] * er, ge13 = o[8], gl[3], gmv[3], gk[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    gZ = fma(o[2 + i], s.l[i], gZ);
+    gbu = fma(-o[2 + i], s.m[i], gbu);
+    gl[i] = o[2 + i] * Z;
+    gmv[i] = -o[2 + i] * bu;
+    ger = fma(o[9 + i], s.k[i], ger);
+    gk[i] = o[9 + i] * er;
+    gP[B1 + i] += o[5 + i];
+  }
+  double gwb = 0.0, gu0 = 0.0, gu1 = 0.0, gbt = 0.0, giut = 0.0, gr0 = 0.0, gr1 = 0.0, ge43 = 0.0;
+  if (gs != 0.0) {  // U_rho s: d s = n d ug / ug - (n + 1) d rho / rho
+    const double n = 1.0 / (p.gam - 1.0), w = gs * g.gdet * P[RHO] * s.u0;
+    gmt = fma(gs * g.gdet, entropy_per_baryon<double>(p, P[RHO], P[UU]), gmt);
+    gP[UU] += w * n / P[UU];
+    gP[RHO] -= w * (n + 1.0) / P[RHO];
+  }
+  if constexpr (MET == KS) {
+    const double* dm = reinterpret_cast<const double*>(&md);
+    const double u2 = P[U2], u3 = P[U3], r2 = P[UR2], r3 = P[UR3];
+    const double c1 = fma(s.bt, s.u1, P[B1]) * s.iut, c2 = fma(s.bt, u2, P[B2]) * s.iut,
+                 c3 = fma(s.bt, u3, P[B3]) * s.iut;  // b^i
+    double G[7], H[7];
+#pragma unroll
+    for (int c = 0; c < 7; ++c) {
+      G[c] = fma(gX[2], dm[2 * c], gX[3] * dm[2 * c + 1]);
+      H[c] = fma(gX[9], dm[2 * c], gX[10] * dm[2 * c + 1]);
+    }
+    gpt += fma(gX[2], md.sg[0], gX[3] * md.sg[1]);
+    ge13 += fma(gX[9], md.sg[0], gX[10] * md.sg[1]);
+    // contractions G(v) of a vector and their halved gradients
+    const double a0 = fma(G[0], s.u0, 0.5 * fma(G[1], s.u1, G[2] * u3));
+    const double a1 = fma(G[3], s.u1, 0.5 * fma(G[1], s.u0, G[4] * u3));
+    const double a2 = G[5] * u2, a3 = fma(G[6], u3, 0.5 * fma(G[2], s.u0, G[4] * s.u1));
+    gwb += a0 * s.u0 + a1 * s.u1 + a2 * u2 + a3 * u3;
+    gu0 += 2.0 * wb * a0;
+    gu1 += 2.0 * wb * a1;
+    gP[U2] += 2.0 * wb * a2;
+    gP[U3] += 2.0 * wb * a3;
+    const double d0 = -2.0 * fma(G[0], s.bt, 0.5 * fma(G[1], c1, G[2] * c3));
+    const double d1 = -2.0 * fma(G[3], c1, 0.5 * fma(G[1], s.bt, G[4] * c3));
+    const double d2 = -2.0 * G[5] * c2, d3 = -2.0 * fma(G[6], c3, 0.5 * fma(G[2], s.bt, G[4] * c1));
+    // b^i = (B^i + b^t u^i) / u^t
+    gbt += d0 + s.iut * (d1 * s.u1 + d2 * u2 + d3 * u3);
+    const double bi = s.bt * s.iut;
+    gu1 = fma(d1, bi, gu1);
+    gP[U2] = fma(d2, bi, gP[U2]);
+    gP[U3] = fma(d3, bi, gP[U3]);
+    gP[B1] = fma(d1, s.iut, gP[B1]);
+    gP[B2] = fma(d2, s.iut, gP[B2]);
+    gP[B3] = fma(d3, s.iut, gP[B3]);
+    giut += (d1 * c1 + d2 * c2 + d3 * c3) * rcp(s.iut);
+    const double e0 = fma(H[0], s.r0, 0.5 * fma(H[1], s.r1, H[2] * r3));
+    const double e1 = fma(H[3], s.r1, 0.5 * fma(H[1], s.r0, H[4] * r3));
+    const double e2 = H[5] * r2, e3 = fma(H[6], r3, 0.5 * fma(H[2], s.r0, H[4] * s.r1));
+    ge43 += e0 * s.r0 + e1 * s.r1 + e2 * r2 + e3 * r3;
+    gr0 += 2.0 * e43 * e0;
+    gr1 += 2.0 * e43 * e1;
+    gP[UR2] += 2.0 * e43 * e2;
+    gP[UR3] += 2.0 * e43 * e3;
+  }
+  ge43 = fma(ger, s.r0, ge43);
+  gr0 = fma(ger, e43, gr0);
+  gP[ER] += fma(4.0 / 3.0, ge43, ge13 * (1.0 / 3.0));
+  // Z = wu - b^t bu, bu = b^t / u^t, wu = wb u^t, mt = rho u^t
+  gbt = fma(-gZ, bu, gbt);
+  gbu = fma(-gZ, s.bt, gbu);
+  gbt = fma(gbu, s.iut, gbt);
+  giut = fma(gbu, s.bt, giut);
+  gwb = fma(gZ, s.u0, gwb);
+  gu0 = fma(gZ, wb, fma(gmt, P[RHO], gu0));
+  gP[RHO] += fma(gmt, s.u0, gwb);
+  gP[UU] += fma(p.gam, gwb, p.gm1 * gpt);
+  frame_T<MET>(g, a01, b1, s, P, gu0, gu1, gl0, gl, gm0, gmv, gbt, giut, gwb + 0.5 * gpt, gr0, gr1, gk0, gk, gP);
+}
+
+// Metric and scaled metric derivatives of the centre of cell (i, j).
+template <int MET>
+__device__ __forceinline__ Geo<MET, double> centre_tables(const DevParams& p, const BoxGeo& bx, const double* geo,
+                                                          int i, int j, MetricDeriv* md) {
+  if constexpr (MET == KS) {
+    const GeoTab T = geotab(geo, bx);
+    const long long x = gidx_c(bx, i, j);
+    *md = md_load(T.M, T.sC, x);
+    return geo_load<MET>(T.C, T.sC, x);
+  } else {
+    return make_geo<MET, double>(p, 0.0, 0.0);
+  }
+}
+
 // ------------------------------------------------------- implicit solve (T)
 template <int MET>
 __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt, const double* __restrict__ K,
@@ -233,18 +420,22 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
 // --------------------------------------------------- explicit update (T)
 // U* = a_s U^n + b_s (U(P_s) + dt X),  X = -sum_d dF_d/dx_d + SM(P_s).
 template <int MET>
-__global__ void ka_update(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt, const double* __restrict__ Ps0) {
+__global__ void __launch_bounds__(128) ka_update(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
+                                                 const double* __restrict__ Ps0, const double* __restrict__ geo) {
   const double A = s == 0 ? 0.0 : (s == 1 ? 0.75 : 1.0 / 3.0);
   const double Bc = s == 0 ? 1.0 : (s == 1 ? 0.25 : 2.0 / 3.0);
-  typedef Dn<4> D4;
   for (long long z = HR_TID; z < bx.nact; z += HR_STRIDE) {
-    double gq[NPR];
+    double gq[NPR], gX[NPR], gP[NPR], P[NPR];
     bool any = false;
+#pragma unroll
     for (int q = 0; q < NPR; ++q) {
       gq[q] = a.gU[q * bx.nact + z];
       any = any || gq[q] != 0.0;
       if (s > 0) a.gUn[q * bx.nact + z] += A * gq[q];
       a.gX[q * bx.nact + z] = Bc * dt * gq[q];
+      gq[q] *= Bc;
+      gX[q] = dt * gq[q];
+      gP[q] = 0.0;
     }
     // S* = A S^n + Bc (S(P_s) + dt X_S), S(P) = U_rho(P) s_gas(P)
     const double gs = a.gS[z];
@@ -254,36 +445,30 @@ __global__ void ka_update(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt, c
     int i, j, k;
     zone_ijk(bx, z, i, j, k);
     const long long t = cell_index(bx, i, j, k);
-    if (!any) {
-      for (int q = 0; q < NPR; ++q) a.gP[q * bx.ntot + t] = 0.0;
-      continue;
+    if (any) {
+      MetricDeriv md{};
+      const Geo<MET, double> g = centre_tables<MET>(p, bx, geo, i, j, &md);
+#pragma unroll
+      for (int q = 0; q < NPR; ++q) P[q] = Ps0[q * bx.ntot + t];
+      cons_T<MET>(p, g, md, P, gq, gX, Bc * gs, gP);
     }
-    const double x1 = xcen(bx, 0, i), x2 = xcen(bx, 1, j);
-    const Geo<MET, D4> g4 = geo_cast<D4>(make_geo<MET, double>(p, x1, x2));
-    for (int ch = 0; ch < 3; ++ch) {
-      D4 PsD[NPR], UsD[NPR], XD[NPR];
-      for (int q = 0; q < NPR; ++q) PsD[q] = D4::seed(Ps0[q * bx.ntot + t], q - 4 * ch);
-      cons_source<MET, D4>(p, g4, x1, x2, PsD, UsD, XD);
-      const D4 Su = gs != 0.0 ? UsD[RHO] * entropy_per_baryon<D4>(p, PsD[RHO], PsD[UU]) : D4(0.0);
-      for (int c = 0; c < 4; ++c) {
-        double v = gs * Su.d[c];
-        for (int q = 0; q < NPR; ++q) v += gq[q] * (UsD[q].d[c] + dt * XD[q].d[c]);
-        a.gP[(4 * ch + c) * bx.ntot + t] = Bc * v;
-      }
-    }
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) a.gP[q * bx.ntot + t] = gP[q];
   }
 }
 
 // U^n = U(P^n): gP^n += (dU/dP)^T gU^n at the end of the sweep.
 template <int MET>
-__global__ void ka_un(DevParams p, BoxGeo bx, AdjBufs a, const double* __restrict__ P0) {
-  typedef Dn<4> D4;
+__global__ void __launch_bounds__(128) ka_un(DevParams p, BoxGeo bx, AdjBufs a, const double* __restrict__ P0,
+                                             const double* __restrict__ geo) {
   for (long long z = HR_TID; z < bx.nact; z += HR_STRIDE) {
-    double gq[NPR];
+    double gq[NPR], gX[NPR], gP[NPR], P[NPR];
     bool any = false;
+#pragma unroll
     for (int q = 0; q < NPR; ++q) {
       gq[q] = a.gUn[q * bx.nact + z];
       any = any || gq[q] != 0.0;
+      gX[q] = gP[q] = 0.0;
     }
     const double gs = a.gSn[z];  // S^n = U_rho(P^n) s_gas(P^n)
     any = any || gs != 0.0;
@@ -291,19 +476,13 @@ __global__ void ka_un(DevParams p, BoxGeo bx, AdjBufs a, const double* __restric
     int i, j, k;
     zone_ijk(bx, z, i, j, k);
     const long long t = cell_index(bx, i, j, k);
-    const double x1 = xcen(bx, 0, i), x2 = xcen(bx, 1, j);
-    const Geo<MET, D4> g4 = geo_cast<D4>(make_geo<MET, double>(p, x1, x2));
-    for (int ch = 0; ch < 3; ++ch) {
-      D4 PsD[NPR], UsD[NPR], XD[NPR];
-      for (int q = 0; q < NPR; ++q) PsD[q] = D4::seed(P0[q * bx.ntot + t], q - 4 * ch);
-      cons_source<MET, D4>(p, g4, x1, x2, PsD, UsD, XD);
-      const D4 Su = gs != 0.0 ? UsD[RHO] * entropy_per_baryon<D4>(p, PsD[RHO], PsD[UU]) : D4(0.0);
-      for (int c = 0; c < 4; ++c) {
-        double v = gs * Su.d[c];
-        for (int q = 0; q < NPR; ++q) v += gq[q] * UsD[q].d[c];
-        a.gN[(4 * ch + c) * bx.nact + z] += v;
-      }
-    }
+    MetricDeriv md{};
+    const Geo<MET, double> g = centre_tables<MET>(p, bx, geo, i, j, &md);
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) P[q] = P0[q * bx.ntot + t];
+    cons_T<MET>(p, g, md, P, gq, gX, gs, gP);
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) a.gN[q * bx.nact + z] += gP[q];
   }
 }
 
@@ -554,7 +733,7 @@ __device__ __forceinline__ void side_build_T(const DevParams& p, const Geo<MET, 
     }
     gc2[w] = gx;
   }
-  const double rho = P[RHO], iwb = rcp(s.wb), ia = MET == MINK ? 1.0 : g.ialpha, al = MET == MINK ? 1.0 : g.alpha;
+  const double rho = P[RHO], iwb = rcp(s.wb);
   double gpg = c.pt, gbsq = 0.5 * c.pt, gwb = c.wb;
   if (!(s.cd & 3u)) {  // c_ms^2 = (Gamma p + b^2) / (w + b^2), unclamped
     gpg = fma(gc2[0] * p.gam, iwb, gpg);
@@ -582,50 +761,19 @@ __device__ __forceinline__ void side_build_T(const DevParams& p, const Geo<MET, 
     gP[UU] = fma(gk * p.kscale, du, gP[UU]);
   }
   (void)dl;
-  // w + b^2, p_tot, b^2
+  // w + b^2, p_tot
   gbsq += gwb;
   gP[RHO] += gwb;
   gP[UU] += fma(p.gm1, gpg, p.gam * gwb);
-  const double i2 = s.iut * s.iut, gBB = gbsq * i2;
-  c.bt = fma(2.0 * gBB, s.bt, c.bt);
-  c.iut = fma(2.0 * gbsq, s.bsq * rcp(s.iut), c.iut);
-  // gas frame
-  double ggm = fma(-c.iut * s.iut, s.igm, c.u0 * ia) - al * c.l0;
-  if (d == 1) c.u1 += c.ud;
-  else gP[U1 + d - 1] += c.ud;
-  gP[U1] += c.u1;
-  ggm = fma(-c.u1, f.a01, ggm);
-  c.l[0] = fma(f.b1, c.l0, c.l[0]);
-  c.m[0] = fma(f.b1, c.m0, c.m[0]);
-  const double gg = 0.5 * ggm * s.igm;
-  double gl[3], gmm[3], t[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    gP[B1 + i] = fma(c.bt, s.l[i], fma(gBB, s.m[i], gP[B1 + i]));
-    gl[i] = fma(c.bt, P[B1 + i], fma(gg, P[U1 + i], c.l[i]));
-    gmm[i] = fma(gBB, P[B1 + i], c.m[i]);
-    gP[U1 + i] = fma(gg, s.l[i], gP[U1 + i]);
+  // u^d, u_r^d
+  if (d == 1) {
+    c.u1 += c.ud;
+  } else {
+    gP[U1 + d - 1] += c.ud;
+    gP[UR1 + d - 1] += c.rd;
   }
-  lower3<MET>(g, gl[0], gl[1], gl[2], t);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) gP[U1 + i] += t[i];
-  lower3<MET>(g, gmm[0], gmm[1], gmm[2], t);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) gP[B1 + i] += t[i];
-  // radiation frame
-  double ggr = fma(c.r0, ia, -al * c.k0);
-  gP[UR1 + d - 1] += c.rd;
-  if (d == 1) ggr = fma(-c.rd, f.a01, ggr);
-  c.k[0] = fma(f.b1, c.k0, c.k[0]);
-  const double gq = 0.5 * ggr * rcp(s.gr);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    gP[UR1 + i] = fma(gq, s.k[i], gP[UR1 + i]);
-    gl[i] = fma(gq, P[UR1 + i], c.k[i]);
-  }
-  lower3<MET>(g, gl[0], gl[1], gl[2], t);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) gP[UR1 + i] += t[i];
+  frame_T<MET>(g, f.a01, f.b1, s, P, c.u0, c.u1, c.l0, c.l, c.m0, c.m, c.bt, c.iut, gbsq, c.r0, d == 1 ? c.rd : 0.0,
+               c.k0, c.k, gP);
 }
 
 template <int MET, int d>

@@ -85,7 +85,7 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
     }
     k_prep64<MET><<<G(nt), 128, 0, st>>>(p, c->dboxes, 1, Pg, c->K, aux, c->geotab);
     HR_ACHECK(cudaMemsetAsync(a.gP, 0, pbytes, st));
-    ka_update<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, Ps);
+    ka_update<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, Ps, c->geotab);
     // fluxes: divergence, then flux-CT
     for (int d = 0; d < 3; ++d) {
       if (!p.act[d]) continue;
@@ -164,7 +164,7 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
     HR_ACHECK(cudaGetLastError());
   }
   // U^n = U(P^n)
-  ka_un<MET><<<G(na), 128, 0, st>>>(p, bx, a, a.Pst);
+  ka_un<MET><<<G(na), 128, 0, st>>>(p, bx, a, a.Pst, c->geotab);
   HR_ACHECK(cudaGetLastError());
   HR_ACHECK(cudaMemcpyAsync(gPin, a.gN, 12 * (size_t)na * sizeof(double), cudaMemcpyDeviceToDevice, st));
   if (gk_out) HR_ACHECK(cudaMemcpyAsync(gk_out, a.gk, sizeof(double), cudaMemcpyDeviceToDevice, st));
