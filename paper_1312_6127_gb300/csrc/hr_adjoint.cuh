@@ -300,9 +300,330 @@ __device__ __forceinline__ Geo<MET, double> centre_tables(const DevParams& p, co
 }
 
 // ------------------------------------------------------- implicit solve (T)
+// The error function and the final primitives of a zone at its solution
+// (pmhd_res64), with every intermediate the reverse sweep reads.
 template <int MET>
-__global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt, const double* __restrict__ K,
-                            const double* __restrict__ Pnext) {
+struct PmhdEval {
+  double l[3], gm, igm, u0, iut, l0, rho, bt, bu, bsq, pg, pt, wb, Z, m0, m[3];
+  double Rt[4], t[3], Er, ie, U2, y, sq, sm1, sp2, rr, E, fa, gr, v0, v[3];
+  double T, ka, ksca, kt, uru, e43, c1, c2, lam, hA, hC;  // ka: absorption over kappa_scale
+  bool neg, lim;
+
+  __device__ __forceinline__ PmhdEval(const DevParams& p, const ImpSys<MET>& s, const double x[4]) {
+    const auto& g = s.g;
+    const auto& c = s.pre;
+    const double al = MET == MINK ? 1.0 : g.alpha;
+    lower3<MET>(g, x[1], x[2], x[3], l);
+    gm = sqrt_rsqrt(fma(x[1], l[0], fma(x[2], l[1], fma(x[3], l[2], 1.0))), &igm);
+    u0 = MET == MINK ? gm : gm * g.ialpha;
+    iut = al * igm;
+    l0 = fma(c.b1, l[0], -al * gm);
+    rho = s.Dlab * iut;
+    bt = fma(s.B[0], l[0], fma(s.B[1], l[1], s.B[2] * l[2]));
+    bu = bt * iut;
+    bsq = fma(bt, bt, c.BB) * (iut * iut);
+    pg = p.gm1 * x[0];
+    pt = fma(0.5, bsq, pg);
+    wb = rho + fma(p.gam, x[0], bsq);
+    Z = fma(-bt, bu, wb * u0);
+    m0 = c.m0;
+    for (int k = 0; k < 3; ++k) m[k] = c.m[k];
+    Rt[0] = s.Rs[0] - (fma(rho, u0, fma(Z, l0, fma(-bu, m0, pt))) - s.Ts[0]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) Rt[1 + k] = s.Rs[1 + k] - (fma(Z, l[k], -bu * m[k]) - s.Ts[1 + k]);
+    raise3(g, c, Rt + 1, t);
+    U2 = c.a2 * fma(Rt[1], t[0], fma(Rt[2], t[1], Rt[3] * t[2]));
+    Er = fma(c.b1, Rt[1], -Rt[0]);
+    neg = !(Er > 0.0);
+    y = neg ? HUGE_VAL : (U2 > 0.0 ? U2 / (Er * Er) : 0.0);
+    lim = y > p.ymax_rad;
+    if (lim) {
+      Er = 1e-150 + sqrt(U2 / p.ymax_rad);
+      y = U2 / (Er * Er);
+    }
+    ie = 1.0 / Er;
+    sq = sqrt64(fma(-3.0, y, 4.0));
+    sm1 = sq - 1.0;
+    sp2 = sq + 2.0;
+    rr = rsqrt64(sp2 * sm1);
+    E = Er * sm1;
+    fa = 1.5 * ie * rr * al;
+    gr = 0.5 * sp2 * rr;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = fa * Rt[1 + k];
+    v0 = fma(c.b1, v[0], -al * gr);
+    T = pg * u0 * s.iDlab;
+    if (p.opacity == 2) {
+      ka = s.kf;
+    } else if (p.opacity == 1) {
+      const double Tl = T > p.Tmin ? T : p.Tmin, T2 = Tl * Tl;
+      ka = p.kabs0 * rho * rho * rsqrt64(T2 * T2 * T2 * Tl);
+    } else {
+      ka = p.kabs0 * rho;
+    }
+    ksca = s.ks * p.kes0 * rho;
+    kt = fma(s.ks, ka, ksca);
+    uru = fma(v[0], x[1], fma(v[1], x[2], fma(v[2], x[3], -gr * gm)));
+    e43 = (4.0 / 3.0) * E;
+    c1 = e43 * uru;
+    c2 = E * (1.0 / 3.0);
+    lam = s.ks * ka * p.a_rad * (T * T) * (T * T);
+    hA = -s.h * (kt * c1);
+    hC = -s.h * (fma(kt, c2, lam) + ksca * fma(c1, uru, -c2));
+  }
+  // gamma^{ij} w_j
+  __device__ __forceinline__ static void raise3(const Geo<MET, double>& g, const ImpPre<double>& c, const double w[3],
+                                                double o[3]) {
+    if constexpr (MET == MINK) {
+      for (int k = 0; k < 3; ++k) o[k] = w[k];
+    } else {
+      o[0] = fma(g.G13, w[2], c.c11 * w[0]);
+      o[1] = g.G22 * w[1];
+      o[2] = fma(g.G33, w[2], g.G13 * w[0]);
+    }
+  }
+
+  // Reverse sweep: gE the cotangents of the error rows, gp those of the final
+  // primitives -> gx of x, gU of U* (times sqrt(-g)), *gks of kappa_scale.
+  __device__ __forceinline__ void reverse(const DevParams& p, const ImpSys<MET>& s, const double x[4],
+                                          const double gE[4], const double gp[NPR], double gx[4], double gU[NPR],
+                                          double* gks) const {
+    const auto& g = s.g;
+    const auto& c = s.pre;
+    const double al = MET == MINK ? 1.0 : g.alpha, a01 = MET == MINK ? 0.0 : g.alpha * g.G01;
+    double gEf = 0.0, gfa = 0.0, gt[3] = {0.0, 0.0, 0.0};
+    if (!neg) {
+      gEf = gp[ER];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        gfa = fma(gp[UR1 + k], t[k], gfa);
+        gt[k] = gp[UR1 + k] * fa;
+      }
+    }
+    // E_k = dT_k - hG_k, hG = hA v + hC u
+    const double ghA = -fma(gE[0], v0, fma(gE[1], v[0], fma(gE[2], v[1], gE[3] * v[2])));
+    const double ghC = -fma(gE[0], l0, fma(gE[1], l[0], fma(gE[2], l[1], gE[3] * l[2])));
+    const double gv0 = -gE[0] * hA;
+    double gl0 = -gE[0] * hC, gv[3], gl[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      gv[k] = -gE[1 + k] * hA;
+      gl[k] = -gE[1 + k] * hC;
+    }
+    // four-force
+    const double hc = -s.h * ghC, ha = -s.h * ghA, T3 = T * T * T;
+    const double gc1 = fma(ha, kt, hc * ksca * uru), gkt = fma(ha, c1, hc * c2), gc2 = hc * (kt - ksca);
+    const double gka = fma(hc * p.a_rad, T3 * T, gkt), gks_ = fma(hc, fma(c1, uru, -c2), gkt);  // of ks ka, ks kes0 rho
+    double guru = fma(hc * ksca, c1, gc1 * e43);
+    double gT = 4.0 * hc * s.ks * ka * p.a_rad * T3;
+    *gks += fma(gka, ka, gks_ * p.kes0 * rho);
+    double grho = fma(gks_ * s.ks, p.kes0, gp[RHO]);
+    if (p.opacity == 1) {
+      grho = fma(2.0 * gka * s.ks, ka / rho, grho);
+      if (T > p.Tmin) gT = fma(-3.5 * gka * s.ks, ka / T, gT);
+    } else if (p.opacity == 0) {
+      grho = fma(gka * s.ks, p.kabs0, grho);
+    }
+    const double gpg = gT * u0 * s.iDlab;
+    double gu0 = gT * pg * s.iDlab, gD = -gT * pg * u0 * (s.iDlab * s.iDlab);
+    gEf += fma(gc1 * uru, 4.0 / 3.0, gc2 * (1.0 / 3.0));
+    // u_r.u = v_i u~^i - gamma_r gamma
+    double ggr = fma(-guru, gm, -al * gv0);
+    const double ggm = -guru * gr;
+    gv[0] = fma(c.b1, gv0, gv[0]);
+    double gR[4];
+    gR[0] = 0.0;
+    double gxu[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      gxu[k] = guru * v[k];
+      gv[k] = fma(guru, x[1 + k], gv[k]);
+      gfa = fma(gv[k], Rt[1 + k], gfa);
+      gR[1 + k] = gv[k] * fa;
+    }
+    // radiation frame
+    double gie = 1.5 * gfa * rr * al;
+    const double grr = fma(1.5 * gfa * ie, al, 0.5 * ggr * sp2), gpr = -0.5 * rr * rr * rr * grr;
+    const double gsp2 = fma(0.5 * ggr, rr, gpr * sm1), gsm1 = fma(gpr, sp2, gEf * Er);
+    double gEr = gEf * sm1, gU2;
+    if (lim) {
+      gEr = fma(-gie, ie * ie, gEr);
+      gU2 = 0.5 * gEr * ie / p.ymax_rad;
+    } else {
+      const double gy = -1.5 * (gsp2 + gsm1) * rcp(sq);
+      gU2 = gy * ie * ie;
+      gie = fma(2.0 * gy * U2, ie, gie);
+      gEr = fma(-gie, ie * ie, gEr);
+      gR[0] -= gEr;
+      gR[1] = fma(c.b1, gEr, gR[1]);
+    }
+    double rt[3];
+    raise3(g, c, gt, rt);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gR[1 + k] += fma(2.0 * gU2 * c.a2, t[k], rt[k]);
+    // R = R* - (T - T*): T's and the conserved inputs' cotangents
+    double gTc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      gTc[k] = gE[k] - gR[k];
+      gU[UU + k] = -gTc[k];
+      gU[ER + k] = gR[k];
+    }
+    double gZ = gTc[0] * l0, gbu = -gTc[0] * m0, gmv[3];
+    const double gm0 = -gTc[0] * bu;
+    gl0 = fma(gTc[0], Z, gl0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      gZ = fma(gTc[1 + k], l[k], gZ);
+      gbu = fma(-gTc[1 + k], m[k], gbu);
+      gl[k] = fma(gTc[1 + k], Z, gl[k]);
+      gmv[k] = -gTc[1 + k] * bu;
+    }
+    const double gwb = gZ * u0, gpt = gTc[0];
+    gu0 = fma(gZ, wb, fma(gTc[0], rho, gu0));
+    grho += fma(gTc[0], u0, gwb);
+    double gbt = -gZ * bu;
+    gbu = fma(-gZ, bt, gbu);
+    gbt = fma(gbu, iut, gbt);
+    double giut = fma(gbu, bt, grho * s.Dlab);
+    gD = fma(grho, iut, gD);
+    gx[0] = gp[UU] + fma(p.gam, gwb, p.gm1 * (gpt + gpg));
+    double P[NPR], gP[NPR];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      P[U1 + k] = x[1 + k];
+      P[B1 + k] = s.B[k];
+      gP[U1 + k] = gp[U1 + k] + gxu[k];
+      gP[B1 + k] = gp[B1 + k];
+    }
+    gas_frame_T<MET>(g, a01, c.b1, *this, P, fma(ggm, al, gu0), 0.0, gl0, gl, gm0, gmv, gbt, giut,
+                     fma(0.5, gpt, gwb), gP);
+    gU[RHO] = gD;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      gx[1 + k] = gP[U1 + k];
+      gU[B1 + k] = gP[B1 + k];
+    }
+  }
+};
+
+// One zone per thread: the floors' transpose (identity unless one acts), then
+// the implicit-function theorem with reverse sweeps of PmhdEval: four for the
+// rows of dE/dx, one for the primitives, one for the solved lambda.  Zones
+// solved by the entropy equation follow in ka_implicit_entropy.
+template <int MET>
+__global__ void __launch_bounds__(128) ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
+                                                   const double* __restrict__ K, const double* __restrict__ geo) {
+  const double Bc = s == 0 ? 1.0 : (s == 1 ? 0.25 : 2.0 / 3.0);
+  const double h = Bc * dt;
+  const double* Ust0 = a.Ust + (long long)s * 12 * bx.nact;
+  const unsigned char* meth = a.meth + (long long)s * bx.nact;
+  const double* Psol0 = a.Psol + (long long)s * 12 * bx.nact;
+  double gk = 0.0;
+  for (long long z = HR_TID; z < bx.nact; z += HR_STRIDE) {
+    double gq[NPR];
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) {
+      gq[q] = a.gN[q * bx.nact + z];
+      any = any || gq[q] != 0.0;
+      a.gU[q * bx.nact + z] = 0.0;
+    }
+    a.gS[z] = 0.0;
+    const int m = meth[z];
+    if (!any || m == METH_ENTROPY) continue;
+    int i, j, k;
+    zone_ijk(bx, z, i, j, k);
+    const long long t = cell_index(bx, i, j, k);
+    Geo<MET, double> g;
+    double igd = 1.0, fl[2] = {p.rf0, p.uf0};
+    const double sgk[3] = {1.0, 1.0, 1.0};  // the error's norms are not read here
+    if constexpr (MET == KS) {
+      const GeoTab T = geotab(geo, bx);
+      const long long x = gidx_c(bx, i, j);
+      g = geo_load<MET>(T.C, T.sC, x);
+      igd = __ldg(T.C + 16 * T.sC + x);
+      fl[0] = __ldg(T.C + 23 * T.sC + x);
+      fl[1] = __ldg(T.C + 24 * T.sC + x);
+    } else {
+      g = make_geo<MET, double>(p, 0.0, 0.0);
+    }
+    if (m == ST_BACKUP) {  // only B = U*[B] / sqrt(-g) is the zone's own
+      for (int c = 0; c < 3; ++c) a.gU[(B1 + c) * bx.nact + z] = gq[B1 + c] * igd;
+      continue;
+    }
+    double Us[NPR], Ps[NPR];
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) {
+      Us[q] = Ust0[q * bx.nact + z];
+      Ps[q] = Psol0[q * bx.nact + z];
+    }
+    {  // floors: gq <- (d floors / d P)^T gq at the solution
+      double Pf[NPR];
+      bool acts = false;
+      for (int q = 0; q < NPR; ++q) Pf[q] = Ps[q];
+      apply_floors<MET>(p, g, fl[0], fl[1], Pf);
+#pragma unroll
+      for (int q = 0; q < NPR; ++q) acts = acts || Pf[q] != Ps[q];
+      if (acts) {
+        typedef Dn<4> D4;
+        const Geo<MET, D4> g4 = geo_cast<D4>(g);
+        double gs[NPR];
+#pragma unroll 1
+        for (int ch = 0; ch < 3; ++ch) {
+          D4 PD[NPR];
+          for (int q = 0; q < NPR; ++q) PD[q] = D4::seed(Ps[q], q - 4 * ch);
+          apply_floors<MET, D4>(p, g4, fl[0], fl[1], PD);
+          for (int c = 0; c < 4; ++c) {
+            double v = 0.0;
+            for (int q = 0; q < NPR; ++q) v += gq[q] * PD[q].d[c];
+            gs[4 * ch + c] = v;
+          }
+        }
+        for (int q = 0; q < NPR; ++q) gq[q] = gs[q];
+      }
+    }
+    ImpSys<MET> sys;
+    build_sys_with<MET, double>(p, g, igd, sgk, Us, h, kfield(p, K, t), sys);
+    const double x[4] = {Ps[UU], Ps[U1], Ps[U2], Ps[U3]};
+    const PmhdEval<MET> ev(p, sys, x);
+    double J[4][4], lam[4], gx[4], gU[NPR], sum[NPR], ks = 0.0;
+    bool ok = true;
+#pragma unroll 1
+    for (int it = 0; it < 6; ++it) {
+      double gE[4], gp[NPR];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) gE[c] = it < 4 ? (c == it ? 1.0 : 0.0) : (it == 4 ? 0.0 : -lam[c]);
+#pragma unroll
+      for (int q = 0; q < NPR; ++q) gp[q] = it == 4 ? gq[q] : 0.0;
+      ks = 0.0;
+      ev.reverse(p, sys, x, gE, gp, gx, gU, &ks);
+      if (it < 4) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (r == it)
+            for (int c = 0; c < 4; ++c) J[c][r] = gx[c];  // transposed
+      } else if (it == 4) {
+        for (int q = 0; q < NPR; ++q) sum[q] = gU[q];
+        ok = solve4(J, gx, lam);
+        if (!ok) break;
+      }
+    }
+    if (!ok) continue;
+    gk += ks;
+#pragma unroll
+    for (int q = 0; q < NPR; ++q) a.gU[q * bx.nact + z] = (sum[q] + gU[q]) * igd;
+  }
+  warp_atomic_add(a.gk, gk);
+}
+
+// The zones solved by the entropy equation (by the entropy PMHD, URAD or PRAD,
+// which solve the same equations; few in any step), on dual numbers: the same
+// transposed solve on the entropy system (Eq. source6), which also depends on
+// S*.
+template <int MET>
+__global__ void ka_implicit_entropy(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
+                                    const double* __restrict__ K) {
   const double Bc = s == 0 ? 1.0 : (s == 1 ? 0.25 : 2.0 / 3.0);
   const double h = Bc * dt;
   const double* Ust0 = a.Ust + (long long)s * 12 * bx.nact;
@@ -312,14 +633,13 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
   typedef Dn<1> D1;
   double gk = 0.0;
   for (long long z = HR_TID; z < bx.nact; z += HR_STRIDE) {
+    if (meth[z] != METH_ENTROPY) continue;
     double gq[NPR];
     bool any = false;
     for (int q = 0; q < NPR; ++q) {
       gq[q] = a.gN[q * bx.nact + z];
       any = any || gq[q] != 0.0;
-      a.gU[q * bx.nact + z] = 0.0;
     }
-    a.gS[z] = 0.0;
     if (!any) continue;
     int i, j, k;
     zone_ijk(bx, z, i, j, k);
@@ -327,23 +647,13 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
     const double x1 = xcen(bx, 0, i), x2 = xcen(bx, 1, j);
     const Geo<MET, double> g = make_geo<MET, double>(p, x1, x2);
     const double igd = 1.0 / g.gdet;
-    const int m = meth[z];
     double Us[NPR], Ps[NPR];
     for (int q = 0; q < NPR; ++q) {
       Us[q] = Ust0[q * bx.nact + z];
       Ps[q] = Psol0[q * bx.nact + z];
     }
-    (void)Pnext;
     const double kz = kfield(p, K, t);
-    if (m == 2) {  // back-up: only B = U*[B] / sqrt(-g) is the zone's own
-      for (int c = 0; c < 3; ++c) a.gU[(B1 + c) * bx.nact + z] = gq[B1 + c] * igd;
-      continue;
-    }
-    // a zone solved by the entropy equation (by the entropy PMHD, URAD or
-    // PRAD, which solve the same equations): the same transposed solve on the
-    // entropy system (Eq. source6), which also depends on S*
-    const bool ent = m == METH_ENTROPY;
-    const double Sz = ent ? a.Sst[(long long)s * bx.nact + z] : 0.0;
+    const double Sz = a.Sst[(long long)s * bx.nact + z];
     const Geo<MET, D4> g4 = geo_cast<D4>(g);
     {  // floors: gq <- (d floors / d P)^T gq at the solution
       double fl[2];
@@ -369,7 +679,7 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
       for (int q = 0; q < NPR; ++q) UsD[q] = D4(Us[q]);
       ImpSysT<MET, D4> sys;
       build_sys<MET, D4>(p, g4, UsD, h, D4(kz), sys);
-      sys.entropy = ent;
+      sys.entropy = true;
       sys.Sstar = D4(Sz * igd);
       pmhd_final<MET, D4>(p, sys, xs, PsD, Eg);
       for (int r = 0; r < 4; ++r)
@@ -386,7 +696,7 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
       for (int q = 0; q < NPR; ++q) UsD[q] = D4::seed(Us[q], q - 4 * ch);
       ImpSysT<MET, D4> sys;
       build_sys<MET, D4>(p, g4, UsD, h, D4(kz), sys);
-      sys.entropy = ent;
+      sys.entropy = true;
       sys.Sstar = D4(Sz * igd);
       pmhd_final<MET, D4>(p, sys, xs, PsD, Eg);
       for (int c = 0; c < 4; ++c) {
@@ -404,7 +714,7 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
       ImpSysT<MET, D1> sys;
       build_sys<MET, D1>(p, g1, UsD, h, D1(kz), sys);
       sys.ks = D1::seed(p.kscale, 0);
-      sys.entropy = ent;
+      sys.entropy = true;
       sys.Sstar = D1(Sz * igd);
       pmhd_final<MET, D1>(p, sys, xs, PsD, Eg);
       for (int r = 0; r < 4; ++r) gk -= lam[r] * Eg[r].d[0];
@@ -412,7 +722,7 @@ __global__ void ka_implicit(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
     for (int q = 0; q < NPR; ++q) a.gU[q * bx.nact + z] = gU[q];
     // S* enters the entropy row only, E_0 = T (S u^t(x) - S*/sqrt(-g)) +
     // h G_mu u^mu with T = p/rho0 at the solution (the factor F_13)
-    if (ent) a.gS[z] = lam[0] * ((p.gam - 1.0) * Ps[UU] / Ps[RHO]) * igd;
+    a.gS[z] = lam[0] * ((p.gam - 1.0) * Ps[UU] / Ps[RHO]) * igd;
   }
   warp_atomic_add(a.gk, gk);
 }

@@ -70,10 +70,10 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
   double* aux = (double*)c->aux;
   double* Pg = c->P;
   for (int s = 2; s >= 0; --s) {
-    const double* Pnext = a.Pst + (size_t)(s + 1) * 12 * nt;
     const double* Ps = a.Pst + (size_t)s * 12 * nt;
     ka_backup_T<<<G(na), 128, 0, st>>>(bx, a.meth + (size_t)s * na, a.gN);
-    ka_implicit<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, K, Pnext);
+    ka_implicit<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, K, c->geotab);
+    ka_implicit_entropy<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, K);
     // forward state of the sub-step: P_s with ghosts, cell factors
     HR_ACHECK(cudaMemcpyAsync(Pg, Ps, pbytes, cudaMemcpyDeviceToDevice, st));
     for (int d = 0; d < 3; ++d) {
