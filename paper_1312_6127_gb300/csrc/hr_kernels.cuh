@@ -110,7 +110,7 @@ __device__ __forceinline__ double kfield(const DevParams& p, const double* K, lo
 // which matters because the step is bound by FP64 arithmetic.
 // Layout of a grid's table (offset BoxGeo::goff, in doubles): [GEO_C][N2][N1]
 // centres, [16][N2][N1] centre derivatives, [GEO_F][N2][n1+1] x1 faces,
-// [GEO_F][n2+1][N1] x2 faces; fields in the order of Geo (g00 g01 g03 g11 g13
+// [GEO_F][n2+1][N1] x2 faces, sqrt(-g) on the x1-x2 edges [n2+1][n1+1]; fields in the order of Geo (g00 g01 g03 g11 g13
 // g22 g33 G00 G01 G11 G13 G22 G33 gdet alpha ialpha) and of MetricDeriv.
 // Centres add 1/sqrt(-g) (plane 16), sqrt(g_dd) of the three directions
 // (17..19), sqrt(gamma^{kk}) of the ZAMO slice (20..22), the density and
@@ -126,12 +126,14 @@ struct GeoTab {
   const double* M;
   const double* F0;
   const double* F1;
+  const double* E;         // [n2+1][n1+1]
   long long sC, sF0, sF1;  // plane sizes
 };
 
 __host__ __device__ __forceinline__ long long geotab_size(const BoxGeo& b) {
   const long long sC = (long long)b.N[0] * b.N[1];
-  return (GEO_C + 16) * sC + GEO_F * ((long long)(b.n[0] + 1) * b.N[1] + (long long)b.N[0] * (b.n[1] + 1));
+  return (GEO_C + 16) * sC + GEO_F * ((long long)(b.n[0] + 1) * b.N[1] + (long long)b.N[0] * (b.n[1] + 1)) +
+         (long long)(b.n[0] + 1) * (b.n[1] + 1);
 }
 
 __device__ __forceinline__ GeoTab geotab(const double* base, const BoxGeo& b) {
@@ -143,6 +145,7 @@ __device__ __forceinline__ GeoTab geotab(const double* base, const BoxGeo& b) {
   t.M = t.C + GEO_C * t.sC;
   t.F0 = t.M + 16 * t.sC;
   t.F1 = t.F0 + GEO_F * t.sF0;
+  t.E = t.F1 + GEO_F * t.sF1;
   return t;
 }
 
@@ -1664,7 +1667,8 @@ static __global__ void k_geo_init(DevParams p, const BoxGeo* __restrict__ boxes,
     double* M = const_cast<double*>(T.M);
     double* F0 = const_cast<double*>(T.F0);
     double* F1 = const_cast<double*>(T.F1);
-    const long long total = 2 * T.sC + T.sF0 + T.sF1;
+    double* Ed = const_cast<double*>(T.E);
+    const long long total = T.sC + T.sF0 + T.sF1 + (long long)(bx.n[0] + 1) * (bx.n[1] + 1);
     for (long long id = HR_TID; id < total; id += HR_STRIDE) {
       if (id < T.sC) {  // centres and their derivatives
         const int i = (int)(id % bx.N[0]) - bx.ng[0], j = (int)(id / bx.N[0]) - bx.ng[1];
@@ -1705,6 +1709,10 @@ static __global__ void k_geo_init(DevParams p, const BoxGeo* __restrict__ boxes,
         geo_store<KS>(F1, T.sF1, e, g);
         F1[16 * T.sF1 + e] = 1.0 / g.gdet;
         F1[17 * T.sF1 + e] = sqrt(g.g22);
+      } else {  // x1-x2 edges
+        const long long e = id - T.sC - T.sF0 - T.sF1;
+        const int i = (int)(e % (bx.n[0] + 1)), j = (int)(e / (bx.n[0] + 1));
+        Ed[e] = make_geo<KS, double>(p, bx.x0[0] + i * bx.dx[0], bx.x0[1] + j * bx.dx[1]).gdet;
       }
     }
   }

@@ -253,7 +253,10 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     nk += 2;
   }
   if (p.emf == 1) {  // staggered field: the 4-state upwind EMFs on the edges
-    k_vel<MET, R><<<grid_for(c->ncell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, (R*)c->vel, c->geotab);
+    if constexpr (std::is_same<R, double>::value)
+      k_vel64<MET><<<grid_for(c->ncell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, (double*)c->vel, c->geotab);
+    else
+      k_vel<MET, R><<<grid_for(c->ncell, c->sms, 256), 256, 0, st>>>(p, bt, nb, c->P, (R*)c->vel, c->geotab);
     mark(c, HARMRAD_K_CT);
     ++nk;
     for (int a = 0; a < 3; ++a)

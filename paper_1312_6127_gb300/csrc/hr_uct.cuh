@@ -38,16 +38,17 @@ __device__ __forceinline__ double gdet_at(const DevParams& p, double x1, double 
 
 // sqrt(-g) at a cell position (q0, q1) of the grid (ghosts included) whose
 // x1 (f0) and/or x2 (f1) coordinate sits on the cell's lower face: from the
-// Kerr-Schild metric tables (centres, x1 faces, x2 faces) where the context
-// has them, else from the closed form.
+// Kerr-Schild metric tables (centres, x1 faces, x2 faces, x1-x2 edges) where the
+// context has them, else from the closed form.
 template <int MET>
 __device__ __forceinline__ double gdet_pos(const DevParams& p, const double* geo, const BoxGeo& bx, bool f0, bool f1,
                                            int q0, int q1) {
   f0 = f0 && bx.n[0] > 1;
   f1 = f1 && bx.n[1] > 1;
   if constexpr (MET == KS) {
-    if (geo && bx.goff >= 0 && !(f0 && f1)) {
+    if (geo && bx.goff >= 0) {
       const GeoTab T = geotab(geo, bx);
+      if (f0 && f1) return __ldg(T.E + (long long)q1 * (bx.n[0] + 1) + q0);
       if (f0) return __ldg(T.F0 + 13 * T.sF0 + gidx_f0(bx, q0, q1));
       if (f1) return __ldg(T.F1 + 13 * T.sF1 + gidx_f1(bx, q0, q1));
       return __ldg(T.C + 13 * T.sC + gidx_c(bx, q0, q1));
@@ -56,6 +57,19 @@ __device__ __forceinline__ double gdet_pos(const DevParams& p, const double* geo
   const double x1 = f0 ? bx.x0[0] + q0 * bx.dx[0] : xcen(bx, 0, q0);
   const double x2 = f1 ? bx.x0[1] + q1 * bx.dx[1] : xcen(bx, 1, q1);
   return gdet_at<MET>(p, x1, x2);
+}
+
+// 1/sqrt(-g) on the d-faces (tables), at the cell position (q0, q1).
+template <int MET>
+__device__ __forceinline__ double igdet_face(const double* geo, const BoxGeo& bx, int d, int q0, int q1) {
+  if constexpr (MET == KS) {
+    const GeoTab T = geotab(geo, bx);
+    if (d == 0 && bx.n[0] > 1) return __ldg(T.F0 + 16 * T.sF0 + gidx_f0(bx, q0, q1));
+    if (d == 1 && bx.n[1] > 1) return __ldg(T.F1 + 16 * T.sF1 + gidx_f1(bx, q0, q1));
+    return __ldg(T.C + 16 * T.sC + gidx_c(bx, q0, q1));
+  } else {
+    return 1.0;
+  }
 }
 
 __device__ __forceinline__ bool periodic_dir(const BoxGeo& bx, int d) {
@@ -174,7 +188,39 @@ __global__ void k_centre_B(DevParams p, const BoxGeo* __restrict__ boxes, int nb
   }
 }
 
-// Lab-frame 3-velocity v^i = u^i / u^t of every cell, ghosts included.
+// Lab-frame 3-velocity v^i = u^i / u^t of every cell, ghosts included, in FP64
+// by u^i alpha / gamma.
+template <int MET>
+__global__ void k_vel64(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const double* __restrict__ P0,
+                        double* __restrict__ V0, const double* __restrict__ geo) {
+  for (int bi = 0; bi < nbox; ++bi) {
+    const BoxGeo& bx = boxes[bi];
+    const double* P = P0 + 12 * bx.coff;
+    double* V = V0 + 3 * bx.coff;
+    for (long long t = first_item(bx.coff); t < bx.ntot; t += HR_STRIDE) {
+      Geo<MET, double> g;
+      double al = 1.0, a01 = 0.0, l[3], ig;
+      if constexpr (MET == KS) {
+        const GeoTab T = geotab(geo, bx);
+        const long long x = (unsigned)t % (unsigned)T.sC, s = T.sC;
+        g.g11 = __ldg(T.C + 3 * s + x);
+        g.g13 = __ldg(T.C + 4 * s + x);
+        g.g22 = __ldg(T.C + 5 * s + x);
+        g.g33 = __ldg(T.C + 6 * s + x);
+        al = __ldg(T.C + 14 * s + x);
+        a01 = al * __ldg(T.C + 8 * s + x);
+      }
+      const double u1 = P[U1 * bx.ntot + t], u2 = P[U2 * bx.ntot + t], u3 = P[U3 * bx.ntot + t];
+      lower3<MET>(g, u1, u2, u3, l);
+      const double gm = sqrt_rsqrt(fma(u1, l[0], fma(u2, l[1], fma(u3, l[2], 1.0))), &ig), iut = al * ig;
+      V[t] = fma(-gm, a01, u1) * iut;
+      V[bx.ntot + t] = u2 * iut;
+      V[2 * bx.ntot + t] = u3 * iut;
+    }
+  }
+}
+
+// The same for split precision.
 template <int MET, typename R>
 __global__ void k_vel(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const double* __restrict__ P0,
                       R* __restrict__ V0, const double* __restrict__ geo) {
@@ -251,15 +297,15 @@ __global__ void k_uct_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
       auto Bat = [&](const double* Fd, int d, int m, int o) {
         int q[3] = {ii[0], ii[1], ii[2]};
         q[m] += o;
-        return Fd[t + o * bx.str[m]] / gdet_pos<MET>(p, geo, bx, d == 0, d == 1, q[0], q[1]);
+        return Fd[t + o * bx.str[m]] * igdet_face<MET>(geo, bx, d, q[0], q[1]);
       };
       double Bb[2], Ba[2];
       {
         const double b0 = Bat(Fb, b, a, 0);
         if (aa) {
           const double bmm = Bat(Fb, b, a, -2), bm = Bat(Fb, b, a, -1), bp = Bat(Fb, b, a, 1);
-          Bb[0] = bm + 0.5 * mc_slope<double>(bmm, bm, b0);
-          Bb[1] = b0 - 0.5 * mc_slope<double>(bm, b0, bp);
+          Bb[0] = fma(0.25, mc_twice(bm - bmm, b0 - bm), bm);
+          Bb[1] = fma(-0.25, mc_twice(b0 - bm, bp - b0), b0);
         } else {
           Bb[0] = Bb[1] = b0;
         }
@@ -268,8 +314,8 @@ __global__ void k_uct_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
         const double b0 = Bat(Fa, a, b, 0);
         if (ab) {
           const double bmm = Bat(Fa, a, b, -2), bm = Bat(Fa, a, b, -1), bp = Bat(Fa, a, b, 1);
-          Ba[0] = bm + 0.5 * mc_slope<double>(bmm, bm, b0);
-          Ba[1] = b0 - 0.5 * mc_slope<double>(bm, b0, bp);
+          Ba[0] = fma(0.25, mc_twice(bm - bmm, b0 - bm), bm);
+          Ba[1] = fma(-0.25, mc_twice(b0 - bm, bp - b0), b0);
         } else {
           Ba[0] = Ba[1] = b0;
         }
@@ -286,8 +332,14 @@ __global__ void k_uct_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
           for (int m = 0; m < 2; ++m) {
             const R* Vm = V + (m == 0 ? a : b) * bx.ntot;
             double val = double(Vm[tc]);
-            if (aa) val += (s1 == 0 ? 0.5 : -0.5) * double(mc_slope<R>(Vm[tc - sa], Vm[tc], Vm[tc + sa]));
-            if (ab) val += (s2 == 0 ? 0.5 : -0.5) * double(mc_slope<R>(Vm[tc - sb], Vm[tc], Vm[tc + sb]));
+            if constexpr (std::is_same<R, double>::value) {
+              const double c = val;
+              if (aa) val = fma(s1 == 0 ? 0.25 : -0.25, mc_twice(c - Vm[tc - sa], Vm[tc + sa] - c), val);
+              if (ab) val = fma(s2 == 0 ? 0.25 : -0.25, mc_twice(c - Vm[tc - sb], Vm[tc + sb] - c), val);
+            } else {
+              if (aa) val += (s1 == 0 ? 0.5 : -0.5) * double(mc_slope<R>(Vm[tc - sa], Vm[tc], Vm[tc + sa]));
+              if (ab) val += (s2 == 0 ? 0.5 : -0.5) * double(mc_slope<R>(Vm[tc - sb], Vm[tc], Vm[tc + sb]));
+            }
             v[m] = val;
           }
           es[s1][s2] = ge * (Bb[s1] * v[0] - Ba[s2] * v[1]);
@@ -317,13 +369,13 @@ __global__ void k_uct_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
       }
       double Wa = wa[0] + wa[1], Wb = wb[0] + wb[1], da = 0.0, db = 0.0;
       if (Wa > 0.0) {
-        da = wa[0] * wa[1] / Wa;
+        da = wa[0] * wa[1] * rcp(Wa);
       } else {
         wa[0] = wa[1] = 1.0;
         Wa = 1.0;
       }
       if (Wb > 0.0) {
-        db = wb[0] * wb[1] / Wb;
+        db = wb[0] * wb[1] * rcp(Wb);
       } else {
         wb[0] = wb[1] = 1.0;
         Wb = 1.0;
@@ -333,7 +385,7 @@ __global__ void k_uct_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
       for (int s1 = 0; s1 < 2; ++s1)
 #pragma unroll
         for (int s2 = 0; s2 < 2; ++s2) sum += wa[s1] * wb[s2] * es[s1][s2];
-      emf[t] = R(sum / (Wa * Wb) - da * ge * (Bb[1] - Bb[0]) + db * ge * (Ba[1] - Ba[0]));
+      emf[t] = R(sum * rcp(Wa * Wb) - da * ge * (Bb[1] - Bb[0]) + db * ge * (Ba[1] - Ba[0]));
     }
   }
 }
