@@ -76,13 +76,7 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
     ka_implicit_entropy<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, K);
     // forward state of the sub-step: P_s with ghosts, cell factors
     HR_ACHECK(cudaMemcpyAsync(Pg, Ps, pbytes, cudaMemcpyDeviceToDevice, st));
-    for (int d = 0; d < 3; ++d) {
-      if (!p.act[d]) continue;
-      long long work = 2LL * bx.ng[d];
-      for (int e = 0; e < 3; ++e)
-        if (e != d) work *= (e < d) ? bx.N[e] : bx.n[e];
-      k_bc_fill<<<G(work), 128, 0, st>>>(p, c->dboxes, 1, Pg, p.opacity == 2 ? c->K : nullptr, d);
-    }
+    fill_ghost_cells(c, Pg);
     k_prep64<MET><<<G(nt), 128, 0, st>>>(p, c->dboxes, 1, Pg, c->K, aux, c->geotab);
     HR_ACHECK(cudaMemsetAsync(a.gP, 0, pbytes, st));
     ka_update<MET><<<G(na), 128, 0, st>>>(p, bx, a, s, dt, Ps, c->geotab);

@@ -211,41 +211,52 @@ __device__ __forceinline__ Geo<MET, R> geo_centre(const DevParams& p, const BoxG
 // enters from the ghost; polar mirrors across the axis from the zone half a
 // turn away in phi, negating the theta components.  The opacity field, when
 // present, is copied like a scalar primitive.
-static __global__ void k_bc_fill(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                 double* __restrict__ P0, double* __restrict__ K0, int d) {
+// NQ variables per thread, blockIdx.y the first of them.  The fill moves little:
+// its time is the latency of a thread's chain, so one grid takes a thread per
+// value (NQ = 1: 64x32x16 0.113 -> 0.063 ms per RK3 step), and a batch, whose
+// threads pass over all its boxes, one per cell (12 boxes: 0.43 ms, 0.93 with
+// NQ = 1).
+template <int d, int NQ>
+__global__ void k_bc_fill(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, double* __restrict__ P0,
+                          double* __restrict__ K0) {
+  const int q0 = NQ == 1 ? blockIdx.y : 0;
   long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     double* P = P0 + 12 * bx.coff;
-    double* K = K0 ? K0 + bx.coff : nullptr;
-    int lo[3], len[3];
-    for (int e = 0; e < 3; ++e) {
-      if (e == d) {
-        lo[e] = 0;
-        len[e] = bx.ng[d];
-      } else if (e < d) {
-        lo[e] = -bx.ng[e];
-        len[e] = bx.n[e] + 2 * bx.ng[e];
-      } else {
-        lo[e] = 0;
-        len[e] = bx.n[e];
-      }
-    }
-    long long total = 2LL * len[0] * len[1] * len[2];
+    double* K = K0 && q0 == 0 ? K0 + bx.coff : nullptr;
+    // directions before d include their ghosts, those after it do not
+    constexpr int e0 = d == 0 ? 1 : 0, e1 = d == 2 ? 1 : 2;
+    const int g0 = e0 < d ? bx.ng[e0] : 0, g1 = e1 < d ? bx.ng[e1] : 0;
+    const int l0 = bx.n[e0] + 2 * g0, l1 = bx.n[e1] + 2 * g1, ng = bx.ng[d];
+    const long long total = 2LL * ng * l0 * l1;
     for (long long id = first_item(done); id < total; id += HR_STRIDE) {
-      long long r = id;
-      int a0 = (int)(r % len[0]);
-      r /= len[0];
-      int a1 = (int)(r % len[1]);
-      r /= len[1];
-      int a2 = (int)(r % len[2]);
-      int side = (int)(r / len[2]);
-      int c[3] = {a0 + lo[0], a1 + lo[1], a2 + lo[2]};
-      int g = c[d];
-      int dst[3] = {c[0], c[1], c[2]}, src[3] = {c[0], c[1], c[2]};
-      int bc = bx.bc[2 * d + side];
+      // x1 fastest: for d = 0 the ghost index, else e0 = x1
+      unsigned r = (unsigned)id;
+      int c[3], g, side;
+      if (d == 0) {
+        g = r % ng;
+        r /= ng;
+        c[e0] = r % l0;
+        r /= l0;
+        c[e1] = r % l1;
+        side = r / l1;
+      } else {
+        c[e0] = r % l0;
+        r /= l0;
+        g = r % ng;
+        r /= ng;
+        c[e1] = r % l1;
+        side = r / l1;
+      }
+      c[e0] -= g0;
+      c[e1] -= g1;
+      const int bc = bx.bc[2 * d + side];
       if (bc == 4) continue;  // fixed ghosts keep the values they were given
-      dst[d] = side == 0 ? -1 - g : bx.n[d] + g;
+      int src[3];
+      src[e0] = c[e0];
+      src[e1] = c[e1];
+      c[d] = side == 0 ? -1 - g : bx.n[d] + g;
       double sgn = 1.0;
       int clamp = 0;
       if (bc == 0) {
@@ -255,16 +266,18 @@ static __global__ void k_bc_fill(DevParams p, const BoxGeo* __restrict__ boxes, 
         clamp = bc == 3 ? 0 : (side == 0 ? -1 : 1);
       } else {
         src[d] = side == 0 ? g : bx.n[d] - 1 - g;
-        if (bx.n[2] > 1) src[2] = (c[2] + bx.n[2] / 2) % bx.n[2];
+        if (bx.n[2] > 1) src[2] = ((d == 2 ? g : c[2]) + bx.n[2] / 2) % bx.n[2];
         sgn = -1.0;
       }
-      long long s = cell_index(bx, src[0], src[1], src[2]);
-      long long t = cell_index(bx, dst[0], dst[1], dst[2]);
+      const long long s = cell_index(bx, src[0], src[1], src[2]);
+      const long long t = cell_index(bx, c[0], c[1], c[2]);
 #pragma unroll
-      for (int q = 0; q < NPR; ++q) {
+      for (int e = 0; e < NQ; ++e) {
+        const int q = q0 + e;
+        const bool normal = q == U1 + d || q == UR1 + d;
         double v = P[q * bx.ntot + s];
-        if (q == U1 + d || q == B1 + d || q == UR1 + d) v *= sgn;
-        if (clamp != 0 && (q == U1 + d || q == UR1 + d)) {
+        if (normal || q == B1 + d) v *= sgn;
+        if (clamp != 0 && normal) {
           const double vc = clamp < 0 ? fmin(v, 0.0) : fmax(v, 0.0);
           if (p.sig) sig_put(p, bx.coff + t, 50 + d, (unsigned long long)q << 8 | (vc != v ? 1u : 0u));
           v = vc;

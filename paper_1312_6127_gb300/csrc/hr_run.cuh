@@ -89,19 +89,25 @@ int face_ghosts(harmrad_ctx* c) {
 }
 
 // Ghost fill of P in every active direction.
-inline int fill_ghost_cells(harmrad_ctx* c) {
+inline int fill_ghost_cells(harmrad_ctx* c, double* P = nullptr) {
   const DevParams& p = c->dp;
   double* K = p.opacity == 2 ? c->K : nullptr;
+  if (!P) P = c->P;
   int nk = 0;
   for (int d = 0; d < 3; ++d) {
     if (!p.act[d]) continue;
-    long long work = all_work(c, [d](const BoxGeo& b) {
+    const long long work = all_work(c, [d](const BoxGeo& b) {
       long long w = 2LL * b.ng[d];
       for (int e = 0; e < 3; ++e)
         if (e != d) w *= (e < d) ? b.N[e] : b.n[e];
       return w;
     });
-    k_bc_fill<<<grid_for(work, c->sms, 256), 256, 0, c->stream>>>(p, c->dboxes, c->nbox, c->P, K, d);
+    const bool one = c->nbox == 1;
+    const dim3 g(grid_for(work, c->sms, 128), one ? NPR : 1);
+    auto run = [&](auto kernel) { kernel<<<g, 128, 0, c->stream>>>(p, c->dboxes, c->nbox, P, K); };
+    if (d == 0) one ? run(k_bc_fill<0, 1>) : run(k_bc_fill<0, NPR>);
+    if (d == 1) one ? run(k_bc_fill<1, 1>) : run(k_bc_fill<1, NPR>);
+    if (d == 2) one ? run(k_bc_fill<2, 1>) : run(k_bc_fill<2, NPR>);
     mark(c, HARMRAD_K_BC);
     ++nk;
   }
