@@ -117,12 +117,14 @@ int Run<MET>::adjoint(harmrad_ctx* c, const double* gPout, double* gPin, double*
       }
       const double* chi_s = a.chi + ((size_t)s * 3 + d) * 2 * nt;
       const double* chi_prev = s > 0 ? a.chi + ((size_t)(s - 1) * 3 + d) * 2 * nt : nullptr;
-      const EdgeSet E{(double*)c->edges, c->ES[d]};
+      const EdgeSet E{(double*)c->edges[d], c->ES[d]};
       double* carry = a.carry + (size_t)d * 2 * nt;
       HR_ACHECK(cudaMemsetAsync(a.gE, 0, 24 * (size_t)nt * sizeof(double), st));
       HR_ACHECK(cudaMemsetAsync(a.gaux, 0, 3 * (size_t)nt * sizeof(double), st));
       const double* flat = p.recon == 0 ? chi_s : aux;  // not read for MC
-      recon<MET>(c, d, Pg, aux, flat, 256, 16);
+      FlatSet fls{};
+      fls.f[d] = const_cast<double*>(flat);
+      recon<MET>(c, d, 1, Pg, aux, fls, 128, 64);
       if (d == 0) {
         ka_face<MET, 0><<<G(wf), 128, 0, st>>>(p, bx, E, K, a.gF[0], a.gE, a.gk, a.gFS[0], c->geotab);
         ka_edges<MET, 0><<<G(wc), 128, 0, st>>>(p, bx, Pg, aux, flat, a.gE, a.gP, a.gchi);

@@ -324,6 +324,9 @@ int launch_step(harmrad_ctx* c, bool with_cfl) {
   return HARMRAD_OK;
 }
 
+// No more zones than one wave of the heavy kernels (2 blocks of 128 threads per SM).
+bool small_grid(long long nact, int sms) { return nact <= 256LL * sms; }
+
 // Default launch shapes.  The heavy kernels hold 2 blocks of 128 threads per SM
 // (200 registers and more): a grid that does not fill one such wave takes blocks
 // of one or two warps, which spread over all SMs and schedulers (64x32x16 torus,
@@ -335,7 +338,7 @@ int launch_step(harmrad_ctx* c, bool with_cfl) {
 harmrad_tuning default_tuning(long long nact, int sms) {
   harmrad_tuning t;
   memset(&t, 0, sizeof(t));
-  const bool small = nact <= 256LL * sms;
+  const bool small = small_grid(nact, sms);
   t.face_block = small ? 32 : 128;
   t.face_blocks_per_sm = 64;
   t.update_block = small ? 32 : 128;
@@ -378,7 +381,8 @@ void free_adjoint(harmrad_ctx* c) {
 void free_all(harmrad_ctx* c) {
   free_adjoint(c);
   void* ptrs[] = {c->P, c->K, c->geotab, c->Un, c->F[0], c->F[1], c->F[2], c->spd[0], c->spd[1], c->spd[2],
-                  c->aux, c->flat[0], c->flat[1], c->flat[2], c->emf, c->edges, c->dt, c->status,
+                  c->aux, c->flat[0], c->flat[1], c->flat[2], c->emf, c->edges[0], c->merged ? c->edges[1] : nullptr,
+                  c->merged ? c->edges[2] : nullptr, c->dt, c->status,
                   c->iters, c->failed, c->qcount, c->czone, c->cbox, c->cdata, c->qzone, c->qbox, c->qdata, c->fzone, c->fbox,
                   c->ftmp, c->stats, c->dtmin, c->stage_buf, c->flag, c->dboxes, c->imex_ust, c->imex_psol,
                   c->imex_M, c->sig, c->Sn, c->FS[0], c->FS[1], c->FS[2], c->ES[0], c->ES[1], c->ES[2], c->Bf[0], c->Bf[1], c->Bf[2],
@@ -479,8 +483,10 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     rc = rc ? rc : dalloc(&c->spd[d], fn * rs);
     rc = rc ? rc : dalloc(&c->flat[d], 2 * fn * rs);
   }
+  const size_t eb = (f64 ? 20 : 24) * nt * rs;
+  rc = rc ? rc : dalloc(&c->edges[0], eb);
   rc = rc ? rc : dalloc(&c->aux, 10 * nt * rs);
-  rc = rc ? rc : dalloc(&c->emf, nt * rs);
+  rc = rc ? rc : dalloc(&c->emf, 3 * nt * rs);
   if (dp.emf == 1) {  // staggered field
     for (int d = 0; d < 3; ++d) {
       rc = rc ? rc : dalloc(&c->Bf[d], nt * sizeof(double));
@@ -490,7 +496,6 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     }
     rc = rc ? rc : dalloc(&c->vel, 3 * nt * rs);
   }
-  rc = rc ? rc : dalloc(&c->edges, (f64 ? 20 : 24) * nt * rs);
   rc = rc ? rc : dalloc(&c->dt, count * sizeof(double));
   rc = rc ? rc : dalloc(&c->status, na);
   rc = rc ? rc : dalloc(&c->iters, na * sizeof(int));
@@ -514,6 +519,18 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     rc = rc ? rc : dalloc(&c->imex_M, 16 * na * sizeof(double));
   }
   rc = rc ? rc : dalloc(&c->flag, sizeof(int));
+  // FP64 grids that do not fill one wave (default_tuning) run all directions of the
+  // reconstruction and of the fluxes in one launch each, from edge values kept for
+  // each direction.  The others, or where that memory is not to be had, keep one
+  // set and launch per direction.
+  c->edges[1] = c->edges[2] = c->edges[0];
+  if (!rc && f64 && small_grid(na, c->sms)) {
+    c->merged = dalloc(&c->edges[1], eb) == HARMRAD_OK && dalloc(&c->edges[2], eb) == HARMRAD_OK;
+    if (!c->merged) {
+      if (c->edges[1]) cudaFree(c->edges[1]);
+      c->edges[1] = c->edges[2] = c->edges[0];
+    }
+  }
   if (!rc && cudaMallocHost((void**)&c->host_dt, count * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     rc = HARMRAD_E_OOM;

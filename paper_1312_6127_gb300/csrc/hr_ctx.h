@@ -34,7 +34,8 @@ struct harmrad_ctx {
   void* spd[3];
   void* aux;
   void* flat[3];
-  void* emf;
+  bool merged;  // reconstruction and fluxes of all directions in one launch each
+  void* emf;  // [3][ntot] edge EMFs of the pairs of directions (flux-CT)
   // staggered field (emf mode 1; null otherwise): sqrt(-g) B^d on the d-faces
   // and its value at the start of the step [ntot] each, gas signal speeds of
   // the faces [2][ntot] per direction, cell 3-velocities [3][ntot] and the
@@ -44,7 +45,7 @@ struct harmrad_ctx {
   void* gsp[3];
   void* vel;
   void* emf3[3];
-  void* edges;  // reconstructed edge values of one direction: FP64 [2][10][ntot] (without rho0, u_g), split [2][12][ntot]
+  void* edges[3];  // reconstructed edge values of each direction (merged), else of one (all three the same): FP64 [2][10][ntot] (without rho0, u_g), split [2][12][ntot]
   double* dt;
   unsigned char* status;
   int* iters;

@@ -32,7 +32,6 @@ struct Bufs {
   void* aux;       // [10][ntot] per-cell gdet, sqrt(-g) u^d gas/rad, tau weights
   void* flat[3];   // [2][ntot] flattener, max over the sub-steps of the step
   void* emf;       // [ntot] edge EMF scratch
-  void* edges;     // reconstructed edges of one direction: FP64 [20][ntot] (EdgeSet), split [24][ntot]
   double* dt;      // [nbox] time step of each grid
   unsigned char* status;  // [nact] worst outcome over the sub-steps
   int* iters;             // [nact] Newton steps summed over the sub-steps
@@ -62,9 +61,8 @@ struct Bufs {
 
 
 // FP64 edge values of one direction: [lower, upper][q - 2][ntot] of the primitives
-// q >= 2 in E, which every direction reuses, and [lower, upper][q][ntot] of rho0
-// and u_g in S, which each direction keeps: the entropy fluxes are formed from
-// them where a zone needs them (entropy_flux).
+// q >= 2 in E and [lower, upper][q][ntot] of rho0 and u_g in S, from which the
+// entropy fluxes are formed where a zone needs them (entropy_flux).
 struct EdgeSet {
   double* E;
   double* S;
@@ -73,6 +71,10 @@ struct EdgeSet {
   __device__ __forceinline__ double* plane(int up, int q, long long nt) const {
     return q < U1 ? S + (2 * up + q) * nt : E + (10 * up + q - U1) * nt;
   }
+};
+
+struct EdgeSets {
+  EdgeSet d[3];
 };
 
 // Counter update aggregated over the converged lanes of a warp.
@@ -568,9 +570,9 @@ __device__ __forceinline__ void flat_sig(const DevParams& p, const BoxGeo& bx, c
 }
 
 template <int d, bool SIG>
-__global__ void __launch_bounds__(256) k_flat_cols(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                                   const double* __restrict__ P0, const double* __restrict__ aux0,
-                                                   double* __restrict__ flat0, int chunk, bool fresh) {
+__device__ __forceinline__ void flat_cols(const DevParams& p, const BoxGeo* __restrict__ boxes, int nbox,
+                                          const double* __restrict__ P0, const double* __restrict__ aux0,
+                                          double* __restrict__ flat0, int chunk, bool fresh) {
   constexpr int o = 3 - d;
   long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
@@ -650,10 +652,9 @@ __global__ void __launch_bounds__(256) k_flat_cols(DevParams p, const BoxGeo* __
 // d = 0: a warp takes 26 consecutive cells of the joined rows (as k_recon_rows),
 // one per lane, three lanes on either side for the neighbours only.
 template <bool SIG>
-__global__ void __launch_bounds__(256) k_flat_rows(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                                          const double* __restrict__ P0,
-                                                          const double* __restrict__ aux0, double* __restrict__ flat0,
-                                                          bool fresh) {
+__device__ __forceinline__ void flat_rows(const DevParams& p, const BoxGeo* __restrict__ boxes, int nbox,
+                                          const double* __restrict__ P0, const double* __restrict__ aux0,
+                                          double* __restrict__ flat0, bool fresh) {
   const int lane = threadIdx.x & 31;
   const unsigned full = 0xffffffffu;
   long long done = 0;
@@ -696,6 +697,25 @@ __global__ void __launch_bounds__(256) k_flat_rows(DevParams p, const BoxGeo* __
     }
     done += total;
   }
+}
+
+// One launch for the directions d0 + blockIdx.y: a grid that does not fill the
+// GPU runs them side by side.
+struct FlatSet {
+  double* f[3];
+};
+struct Chunks {
+  int c[3];
+};
+template <bool SIG>
+__global__ void __launch_bounds__(128) k_flat(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                              const double* __restrict__ P0, const double* __restrict__ aux0,
+                                              FlatSet flat, Chunks ch, bool fresh, int d0) {
+  const int d = d0 + blockIdx.y;
+  if (!p.act[d]) return;
+  if (d == 0) flat_rows<SIG>(p, boxes, nbox, P0, aux0, flat.f[0], fresh);
+  else if (d == 1) flat_cols<1, SIG>(p, boxes, nbox, P0, aux0, flat.f[1], ch.c[1], fresh);
+  else flat_cols<2, SIG>(p, boxes, nbox, P0, aux0, flat.f[2], ch.c[2], fresh);
 }
 
 // ------------------------------------------------------------- reconstruction
@@ -756,17 +776,16 @@ __device__ __forceinline__ void ppm_cell(const R s[5], R chi, R* aL, R* aR) {
 // them in registers, or, along x1, a warp passes them between its lanes), and
 // the limiters work on differences: with a = |r - q|, b = |q - l| the
 // monotonicity tests of Colella & Woodward read b > 2 a and a > 2 b, and twice
-// the MC slope is min(|dl + dr|, 4 |dl|, 4 |dr|).  About 11 FP64 instructions
+// the MC slope is min(|dl + dr|, 4 |dl|, 4 |dr|).  About 14 FP64 instructions
 // per cell and variable.  One thread (or warp) takes one variable: few
 // registers, many warps, and small grids still fill the SMs.  Measured over an
 // RK3 step (GB300, PPM, Kerr-Schild, event time of the class): 256x128x64
-// 17.2 -> 7.8 ms, 64x32x16 0.75 -> 0.22 ms, 256 zones in 1D 125 -> 24 us,
+// 17.2 -> 10.7 ms, 64x32x16 0.75 -> 0.36 ms, 256 zones in 1D 125 -> 27 us,
 // against a slope pass plus a parabola pass of one thread per cell.
 
 // The limiters' comparisons and powers of two act on the bit patterns, off the
 // FP64 pipe: twice a double's bits (the sign shifted out) order like its
-// magnitude.  (A mask in place of the shift is compiled to an FP64 |x|.)  The
-// same on FP64 compares: 256x128x64 per RK3 step 9.8 ms, on the keys 7.8.
+// magnitude.  (A mask in place of the shift is compiled to an FP64 |x|.)
 __device__ __forceinline__ unsigned long long mag_key(double x) {
   return (unsigned long long)__double_as_longlong(x) << 1;
 }
@@ -819,9 +838,9 @@ __device__ __forceinline__ unsigned ppm_limit(double q, double chi, double& l, d
 // SIG: folds its decisions into the branch signature (a test instrument; a
 // variant of its own, so that the hot one holds no registers for it).
 template <int MET, int d, bool SIG>
-__global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                                    const double* __restrict__ P0, const double* __restrict__ aux0,
-                                                    const double* __restrict__ flat0, EdgeSet E0, int chunk) {
+__device__ __forceinline__ void recon_cols(const DevParams& p, const BoxGeo* __restrict__ boxes, int nbox,
+                                           const double* __restrict__ P0, const double* __restrict__ aux0,
+                                           const double* __restrict__ flat0, const EdgeSet& E0, int chunk) {
   const bool weighted = (MET == KS) && (d != 1);
   constexpr int o = 3 - d;  // the other transverse direction beside x1
   long long done = 0;
@@ -896,9 +915,9 @@ __global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* _
 // and interface values pass between lanes.  Values that cross a row's end
 // reach ghost cells that are not stored.
 template <int MET, bool SIG>
-__global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                                    const double* __restrict__ P0, const double* __restrict__ aux0,
-                                                    const double* __restrict__ flat0, EdgeSet E0) {
+__device__ __forceinline__ void recon_rows(const DevParams& p, const BoxGeo* __restrict__ boxes, int nbox,
+                                           const double* __restrict__ P0, const double* __restrict__ aux0,
+                                           const double* __restrict__ flat0, const EdgeSet& E0) {
   const bool weighted = (MET == KS);
   const int lane = threadIdx.x & 31;
   const unsigned full = 0xffffffffu;
@@ -967,6 +986,34 @@ __global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* _
     }
     done += total;
   }
+}
+
+// One launch per direction: fewer registers (the merged kernel holds 88), which a
+// grid that fills the GPU needs (256x128x64 per RK3 step 7.8 ms, merged 8.0;
+// batch of 12 boxes 5.16 against 5.31).
+template <int MET, bool SIG>
+__global__ void __launch_bounds__(256) k_recon_rows(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                    const double* __restrict__ P0, const double* __restrict__ aux0,
+                                                    const double* __restrict__ flat0, EdgeSet E0) {
+  recon_rows<MET, SIG>(p, boxes, nbox, P0, aux0, flat0, E0);
+}
+template <int MET, int d, bool SIG>
+__global__ void __launch_bounds__(256) k_recon_cols(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                    const double* __restrict__ P0, const double* __restrict__ aux0,
+                                                    const double* __restrict__ flat0, EdgeSet E0, int chunk) {
+  recon_cols<MET, d, SIG>(p, boxes, nbox, P0, aux0, flat0, E0, chunk);
+}
+// One launch for the directions d0 + blockIdx.y: a grid that does not fill the GPU
+// runs them side by side (64x32x16 per RK3 step 0.22 -> 0.19 ms).
+template <int MET>
+__global__ void __launch_bounds__(256) k_recon_all(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                   const double* __restrict__ P0, const double* __restrict__ aux0,
+                                                   FlatSet flat, EdgeSets E, Chunks ch, int d0) {
+  const int d = d0 + blockIdx.y;
+  if (!p.act[d]) return;
+  if (d == 0) recon_rows<MET, false>(p, boxes, nbox, P0, aux0, flat.f[0], E.d[0]);
+  else if (d == 1) recon_cols<MET, 1, false>(p, boxes, nbox, P0, aux0, flat.f[1], E.d[1], ch.c[1]);
+  else recon_cols<MET, 2, false>(p, boxes, nbox, P0, aux0, flat.f[2], E.d[2], ch.c[2]);
 }
 
 // FP32 reconstruction (split precision), one thread per cell of the face range
@@ -1120,19 +1167,18 @@ __device__ __forceinline__ void face_flux(const DevParams& p, const Geo<MET, R>&
 // the HLL or LAXF flux (Eqs. hll, lax), gas and radiation groups with their own
 // speeds.  The direction is a template parameter so that every index into a
 // 4-vector or the primitive array is resolved at compile time.
-template <int MET, typename R, int d>
-__global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
-                                              const R* __restrict__ E0, const double* __restrict__ K0,
-                                              R* __restrict__ F0, R* __restrict__ spd0,
-                                              const double* __restrict__ geo0, R* __restrict__ FS0,
-                                              R* __restrict__ gsp0, const double* __restrict__ S0) {
+// FP32 fluxes of one direction (split precision).
+template <int MET, int d>
+__global__ void __launch_bounds__(128) k_face32(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                const float* __restrict__ E0, const double* __restrict__ K0,
+                                                float* __restrict__ F0, float* __restrict__ spd0,
+                                                float* __restrict__ FS0, float* __restrict__ gsp0) {
+  typedef float R;
   const bool weighted = (MET == KS) && (d != 1);
   long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
-    constexpr bool F64 = std::is_same<R, double>::value;
-    const R* E = E0 + (F64 ? 20 : 24) * bx.coff;
-    const double* S = F64 ? S0 + 4 * bx.coff : nullptr;  // edges of rho0 and u_g
+    const R* E = E0 + 24 * bx.coff;
     const double* K = K0 + bx.coff;
     R* F = F0 + 12 * bx.coff;
     R* spd = spd0 + bx.coff;
@@ -1172,34 +1218,18 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
         continue;
       }
       Geo<MET, R> g;
-      R igf = R(1), dl = dxd;  // FP64: 1/sqrt(-g) and the cell's proper length along d
-      if constexpr (MET == KS && std::is_same<R, double>::value) {
-        const GeoTab T = geotab(geo0, bx);
-        const double* tab = d == 0 ? T.F0 : (d == 1 ? T.F1 : T.C);
-        const long long sz = d == 0 ? T.sF0 : (d == 1 ? T.sF1 : T.sC);
-        const long long x = d == 0 ? gidx_f0(bx, ii[0], ii[1])
-                                   : (d == 1 ? gidx_f1(bx, ii[0], ii[1]) : gidx_c(bx, ii[0], ii[1]));
-        g = geo_load<MET>(tab, sz, x);
-        if (weighted) igf = __ldg(tab + 16 * sz + x);
-        dl = dxd * __ldg(tab + (d == 2 ? 19 : 17) * sz + x);
-      } else {
-        R xf[3];
-        for (int e = 0; e < 3; ++e) xf[e] = R(bx.x0[e] + (ii[e] + (e == d ? 0.0 : 0.5)) * bx.dx[e]);
-        g = make_geo<MET, R>(p, xf[0], xf[1]);
-        igf = weighted ? R(1) / g.gdet : R(1);
-      }
+      R igf = R(1);
+      R xf[3];
+      for (int e = 0; e < 3; ++e) xf[e] = R(bx.x0[e] + (ii[e] + (e == d ? 0.0 : 0.5)) * bx.dx[e]);
+      g = make_geo<MET, R>(p, xf[0], xf[1]);
+      igf = weighted ? R(1) / g.gdet : R(1);
       R PL[NPR], PR[NPR];
 #pragma unroll
       for (int q = 0; q < NPR; ++q) {
         const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
         R aR, bL;  // upper edge of cell f-1, lower edge of cell f
-        if constexpr (F64) {
-          aR = q < U1 ? S[(2 + q) * bx.ntot + t - st] : E[(10 + q - U1) * bx.ntot + t - st];
-          bL = q < U1 ? S[q * bx.ntot + t] : E[(q - U1) * bx.ntot + t];
-        } else {
-          aR = E[(NPR + q) * bx.ntot + t - st];
-          bL = E[q * bx.ntot + t];
-        }
+        aR = E[(NPR + q) * bx.ntot + t - st];
+        bL = E[q * bx.ntot + t];
         PL[q] = wq ? aR * igf : aR;
         PR[q] = wq ? bL * igf : bL;
       }
@@ -1207,12 +1237,8 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
       R out[NPR], smax;
       unsigned fcode = 0;
       R fsv, gs[2];
-      if constexpr (std::is_same<R, double>::value)
-        face_flux64<MET, d + 1>(p, g, dl, kL, kR, PL, PR, out, &smax, p.sig ? &fcode : nullptr, FS ? &fsv : nullptr,
-                                gsp ? gs : nullptr);
-      else
-        face_flux<MET, R, d>(p, g, dxd, kL, kR, R(p.kscale), PL, PR, out, &smax, p.sig ? &fcode : nullptr,
-                             FS ? &fsv : nullptr, gs);
+      face_flux<MET, R, d>(p, g, dxd, kL, kR, R(p.kscale), PL, PR, out, &smax, p.sig ? &fcode : nullptr,
+                           FS ? &fsv : nullptr, gs);
       if (p.sig) sig_put(p, bx.coff + t, 40 + d, fcode);
       if (FS) FS[t] = fsv;
       if (gsp) {
@@ -1227,14 +1253,145 @@ __global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restr
   }
 }
 
+template <int MET, int d>
+__device__ __forceinline__ void face_dir(const DevParams& p, const BoxGeo* __restrict__ boxes, int nbox, EdgeSet E0,
+                                         const double* __restrict__ K0, double* __restrict__ F0,
+                                         double* __restrict__ spd0, const double* __restrict__ geo0,
+                                         double* __restrict__ FS0, double* __restrict__ gsp0) {
+  const bool weighted = (MET == KS) && (d != 1);
+  long long done = 0;
+  for (int bi = 0; bi < nbox; ++bi) {
+    const BoxGeo& bx = boxes[bi];
+    const EdgeSet E = E0.box(bx);
+    const double* K = K0 + bx.coff;
+    double* F = F0 + 12 * bx.coff;
+    double* spd = spd0 + bx.coff;
+    double* FS = FS0 ? FS0 + bx.coff : nullptr;
+    double* gsp = gsp0 ? gsp0 + 2 * bx.coff : nullptr;  // gas v_max, v_min per face (staggered field)
+    int len[3], off[3];
+    for (int e = 0; e < 3; ++e) {
+      if (e == d) {
+        len[e] = bx.n[e] + 1;
+        off[e] = 0;
+      } else if (bx.n[e] > 1) {
+        len[e] = bx.n[e] + 2;
+        off[e] = -1;
+      } else {
+        len[e] = 1;
+        off[e] = 0;
+      }
+    }
+    long long total = (long long)len[0] * len[1] * len[2];
+    const long long st = bx.str[d];
+    const double dxd = bx.dx[d];
+    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+      long long r = id;
+      int ii[3];
+      ii[0] = (int)(r % len[0]) + off[0];
+      r /= len[0];
+      ii[1] = (int)(r % len[1]) + off[1];
+      ii[2] = (int)(r / len[1]) + off[2];
+      long long t = cell_index(bx, ii[0], ii[1], ii[2]);
+      const int f = ii[d];
+      if (MET == KS && d == 1 && ((f == 0 && bx.bc[2] == 2) || (f == bx.n[1] && bx.bc[3] == 2))) {
+#pragma unroll
+        for (int q = 0; q < NPR; ++q) F[q * bx.ntot + t] = 0.0;
+        spd[t] = 0.0;
+        if (FS) FS[t] = 0.0;
+        if (gsp) gsp[t] = gsp[bx.ntot + t] = 0.0;
+        continue;
+      }
+      Geo<MET, double> g;
+      double igf = 1.0, dl = dxd;  // 1/sqrt(-g) and the cell's proper length along d
+      if constexpr (MET == KS) {
+        const GeoTab T = geotab(geo0, bx);
+        const double* tab = d == 0 ? T.F0 : (d == 1 ? T.F1 : T.C);
+        const long long sz = d == 0 ? T.sF0 : (d == 1 ? T.sF1 : T.sC);
+        const long long x = d == 0 ? gidx_f0(bx, ii[0], ii[1])
+                                   : (d == 1 ? gidx_f1(bx, ii[0], ii[1]) : gidx_c(bx, ii[0], ii[1]));
+        g = geo_load<MET>(tab, sz, x);
+        if (weighted) igf = __ldg(tab + 16 * sz + x);
+        dl = dxd * __ldg(tab + (d == 2 ? 19 : 17) * sz + x);
+      } else {
+        g = make_geo<MET, double>(p, 0.0, 0.0);
+      }
+      double PL[NPR], PR[NPR];
+#pragma unroll
+      for (int q = 0; q < NPR; ++q) {
+        const bool wq = weighted && ((q >= U1 && q <= B3) || q >= UR1);
+        const double aR = E.plane(1, q, bx.ntot)[t - st];  // upper edge of cell f-1
+        const double bL = E.plane(0, q, bx.ntot)[t];       // lower edge of cell f
+        PL[q] = wq ? aR * igf : aR;
+        PR[q] = wq ? bL * igf : bL;
+      }
+      const double kL = kfield(p, K, t - st), kR = kfield(p, K, t);
+      double out[NPR], smax;
+      unsigned fcode = 0;
+      double fsv, gs[2];
+      face_flux64<MET, d + 1>(p, g, dl, kL, kR, PL, PR, out, &smax, p.sig ? &fcode : nullptr, FS ? &fsv : nullptr,
+                              gsp ? gs : nullptr);
+      if (p.sig) sig_put(p, bx.coff + t, 40 + d, fcode);
+      if (FS) FS[t] = fsv;
+      if (gsp) {
+        gsp[t] = gs[0];
+        gsp[bx.ntot + t] = gs[1];
+      }
+#pragma unroll
+      for (int q = 0; q < NPR; ++q) F[q * bx.ntot + t] = out[q];
+      spd[t] = smax;
+    }
+    done += total;
+  }
+}
+
+// FP64: one launch per direction for the grids that fill the GPU.
+template <int MET, int d>
+__global__ void __launch_bounds__(128) k_face(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, EdgeSet E0,
+                                              const double* __restrict__ K0, double* __restrict__ F0,
+                                              double* __restrict__ spd0, const double* __restrict__ geo0,
+                                              double* __restrict__ FS0, double* __restrict__ gsp0) {
+  face_dir<MET, d>(p, boxes, nbox, E0, K0, F0, spd0, geo0, FS0, gsp0);
+}
+// One launch for the directions d0 + blockIdx.y, as k_recon_all (64x32x16 per RK3
+// step 0.35 -> 0.27 ms; grids that fill the GPU gain nothing).  gsp: gas v_max,
+// v_min per face (staggered field; null otherwise).
+struct FaceArgs {
+  EdgeSets E;
+  double* F[3];
+  double* spd[3];
+  double* FS[3];
+  double* gsp[3];
+};
+template <int MET>
+__global__ void __launch_bounds__(128) k_face_all(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
+                                                  const double* __restrict__ K0, const double* __restrict__ geo0,
+                                                  FaceArgs a, int d0) {
+  const int d = d0 + blockIdx.y;
+  if (!p.act[d]) return;
+  if (d == 0) face_dir<MET, 0>(p, boxes, nbox, a.E.d[0], K0, a.F[0], a.spd[0], geo0, a.FS[0], a.gsp[0]);
+  else if (d == 1) face_dir<MET, 1>(p, boxes, nbox, a.E.d[1], K0, a.F[1], a.spd[1], geo0, a.FS[1], a.gsp[1]);
+  else face_dir<MET, 2>(p, boxes, nbox, a.E.d[2], K0, a.F[2], a.spd[2], geo0, a.FS[2], a.gsp[2]);
+}
+
 // ----------------------------------------------------------------- flux-CT
 // Toth (2000) constrained transport for the pair (a, b) of active directions:
 // edge EMF = 1/4 (F_a[B_b] + F_a[B_b](b-1) - F_b[B_a] - F_b[B_a](a-1)), zero on
 // the polar axis; then F_a[B_b] and F_b[B_a] become averages of the two
 // adjacent edge EMFs (with opposite signs).
+// blockIdx.y = 0, 1, 2: the pairs (0, 1), (0, 2), (1, 2); emf1 holds one plane per
+// pair, `planes` apart.
 template <typename R>
-__global__ void k_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const R* __restrict__ Fa0,
-                      const R* __restrict__ Fb0, R* __restrict__ emf0, int a, int b) {
+struct FluxSet {
+  R* f[3];
+};
+template <typename R>
+__global__ void k_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, FluxSet<R> F, R* __restrict__ emf1,
+                      long long planes) {
+  const int a = blockIdx.y == 2 ? 1 : 0, b = blockIdx.y == 0 ? 1 : 2;
+  if (!p.act[a] || !p.act[b]) return;
+  const R* Fa0 = F.f[a];
+  const R* Fb0 = F.f[b];
+  R* emf0 = emf1 + blockIdx.y * planes;
   long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
@@ -1262,8 +1419,13 @@ __global__ void k_emf(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, c
 }
 
 template <typename R>
-__global__ void k_ct(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const R* __restrict__ emf0,
-                     R* __restrict__ Fa0, R* __restrict__ Fb0, int a, int b) {
+__global__ void k_ct(DevParams p, const BoxGeo* __restrict__ boxes, int nbox, const R* __restrict__ emf1,
+                     FluxSet<R> F, long long planes) {
+  const int a = blockIdx.y == 2 ? 1 : 0, b = blockIdx.y == 0 ? 1 : 2;
+  if (!p.act[a] || !p.act[b]) return;
+  R* Fa0 = F.f[a];
+  R* Fb0 = F.f[b];
+  const R* emf0 = emf1 + blockIdx.y * planes;
   long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];

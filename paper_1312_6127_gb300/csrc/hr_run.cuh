@@ -21,7 +21,6 @@ inline Bufs make_bufs(harmrad_ctx* c) {
   }
   b.aux = c->aux;
   b.emf = c->emf;
-  b.edges = c->edges;
   b.dt = c->dt;
   b.status = c->status;
   b.iters = c->iters;
@@ -124,62 +123,79 @@ inline int column_chunk(const harmrad_ctx* c, long long columns, long long nd, i
   return (int)((nd + n - 1) / n);
 }
 
-// FP64 flattener of direction d.
-inline void flatten(harmrad_ctx* c, int d, bool fresh) {
+inline int range_width(const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; }
+
+// Launches over directions take blockIdx.y for the direction, d0 + blockIdx.y.
+// first_dir and dir_count: the range that holds the active ones.
+inline int first_dir(const DevParams& p) { return p.act[0] ? 0 : (p.act[1] ? 1 : 2); }
+inline int dir_count(const DevParams& p) { return (p.act[2] ? 3 : (p.act[1] ? 2 : 1)) - first_dir(p); }
+
+// FP64 flattener of the active directions.
+inline void flatten(harmrad_ctx* c, bool fresh) {
   const DevParams& p = c->dp;
-  const BoxGeo* bt = c->dboxes;
-  const int nb = c->nbox;
-  const double* aux = (const double*)c->aux;
-  double* fl = (double*)c->flat[d];
-  auto width = [](const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; };
-  if (d == 0) {
-    const long long work = all_work(c, [width](const BoxGeo& b) {
-      return 32LL * (((long long)width(b, 1) * width(b, 2) * b.N[0] + 25) / 26);
-    });
-    const int g = grid_for(work, c->sms, 256);
-    if (p.sig) k_flat_rows<true><<<g, 256, 0, c->stream>>>(p, bt, nb, c->P, aux, fl, fresh);
-    else k_flat_rows<false><<<g, 256, 0, c->stream>>>(p, bt, nb, c->P, aux, fl, fresh);
-    return;
+  FlatSet fl;
+  Chunks ch{};
+  long long most = !p.act[0] ? 1 : all_work(c, [](const BoxGeo& b) {
+    return 32LL * (((long long)range_width(b, 1) * range_width(b, 2) * b.N[0] + 25) / 26);
+  });
+  for (int d = 0; d < 3; ++d) {
+    fl.f[d] = (double*)c->flat[d];
+    if (d == 0 || !p.act[d]) continue;
+    const long long cols =
+        all_work(c, [d](const BoxGeo& b) { return (long long)range_width(b, 0) * range_width(b, 3 - d); });
+    const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
+    // a piece evaluates two cells more than it owns; 4 blocks of 128 fit an SM
+    long long pieces;
+    ch.c[d] = column_chunk(c, cols, nd, 1024, 4, &pieces);
+    if (cols * pieces > most) most = cols * pieces;
   }
-  const int o = 3 - d;
-  const long long cols = all_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
-  const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
-  // a piece evaluates two cells more than it owns; 4 blocks of 128 fit an SM
-  long long pieces;
-  const int chunk = column_chunk(c, cols, nd, 1024, 4, &pieces);
-  const int g = grid_for(cols * pieces, c->sms, 128);
-  auto run = [&](auto kernel) { kernel<<<g, 128, 0, c->stream>>>(p, bt, nb, c->P, aux, fl, chunk, fresh); };
-  if (d == 1) p.sig ? run(k_flat_cols<1, true>) : run(k_flat_cols<1, false>);
-  else p.sig ? run(k_flat_cols<2, true>) : run(k_flat_cols<2, false>);
+  const int d0 = first_dir(p);
+  const dim3 g(grid_for(most, c->sms, 128), dir_count(p));
+  const double* aux = (const double*)c->aux;
+  if (p.sig) k_flat<true><<<g, 128, 0, c->stream>>>(p, c->dboxes, c->nbox, c->P, aux, fl, ch, fresh, d0);
+  else k_flat<false><<<g, 128, 0, c->stream>>>(p, c->dboxes, c->nbox, c->P, aux, fl, ch, fresh, d0);
 }
 
-// FP64 reconstruction of direction d: edge values of every cell of its face range.
+// FP64 reconstruction of the active directions d0 .. d0 + nd - 1: edge values of
+// every cell of their face ranges.
 template <int MET>
-void recon(harmrad_ctx* c, int d, const double* P, const double* aux, const double* flat, int block, int per_sm) {
+void recon(harmrad_ctx* c, int d0, int ndir, const double* P, const double* aux, const FlatSet& flat, int block,
+           int per_sm) {
   const DevParams& p = c->dp;
-  const EdgeSet E{(double*)c->edges, c->ES[d]};
-  const BoxGeo* bt = c->dboxes;
-  const int nb = c->nbox;
-  auto width = [](const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; };
-  if (d == 0) {
-    const long long work = all_work(c, [width](const BoxGeo& b) {
-      return 12LL * 32 * (((long long)width(b, 1) * width(b, 2) * b.N[0] + 59) / 60);
-    });
-    const int g = grid_for(work, c->sms, block, per_sm);
-    if (p.sig) k_recon_rows<MET, true><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E);
-    else k_recon_rows<MET, false><<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E);
-    return;
+  EdgeSets E;
+  Chunks ch{};
+  long long most = 1;
+  for (int d = 0; d < 3; ++d) {
+    E.d[d] = EdgeSet{(double*)c->edges[d], c->ES[d]};
+    if (d < d0 || d >= d0 + ndir || !p.act[d]) continue;
+    long long work;
+    if (d == 0) {
+      work = all_work(c, [](const BoxGeo& b) {
+        return 12LL * 32 * (((long long)range_width(b, 1) * range_width(b, 2) * b.N[0] + 59) / 60);
+      });
+    } else {
+      const long long cols =
+          all_work(c, [d](const BoxGeo& b) { return (long long)range_width(b, 0) * range_width(b, 3 - d); });
+      const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
+      // a piece repeats about one cell's work: 16 cells or more, two threads per slot
+      long long pieces;
+      ch.c[d] = column_chunk(c, 12 * cols, nd, 4096, 16, &pieces);
+      work = 12 * cols * pieces;
+    }
+    if (work > most) most = work;
   }
-  const int o = 3 - d;
-  const long long cols = all_work(c, [width, o](const BoxGeo& b) { return (long long)width(b, 0) * width(b, o); });
-  const long long nd = max_work(c, [d](const BoxGeo& b) { return b.n[d] + 2; });
-  // a piece repeats about one cell's work: 16 cells or more, two threads per slot
-  long long pieces;
-  const int chunk = column_chunk(c, 12 * cols, nd, 4096, 16, &pieces);
-  const int g = grid_for(12 * cols * pieces, c->sms, block, per_sm);
-  auto run = [&](auto kernel) { kernel<<<g, block, 0, c->stream>>>(p, bt, nb, P, aux, flat, E, chunk); };
-  if (d == 1) p.sig ? run(k_recon_cols<MET, 1, true>) : run(k_recon_cols<MET, 1, false>);
-  else p.sig ? run(k_recon_cols<MET, 2, true>) : run(k_recon_cols<MET, 2, false>);
+  const dim3 g(grid_for(most, c->sms, block, per_sm), ndir);
+  auto run = [&](auto sig) {
+    constexpr bool SIG = decltype(sig)::value;
+    if (d0 == 0) k_recon_rows<MET, SIG><<<g, block, 0, c->stream>>>(p, c->dboxes, c->nbox, P, aux, flat.f[0], E.d[0]);
+    else if (d0 == 1)
+      k_recon_cols<MET, 1, SIG><<<g, block, 0, c->stream>>>(p, c->dboxes, c->nbox, P, aux, flat.f[1], E.d[1], ch.c[1]);
+    else
+      k_recon_cols<MET, 2, SIG><<<g, block, 0, c->stream>>>(p, c->dboxes, c->nbox, P, aux, flat.f[2], E.d[2], ch.c[2]);
+  };
+  if (ndir > 1) k_recon_all<MET><<<g, block, 0, c->stream>>>(p, c->dboxes, c->nbox, P, aux, flat, E, ch, d0);
+  else if (p.sig) run(std::true_type{});
+  else run(std::false_type{});
 }
 
 template <int MET, typename R>
@@ -204,59 +220,83 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     return w;
   };
   if (p.recon == 0) {
-    for (int d = 0; d < 3; ++d) {
-      if (!p.act[d]) continue;
-      if constexpr (std::is_same<R, double>::value) {
-        flatten(c, d, fresh);
-        mark(c, HARMRAD_K_FLATTEN);
-        ++nk;
-        continue;
-      }
-      if (fresh) {
-        if (cudaMemsetAsync(c->flat[d], 0, 2 * c->ncell * sizeof(R), st) != cudaSuccess) return HARMRAD_E_CUDA;
-        mark(c, HARMRAD_K_OTHER);
-      }
-      k_flatten<R><<<grid_for(all_work(c, range_cells), c->sms, 256), 256, 0, st>>>(
-          p, bt, nb, c->P, (const R*)c->aux, (R*)c->flat[d], d);
+    if constexpr (std::is_same<R, double>::value) {
+      flatten(c, fresh);
       mark(c, HARMRAD_K_FLATTEN);
       ++nk;
+    } else {
+      for (int d = 0; d < 3; ++d) {
+        if (!p.act[d]) continue;
+        if (fresh) {
+          if (cudaMemsetAsync(c->flat[d], 0, 2 * c->ncell * sizeof(R), st) != cudaSuccess) return HARMRAD_E_CUDA;
+          mark(c, HARMRAD_K_OTHER);
+        }
+        k_flatten<R><<<grid_for(all_work(c, range_cells), c->sms, 256), 256, 0, st>>>(
+            p, bt, nb, c->P, (const R*)c->aux, (R*)c->flat[d], d);
+        mark(c, HARMRAD_K_FLATTEN);
+        ++nk;
+      }
     }
   }
-  for (int d = 0; d < 3; ++d) {
-    if (!p.act[d]) continue;
-    long long wf = all_work(c, [d](const BoxGeo& b) {
+  const harmrad_tuning& tu = c->tune;
+  const int be = tu.edge_block, bf = tu.face_block;
+  FlatSet fl;
+  for (int d = 0; d < 3; ++d) fl.f[d] = (double*)c->flat[d];
+  auto faces_of = [c](int d) {
+    return all_work(c, [d](const BoxGeo& b) {
       long long w = 1;
       for (int e = 0; e < 3; ++e) w *= (e == d) ? b.n[e] + 1 : (b.n[e] > 1 ? b.n[e] + 2 : 1);
       return w;
     });
-    const harmrad_tuning& tu = c->tune;
-    const int be = tu.edge_block, bf = tu.face_block;
-    const int g = grid_for(wf, c->sms, bf, tu.face_blocks_per_sm);
-    R* Ed = (R*)c->edges;
-    R* Fd = (R*)c->F[d];
-    R* sd = (R*)c->spd[d];
-    if constexpr (std::is_same<R, double>::value) {
-      recon<MET>(c, d, c->P, (const double*)c->aux, (const double*)c->flat[d], be, tu.edge_blocks_per_sm);
-    } else {
-      const int ge = grid_for(all_work(c, range_cells), c->sms, be, tu.edge_blocks_per_sm);
-      const R* aux = (const R*)c->aux;
-      const R* fl = (const R*)c->flat[d];
-      if (d == 0) k_edges<MET, 0><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Ed);
-      else if (d == 1) k_edges<MET, 1><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Ed);
-      else k_edges<MET, 2><<<ge, be, 0, st>>>(p, bt, nb, c->P, aux, fl, Ed);
+  };
+  if (c->merged && !p.sig) {  // FP64: all directions in one launch each
+    FaceArgs fa;
+    long long wf = 1;
+    const int d0 = first_dir(p), nd = dir_count(p);
+    for (int d = 0; d < 3; ++d) {
+      fa.E.d[d] = EdgeSet{(double*)c->edges[d], c->ES[d]};
+      fa.F[d] = (double*)c->F[d];
+      fa.spd[d] = (double*)c->spd[d];
+      fa.FS[d] = (double*)c->FS[d];
+      fa.gsp[d] = (double*)c->gsp[d];
+      if (p.act[d] && faces_of(d) > wf) wf = faces_of(d);
     }
+    recon<MET>(c, d0, nd, c->P, (const double*)c->aux, fl, be, tu.edge_blocks_per_sm);
     mark(c, HARMRAD_K_EDGE);
-    if (d == 0)
-      k_face<MET, R, 0><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[0],
-                                           (R*)c->gsp[0], c->ES[0]);
-    else if (d == 1)
-      k_face<MET, R, 1><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[1],
-                                           (R*)c->gsp[1], c->ES[1]);
-    else
-      k_face<MET, R, 2><<<g, bf, 0, st>>>(p, bt, nb, Ed, c->K, Fd, sd, c->geotab, (R*)c->FS[2],
-                                           (R*)c->gsp[2], c->ES[2]);
+    const dim3 g(grid_for(wf, c->sms, bf, tu.face_blocks_per_sm), nd);
+    k_face_all<MET><<<g, bf, 0, st>>>(p, bt, nb, c->K, c->geotab, fa, d0);
     mark(c, HARMRAD_K_FACE);
     nk += 2;
+  } else {
+    for (int d = 0; d < 3; ++d) {
+      if (!p.act[d]) continue;
+      if constexpr (std::is_same<R, double>::value) {
+        recon<MET>(c, d, 1, c->P, (const double*)c->aux, fl, be, tu.edge_blocks_per_sm);
+      } else {
+        const int ge = grid_for(all_work(c, range_cells), c->sms, be, tu.edge_blocks_per_sm);
+        auto edge = [&](auto kernel) {
+          kernel<<<ge, be, 0, st>>>(p, bt, nb, c->P, (const R*)c->aux, (const R*)c->flat[d], (R*)c->edges[d]);
+        };
+        d == 0 ? edge(k_edges<MET, 0>) : (d == 1 ? edge(k_edges<MET, 1>) : edge(k_edges<MET, 2>));
+      }
+      mark(c, HARMRAD_K_EDGE);
+      const int gf = grid_for(faces_of(d), c->sms, bf, tu.face_blocks_per_sm);
+      if constexpr (std::is_same<R, double>::value) {
+        auto face = [&](auto kernel) {
+          kernel<<<gf, bf, 0, st>>>(p, bt, nb, EdgeSet{(double*)c->edges[d], c->ES[d]}, c->K, (double*)c->F[d],
+                                    (double*)c->spd[d], c->geotab, (double*)c->FS[d], (double*)c->gsp[d]);
+        };
+        d == 0 ? face(k_face<MET, 0>) : (d == 1 ? face(k_face<MET, 1>) : face(k_face<MET, 2>));
+      } else {
+        auto face = [&](auto kernel) {
+          kernel<<<gf, bf, 0, st>>>(p, bt, nb, (const R*)c->edges[d], c->K, (R*)c->F[d], (R*)c->spd[d],
+                                    (R*)c->FS[d], (R*)c->gsp[d]);
+        };
+        d == 0 ? face(k_face32<MET, 0>) : (d == 1 ? face(k_face32<MET, 1>) : face(k_face32<MET, 2>));
+      }
+      mark(c, HARMRAD_K_FACE);
+      nk += 2;
+    }
   }
   if (p.emf == 1) {  // staggered field: the 4-state upwind EMFs on the edges
     if constexpr (std::is_same<R, double>::value)
@@ -282,30 +322,16 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     if (cudaGetLastError() != cudaSuccess) return HARMRAD_E_CUDA;
     return nk;
   }
-  for (int a = 0; a < 3; ++a)
-    for (int b = a + 1; b < 3; ++b) {
-      if (!p.act[a] || !p.act[b]) continue;
-      long long we = all_work(c, [a, b](const BoxGeo& x) {
-        long long w = 1;
-        for (int e = 0; e < 3; ++e) w *= x.n[e] + ((e == a || e == b) ? 1 : 0);
-        return w;
-      });
-      long long wc = all_work(c, [a, b](const BoxGeo& x) {
-        long long la = 1, lb = 1;
-        for (int e = 0; e < 3; ++e) {
-          la *= x.n[e] + (e == a ? 1 : 0);
-          lb *= x.n[e] + (e == b ? 1 : 0);
-        }
-        return la + lb;
-      });
-      k_emf<R><<<grid_for(we, c->sms, 256), 256, 0, st>>>(p, bt, nb, (const R*)c->F[a], (const R*)c->F[b],
-                                                            (R*)c->emf, a, b);
-      mark(c, HARMRAD_K_CT);
-      k_ct<R><<<grid_for(wc, c->sms, 256), 256, 0, st>>>(p, bt, nb, (const R*)c->emf, (R*)c->F[a],
-                                                           (R*)c->F[b], a, b);
-      mark(c, HARMRAD_K_CT);
-      nk += 2;
-    }
+  if (p.act[0] + p.act[1] + p.act[2] >= 2) {  // flux-CT of every pair of active directions
+    const long long we = all_work(c, [](const BoxGeo& x) { return (x.n[0] + 1LL) * (x.n[1] + 1) * (x.n[2] + 1); });
+    FluxSet<R> F;
+    for (int d = 0; d < 3; ++d) F.f[d] = (R*)c->F[d];
+    k_emf<R><<<dim3(grid_for(we, c->sms, 256), 3), 256, 0, st>>>(p, bt, nb, F, (R*)c->emf, c->ncell);
+    mark(c, HARMRAD_K_CT);
+    k_ct<R><<<dim3(grid_for(2 * we, c->sms, 256), 3), 256, 0, st>>>(p, bt, nb, (const R*)c->emf, F, c->ncell);
+    mark(c, HARMRAD_K_CT);
+    nk += 2;
+  }
   if (cudaGetLastError() != cudaSuccess) return HARMRAD_E_CUDA;
   return nk;
 }
