@@ -453,7 +453,9 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     return HARMRAD_E_CUDA;
   }
   c->tune = default_tuning(c->nact, c->sms);
-  if (count > 1) c->tune.newton_split = 5;  // batches: heavy-tailed Newton counts expected (3: 51.3 ms, 5: 48.2)
+  // batches: heavy-tailed Newton counts (update of 12 boxes per RK3 step with 0, 3, 5, 6, 8: 54.1, 35.3, 27.7, 26.1,
+  // 26.8 ms)
+  if (count > 1) c->tune.newton_split = 6;
   if (stream) {
     c->stream = (cudaStream_t)stream;
   } else {

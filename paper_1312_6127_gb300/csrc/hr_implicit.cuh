@@ -21,6 +21,8 @@
 // R^mu_a u^a = 4/3 Ebar (u_r.u) u_r^mu + 1/3 Ebar u^mu, so G_nu (Eq. Gcov) is a
 // combination of u_r_nu and u_nu and needs no 4x4 contraction.
 #pragma once
+#include <climits>
+
 #include "hr_phys.cuh"
 #include "hr_tangent.cuh"
 
@@ -563,12 +565,17 @@ __device__ __forceinline__ bool pmhd_newton_dx(const DevParams& p, const ImpSys<
 
 // PMHD Newton iterations from the state st until a stopping rule ends the
 // iteration (returns true) or the next iteration's index reaches kstop
-// (returns false; st holds what the remaining iterations need).  best_x /
-// best_eT hold the lowest-error iterate (best_eT = inf if no residual was
+// (returns false; st holds what the remaining iterations need).  With a kstop a
+// zone that turns to finite differences pauses there as well: its iterations
+// cost four more residuals, for which the other lanes of its warp would wait.
+// best_x / best_eT hold the lowest-error iterate (best_eT = inf if no residual was
 // finite).
 template <int MET, bool FAST>
 __device__ __forceinline__ bool newton_pmhd_run(const DevParams& p, const ImpSys<MET, FAST>& s, NewtonState& st, int kstop) {
   TanStage ts;
+  // (split precision keeps the pauses at kstop alone: the queue's kernel works
+  // with the FP64 functions)
+  const bool defer = FAST && kstop != INT_MAX;
   for (;; ++st.k) {
     if (st.k >= kstop) return false;
     ImpRes r;
@@ -583,7 +590,10 @@ __device__ __forceinline__ bool newton_pmhd_run(const DevParams& p, const ImpSys
     if (r.eT < p.newton_tol) break;
     // a step with the FP32 Jacobian that raised e_T: finite differences for
     // the rest of the solve
-    if (st.jac32 && r.eT > st.hs.t1) st.jac32 = 0;
+    if (st.jac32 && r.eT > st.hs.t1) {
+      st.jac32 = 0;
+      if (defer) return false;
+    }
     if (stalled(st.hs, st.k, r.eT, r.eI)) break;
     if (st.k >= p.newton_max) break;
     if (r.eI < 1e-9) st.eps = 1e-10;

@@ -36,7 +36,7 @@ struct Bufs {
   unsigned char* status;  // [nact] worst outcome over the sub-steps
   int* iters;             // [nact] Newton steps summed over the sub-steps
   unsigned char* failed;  // [nact] back-up flag of the current sub-step
-  int* qcount;            // [4] retry queue, back-up list, Newton continuation queue lengths
+  int* qcount;            // [4] lengths: retry queue, back-up list, Newton continuation queue, its finite-difference end
   int* qzone;             // [nact] retry queue: zone index within its grid
   int* qbox;              // [nact] retry queue: grid of the entry
   double* qdata;          // [nact][19] retry queue payload: U*, PMHD best x, e_T, h, S*
@@ -46,6 +46,7 @@ struct Bufs {
   int* czone;             // [nact] Newton continuation queue: zone index within its grid
   int* cbox;              // [nact] Newton continuation queue: grid of the entry
   double* cdata;          // [nact][CSTRIDE] continuation payload: U*, Newton state
+  int ncont;              // nact of the context: the queue's finite-difference zones fill it from the end
   unsigned long long* stats;  // [8] counters
   unsigned long long* dtmin;  // [nbox] CFL minimum (ordered bits of a positive double)
   const double* geo;          // metric tables of Kerr-Schild grids (null otherwise)
@@ -2483,7 +2484,7 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
           accept = pmhd_finish<MET>(p, bx, bi, z, t, fl, g, s, Ust, h, ns.best_x, ns.best_eT, ns.steps, P, b, Sst);
           done_steps = (unsigned)ns.steps;
         } else {
-          const int slot = atomicAdd(&b.qcount[2], 1);
+          const int slot = ns.jac32 ? atomicAdd(&b.qcount[2], 1) : b.ncont - 1 - atomicAdd(&b.qcount[3], 1);
           b.czone[slot] = (int)z;
           b.cbox[slot] = bi;
           double* cd = b.cdata + (long long)slot * CSTRIDE;
@@ -2507,8 +2508,11 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
 template <int MET>
 __global__ void __launch_bounds__(128) k_newton_cont(DevParams p, const BoxGeo* __restrict__ boxes, Bufs b,
                                                      double hfac) {
-  const int nq = b.qcount[2];
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nq; e += gridDim.x * blockDim.x) {
+  // the finite-difference zones first, in warps of their own
+  const int nfd = b.qcount[3], pad = (nfd + 31) & ~31, nq = pad + b.qcount[2];
+  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < nq; it += gridDim.x * blockDim.x) {
+    if (it >= nfd && it < pad) continue;
+    const int e = it < nfd ? b.ncont - 1 - it : it - pad;
     const int bi = b.cbox[e];
     const BoxGeo& bx = boxes[bi];
     const long long z = b.czone[e];
@@ -2529,7 +2533,7 @@ __global__ void __launch_bounds__(128) k_newton_cont(DevParams p, const BoxGeo* 
     const double h = hfac * b.dt[bi];  // the sub-step's implicit step fraction
     ImpSys<MET> s;
     build_sys<MET>(p, g, Ust, h, kfield(p, b.K + bx.coff, t), s);
-    newton_pmhd_run<MET>(p, s, ns, 1 << 30);
+    newton_pmhd_run<MET>(p, s, ns, INT_MAX);
     const bool accept = pmhd_finish<MET>(p, bx, bi, z, t, fl, g, s, Ust, h, ns.best_x, ns.best_eT, ns.steps,
                                          b.P + 12 * bx.coff, b, cd[NPR + 22]);
     if (accept) atomicAdd(&b.stats[ST_PMHD], 1ULL);

@@ -26,6 +26,7 @@ inline Bufs make_bufs(harmrad_ctx* c) {
   b.iters = c->iters;
   b.failed = c->failed;
   b.qcount = c->qcount;
+  b.ncont = (int)c->nact;
   b.qzone = c->qzone;
   b.qbox = c->qbox;
   b.qdata = c->qdata;
@@ -406,13 +407,14 @@ int solve_impl(harmrad_ctx* c, int stage, const ImexStage& im) {
   int nk = 4 + nf;
   if (split > 0) {
     // the continuation queue, the retry queue and the back-up list are
-    // short: one persistent wave of blocks each
+    // short: one persistent wave of blocks each, of one warp so that a queue shorter
+    // than the wave spreads over all SMs
     const double hfac = im.on ? im.g : (stage == 0 ? 1.0 : (stage == 1 ? 0.25 : 2.0 / 3.0));
-    k_newton_cont<MET><<<c->sms * 2, 128, 0, st>>>(p, c->dboxes, b, hfac);
+    k_newton_cont<MET><<<c->sms * 8, 32, 0, st>>>(p, c->dboxes, b, hfac);
     mark(c, HARMRAD_K_UPDATE);
     ++nk;
   }
-  k_retry<MET><<<c->sms * 2, 128, 0, st>>>(p, c->dboxes, b, stage);
+  k_retry<MET><<<c->sms * 8, 32, 0, st>>>(p, c->dboxes, b, stage);
   mark(c, HARMRAD_K_RETRY);
   if (im.on && im.g > 0.0) {
     k_imex_store<MET><<<grid_for(c->nact, c->sms, 256), 256, 0, st>>>(p, c->dboxes, c->nbox, b, stage, im.g);
