@@ -67,4 +67,27 @@ __device__ __forceinline__ double sqrt64(double x) {
   return fma(x, y, x * (y * q));
 }
 
+// FP64 <-> FP32 with the bits of the language's conversions, by integer
+// operations: the hardware's conversion is an FP64 pipe instruction like any
+// other, and a zone's FP32 Jacobian takes about fifty.  Numbers beyond the normal
+// FP32 range go to the language's conversion.
+static __device__ __noinline__ float narrow_any(double x) { return (float)x; }
+static __device__ __noinline__ double widen_any(float x) { return (double)x; }
+
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  if ((hi & 0x7ff00000u) - (897u << 20) >= (254u << 20))
+    return ((hi << 1) | lo) == 0 ? __uint_as_float(hi) : narrow_any(x);
+  // round to nearest even at bit 29; the exponent's bias 1023 -> 127
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x) + 0x0fffffffu + ((lo >> 29) & 1u);
+  return __uint_as_float(((unsigned)(b >> 29) - (896u << 23)) | (hi & 0x80000000u));
+}
+
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x);
+  if ((u & 0x7f800000u) - 0x00800000u >= 0x7f000000u)
+    return (u << 1) == 0 ? __hiloint2double((int)u, 0) : widen_any(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
 }  // namespace hr

@@ -134,17 +134,21 @@ __device__ __forceinline__ void tan_stage_zone(const Sys& s, TanStage& ts) {
 }
 
 // the FP32 inputs of one column pass: from the staged copy (v[15..31]), or,
-// on the Minkowski path, which has no metric to stage, converted in registers
+// on the Minkowski path, which has no metric to stage, converted in registers.
+// There narrow and widen take the conversions off the FP64 pipe (93x71x45 box,
+// update per RK3 step 2.71 -> 2.50 ms; batch of 12 boxes 29.9 -> 27.7); the
+// Kerr-Schild kernel spills more with them than it gains (256x128x64: 17.6 ->
+// 18.2 ms) and keeps the language's.
 struct TanIn {
   float x[4], rt[4], Dlab, iDlab, B[3], h, ks, kf;
   template <class Sys>
   __device__ __forceinline__ TanIn(const Sys& s, const double xd[4], const double Rt64[4])
-      : Dlab((float)s.Dlab), iDlab((float)s.iDlab), B{(float)s.B[0], (float)s.B[1], (float)s.B[2]},
-        h((float)s.h), ks((float)s.ks), kf((float)s.kf) {
+      : Dlab(narrow(s.Dlab)), iDlab(narrow(s.iDlab)), B{narrow(s.B[0]), narrow(s.B[1]), narrow(s.B[2])},
+        h(narrow(s.h)), ks(narrow(s.ks)), kf(narrow(s.kf)) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      x[i] = (float)xd[i];
-      rt[i] = (float)Rt64[i];
+      x[i] = narrow(xd[i]);
+      rt[i] = narrow(Rt64[i]);
     }
   }
   __device__ __forceinline__ explicit TanIn(const TanStage& ts)
@@ -264,13 +268,14 @@ __device__ __forceinline__ bool pmhd_jac_column(const DevParams& p, const TanIn&
 
 // The PMHD Jacobian (J[i][c] = dE_i/dx_c) from four FP32 tangent passes; ts
 // holds the solve's staged inputs (tan_stage_zone; Kerr-Schild only).
+template <int MET>
 __device__ __forceinline__ void jac_store_column(double J[4][4], int j, const float col[4]) {
   // column j written through compile-time indices
 #pragma unroll
   for (int c = 0; c < 4; ++c)
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if (c == j) J[i][c] = (double)col[i];
+      if (c == j) J[i][c] = MET == MINK ? widen(col[i]) : (double)col[i];
 }
 
 template <int MET, class Sys>
@@ -284,7 +289,7 @@ __device__ __forceinline__ bool pmhd_jacobian_fp32(const DevParams& p, const Sys
     for (int j = 0; j < 4; ++j) {
       float col[4];
       ok = pmhd_jac_column<MET>(p, ti, g, j, col) && ok;
-      jac_store_column(J, j, col);
+      jac_store_column<MET>(J, j, col);
     }
   } else {
     if (!ts.zone) tan_stage_zone<MET>(s, ts);
@@ -297,7 +302,7 @@ __device__ __forceinline__ bool pmhd_jacobian_fp32(const DevParams& p, const Sys
     for (int j = 0; j < 4; ++j) {
       float col[4];
       ok = pmhd_jac_column<MET>(p, TanIn(ts), GeoF<MET>(ts.v), j, col) && ok;
-      jac_store_column(J, j, col);
+      jac_store_column<MET>(J, j, col);
     }
   }
   return ok;
