@@ -92,6 +92,9 @@ __device__ __forceinline__ void warp_add(unsigned long long* dst, unsigned v) {
 // First item of this thread among the items of a grid whose predecessors in
 // the context hold `done` items: the grids' items form one sequence dealt to
 // the threads in turn, so that a batch of small grids loads every block alike.
+// (The FP32 kernels of split precision pass over each grid from its first item:
+// with another loop around them their sums are fused and rounded differently, and
+// the FP32 stages answer round-off with up to 3e-7.)
 __device__ __forceinline__ long long first_item(long long done) {
   if (done == 0) return HR_TID;
   const long long r = HR_TID - done % HR_STRIDE;
@@ -306,7 +309,7 @@ __global__ void k_prep(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
     const double* P = P0 + 12 * bx.coff;
     const double* K = K0 + bx.coff;
     R* aux = aux0 + 10 * bx.coff;
-    for (long long t = first_item(bx.coff); t < bx.ntot; t += HR_STRIDE) {
+    for (long long t = HR_TID; t < bx.ntot; t += HR_STRIDE) {
       long long r = t;
       int i = (int)(r % bx.N[0]) - bx.ng[0];
       r /= bx.N[0];
@@ -474,7 +477,6 @@ template <typename R>
 __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbox,
                           const double* __restrict__ P0, const R* __restrict__ aux0,
                           R* __restrict__ flat0, int d) {
-  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const double* P = P0 + 12 * bx.coff;
@@ -492,7 +494,7 @@ __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
     }
     long long total = (long long)len[0] * len[1] * len[2];
     const long long st = bx.str[d];
-    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
       long long r = id;
       int i = (int)(r % len[0]) + off[0];
       r /= len[0];
@@ -516,7 +518,6 @@ __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
       flat[t] = Fg > og ? Fg : og;
       flat[bx.ntot + t] = Fr > orr ? Fr : orr;
     }
-    done += total;
   }
 }
 
@@ -1026,7 +1027,6 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
                                                const float* __restrict__ flat0, float* __restrict__ E0) {
   typedef float R;
   const bool weighted = (MET == KS) && (d != 1);
-  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const double* P = P0 + 12 * bx.coff;
@@ -1045,7 +1045,7 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
     }
     long long total = (long long)len[0] * len[1] * len[2];
     const long long st = bx.str[d];
-    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
       long long r = id;
       int i = (int)(r % len[0]) + off[0];
       r /= len[0];
@@ -1083,7 +1083,6 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
         E[(NPR + q) * bx.ntot + t] = aR;
       }
     }
-    done += total;
   }
 }
 
@@ -1176,7 +1175,6 @@ __global__ void __launch_bounds__(128) k_face32(DevParams p, const BoxGeo* __res
                                                 float* __restrict__ FS0, float* __restrict__ gsp0) {
   typedef float R;
   const bool weighted = (MET == KS) && (d != 1);
-  long long done = 0;
   for (int bi = 0; bi < nbox; ++bi) {
     const BoxGeo& bx = boxes[bi];
     const R* E = E0 + 24 * bx.coff;
@@ -1201,7 +1199,7 @@ __global__ void __launch_bounds__(128) k_face32(DevParams p, const BoxGeo* __res
     long long total = (long long)len[0] * len[1] * len[2];
     const long long st = bx.str[d];
     const R dxd = R(bx.dx[d]);
-    for (long long id = first_item(done); id < total; id += HR_STRIDE) {
+    for (long long id = HR_TID; id < total; id += HR_STRIDE) {
       long long r = id;
       int ii[3];
       ii[0] = (int)(r % len[0]) + off[0];
@@ -1250,7 +1248,6 @@ __global__ void __launch_bounds__(128) k_face32(DevParams p, const BoxGeo* __res
       for (int q = 0; q < NPR; ++q) F[q * bx.ntot + t] = out[q];
       spd[t] = smax;
     }
-    done += total;
   }
 }
 
