@@ -1252,9 +1252,9 @@ __device__ __forceinline__ void build_sys_with(const DevParams& p, const Geo<MET
   }
 }
 
-template <int MET, typename T = double>
+template <int MET, typename T = double, bool FAST>
 __device__ __forceinline__ void build_sys(const DevParams& p, const Geo<MET, T>& g, const T Us[12], double h,
-                                          T kf, ImpSysT<MET, T>& s) {
+                                          T kf, ImpSysT<MET, T, FAST>& s) {
   // orthonormal (ZAMO) size of covariant spatial components:
   // sqrt(gamma^{kk}), gamma^{kk} = g^{kk} - (g^{tk})^2 / g^{tt} > 0 everywhere
   // on the slice, inside the horizon too

@@ -484,7 +484,9 @@ __global__ void k_zone_implicit(DevParams p, BoxGeo bg, int n, const double* __r
       Ust[q] = Us[NPR * z + q];
       P0[q] = Ps[NPR * z + q];
     }
-    ImpSys<MET> s;
+    // PMHD term by term: the outcome of a zone near a method's threshold (a whole
+    // value) follows the last bits of the residual
+    ImpSys<MET, false> s;
     build_sys<MET>(p, g, Ust, hh[z], 1.0, s);
     double x0[4] = {P0[UU], P0[U1], P0[U2], P0[U3]};
     double kabs, ksca;
@@ -494,7 +496,7 @@ __global__ void k_zone_implicit(DevParams p, BoxGeo bg, int n, const double* __r
       if (p.act[d - 1]) dl = fmax(dl, sqrt(g.gdd(d)) * bg.dx[d - 1]);
     if ((kabs + ksca) * dl < 2.0 / 3.0) {
       double go[5], T3[3] = {s.Ts[1], s.Ts[2], s.Ts[3]};
-      if (gas_invert<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, P0, 1e-9, go) == 0) {
+      if (gas_invert_ieee<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, P0, 1e-9, go) == 0) {
         x0[0] = go[1];
         x0[1] = go[2];
         x0[2] = go[3];
@@ -514,6 +516,8 @@ __global__ void k_zone_implicit(DevParams p, BoxGeo bg, int n, const double* __r
       int rs;
       const double tau = zone_tau<MET>(p, g, bg.dx, P0, 1.0);
       const double sz = Sst ? Sst[z] : NAN;
+      ImpSys<MET> s;
+      build_sys<MET>(p, g, Ust, hh[z], 1.0, s);
       method = retry_sequence<MET>(p, g, s, P0, bx, beT, tau, Pn, &eT, &rs, subdom, sz);
       steps += rs;
       if (method == ST_BACKUP) {  // the entropy (S* given), then the cold-MHD equations

@@ -96,10 +96,10 @@ __global__ void k_zi_clear(void* base) {
 }
 
 // Geometry, explicit state and the PMHD guess of one zone.
-template <int MET>
+template <int MET, bool FAST>
 __device__ void zi_setup(const hr::DevParams& p, int z, const double* x, const double* Us,
                          const double* Ps, const double* hh, hr::Geo<MET, double>& g,
-                         hr::ImpSys<MET>& s, double P0[hr::NPR]) {
+                         hr::ImpSys<MET, FAST>& s, double P0[hr::NPR]) {
   using namespace hr;
   double x1 = x[4 * z + 1], x2 = x[4 * z + 2];
   g = make_geo<MET, double>(p, x1, x2);
@@ -120,7 +120,7 @@ __global__ void k_zi_pmhd(hr::DevParams p, hr::BoxGeo bg, int n, const double* _
   QueueView qv = queue_view(base);
   for (int z = blockIdx.x * blockDim.x + threadIdx.x; z < n; z += gridDim.x * blockDim.x) {
     Geo<MET, double> g;
-    ImpSys<MET> s;
+    ImpSys<MET, false> s;  // term by term, as k_zone_implicit
     double P0[NPR];
     zi_setup<MET>(p, z, x, Us, Ps, hh, g, s, P0);
     double x0[4] = {P0[UU], P0[U1], P0[U2], P0[U3]};
@@ -131,7 +131,7 @@ __global__ void k_zi_pmhd(hr::DevParams p, hr::BoxGeo bg, int n, const double* _
       if (p.act[d - 1]) dl = fmax(dl, sqrt(g.gdd(d)) * bg.dx[d - 1]);
     if ((kabs + ksca) * dl < 2.0 / 3.0) {
       double go[5], T3[3] = {s.Ts[1], s.Ts[2], s.Ts[3]};
-      if (gas_invert<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, P0, 1e-9, go) == 0) {
+      if (gas_invert_ieee<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, P0, 1e-9, go) == 0) {
         x0[0] = go[1];
         x0[1] = go[2];
         x0[2] = go[3];
