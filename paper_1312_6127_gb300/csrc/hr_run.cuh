@@ -127,9 +127,12 @@ inline int column_chunk(const harmrad_ctx* c, long long columns, long long nd, i
 inline int range_width(const BoxGeo& b, int e) { return b.n[e] > 1 ? b.n[e] + 2 : 1; }
 
 // Launches over directions take blockIdx.y for the direction, d0 + blockIdx.y.
-// first_dir and dir_count: the range that holds the active ones.
+// first_dir and dir_count: the range that holds the active ones (none in a grid
+// of one zone, which launches nothing for them).
 inline int first_dir(const DevParams& p) { return p.act[0] ? 0 : (p.act[1] ? 1 : 2); }
-inline int dir_count(const DevParams& p) { return (p.act[2] ? 3 : (p.act[1] ? 2 : 1)) - first_dir(p); }
+inline int dir_count(const DevParams& p) {
+  return p.act[0] || p.act[1] || p.act[2] ? (p.act[2] ? 3 : (p.act[1] ? 2 : 1)) - first_dir(p) : 0;
+}
 
 // FP64 flattener of the active directions.
 inline void flatten(harmrad_ctx* c, bool fresh) {
@@ -220,7 +223,7 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     for (int e = 0; e < 3; ++e) w *= b.n[e] > 1 ? b.n[e] + 2 : 1;
     return w;
   };
-  if (p.recon == 0) {
+  if (p.recon == 0 && dir_count(p) > 0) {
     if constexpr (std::is_same<R, double>::value) {
       flatten(c, fresh);
       mark(c, HARMRAD_K_FLATTEN);
@@ -250,7 +253,7 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
       return w;
     });
   };
-  if (c->merged && !p.sig) {  // FP64: all directions in one launch each
+  if (c->merged && !p.sig && dir_count(p) > 0) {  // FP64: all directions in one launch each
     FaceArgs fa;
     long long wf = 1;
     const int d0 = first_dir(p), nd = dir_count(p);
