@@ -44,8 +44,9 @@ struct ImpPre<double> {
 // evaluates the same functions on dual numbers.  FAST: FP64 with pmhd_res64
 // and hr_math.cuh; otherwise the term-by-term functions with the language's
 // divisions (dual numbers, and split precision, whose FP32 stages round the
-// primitives so that a last-bit change here moves a rounding there: its
-// results are kept to the bit).
+// primitives so that a last-bit change here moves a rounding there: values of
+// the 256x128x64 torus move by up to 2.8e-7 with the FP64 functions, by 3e-12
+// with these).  Every kernel of a context that solves takes the same ones.
 template <int MET, typename T = double, bool FAST = std::is_same<T, double>::value>
 struct ImpSysT {
   static constexpr bool fast = FAST;
@@ -574,8 +575,7 @@ __device__ __forceinline__ bool pmhd_newton_dx(const DevParams& p, const ImpSys<
 template <int MET, bool FAST>
 __device__ __forceinline__ bool newton_pmhd_run(const DevParams& p, const ImpSys<MET, FAST>& s, NewtonState& st, int kstop) {
   TanStage ts;
-  // (split precision keeps the pauses at kstop alone: the queue's kernel works
-  // with the FP64 functions)
+  // (split precision pauses at kstop alone)
   const bool defer = FAST && kstop != INT_MAX;
   for (;; ++st.k) {
     if (st.k >= kstop) return false;
@@ -691,8 +691,8 @@ __device__ int newton_pmhd(const DevParams& p, const ImpSys<MET, FAST>& s, const
 // and their error rows drop out (identity row and column, zero error); the
 // Jacobian columns come from two-sided differences with the PMHD offsets;
 // x_new = x - D J^-1 E.  Returns false if the system is singular.
-template <int MET>
-__device__ bool pmhd_damped_step(const DevParams& p, const ImpSys<MET>& s, const double x[4], const ImpRes& r,
+template <int MET, bool FAST>
+__device__ bool pmhd_damped_step(const DevParams& p, const ImpSys<MET, FAST>& s, const double x[4], const ImpRes& r,
                                  unsigned mask, double D, double eps, double xn[4]) {
   const double umag = fmax(1.0, sqrt(s.g.sq3(x[1], x[2], x[3])));
   double J[4][4], E[4];
@@ -715,7 +715,7 @@ __device__ bool pmhd_damped_step(const DevParams& p, const ImpSys<MET>& s, const
   }
   for (int i = 0; i < 4; ++i) E[i] = (mask >> i & 1u) ? r.Eg[i] : 0.0;
   double dx[4];
-  if (!solve4(J, E, dx)) return false;
+  if (!solve4<FAST>(J, E, dx)) return false;
   for (int i = 0; i < 4; ++i) xn[i] = x[i] - D * dx[i];
   return true;
 }
@@ -730,8 +730,8 @@ __device__ bool pmhd_damped_step(const DevParams& p, const ImpSys<MET>& s, const
 // after a step becomes |u_g|/2; the second such reset in stage 1 or 2 keeps
 // the prior iterate and ends the stage.  best_x / best_eT: the lowest-e_T
 // iterate of all stages (inf if no residual was finite).  Returns the steps.
-template <int MET>
-__device__ int newton_pmhd_staged(const DevParams& p, const ImpSys<MET>& s, const double x0[4], double best_x[4],
+template <int MET, bool FAST>
+__device__ int newton_pmhd_staged(const DevParams& p, const ImpSys<MET, FAST>& s, const double x0[4], double best_x[4],
                                   double* best_eT) {
   double x[4] = {x0[0], x0[1], x0[2], x0[3]};
   *best_eT = HUGE_VAL;
@@ -803,8 +803,8 @@ __device__ int newton_pmhd_staged(const DevParams& p, const ImpSys<MET>& s, cons
 // G_S of Eq. GS, times F_13 = T) in place of the radiation energy row; returns
 // its normalised error (its terms plus the gas energy row's norm, Tc0 and G0
 // the iterate's T^t_t + rho0 u^t and G_t) for normalise.
-template <int MET>
-__device__ __forceinline__ double entropy_rad_row(const DevParams& p, const ImpSys<MET>& s, double rho, double ug,
+template <int MET, bool FAST>
+__device__ __forceinline__ double entropy_rad_row(const DevParams& p, const ImpSys<MET, FAST>& s, double rho, double ug,
                                                   const double ucon[4], const double G[4], double Tc0, ImpRes& r) {
   const double Tg = (p.gam - 1.0) * ug / rho;
   const double Gu = G[0] * ucon[0] + G[1] * ucon[1] + G[2] * ucon[2] + G[3] * ucon[3];
@@ -827,10 +827,18 @@ __device__ __forceinline__ void entropy_ug_guess(const DevParams& p, double Sst,
   if (isfinite(pg) && pg > 0.0) x[0] = pg / (p.gam - 1.0);
 }
 
+// The 1D_W gas inversion with the system's arithmetic: T^t_t + rho0 u^t, T^t_i.
+template <int MET, bool FAST>
+__device__ __forceinline__ int gas_invert_sys(const DevParams& p, const ImpSys<MET, FAST>& s, double taue,
+                                              const double Tt[3], const double Pg[NPR], double tol, double out[5]) {
+  return FAST ? gas_invert<MET>(p, s.g, s.Dlab, taue, Tt, s.B, Pg, tol, out)
+              : gas_invert_ieee<MET>(p, s.g, s.Dlab, taue, Tt, s.B, Pg, tol, out);
+}
+
 // URAD error function: iterate R^t_nu; gas from 1D_W inversion of
 // T^t_nu = T*^t_nu - (x - R*^t_nu); radiation from the M1 inversion of x.
-template <int MET>
-__device__ __forceinline__ bool urad_res(const DevParams& p, const ImpSys<MET>& s, const double x[4],
+template <int MET, bool FAST>
+__device__ __forceinline__ bool urad_res(const DevParams& p, const ImpSys<MET, FAST>& s, const double x[4],
                                          const double Pg[5], double tol_inv, ImpRes& r,
                                          double gas_out[5], double Pr[4], bool norm) {
   const auto& g = s.g;
@@ -843,7 +851,7 @@ __device__ __forceinline__ bool urad_res(const DevParams& p, const ImpSys<MET>& 
   Pg12[U2] = Pg[3];
   Pg12[U3] = Pg[4];
   double T3[3] = {Tt[1], Tt[2], Tt[3]};
-  if (gas_invert<MET>(p, g, s.Dlab, Tt[0], T3, s.B, Pg12, tol_inv, gas_out) != 0) {
+  if (gas_invert_sys<MET>(p, s, Tt[0], T3, Pg12, tol_inv, gas_out) != 0) {
     r.ok = false;
     return false;
   }
@@ -885,8 +893,8 @@ __device__ __forceinline__ bool urad_res(const DevParams& p, const ImpSys<MET>& 
 // PRAD error function: iterate the radiation primitives (Ebar, u~^i_rad);
 // R^t_nu from them in closed form; gas from 1D_W inversion of
 // T^t_nu = T*^t_nu - (R^t_nu - R*^t_nu) (Sec. 4.8).
-template <int MET>
-__device__ __forceinline__ bool prad_res(const DevParams& p, const ImpSys<MET>& s, const double x[4],
+template <int MET, bool FAST>
+__device__ __forceinline__ bool prad_res(const DevParams& p, const ImpSys<MET, FAST>& s, const double x[4],
                                          const double Pg[5], double tol_inv, ImpRes& r,
                                          double gas_out[5], double Rx[4], bool norm) {
   const auto& g = s.g;
@@ -905,7 +913,7 @@ __device__ __forceinline__ bool prad_res(const DevParams& p, const ImpSys<MET>& 
   Pg12[U2] = Pg[3];
   Pg12[U3] = Pg[4];
   double T3[3] = {Tt[1], Tt[2], Tt[3]};
-  if (gas_invert<MET>(p, g, s.Dlab, Tt[0], T3, s.B, Pg12, tol_inv, gas_out) != 0) {
+  if (gas_invert_sys<MET>(p, s, Tt[0], T3, Pg12, tol_inv, gas_out) != 0) {
     r.ok = false;
     return false;
   }
@@ -947,8 +955,8 @@ __device__ __forceinline__ bool prad_res(const DevParams& p, const ImpSys<MET>& 
 // reflects R^t_t > 0 and PRAD Ebar < 0 to half their size.  Pg (gas guess:
 // rho, u_g, u~^i) is updated by every successful residual.  best_x / best_Pg
 // / best_eT hold the best iterate.
-template <int MET, bool PRAD>
-__device__ int newton_rad(const DevParams& p, const ImpSys<MET>& s, const double x0[4], double Pg[5],
+template <int MET, bool PRAD, bool FAST>
+__device__ int newton_rad(const DevParams& p, const ImpSys<MET, FAST>& s, const double x0[4], double Pg[5],
                           double best_x[4], double best_Pg[5], double* best_eT) {
   double x[4] = {x0[0], x0[1], x0[2], x0[3]};
   double xprev[4] = {x0[0], x0[1], x0[2], x0[3]};
@@ -1020,7 +1028,7 @@ __device__ int newton_rad(const DevParams& p, const ImpSys<MET>& s, const double
     }
     if (!jok) break;
     double E[4] = {r.Er[0], r.Er[1], r.Er[2], r.Er[3]}, dx[4];
-    if (!solve4(J, E, dx)) break;
+    if (!solve4<FAST>(J, E, dx)) break;
     double xn[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) xn[i] = x[i] - dx[i];
@@ -1067,8 +1075,8 @@ __device__ int newton_rad(const DevParams& p, const ImpSys<MET>& s, const double
 // with 40 x 6 gas inversions in all.  The energy unknown reflected to half
 // its size when a step puts it on the wrong side; the second reflection in
 // stage 1 or 2 keeps the prior iterate and ends the stage.
-template <int MET, bool PRAD>
-__device__ int newton_rad_staged(const DevParams& p, const ImpSys<MET>& s, const double x0[4], double Pg[5],
+template <int MET, bool PRAD, bool FAST>
+__device__ int newton_rad_staged(const DevParams& p, const ImpSys<MET, FAST>& s, const double x0[4], double Pg[5],
                                  double best_x[4], double best_Pg[5], double* best_eT) {
   double x[4] = {x0[0], x0[1], x0[2], x0[3]};
   double xprev[4] = {x0[0], x0[1], x0[2], x0[3]};
@@ -1131,7 +1139,7 @@ __device__ int newton_rad_staged(const DevParams& p, const ImpSys<MET>& s, const
     }
     for (int i = 0; i < 4; ++i) E[i] = (mask >> i & 1u) ? r.Er[i] : 0.0;
     double dx[4];
-    if (!solve4(J, E, dx)) return false;
+    if (!solve4<FAST>(J, E, dx)) return false;
     for (int i = 0; i < 4; ++i) xn[i] = x[i] - D * dx[i];
     return true;
   };
@@ -1203,8 +1211,8 @@ __device__ int newton_rad_staged(const DevParams& p, const ImpSys<MET>& s, const
   return steps;
 }
 
-template <int MET>
-__device__ __forceinline__ int newton_urad(const DevParams& p, const ImpSys<MET>& s, const double x0[4],
+template <int MET, bool FAST>
+__device__ __forceinline__ int newton_urad(const DevParams& p, const ImpSys<MET, FAST>& s, const double x0[4],
                                            double Pg[5], double best_x[4], double best_Pg[5], double* best_eT) {
   return newton_rad<MET, false>(p, s, x0, Pg, best_x, best_Pg, best_eT);
 }

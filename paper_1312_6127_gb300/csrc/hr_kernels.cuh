@@ -1599,8 +1599,8 @@ __device__ __forceinline__ double zone_tau(const DevParams& p, const Geo<MET, do
 // PMHD iterate and its error (inf if none).  Returns the outcome: ST_PMHD,
 // ST_URAD (URAD or PRAD), or ST_BACKUP when no residual was finite or the
 // best e_T exceeds 1e-7; *eT_out its error, *steps_out the Newton steps.
-template <int MET>
-__device__ int retry_sequence(const DevParams& p, const Geo<MET, double>& g, const ImpSys<MET>& s,
+template <int MET, bool FAST>
+__device__ int retry_sequence(const DevParams& p, const Geo<MET, double>& g, const ImpSys<MET, FAST>& s,
                               const double Ps[NPR], const double px[4], double peT, double tau, double Pn[NPR],
                               double* eT_out, int* steps_out, bool subdom = false, double Sst = NAN) {
   const bool pfin = isfinite(peT);
@@ -2137,8 +2137,8 @@ __device__ __forceinline__ bool cold_allowed(const Geo<MET, double>& g, const do
 // METH_ENTROPY (the entropy PMHD's solution), METH_ENTROPY_RAD (the entropy
 // URAD's or PRAD's) or METH_COLD with Pn and *eT set, 0 if none gives a
 // solution; adds the Newton steps to *steps.  emode 0: no entropy equation.
-template <int MET>
-__device__ int backup_equations(const DevParams& p, const Geo<MET, double>& g, const ImpSys<MET>& s,
+template <int MET, bool FAST>
+__device__ int backup_equations(const DevParams& p, const Geo<MET, double>& g, const ImpSys<MET, FAST>& s,
                                 const double Ust[NPR], const double Ps[NPR], double Sst, int emode,
                                 double tau, double Pn[NPR], double* eT, int* steps,
                                 const double* px = nullptr, double peT = HUGE_VAL) {
@@ -2148,11 +2148,11 @@ __device__ int backup_equations(const DevParams& p, const Geo<MET, double>& g, c
   double x0[4] = {Ps[UU], Ps[U1], Ps[U2], Ps[U3]};
   if (tau < 2.0 / 3.0) {
     double go[5], T3[3] = {s.Ts[1], s.Ts[2], s.Ts[3]};
-    if (gas_invert<MET>(p, g, s.Dlab, s.Ts[0], T3, s.B, Ps, 1e-9, go) == 0)
+    if (gas_invert_sys<MET>(p, s, s.Ts[0], T3, Ps, 1e-9, go) == 0)
       for (int c = 0; c < 4; ++c) x0[c] = go[1 + c];
   }
   if (ent) {
-    ImpSys<MET> se = s;
+    ImpSys<MET, FAST> se = s;
     se.entropy = true;
     se.Sstar = Sst / g.gdet;
     double bxe[4] = {0.0, 0.0, 0.0, 0.0}, beT = HUGE_VAL;
@@ -2223,7 +2223,7 @@ __device__ int backup_equations(const DevParams& p, const Geo<MET, double>& g, c
     }
   }
   if (cold) {
-    ImpSys<MET> sc = s;
+    ImpSys<MET, FAST> sc = s;
     sc.entropy = false;
     sc.cold = true;
     double bxc[4] = {0.0, 0.0, 0.0, 0.0}, beT = HUGE_VAL;
@@ -2507,7 +2507,9 @@ __device__ __forceinline__ void update_box(const DevParams& p, const BoxGeo& bx,
 // queue's other end, into warps of their own.  Update class of 12 boxes per RK3
 // step 43.9 -> 29.9 ms (11 lanes of 32 were active in an FP64 instruction of the
 // update kernel, 18 now).
-template <int MET>
+// FAST: the functions of the context's update kernel (ImpSysT), so that a queue
+// changes no byte of the result, in split precision (false) as in FP64.
+template <int MET, bool FAST>
 __global__ void __launch_bounds__(128) k_newton_cont(DevParams p, const BoxGeo* __restrict__ boxes, Bufs b,
                                                      double hfac) {
   // the finite-difference zones first, in warps of their own
@@ -2533,7 +2535,7 @@ __global__ void __launch_bounds__(128) k_newton_cont(DevParams p, const BoxGeo* 
     NewtonState ns;
     newton_state_load(cd + NPR, ns);
     const double h = hfac * b.dt[bi];  // the sub-step's implicit step fraction
-    ImpSys<MET> s;
+    ImpSys<MET, FAST> s;
     build_sys<MET>(p, g, Ust, h, kfield(p, b.K + bx.coff, t), s);
     newton_pmhd_run<MET>(p, s, ns, INT_MAX);
     const bool accept = pmhd_finish<MET>(p, bx, bi, z, t, fl, g, s, Ust, h, ns.best_x, ns.best_eT, ns.steps,
@@ -2592,8 +2594,8 @@ __global__ void k_imex_store(DevParams p, const BoxGeo* __restrict__ boxes, int 
 // Persistent grid over the retry queue (its length is read on the device, so
 // the launch needs no host round trip and can live in a CUDA graph): URAD,
 // then PRAD (retry_sequence); e_T > 1e-7 sends the zone to the
-// neighbour-average back-up.
-template <int MET>
+// neighbour-average back-up.  FAST: as k_newton_cont.
+template <int MET, bool FAST>
 __global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __restrict__ boxes, Bufs b, int stage) {
   const int nq = b.qcount[0];
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nq; e += gridDim.x * blockDim.x) {
@@ -2621,7 +2623,7 @@ __global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __rest
     const bool subdom = qd[16] < 0.0;
     const double peT = subdom ? HUGE_VAL : qd[16];
     const double h = qd[17];
-    ImpSys<MET> s;
+    ImpSys<MET, FAST> s;
     build_sys<MET>(p, g, Ust, h, kfield(p, K, t), s);
     const long long zg = bx.aoff + z;
     double Pn[NPR], eT;
@@ -2631,7 +2633,7 @@ __global__ void __launch_bounds__(128) k_retry(DevParams p, const BoxGeo* __rest
     double Sst = qd[18];
     // FP64: the explicit entropy, where the sequence reads it
     auto entropy = [&] {
-      if (p.precision != 0 || !b.Sn) return;
+      if (!FAST || !b.Sn) return;
       double u[4], v[4], gm;
       fourvel<MET, double>(g, Ps[U1], Ps[U2], Ps[U3], u, v, &gm);
       Sst = entropy_star(p, bx, b, z, t, stage, b.dt[bi], g.gdet * Ps[RHO] * u[0], Ps[RHO], Ps[UU]);

@@ -953,8 +953,7 @@ __device__ __forceinline__ int gas_invert(const DevParams& p, const Geo<MET, dou
 }
 
 // The same inversion in the language's divisions and square roots, for split
-// precision: its FP32 stages round the primitives, so a last-bit change here
-// moves a rounding there, and its results are kept to the bit.
+// precision (ImpSysT) and the point-wise solves.
 template <int MET>
 __device__ __forceinline__ int gas_invert_ieee(const DevParams& p, const Geo<MET, double>& g, double Dlab,
                                           double taue, const double Tt[3], const double B[3],

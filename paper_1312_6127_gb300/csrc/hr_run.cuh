@@ -413,11 +413,11 @@ int solve_impl(harmrad_ctx* c, int stage, const ImexStage& im) {
     // short: one persistent wave of blocks each, of one warp so that a queue shorter
     // than the wave spreads over all SMs
     const double hfac = im.on ? im.g : (stage == 0 ? 1.0 : (stage == 1 ? 0.25 : 2.0 / 3.0));
-    k_newton_cont<MET><<<c->sms * 8, 32, 0, st>>>(p, c->dboxes, b, hfac);
+    k_newton_cont<MET, std::is_same<R, double>::value><<<c->sms * 8, 32, 0, st>>>(p, c->dboxes, b, hfac);
     mark(c, HARMRAD_K_UPDATE);
     ++nk;
   }
-  k_retry<MET><<<c->sms * 8, 32, 0, st>>>(p, c->dboxes, b, stage);
+  k_retry<MET, std::is_same<R, double>::value><<<c->sms * 8, 32, 0, st>>>(p, c->dboxes, b, stage);
   mark(c, HARMRAD_K_RETRY);
   if (im.on && im.g > 0.0) {
     k_imex_store<MET><<<grid_for(c->nact, c->sms, 256), 256, 0, st>>>(p, c->dboxes, c->nbox, b, stage, im.g);
