@@ -450,25 +450,31 @@ int harmrad_adjoint_set_input(harmrad_ctx* ctx, const double* P, double dt, int 
 
 /* Launch shapes of the three heaviest kernels: threads per block and the cap
  * on blocks per SM of their grid-stride grids (the grid is the smaller of the
- * work and sms x cap blocks).  Shapes change no result: every zone and face
- * runs the same arithmetic under any shape. */
+ * work and sms x cap blocks).  A context of at most 256 zones per SM launches
+ * blocks of at most 32 threads (reconstruction 64), whatever the larger number
+ * here.  Shapes change no result: every zone and face runs the same arithmetic
+ * under any shape. */
 typedef struct harmrad_tuning {
   int face_block, face_blocks_per_sm;      /* face physics + Riemann; block 32..128 */
   int update_block, update_blocks_per_sm;  /* update + implicit solve; block 32..128 */
   int edge_block, edge_blocks_per_sm;      /* reconstruction; block 32..256 */
   int newton_split;  /* PMHD iterations the update kernel runs before a zone moves to the
                         compacted continuation queue (0: none, the zone finishes in place);
-                        1..60.  The resumed iteration is the same arithmetic. */
+                        1..60.  In FP64 a zone that turns to finite differences moves
+                        there at once.  The resumed iteration is the same arithmetic. */
   double face_ms, update_ms, edge_ms;      /* autotune: best device ms per step */
 } harmrad_tuning;
 
 /* Autotune the launch shapes on the context's current state: time `reps`
  * eager steps (dt <= 0: CFL) for each candidate shape, with CUDA events on the
- * context's stream, keep the fastest per kernel class, restore the primitives
- * and drop the captured graphs (the next step re-captures).  Candidates:
- * blocks of 64 or 128 threads (edges 128 or 256) with caps of 4..64 blocks per
- * SM, and Newton splits of 0 (no continuation queue), 3 and 5.  Writes the chosen shapes to *out (may be NULL).  Synchronises; allocates
- * a scratch copy of the primitives for the duration of the call. */
+ * context's stream, keep the fastest per kernel class (the current one unless
+ * another is 1 % faster), restore the primitives and drop the captured graphs
+ * (the next step re-captures).  Candidates: the context's current shapes (the
+ * defaults, unless set), and blocks of 64 or 128 threads (edges 128 or 256)
+ * with caps of 4..64 blocks per SM and Newton splits of 0 (no continuation
+ * queue), 3 and 5.  Writes the chosen shapes to *out (may be NULL).
+ * Synchronises; allocates a scratch copy of the primitives for the duration of
+ * the call. */
 int harmrad_autotune(harmrad_ctx* ctx, int reps, harmrad_tuning* out);
 
 /* Read or set the launch shapes (set: values outside the ranges above give

@@ -324,28 +324,22 @@ int launch_step(harmrad_ctx* c, bool with_cfl) {
   return HARMRAD_OK;
 }
 
-// No more zones than one wave of the heavy kernels (2 blocks of 128 threads per SM).
-bool small_grid(long long nact, int sms) { return nact <= 256LL * sms; }
-
-// Default launch shapes.  The heavy kernels hold 2 blocks of 128 threads per SM
-// (200 registers and more): a grid that does not fill one such wave takes blocks
-// of one or two warps, which spread over all SMs and schedulers (64x32x16 torus,
-// 32-thread against 128-thread blocks: update 0.57 against 0.62 ms per step,
-// reconstruction 0.26 against 0.34); a larger one is fastest with full blocks
-// (256x128x64: update 17.6 ms against 20.9 with 32 threads).  Blocks beyond the
-// resident ones (cap 64 per SM, 16 before: update 20.5 ms) even out zones of
-// unlike Newton counts.
-harmrad_tuning default_tuning(long long nact, int sms) {
+// Default launch shapes: full blocks (256x128x64 torus: update 17.6 ms per step
+// against 21.0 with 32 threads; a small grid launches smaller ones, fit_block).
+// Blocks beyond the resident ones (cap 64 per SM, 16 before: update 20.5 ms) even
+// out zones of unlike Newton counts.  Batches have heavy-tailed Newton counts and
+// split the solve (update of 12 boxes per RK3 step with a split at 0, 3, 5, 6, 8:
+// 54.1, 35.3, 27.7, 26.1, 26.8 ms).
+harmrad_tuning default_tuning(int nbox) {
   harmrad_tuning t;
   memset(&t, 0, sizeof(t));
-  const bool small = small_grid(nact, sms);
-  t.face_block = small ? 32 : 128;
+  t.face_block = 128;
   t.face_blocks_per_sm = 64;
-  t.update_block = small ? 32 : 128;
+  t.update_block = 128;
   t.update_blocks_per_sm = 64;
-  t.edge_block = small ? 64 : 256;
+  t.edge_block = 256;
   t.edge_blocks_per_sm = 64;
-  t.newton_split = 0;
+  t.newton_split = nbox > 1 ? 6 : 0;
   return t;
 }
 
@@ -452,10 +446,7 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     free(c);
     return HARMRAD_E_CUDA;
   }
-  c->tune = default_tuning(c->nact, c->sms);
-  // batches: heavy-tailed Newton counts (update of 12 boxes per RK3 step with 0, 3, 5, 6, 8: 54.1, 35.3, 27.7, 26.1,
-  // 26.8 ms)
-  if (count > 1) c->tune.newton_split = 6;
+  c->tune = default_tuning(count);
   if (stream) {
     c->stream = (cudaStream_t)stream;
   } else {
@@ -521,12 +512,12 @@ int create(const harmrad_params* p, int count, void* stream, harmrad_ctx** out) 
     rc = rc ? rc : dalloc(&c->imex_M, 16 * na * sizeof(double));
   }
   rc = rc ? rc : dalloc(&c->flag, sizeof(int));
-  // FP64 grids that do not fill one wave (default_tuning) run all directions of the
+  // FP64 grids that do not fill one wave (small_grid) run all directions of the
   // reconstruction and of the fluxes in one launch each, from edge values kept for
   // each direction.  The others, or where that memory is not to be had, keep one
   // set and launch per direction.
   c->edges[1] = c->edges[2] = c->edges[0];
-  if (!rc && f64 && small_grid(na, c->sms)) {
+  if (!rc && f64 && hr::small_grid(na, c->sms)) {
     c->merged = dalloc(&c->edges[1], eb) == HARMRAD_OK && dalloc(&c->edges[2], eb) == HARMRAD_OK;
     if (!c->merged) {
       if (c->edges[1]) cudaFree(c->edges[1]);
@@ -1065,15 +1056,19 @@ int harmrad_autotune(harmrad_ctx* c, int reps, harmrad_tuning* out) {
   struct Shape {
     int block, cap, split;
   };
-  // candidate i pairs the i-th shape of each class; the classes are timed
-  // separately within the same step
+  // candidate 0 is the context's current shape of each class, candidate i > 0 pairs
+  // the shapes i - 1 of the lists; the classes are timed separately within the
+  // same step.  A class leaves its current shape only for one that is 1 % faster:
+  // two timings of one shape differ by less, and the defaults are near the best
+  // (256x128x64 torus, update at 64 blocks per SM: 17.6 ms, with a split of 3
+  // 18.5; 12 boxes at a split of 5, 6: 27.7, 26.1)
   const Shape fc[] = {{128, 16, 0}, {64, 16, 0}, {128, 8, 0}, {128, 32, 0}, {64, 32, 0},
                       {128, 64, 0}, {128, 4, 0}, {128, 32, 0}, {64, 64, 0}};
-  const Shape uc[] = {{128, 16, 0}, {64, 16, 3}, {128, 8, 5}, {128, 32, 0}, {64, 32, 3},
-                      {128, 64, 3}, {64, 64, 0}, {128, 32, 3}, {128, 32, 5}};
+  const Shape uc[] = {{128, 64, 0}, {64, 16, 3}, {128, 8, 5}, {128, 32, 0}, {64, 32, 3},
+                      {128, 64, 3}, {64, 64, 0}, {128, 64, 5}, {128, 16, 0}};
   const Shape ec[] = {{256, 16, 0}, {128, 16, 0}, {256, 8, 0}, {256, 32, 0}, {128, 32, 0},
                       {256, 64, 0}, {128, 64, 0}, {256, 32, 0}, {128, 8, 0}};
-  const int ncand = 9;
+  const int ncand = 10;
   const size_t bytes = 12 * (size_t)c->ncell * sizeof(double);
   double* save = nullptr;
   if (cudaMalloc((void**)&save, bytes) != cudaSuccess) {
@@ -1081,22 +1076,24 @@ int harmrad_autotune(harmrad_ctx* c, int reps, harmrad_tuning* out) {
     return HARMRAD_E_OOM;
   }
   const harmrad_tuning orig = c->tune;
-  harmrad_tuning best = orig;
-  best.face_ms = best.update_ms = best.edge_ms = HUGE_VAL;
+  harmrad_tuning cand[ncand];
+  cand[0] = orig;
+  for (int i = 1; i < ncand; ++i) {
+    harmrad_tuning& t = cand[i];
+    t = orig;
+    t.face_block = fc[i - 1].block;
+    t.face_blocks_per_sm = fc[i - 1].cap;
+    t.update_block = uc[i - 1].block;
+    t.update_blocks_per_sm = uc[i - 1].cap;
+    t.newton_split = uc[i - 1].split;
+    t.edge_block = ec[i - 1].block;
+    t.edge_blocks_per_sm = ec[i - 1].cap;
+  }
+  for (harmrad_tuning& t : cand) t.face_ms = t.update_ms = t.edge_ms = HUGE_VAL;
   int rc = HARMRAD_OK;
   if (cudaMemcpyAsync(save, c->P, bytes, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess) rc = HARMRAD_E_CUDA;
   for (int it = -1; it < reps * ncand && rc >= 0; ++it) {
-    harmrad_tuning t = orig;
-    if (it >= 0) {  // it = -1: one untimed step loads every kernel
-      int i = it % ncand;
-      t.face_block = fc[i].block;
-      t.face_blocks_per_sm = fc[i].cap;
-      t.update_block = uc[i].block;
-      t.update_blocks_per_sm = uc[i].cap;
-      t.newton_split = uc[i].split;
-      t.edge_block = ec[i].block;
-      t.edge_blocks_per_sm = ec[i].cap;
-    }
+    harmrad_tuning& t = cand[it < 0 ? 0 : it % ncand];  // it = -1: one untimed step loads every kernel
     c->tune = t;
     harmrad_kernel_times kt;
     rc = harmrad_profile_step(c, 0.0, &kt);
@@ -1106,19 +1103,26 @@ int harmrad_autotune(harmrad_ctx* c, int reps, harmrad_tuning* out) {
       break;
     }
     if (it < 0) continue;
-    if (kt.ms[HARMRAD_K_FACE] < best.face_ms) {
-      best.face_ms = kt.ms[HARMRAD_K_FACE];
+    t.face_ms = fmin(t.face_ms, kt.ms[HARMRAD_K_FACE]);
+    t.update_ms = fmin(t.update_ms, kt.ms[HARMRAD_K_UPDATE]);
+    t.edge_ms = fmin(t.edge_ms, kt.ms[HARMRAD_K_EDGE]);
+  }
+  harmrad_tuning best = cand[0];
+  for (int i = 1; i < ncand; ++i) {
+    const harmrad_tuning& t = cand[i];
+    if (t.face_ms < best.face_ms && t.face_ms < 0.99 * cand[0].face_ms) {
+      best.face_ms = t.face_ms;
       best.face_block = t.face_block;
       best.face_blocks_per_sm = t.face_blocks_per_sm;
     }
-    if (kt.ms[HARMRAD_K_UPDATE] < best.update_ms) {
-      best.update_ms = kt.ms[HARMRAD_K_UPDATE];
+    if (t.update_ms < best.update_ms && t.update_ms < 0.99 * cand[0].update_ms) {
+      best.update_ms = t.update_ms;
       best.update_block = t.update_block;
       best.update_blocks_per_sm = t.update_blocks_per_sm;
       best.newton_split = t.newton_split;
     }
-    if (kt.ms[HARMRAD_K_EDGE] < best.edge_ms) {
-      best.edge_ms = kt.ms[HARMRAD_K_EDGE];
+    if (t.edge_ms < best.edge_ms && t.edge_ms < 0.99 * cand[0].edge_ms) {
+      best.edge_ms = t.edge_ms;
       best.edge_block = t.edge_block;
       best.edge_blocks_per_sm = t.edge_blocks_per_sm;
     }

@@ -41,4 +41,7 @@ inline int grid_for(long long work, int sms, int block, int per_sm = 16) {
   return (int)g;
 }
 
+// No more zones than one wave of the heavy kernels (2 blocks of 128 threads per SM).
+inline bool small_grid(long long nact, int sms) { return nact <= 256LL * sms; }
+
 }  // namespace hr

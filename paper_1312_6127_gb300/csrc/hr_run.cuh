@@ -52,6 +52,16 @@ inline Bufs make_bufs(harmrad_ctx* c) {
   return b;
 }
 
+// Threads per block of a heavy kernel's launch: the tuned number, but at most
+// `small` in a grid that does not fill one wave, whose blocks of one or two warps
+// spread over all SMs and schedulers (per RK3 step with 32 and 128 threads, the
+// reconstruction with 64 and 256: 32x32x32 box update 0.417, 0.458, reconstruction
+// 0.079, 0.086 ms; 64x32x16 torus 0.567, 0.620 and 0.188, 0.217; 64 and 128 threads
+// lie between, or within 7 % on either side).
+inline int fit_block(const harmrad_ctx* c, int block, int small) {
+  return small_grid(c->nact, c->sms) && block > small ? small : block;
+}
+
 // Largest per-grid count, and the work of all grids (the kernels deal the grids'
 // items to the threads as one sequence, first_item), for sizing a launch.
 template <typename Fn>
@@ -243,7 +253,7 @@ int faces_impl(harmrad_ctx* c, bool fresh) {
     }
   }
   const harmrad_tuning& tu = c->tune;
-  const int be = tu.edge_block, bf = tu.face_block;
+  const int be = fit_block(c, tu.edge_block, 64), bf = fit_block(c, tu.face_block, 32);
   FlatSet fl;
   for (int d = 0; d < 3; ++d) fl.f[d] = (double*)c->flat[d];
   auto faces_of = [c](int d) {
@@ -363,7 +373,7 @@ int solve_impl(harmrad_ctx* c, int stage, const ImexStage& im) {
   if (cudaMemsetAsync(c->failed, 0, c->nact, st) != cudaSuccess) return HARMRAD_E_CUDA;
   mark(c, HARMRAD_K_OTHER);
   Bufs b = make_bufs(c);
-  const int bu = c->tune.update_block;
+  const int bu = fit_block(c, c->tune.update_block, 32);
   const int gu = grid_for(c->nact, c->sms, bu, c->tune.update_blocks_per_sm);
   const int split = c->tune.newton_split;
   const bool one = c->nbox == 1;

@@ -1,0 +1,49 @@
+"""The autotuner against the shapes that the context had: no kernel class is
+slower with the chosen ones.  Best of five steps on either side, after one
+untimed; two such minima of one shape differ by less than 1 %, the tuner may take
+a shape 1 % slower on such a timing, and as much again is left: 3 %."""
+import pytest
+
+from paper_1312_6127_gb300 import harmrad as H
+from paper_1312_6127_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def torus(n):
+    cfg, P = W.torus(n, seed=12345)
+    return H.Grid(cfg), P
+
+
+def batch():
+    cfgs, Ps, Ks = W.box_batch(8, seed=5, edge=(24, 64))
+    b = H.Batch(cfgs)
+    b.set_opacity_field(Ks)
+    return b, Ps
+
+
+CASES = {"small torus": lambda: torus((64, 32, 16)), "torus": lambda: torus((128, 64, 32)), "batch": batch}
+
+
+@pytest.mark.parametrize("case", list(CASES))
+def test_tuned_classes_are_no_slower(case):
+    g, P = CASES[case]()
+
+    def times(shape):
+        g.set_tuning(**shape)
+        best = {}
+        for i in range(6):
+            g.set_prims(P)
+            kt = g.profile_step()
+            for k in ("face", "update", "edge"):
+                if i > 0:
+                    best[k] = min(best.get(k, 1e9), kt[k][0])
+        return best
+
+    g.set_prims(P)
+    before = g.tuning()
+    after = g.autotune(reps=2)
+    a, b = times(before), times(after)
+    print(case, before, after, a, b)
+    for k in a:
+        assert b[k] <= 1.03 * a[k], (k, a[k], b[k])
