@@ -337,21 +337,22 @@ void prim_to_cons(const orc_params& p, const Geom& G, const double Gam[4][4][4],
 // Lab-frame characteristic speeds along direction d for a fluid with
 // 4-velocity u and rest-frame signal speed^2 c2 (Sec. 4.4): the covector
 // k_mu = delta^d_mu - v delta^t_mu must satisfy (k.u)^2 = c2 (k.k + (k.u)^2).
-// In extended precision: for small c2 (cold gas, optically thick radiation) the
-// discriminant is c2 times a number of order one, left over from terms of
-// order one, and loses -log10(c2) digits.
+// In w = v - u^d/u^t (k.u = -w u^t there) it reads a w^2 + 2 c2 b w - c2 N = 0
+// with a = (1 - c2) (u^t)^2 - c2 g^{tt}, b = g^{td} - v0 g^{tt} and N the
+// square of k at v0 = u^d/u^t: every term carries its c2, so that small c2 (cold
+// gas, optically thick radiation) costs no digits, as the roots in v itself do.
 void char_speeds(const Geom& G, const double ucon[4], double c2, int d, double* vmin,
                  double* vmax) {
-  const long double Au = ucon[d], Bu = ucon[0];
-  const long double AA = G.gcon[d][d], BB = G.gcon[0][0], AB = G.gcon[0][d];
-  const long double qa = Bu * Bu - c2 * (BB + Bu * Bu);
-  const long double qb = -2.0L * (Au * Bu - c2 * (AB + Au * Bu));
-  const long double qc = Au * Au - c2 * (AA + Au * Au);
-  long double disc = qb * qb - 4.0L * qa * qc;
-  if (disc < 0.0L) disc = 0.0L;
-  const long double sd = std::sqrt(disc);
-  const double v1 = (double)((-qb + sd) / (2.0L * qa));
-  const double v2 = (double)((-qb - sd) / (2.0L * qa));
+  const double gdd = G.gcon[d][d], gtt = G.gcon[0][0], gtd = G.gcon[0][d];
+  const double v0 = ucon[d] / ucon[0];
+  const double a = (1.0 - c2) * ucon[0] * ucon[0] - c2 * gtt;
+  const double b = gtd - v0 * gtt;
+  const double N = gdd - v0 * (2.0 * gtd - v0 * gtt);
+  double disc = c2 * (c2 * b * b + N * a);
+  if (disc < 0.0) disc = 0.0;
+  const double s = std::sqrt(disc);
+  const double v1 = v0 + (s - c2 * b) / a;
+  const double v2 = v0 - (s + c2 * b) / a;
   *vmax = std::max(v1, v2);
   *vmin = std::min(v1, v2);
 }
