@@ -304,7 +304,11 @@ int harmrad_zone_physics(const harmrad_params* p, int n, const double* x, const 
  * explicit entropy: PMHD, URAD, PRAD, then the cold-MHD equations for a cold,
  * momentum-dominated zone.  The grid step then replaces a cold-MHD zone's u_g
  * by its neighbours' average; a single zone has no neighbours, so Pout keeps
- * the solve's u_g (the guess's). */
+ * the solve's u_g (the guess's).  The PMHD residual is evaluated term by term,
+ * as in a split-precision step; an FP64 step arranges the same sums otherwise, so
+ * that a zone whose error ends within round-off of a method's threshold can come
+ * out of the step by another method than here (about one retried zone in a
+ * hundred; both lie as close to the equations). */
 int harmrad_zone_implicit(const harmrad_params* p, int n, const double* x, const double* Ustar,
                           const double* Ps, const double* h, double* Pout, double* eT, int* iters,
                           unsigned char* method, void* stream);
