@@ -6,12 +6,12 @@
 // (PTX rcp.approx.ftz.f64, rsqrt.approx.ftz.f64: about 20 bits, computed off the
 // FP64 pipe) takes one step of the cubically convergent iteration for 1/x
 // (y (1 + e + e^2), e = 1 - x y) or 1/sqrt(x) (y (1 + e/2 + 3 e^2/8),
-// e = 1 - x y^2; Householder's family), which leaves 2^-60 of truncation:
-// below the rounding of the last operation (sqrt(x) = x y + x y q with one
-// rounding of the sum, y q the correction).  1/x costs 3 FP64 instructions,
-// 1/sqrt(x) 5, sqrt(x) 7, both together 8.  Measured over 4 million arguments
-// between 2^-1020 and 2^1020 against extended precision: largest error 0.507
-// ulp, mean 0.25, as the library's rsqrt.  Arguments outside the range where
+// e = 1 - x y^2; Householder's family), which leaves e^3 and 5 e^3/16 of
+// truncation, 2^-60 and 2^-58.7 for |e| of 2^-20 and 2^-19: below the rounding of
+// the last operation (sqrt(x) = x y + x y q with one rounding of the sum, y q the
+// correction).  1/x costs 3 FP64 instructions, 1/sqrt(x) 5, sqrt(x) 7, both
+// together 8.  Largest errors over a million arguments of every exponent, against
+// extended precision: 1/x 0.504 ulp, 1/sqrt(x) 0.505, sqrt(x) 0.515.  Arguments outside the range where
 // the seed and the residual are normal numbers (zero, subnormal, infinite,
 // NaN, negative under the root, above 2^1022) go to the language's operation.
 #pragma once
