@@ -4,10 +4,12 @@
 // inside each, the operations of the sub-step in reverse: implicit solve,
 // explicit update, flux-CT, Riemann fluxes, reconstruction, flattener, cell
 // factors and ghost fill.  Each kernel applies the transpose of its forward
-// operation's local Jacobian to the incoming cotangent; the local Jacobians
-// come from evaluating the forward device functions on dual numbers (Dn<N>),
-// so every branch (limiters, wave-speed maxima, flattener clamps) takes the
-// derivative of the branch the forward step took.
+// operation's local Jacobian to the incoming cotangent along the branches
+// (limiters, wave-speed maxima, flattener clamps) that the forward step took:
+// by a reverse sweep written out by hand for the fluxes, the reconstruction,
+// the explicit update and the implicit solve; by evaluating the forward device
+// functions on dual numbers (Dn<N>) for the flattener, the cell factors, the
+// floors where one acts, and the zones that the entropy equation solved.
 //
 // The implicit solve is differentiated through its solution, not through the
 // Newton iterations (implicit-function theorem): at the root x* of the PMHD
@@ -43,7 +45,7 @@ struct AdjBufs {
   double* gemf;         // [ntot] cotangent of the edge EMFs of one pair of directions
   double* gk;           // [1] cotangent of kappa_scale
   // the entropy (Sec. 2, Eq. S), for zones solved by the entropy equation
-  double* Sst;          // [3][nact] explicit entropy S* of every zone and sub-step
+  double* Sst;          // [3][nact] explicit entropy S* of the zones whose retry read it (valid where meth is 3)
   double* gS;           // [nact] cotangent of S*
   double* gSn;          // [nact] cotangent of S^n, the step's initial conserved entropy
   double* gXS;          // [nact] cotangent of the entropy's explicit rate X_S = -div F_S

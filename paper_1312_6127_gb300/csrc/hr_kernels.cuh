@@ -31,7 +31,7 @@ struct Bufs {
   void* spd[3];    // [ntot] per-face max signal speed
   void* aux;       // [10][ntot] per-cell gdet, sqrt(-g) u^d gas/rad, tau weights
   void* flat[3];   // [2][ntot] flattener, max over the sub-steps of the step
-  void* emf;       // [ntot] edge EMF scratch
+  void* emf;       // [3][ntot] edge EMFs of the pairs of directions
   double* dt;      // [nbox] time step of each grid
   unsigned char* status;  // [nact] worst outcome over the sub-steps
   int* iters;             // [nact] Newton steps summed over the sub-steps
@@ -55,7 +55,7 @@ struct Bufs {
   double* ust_rec;            // [12][nact] U* of every zone of the sub-step
   unsigned char* meth_rec;    // [nact] outcome of every zone of the sub-step
   double* psol_rec;           // [12][nact] solution of every zone before the floors
-  double* sst_rec;            // [nact] explicit entropy S* of every zone of the sub-step
+  double* sst_rec;            // [nact] explicit entropy S* of the zones whose retry read it in the sub-step
   double* imexM;              // IMEX: [4 stages][4 gas rows][nact] per grid, grid b at 16 aoff_b
   double* Bf[3];              // staggered field: sqrt(-g) B^d on the d-faces [ntot] (null: flux-CT)
 };
@@ -529,14 +529,14 @@ __global__ void k_flatten(DevParams p, const BoxGeo* __restrict__ boxes, int nbo
 // the wider difference only where the jump is a shock.  About 12 FP64
 // instructions per cell where nothing compresses.  `fresh`: the first sub-step
 // (no earlier value to keep).  Measured over an RK3 step: 256x128x64 torus
-// 3.05 -> 1.38 ms, 64x32x16 0.18 -> 0.10 ms.
+// 3.05 -> 1.38 ms, 64x32x16 0.18 -> 0.10.
 
-// f(m) from the jump dp across the cell, the blended pressures pp, pm beside it
-// and the wider jump d2.
+// f(m) from the jump dp across the cell and the wider jump d2.
 __device__ __forceinline__ double flat_value(double dp, double d2) {
   const double f = d2 != 0.0 ? 10.0 * (dp / d2 - 0.75) : -7.5;
   return f < 0.0 ? 0.0 : (f > 1.0 ? 1.0 : f);
 }
+// The jump dp is a shock beside the blended pressures pp, pm.
 __device__ __forceinline__ bool flat_shock(double dp, double pp, double pm) {
   return fabs(dp) > 0.33 * (pp < pm ? pp : pm);
 }
@@ -768,9 +768,10 @@ __device__ __forceinline__ void ppm_cell(const R s[5], R chi, R* aL, R* aR) {
 // FP64 reconstruction of one direction: the PPM parabola (or MC line) of every
 // primitive in every cell of the face range (cells -1..n_d along d, transverse
 // range widened by one layer), flattened by the cell's GAS or RAD flattener and
-// stored as its two edge values (EdgeSet); the face kernel reads the upper edge of cell f-1 and the lower edge of cell f.  In r
-// and phi on the Kerr-Schild grid the velocity and field components are
-// reconstructed as sqrt(-g) times the primitive (Sec. 4.3).
+// stored as its two edge values (EdgeSet); the face kernel reads the upper edge
+// of cell f-1 and the lower edge of cell f.  In r and phi on the Kerr-Schild grid
+// the velocity and field components are reconstructed as sqrt(-g) times the
+// primitive (Sec. 4.3).
 //
 // Bound by FP64 instructions (each holds an SM's FP64 pipe for 16 clocks), so
 // nothing is computed twice: neighbouring cells share the difference, the MC
@@ -778,12 +779,12 @@ __device__ __forceinline__ void ppm_cell(const R s[5], R chi, R* aL, R* aR) {
 // them in registers, or, along x1, a warp passes them between its lanes), and
 // the limiters work on differences: with a = |r - q|, b = |q - l| the
 // monotonicity tests of Colella & Woodward read b > 2 a and a > 2 b, and twice
-// the MC slope is min(|dl + dr|, 4 |dl|, 4 |dr|).  About 14 FP64 instructions
+// the MC slope is min(|dl + dr|, 4 |dl|, 4 |dr|).  About 11 FP64 instructions
 // per cell and variable.  One thread (or warp) takes one variable: few
 // registers, many warps, and small grids still fill the SMs.  Measured over an
-// RK3 step (GB300, PPM, Kerr-Schild, event time of the class): 256x128x64
-// 17.2 -> 10.7 ms, 64x32x16 0.75 -> 0.36 ms, 256 zones in 1D 125 -> 27 us,
-// against a slope pass plus a parabola pass of one thread per cell.
+// RK3 step (GB300, PPM, event time of the class) against a slope pass plus a
+// parabola pass of one thread per cell: Kerr-Schild torus 256x128x64 17.2 -> 7.8
+// ms, 64x32x16 0.75 -> 0.19, 256 zones in 1D 0.125 -> 0.024.
 
 // The limiters' comparisons and powers of two act on the bit patterns, off the
 // FP64 pipe: twice a double's bits (the sign shifted out) order like its
@@ -791,7 +792,8 @@ __device__ __forceinline__ void ppm_cell(const R s[5], R chi, R* aL, R* aR) {
 __device__ __forceinline__ unsigned long long mag_key(double x) {
   return (unsigned long long)__double_as_longlong(x) << 1;
 }
-// |a| < 2^k |b|, for normal numbers and zero
+// |a| < 2^k |b|, for normal numbers and zero (a subnormal b counts as up to
+// 2^(k-1022); a slope limited by it is off by that much at most)
 __device__ __forceinline__ bool mag_less(double a, double b, int k = 0) {
   return mag_key(a) < mag_key(b) + ((unsigned long long)k << 53);
 }
@@ -1090,7 +1092,7 @@ __global__ void __launch_bounds__(256) k_edges(DevParams p, const BoxGeo* __rest
 // reconstructed states: both states' gas and radiation signal speeds, then
 // HLL or LAXF (Eqs. hll, lax), the gas and radiation groups with their own
 // speeds; F[B_d] = 0.  smax: the largest signal speed (for the CFL step).
-// Used by the face kernel and, on dual numbers, by the adjoint.
+// Split precision's face kernel (FP64: face_flux64).
 template <int MET, typename R, int d>
 __device__ __forceinline__ void face_flux(const DevParams& p, const Geo<MET, R>& g, R dxd, R kL, R kR, R ks,
                                           const R PL[NPR], const R PR[NPR], R out[NPR], R* smax,
@@ -2242,9 +2244,11 @@ __device__ int backup_equations(const DevParams& p, const Geo<MET, double>& g, c
 // (Sec. 4.7, 4.11), few in any run, or by all zones in the entropy-everywhere
 // mode.  Two logarithms per face were a quarter of the face kernel when every
 // face formed its flux (256x128x64 torus, per RK3 step: faces 17.4 -> 13.8 ms,
-// update 21.7 -> 20.5 ms without, at the launch shapes of then); the face kernel now keeps the left state's mass flux
-// mL, and the flux is s_L mL + s_R (F_rho - mL) with the entropy per baryon s
-// of the kept edges (Sec. 2, Eq. S).
+// update 21.7 -> 20.5 ms without, at 16 blocks per SM); the face kernel keeps the
+// left state's mass flux mL, and the flux is s_L mL + s_R (F_rho - mL) with the
+// entropy per baryon s of the kept edges (Sec. 2, Eq. S).  The mode that reads it
+// everywhere forms each face's flux from either side and still gains with the rest
+// (128x64x32 torus, step: 16.9 -> 11.2 ms).
 static __device__ __forceinline__ double entropy_flux(const DevParams& p, const BoxGeo& bx, const Bufs& b, int d,
                                                       long long t) {
   const double* S = b.ES[d] + 4 * bx.coff;

@@ -11,9 +11,10 @@
 // the last operation (sqrt(x) = x y + x y q with one rounding of the sum, y q the
 // correction).  1/x costs 3 FP64 instructions, 1/sqrt(x) 5, sqrt(x) 7, both
 // together 8.  Largest errors over a million arguments of every exponent, against
-// extended precision: 1/x 0.504 ulp, 1/sqrt(x) 0.505, sqrt(x) 0.515.  Arguments outside the range where
-// the seed and the residual are normal numbers (zero, subnormal, infinite,
-// NaN, negative under the root, above 2^1022) go to the language's operation.
+// extended precision: 1/x 0.504 ulp, 1/sqrt(x) 0.505, sqrt(x) 0.515.  Arguments
+// outside the range where the seed and the residual are normal numbers (zero,
+// subnormal, infinite, NaN, negative under the root, above 2^1022) go to the
+// language's operation.
 #pragma once
 #include <cuda_runtime.h>
 

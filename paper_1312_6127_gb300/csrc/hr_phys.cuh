@@ -431,15 +431,7 @@ __device__ __forceinline__ void face_speeds(const DevParams& p, const Geo<MET, R
   const R rho = P[RHO], ug = P[UU];
   const R pg = R(p.gam - 1.0) * ug;
   const R w = rho + ug + pg;
-  R cs2, va2;
-  if constexpr (std::is_same<R, double>::value) {  // one division (w^2 stays in FP64's range)
-    const R iw = R(1) / (w * (w + bsq));
-    cs2 = R(p.gam) * pg * (w + bsq) * iw;
-    va2 = bsq * w * iw;
-  } else {
-    cs2 = R(p.gam) * pg / w;
-    va2 = bsq / (w + bsq);
-  }
+  const R cs2 = R(p.gam) * pg / w, va2 = bsq / (w + bsq);
   R cms2 = cs2 + va2 - cs2 * va2;
   if (code) *code = (cms2 > R(1) ? 1u : 0u) | (cms2 < R(0) ? 2u : 0u);
   cms2 = cms2 > R(1) ? R(1) : (cms2 < R(0) ? R(0) : cms2);
@@ -518,7 +510,7 @@ __device__ __forceinline__ void face_accum(const DevParams& p, const Geo<MET, R>
 // ------------------------------------------------- FP64 face (hot path)
 // The Riemann flux of one face in FP64, arranged for few FP64 instructions
 // (face_speeds and face_accum above state the same physics term by term and
-// serve FP32 and the adjoint's dual numbers).  With l_i = g_ij u~^j = u_i (the
+// serve FP32).  With l_i = g_ij u~^j = u_i (the
 // ZAMO's n_i vanish): gamma^2 = 1 + u~^i l_i and u_t = -alpha gamma + beta^i l_i,
 // beta^i = alpha^2 g^{ti}; likewise B_mu from m_i = g_ij B^j.  With
 // b_mu = (B_mu + b^t u_mu) / u^t a state's share aF F^d + aU U of every gas row
