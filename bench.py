@@ -227,6 +227,23 @@ def make_context(args, H, W, workload, prec, stream, rank, integ):
     return g, g.nact, wl, ("batch48", "batch48_" + pname)
 
 
+def tune(g, args, workload):
+    """Launch shapes for the state that is timed: a batch's solves settle within
+    its first steps, and the best Newton split with them (update of the 48 boxes
+    per step with a split of 6 and 5: 557 and 572 ms at first, 370 and 322
+    later), so it is tuned after the warm-up steps and then set back."""
+    if args.no_autotune:
+        return g.tuning()
+    if workload != "batch48":
+        return g.autotune(reps=1)
+    P = g.get_prims(device=True)
+    for _ in range(args.warmup):
+        g.step(0.0)
+    shapes = g.autotune(reps=1)
+    g.set_prims(P)
+    return shapes
+
+
 def time_steps(g, args, stream, dist, local):
     """W warm-up steps, then K timed CUDA-graph steps bracketed by a barrier
     and a synchronize; clocks sampled during the timed region."""
@@ -383,7 +400,7 @@ def main():
     integ = INTEGRATORS[args.integrator]
     peak_tf, peak_note = fp64_peak(H)
     g, nact, wl, key = make_context(args, H, W, args.workload, prec, stream, rank, integ)
-    tuning = g.tuning() if args.no_autotune else g.autotune(reps=1)
+    tuning = tune(g, args, args.workload)
     ms, clk = time_steps(g, args, stream, dist, local)
     ms = job_time_ms(ms, dist, "cuda")
     st = g.stats()
@@ -421,7 +438,7 @@ def main():
         for name, wk, pr in (("split", "torus", H.PREC_SPLIT), ("batch48", "batch48", H.PREC_FP64),
                              ("uct", "torus_uct", H.PREC_FP64)):
             gx, nx, wlx, keyx = make_context(args, H, W, wk, pr, stream, rank, integ)
-            tx = gx.tuning() if args.no_autotune else gx.autotune(reps=1)
+            tx = tune(gx, args, wk)
             msx, clkx = time_steps(gx, args, stream, None, local)
             stx = gx.stats()
             sub = {"value": job_throughput(nx, args.steps, 1, msx), "unit": UNIT,

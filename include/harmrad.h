@@ -469,7 +469,8 @@ typedef struct harmrad_tuning {
   double face_ms, update_ms, edge_ms;      /* autotune: best device ms per step */
 } harmrad_tuning;
 
-/* Autotune the launch shapes on the context's current state: time `reps`
+/* Autotune the launch shapes on the context's current state (the best split
+ * follows the solves: tune on a state like those to come): time `reps`
  * eager steps (dt <= 0: CFL) for each candidate shape, with CUDA events on the
  * context's stream, keep the fastest per kernel class (the current one unless
  * another is 1 % faster), restore the primitives and drop the captured graphs
