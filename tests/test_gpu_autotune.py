@@ -1,5 +1,5 @@
 """The autotuner against the shapes that the context had: no kernel class is
-slower with the chosen ones.  Best of five steps on either side, after one
+slower with the chosen ones.  Best of ten steps on either side, in turn, after one
 untimed; two such minima of one shape differ by less than 1 %, the tuner may take
 a shape 1 % slower on such a timing, and as much again is left: 3 %."""
 import pytest
@@ -29,21 +29,18 @@ CASES = {"small torus": lambda: torus((64, 32, 16)), "torus": lambda: torus((128
 def test_tuned_classes_are_no_slower(case):
     g, P = CASES[case]()
 
-    def times(shape):
-        g.set_tuning(**shape)
-        best = {}
-        for i in range(6):
+    g.set_prims(P)
+    before = g.tuning()
+    after = g.autotune(reps=2)
+    a, b = {}, {}
+    for i in range(11):
+        for shape, best in ((before, a), (after, b)):
+            g.set_tuning(**shape)
             g.set_prims(P)
             kt = g.profile_step()
             for k in ("face", "update", "edge"):
                 if i > 0:
                     best[k] = min(best.get(k, 1e9), kt[k][0])
-        return best
-
-    g.set_prims(P)
-    before = g.tuning()
-    after = g.autotune(reps=2)
-    a, b = times(before), times(after)
     print(case, before, after, a, b)
     for k in a:
         assert b[k] <= 1.03 * a[k], (k, a[k], b[k])
